@@ -62,15 +62,20 @@ plan_kernel(const int32_t* __restrict__ offs, int G, int N, int rows_per_item, i
         }
         __syncthreads();
         const int base = s_carry + (wid ? s_warp[wid - 1] : 0) + incl - tiles;
-        for (int t = 0; t < tiles; ++t) {
-            if (base + t < max_items) {
+        // a warp writes the items of its 32 graphs together, 32 items a step: one thread that wrote all items of a
+        // large graph by itself took 20 us for 782 of them and 31 us for 977 (now 3 to 4)
+        for (unsigned left = __ballot_sync(0xFFFFFFFFu, tiles > 0); left; left &= left - 1u) {
+            const int src = __ffs(left) - 1;
+            const int g_lo = __shfl_sync(0xFFFFFFFFu, lo, src), g_hi = __shfl_sync(0xFFFFFFFFu, hi, src);
+            const int g_base = __shfl_sync(0xFFFFFFFFu, base, src), g_tiles = __shfl_sync(0xFFFFFFFFu, tiles, src);
+            for (int t = lane; t < g_tiles && g_base + t < max_items; t += 32) {
                 WorkItem it;
-                it.row0 = lo + t * rows_per_item;
-                it.nrows = min(rows_per_item, hi - it.row0);
-                it.key_lo = lo;
-                it.key_hi = hi;
-                it.tile0 = lo / 128 + g;
-                items[base + t] = it;
+                it.row0 = g_lo + t * rows_per_item;
+                it.nrows = min(rows_per_item, g_hi - it.row0);
+                it.key_lo = g_lo;
+                it.key_hi = g_hi;
+                it.tile0 = g_lo / 128 + g - lane + src;
+                items[g_base + t] = it;
             }
         }
         __syncthreads();
