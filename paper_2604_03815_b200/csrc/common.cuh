@@ -35,6 +35,8 @@ struct Canaries {
     int n = 0;
 };
 
+constexpr int kRedoSplitMax = 48;
+
 struct StatusBlock {
     int status;      // kmip_status_t recorded by the device (first error wins)
     int detail;      // where it happened (kernel-specific code)
@@ -44,7 +46,8 @@ struct StatusBlock {
     // (key tile, query tile) pairs, pairs scored - summed over the CTAs (kmip_attn_sweep_counters)
     unsigned long long counters[4];
     int n_redo;      // forward, fp16 prefilter: rows the rescoring kernel sent to the exact kernel
-    int reserved[51];
+    int redo_done[kRedoSplitMax];  // parts finished of each of the first redo rows (score_select_exact.cu)
+    int reserved[51 - kRedoSplitMax];
 };
 static_assert(sizeof(StatusBlock) == kStatusBytes, "status block size");
 

@@ -120,3 +120,15 @@ def test_rows_with_one_dominant_and_many_tiny_queries():
     w = wl.iid_workload("s", 5400, [4000], 2, 32, 16, wl.MODE_BF16_TC, input_scale=1.0 / np.sqrt(32.0))
     w.Q[17] = wl.round_to_bf16(w.Q[17] * np.float32(1e6))
     _check(w, 0.95)
+
+
+@pytest.mark.parametrize("n_tied,k", [(1, 32), (5, 8), (48, 16), (60, 32), (1300, 16)])
+def test_few_undecidable_rows(n_tied, k):
+    """`n_tied` queries score equally on hundreds of keys (zero vectors: every score is 0), the others do not: from one
+    row that the whole grid shares, over the most rows that are cut into parts, to a block and to a warp per row."""
+    N, H, d = 2900, 1, 32
+    w = wl.iid_workload("s", 5500 + n_tied + k, [N], H, d, k, wl.MODE_BF16_TC, input_scale=1.0 / np.sqrt(32.0))
+    rows = (np.arange(n_tied) * 2) % N
+    w.Q[rows] = 0.0
+    st = _check(w, 0.98)
+    assert st["redo"] == n_tied
