@@ -365,12 +365,11 @@ int kmip_test_gemm_tn(const void* A, const void* B, void* C, int32_t M, int32_t 
     if (workspace_bytes < kStatusBytes) return KMIP_ERR_WORKSPACE;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     if (cudaMemsetAsync(workspace, 0, kStatusBytes, st) != cudaSuccess) return KMIP_ERR_CUDA;
-    const void* As[3] = {A, A, A};
-    const void* Bs[3] = {B, B, B};
-    void* Cs[3] = {C, C, C};
-    if (launch_gemm_tn(As, K, Bs, K, Cs, nullptr, 1, 1, M, N, K, N, 0, 0, 0, 0, out_f32 != 0, static_cast<StatusBlock*>(workspace),
-                       st) != cudaSuccess)
-        return KMIP_ERR_CUDA;
+    GemmCall g{};
+    g.A[0] = A; g.B[0] = B; g.C[0] = C;
+    g.M = M; g.N = N; g.K = K; g.lda = g.ldb = K; g.ldc = N;
+    g.out_f32 = out_f32 != 0;
+    if (launch_gemm(g, static_cast<StatusBlock*>(workspace), st) != cudaSuccess) return KMIP_ERR_CUDA;
     return KMIP_OK;
 }
 

@@ -359,10 +359,26 @@ cudaError_t launch_softmax_gather(const FwdArgs& a);
 // ev (optional): three events recorded after the rows, inverse-index and segment stages
 cudaError_t launch_backward(const BwdArgs& a, const BwdWorkspace& w, cudaEvent_t* ev);
 
-// gemm_tn.cu: C = scale * A B^T on the tensor cores (bf16 operands with K contiguous, fp32 accumulation); see there
-cudaError_t launch_gemm_tn(const void* const* A, int lda, const void* const* B, int ldb, void* const* C, const float* scale,
-                           int n_batch, int n_kseg, int M, int N, int K, int ldc, int row_pad, int row_real, int col_pad,
-                           int col_real, bool out_f32, StatusBlock* sb, cudaStream_t stream);
+// gemm_tn.cu: C_z = A_z B_z^T on the tensor cores (bf16 operands, fp32 accumulation); see there
+struct GemmCall {
+    const void *A[4], *B[4];
+    void* C[4];
+    int M, N, K, lda, ldb, ldc;
+    bool a_mn = false, b_mn = false;  // stored [K, M] / [K, N] instead of [M, K] / [N, K]
+    bool out_f32 = false;
+    int n_batch = 1, n_kseg = 1, n_split = 1;
+    const StatusBlock* merge_from = nullptr;  // a device-side problem recorded there is copied into the call's status block
+};
+cudaError_t launch_gemm(const GemmCall& g, StatusBlock* sb, cudaStream_t stream);
+// parts of the K axis for a split launch whose partial sums have to fit `partial_bytes`
+int gemm_splits(int M, int N, int K, int n_batch, size_t partial_bytes);
+struct ReduceOut {
+    void* dst[4];
+    float scale[4];
+    int transposed[4];
+};
+cudaError_t launch_reduce_partials(const float* partial, int n_split, int M, int N, int pad, int real, int n_batch, const ReduceOut& out,
+                                   cudaStream_t stream);
 
 // layer.cu: the full layer of Eq. 2 (bf16).  All pointers are device memory.
 struct LayerArgs {
@@ -381,10 +397,9 @@ struct LayerArgs {
     cudaStream_t stream;
 };
 struct LayerWorkspace {
-    size_t wq_pad, wk_pad, wv_pad, wo_pad;         // padded weights
-    size_t wqT, wkT, wvT, woT;                     // their transposes (backward)
+    size_t wq_pad, wk_pad, wv_pad, wo_pad;         // padded weights (unused when the head width needs no padding)
     size_t d_o, d_q, d_k, d_v;                     // [N, H*d_pad] gradients around the attention core
-    size_t xT, dyT, oT, dqT, dkT, dvT;             // transposed activations for the weight gradients
+    size_t partial, partial_bytes;                 // fp32 partial sums of the weight gradients
     size_t attn, attn_bytes;                       // workspace of the attention call
     size_t total;
 };

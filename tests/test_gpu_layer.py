@@ -136,3 +136,30 @@ def test_layer_calls_reject_bad_arguments():
     attn_b = kb.kmip_attn_workspace_bytes(100_000, 1, 4, 32, 16, kb.KMIP_BF16_TC, kb.PASS_BACKWARD)
     assert attn_f < f < attn_f + (1 << 20)                                          # + four padded weight copies
     assert attn_b + 10 * 100_000 * 128 * 2 <= b < attn_b + 10 * 100_008 * 128 * 2 + (1 << 21)   # + ten [N, 128] bf16 arrays
+
+
+@pytest.mark.parametrize("N,d_model,H,d_head", [(1, 8, 1, 16), (63, 72, 3, 10), (257, 264, 4, 64), (513, 64, 2, 128), (40001, 136, 4, 32)])
+def test_weight_gradient_partial_sums(N, d_model, H, d_head):
+    """dW_O = dY^T O with the node axis cut into parts (from one part to more than the SMs hold), operands read along
+    either axis, tiles ragged in every dimension, padded and unpadded heads: against fp64 on the saved O.  One bf16
+    rounding of the result (2^-8 relative to the largest element bounds it) and fp32 sums of N terms."""
+    from paper_2604_03815_b200 import binding as kb
+    g = torch.Generator().manual_seed(N + d_model)
+    bf = lambda *s: torch.randn(*s, generator=g).to(torch.bfloat16).cuda()
+    d_pad, k, inner = next(v for v in (16, 32, 64, 128) if v >= d_head), min(4, N), H * d_head
+    mk = lambda *s, dt=torch.bfloat16: torch.full(s, float("nan") if dt.is_floating_point else -7, dtype=dt, device="cuda")
+    t = {"x": bf(N, d_model), "w_q": bf(inner, d_model) * 0.1, "w_k": bf(inner, d_model) * 0.1, "w_v": bf(inner, d_model) * 0.1,
+         "w_o": bf(d_model, inner) * 0.1, "q": mk(N, H, d_pad), "k": mk(N, H, d_pad), "v": mk(N, H, d_pad), "o": mk(N, H, d_pad),
+         "topk_idx": mk(N, H, k, dt=torch.int32), "topk_score": mk(N, H, k, dt=torch.float32), "y": mk(N, d_model),
+         "d_y": bf(N, d_model), "d_x": mk(N, d_model), "dw_q": mk(inner, d_model), "dw_k": mk(inner, d_model),
+         "dw_v": mk(inner, d_model), "dw_o": mk(d_model, inner)}
+    offs = torch.tensor([0, N], dtype=torch.int32, device="cuda")
+    for pass_, fn in ((kb.PASS_FORWARD, kb.kmip_layer_forward), (kb.PASS_BACKWARD, kb.kmip_layer_backward)):
+        ws = torch.full((kb.kmip_layer_workspace_bytes(N, 1, d_model, H, d_head, k, pass_),), 0xFF, dtype=torch.uint8, device="cuda")
+        assert fn(t, offs, N, d_model, H, d_head, k, ws) == kb.KMIP_OK and kb.kmip_last_status(ws) == kb.KMIP_OK
+    o = t["o"][..., :d_head].reshape(N, inner).double()
+    for got, ref in ((t["y"], o @ t["w_o"].double().T), (t["dw_o"], t["d_y"].double().T @ o)):
+        assert float((got.double() - ref).abs().max()) <= 2.0 ** -8 * float(ref.abs().max()) + 1e-5 * np.sqrt(N)
+    assert all(torch.isfinite(t[n].float()).all() for n in ("d_x", "dw_q", "dw_k", "dw_v"))
+    q = t["x"].double() @ t["w_q"].double().T * np.sqrt(d_pad / d_head)
+    assert float((t["q"][..., :d_head].reshape(N, inner).double() - q).abs().max()) <= 2.0 ** -6 * float(q.abs().max())
