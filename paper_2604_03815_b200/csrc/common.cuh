@@ -90,7 +90,9 @@ struct FwdWorkspace {
     int max_tiles;
     int list;          // groups kept per row by the half-precision prefilter
     bool tc;           // a tensor-core sweep runs (bf16 storage and a supported (d, k))
-    bool f16;          // ... namely the half-precision prefilter (score_select_f16.cu)
+    bool f16;          // the half-precision prefilter runs (bf16: instead of that sweep; fp32: instead of the CUDA-core ones)
+    bool in_outputs;   // ... with its lists, the redo list and the operand copies that have no place here in the call's
+                       // output arrays, which nothing else uses until the last stages write them (f16_buffers)
     bool reorder;      // the sweep runs the rows of large graphs in locality order (reorder.cu)
     bool prune;        // the sweep skips key tiles that cannot hold a candidate (prune.cu)
     Canaries canaries;
@@ -100,9 +102,9 @@ constexpr int64_t kReorderMinNodes = 32768;  // below this the extra launches co
 
 bool score_select_tc_supported(int32_t d, int32_t k);
 bool score_select_f16_supported(int32_t d, int32_t k);
+bool score_select_f16_in_outputs_supported(int64_t N, int32_t H, int32_t d, int32_t k, int mode);
 int score_select_f16_list(int32_t k);
-int score_select_f16_rows_per_item(int32_t k);
-int score_select_f16x4_rows_per_item();
+int score_select_f16_list_in_outputs(int32_t k);
 
 // Which sweep the plan is for: the one the mode selects, or one a test entry point asks for.
 enum PlanVariant { kPlanByMode = 0, kPlanNoTensorCore = 1, kPlanTcFp32Acc = 2, kPlanTcFp16Acc = 3,
@@ -122,13 +124,15 @@ inline FwdWorkspace plan_fwd_workspace(int64_t N, int32_t G, int32_t H, int32_t 
                                   : variant != kPlanNoTensorCore;
     w.f16 = variant == kPlanByMode ? (w.tc && mode == KMIP_BF16_TC && score_select_f16_supported(d, k))
                                    : variant == kPlanTcFp16Acc;
-    w.list = w.f16 ? score_select_f16_list(k) : 0;
+    w.in_outputs = variant == kPlanByMode && !w.f16 && score_select_f16_in_outputs_supported(N, H, d, k, mode);
+    w.f16 = w.f16 || w.in_outputs;
+    w.list = w.in_outputs ? score_select_f16_list_in_outputs(k) : w.f16 ? score_select_f16_list(k) : 0;
     w.max_items = (int)(N / 128 + g + 1);
     w.items_off = region(kStatusBytes);
     w.kpack_off = region(w.items_off + sizeof(WorkItem) * (size_t)w.max_items);
     w.reorder = w.tc && N >= kReorderMinNodes && variant != kPlanTcFp32AccInOrder;
     w.qperm_off = region(w.kpack_off + (w.tc ? (size_t)N * H * d * 2 : 0));
-    w.perm_off = region(w.qperm_off + ((w.reorder || w.f16) ? (size_t)N * H * d * 2 : 0));
+    w.perm_off = region(w.qperm_off + ((w.reorder || (w.f16 && !w.in_outputs)) ? (size_t)N * H * d * 2 : 0));
     w.code_off = region(w.perm_off + (w.reorder ? (size_t)N * 4 : 0));
     w.prune = variant == kPlanByMode && mode == KMIP_BF16_TC_PRUNED && w.reorder;
     w.max_tiles = (int)(N / 128 + g + 2);  // tile0 of a graph = floor(first row / 128) + graph index
@@ -141,9 +145,9 @@ inline FwdWorkspace plan_fwd_workspace(int64_t N, int32_t G, int32_t H, int32_t 
     w.qnorm_off = region(w.gmax_off + p * (size_t)g * 4);
     w.qstat_off = region(w.qnorm_off + p * (size_t)N * H * 4);
     w.kstat_off = region(w.qstat_off + p * (size_t)w.max_items * 3 * H * rec);
-    const size_t f = w.f16 ? 1 : 0, rows = (size_t)N * H;
+    const size_t f = w.f16 && !w.in_outputs ? 1 : 0, rows = (size_t)N * H;
     w.f16stat_off = region(w.kstat_off + p * (size_t)w.max_tiles * H * rec);
-    w.cand_word_off = region(w.f16stat_off + f * 16 * (size_t)H);
+    w.cand_word_off = region(w.f16stat_off + (w.f16 ? 16 : 0) * (size_t)H);
     w.cand_half_off = region(w.cand_word_off + f * rows * w.list * 4);
     w.redo_off = region(w.cand_half_off + f * rows * w.list * 2);
     w.total = region(w.redo_off + f * rows * 4);  // checks builds: a last canary block behind the last region
@@ -326,6 +330,9 @@ cudaError_t launch_reorder_keys(const FwdArgs& a, const FwdWorkspace& w);
 // prune.cu: centroid / radius / norm statistics of every item's query rows and of every key tile
 cudaError_t launch_prune_stats(const FwdArgs& a, const FwdWorkspace& w);
 constexpr int kMinRowsToSort = 8192;  // smaller graphs keep their row and key order
+// fp32 mode: smallest N * H that runs the half-precision prefilter.  Its launches cost about 100 us, and one warp per row
+// takes 58 us at 1024 rows (one graph, d = 32), 167 at 2048 (filter: 114) and 601 at 4096 (150).
+constexpr int64_t kF16MinRowsFp32 = 1536;
 // score_select_exact.cu: CUDA-core scores + running top-k, any supported (d, k), fp32 or bf16 storage
 cudaError_t launch_score_select_exact(const FwdArgs& a);
 int sm_count();  // multiprocessors of the current device (cached per device)
@@ -334,12 +341,51 @@ int sm_count();  // multiprocessors of the current device (cached per device)
 int score_select_tc_rows_per_item(int32_t d, int32_t k);
 cudaError_t launch_score_select_tc(const FwdArgs& a, const FwdWorkspace& w);
 cudaError_t launch_score_dump_tc(const FwdArgs& a, const FwdWorkspace& w, float* dump);
-// Half-precision prefilter of the tensor-core mode, head widths 16 and 32, k <= 32:
-// f16_convert.cu (norm maxima, scaled fp16 copies of K and Q), score_select_f16.cu (sweep: 384-row work items),
+// Half-precision prefilter (k <= 32; bf16 storage: head widths 16, 32, 64, fp32 storage: the same on large problems):
+// f16_convert.cu (norm maxima, scaled fp16 copies of K and Q), score_select_f16.cu / score_select_f16x4.cu (sweeps),
 // refine_f16.cu (exact rescoring, redo list), score_select_exact.cu (the listed rows again, from all keys)
+
+// The groups a row kept: `slots` entries per (node, head) row, the group and the fp16 maximum of its scores.
+//   compact = 0  32-bit words (first key of the 16-key window, bit 31 = its odd keys)
+//   compact = 1  16-bit numbers inside the graph: 2 * window + (odd keys)
+struct GroupLists {
+    unsigned char* word;
+    unsigned char* half;
+    long long word_pitch, half_pitch;  // bytes from row to row
+    int slots, compact;
+};
+struct F16Buffers {
+    void *k16, *q16;        // [H, N, d] and [N, H, d] (sweep order) fp16
+    GroupLists lists;
+    int* redo;              // [N * H]
+    void* scratch;          // of the redo pass, 8-byte entries
+    long long scratch_words;
+};
+inline F16Buffers f16_buffers(const FwdArgs& a, const FwdWorkspace& w) {
+    const size_t rows = (size_t)a.N * a.H, copy = rows * a.d * 2, out_bytes = rows * a.d * (a.mode == KMIP_FP32_EXACT ? 4 : 2);
+    unsigned char* out = static_cast<unsigned char*>(a.out);
+    F16Buffers b;
+    b.k16 = a.ws + w.kpack_off;
+    b.q16 = a.ws + w.qperm_off;
+    b.lists = {a.ws + w.cand_word_off, a.ws + w.cand_half_off, 4ll * w.list, 2ll * w.list, w.list, 0};
+    b.redo = reinterpret_cast<int*>(a.ws + w.redo_off);
+    size_t used = 0;  // bytes of `out` taken after the sweep
+    if (w.in_outputs) {
+        // until the sweep is done `out` holds the copies; then the redo list and the redo pass's scratch
+        if (a.mode == KMIP_FP32_EXACT) { b.k16 = out; b.q16 = out + copy; }
+        else if (!w.reorder) b.q16 = out;
+        b.lists = {reinterpret_cast<unsigned char*>(a.topk_idx), reinterpret_cast<unsigned char*>(a.topk_score), 4ll * a.k, 4ll * a.k, w.list, 1};
+        b.redo = reinterpret_cast<int*>(out);
+        used = align_up(rows * 4, 16);
+    }
+    b.scratch = out + used;
+    b.scratch_words = out_bytes > used ? (long long)((out_bytes - used) / 8) : 0;
+    return b;
+}
+int score_select_f16_rows_per_item(const FwdWorkspace& w, int32_t d, int32_t k);
 cudaError_t launch_f16_convert(const FwdArgs& a, const FwdWorkspace& w);
 cudaError_t launch_score_select_f16(const FwdArgs& a, const FwdWorkspace& w);
-cudaError_t launch_score_select_f16x4(const FwdArgs& a, const FwdWorkspace& w);  // k <= 16, called by the above
+cudaError_t launch_score_select_f16x4(const FwdArgs& a, const FwdWorkspace& w);  // called by the above
 cudaError_t launch_score_dump_f16(const FwdArgs& a, const FwdWorkspace& w, float* dump);
 cudaError_t launch_refine_f16(const FwdArgs& a, const FwdWorkspace& w);
 cudaError_t launch_score_select_exact_redo(const FwdArgs& a, const FwdWorkspace& w);

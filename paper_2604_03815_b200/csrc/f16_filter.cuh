@@ -17,13 +17,14 @@ namespace kmip {
 constexpr int kF16List32 = KMIP_F16_LIST32;
 
 // Per head: largest squared norm of a query row, of a key row, and of the first 16 elements of a key
-// row (the partial sum after the first tensor-core step of a 32-wide head); float bits, maxima taken
+// row (the partial sum after the first tensor-core step of a wider head); largest squared norm of what the conversion
+// of a key row to fp16 lost (fp32 storage only; bf16 values convert exactly up to underflow).  Float bits, maxima taken
 // with integer atomics (the values are non-negative).
 struct F16HeadStat {
     float q_n2max;
     float k_n2max;
     float k_first16_n2max;
-    float pad;
+    float k_lost_n2max;  // of the SCALED row
 };
 
 // Power of two s such that s * sqrt(n2max) lies in [32, 64) (up to the rounding of the square root):
@@ -39,12 +40,13 @@ __host__ __device__ inline float f16_scale_from_n2max(float n2max) {
 
 // |fp16 score T - exact scaled score| <= a + r * |T| for every key of the head, given the row's scaled
 // norms.  The tensor cores round the fp16 accumulator to nearest once per 16-deep step: the last
-// rounding is at most 2^-11 |T|, the one before (32-wide heads) at most 2^-11 times the partial sum,
-// itself at most |q[0:16]| |k[0:16]|.  2^-18 |q||k| covers the internal summation, 2.5e-5 the elements
-// that underflowed in the conversion (scaled norms are below 64) and subnormal results.
+// rounding is at most 2^-11 |T|, an earlier one at most 2^-11 times the partial sum, itself at most
+// |q[0:16 s]| |k[0:16 s]| (`partial`: the sum of these products over the steps before the last).  2^-18 |q||k| covers
+// the internal summation, 2.5e-5 the elements that underflowed in the conversion (scaled norms are below 64) and
+// subnormal results; `lost` what rounding fp32 operands to fp16 changed (at most |q| |dk| + |dq| |k|; 0 for bf16).
 constexpr float kF16RelErr = 4.8923e-4f;  // 2^-11 (1 + 2^-9)
-__host__ __device__ inline float f16_abs_err(int ksteps, float nq_first16, float nk_first16_max, float nq, float nk_max) {
-    return (ksteps > 1 ? kF16RelErr * nq_first16 * nk_first16_max : 0.0f) + 3.8147e-6f * nq * nk_max + 2.5e-5f;
+__host__ __device__ inline float f16_abs_err(float partial, float nq, float nk_max, float lost) {
+    return kF16RelErr * partial + 3.8147e-6f * nq * nk_max + 2.5e-5f + lost;
 }
 
 }  // namespace kmip

@@ -12,12 +12,13 @@ constexpr int kPlanThreads = 1024;
 
 __global__ void __launch_bounds__(kPlanThreads)
 plan_kernel(const int32_t* __restrict__ offs, int G, int N, int rows_per_item, int max_items,
-            WorkItem* __restrict__ items, StatusBlock* __restrict__ sb) {
+            WorkItem* __restrict__ items, StatusBlock* __restrict__ sb, float* __restrict__ clear, int n_clear) {
     __shared__ int s_warp[32];
     __shared__ int s_carry;
     __shared__ int s_bad;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     if (tid == 0) { s_carry = 0; s_bad = 0; }
+    for (int x = tid; x < n_clear; x += kPlanThreads) clear[x] = 0.0f;  // statistics that later kernels take maxima into
     __syncthreads();
 
     if (offs != nullptr) {
@@ -133,7 +134,8 @@ cudaError_t launch_pack_keys(const FwdArgs& a, const FwdWorkspace& w) {
 cudaError_t launch_plan(const FwdArgs& a, const FwdWorkspace& w, int rows_per_item) {
     plan_kernel<<<1, kPlanThreads, 0, a.stream>>>(
         a.graph_offsets, a.G, (int)a.N, rows_per_item, w.max_items,
-        reinterpret_cast<WorkItem*>(a.ws + w.items_off), reinterpret_cast<StatusBlock*>(a.ws));
+        reinterpret_cast<WorkItem*>(a.ws + w.items_off), reinterpret_cast<StatusBlock*>(a.ws),
+        reinterpret_cast<float*>(a.ws + w.f16stat_off), w.f16 ? 4 * a.H : 0);
     return cudaGetLastError();
 }
 

@@ -6,9 +6,8 @@
 //      is at least lowS = m_k - err(m_k), so the true k-th best score t_k is at least lowS, and a group
 //      whose maximum g satisfies g + err(g) < lowS cannot hold one of the k best keys: it is skipped.
 //      err(T) = a + r |T| bounds |fp16 score - exact scaled score| (f16_filter.cuh).
-//   2. The keys of the other groups are scored again - fp32 fused multiply-adds over the bf16 values in
-//      index order (the mixed-precision instruction: exact product, one rounding, the same bits as convert +
-//      fmaf), read from K in place - and the k best under (score desc, key asc) are kept with the
+//   2. The keys of the other groups are scored again - fp32 fused multiply-adds in index order (over bf16 values the
+//      mixed-precision instruction: exact product, one rounding, the same bits as convert + fmaf), read from K in place - and the k best under (score desc, key asc) are kept with the
 //      running top-k buffer of the CUDA-core kernel.
 //   3. If the sweep's list was full, groups it dropped have maxima at most g_min, the smallest one
 //      kept.  When g_min + err(g_min) reaches the k-th best exact score found, a dropped group could
@@ -32,45 +31,93 @@ namespace {
 constexpr int kWarpsPerBlock = 8;
 constexpr unsigned FULL = 0xFFFFFFFFu;
 
-// End of the graph that holds node i.  Batches of up to kOffsCached - 1 graphs search a copy of the offsets in
+// Range of the graph that holds node i.  Batches of up to kOffsCached - 1 graphs search a copy of the offsets in
 // shared memory: seven dependent global loads per row would otherwise be the longest chain of a small-graph batch.
 constexpr int kOffsCached = 1024;
-__device__ inline int graph_end_of(const int32_t* offs, const int* s_offs, int G, int N, int i) {
-    if (offs == nullptr) return N;
+__device__ inline void graph_range_of(const int32_t* offs, const int* s_offs, int G, int N, int i, int& lo, int& hi) {
+    if (offs == nullptr) { lo = 0; hi = N; return; }
     int a = 0, b = G;
     if (G < kOffsCached) {
         while (b - a > 1) {
             const int m = (a + b) >> 1;
             if (s_offs[m] <= i) a = m; else b = m;
         }
-        return max(0, min(N, s_offs[a + 1]));
+        lo = max(0, s_offs[a]);
+        hi = max(0, min(N, s_offs[a + 1]));
+        return;
     }
     while (b - a > 1) {
         const int m = (a + b) >> 1;
         if (__ldg(offs + m) <= i) a = m; else b = m;
     }
-    return max(0, min(N, __ldg(offs + a + 1)));
+    lo = max(0, __ldg(offs + a));
+    hi = max(0, min(N, __ldg(offs + a + 1)));
 }
 
 // fp16 bits -> 16-bit key whose unsigned order is the order of the values (no NaNs reach this point)
 __device__ __forceinline__ unsigned f16_ordered(unsigned hb) { return (hb & 0x8000u) ? (~hb & 0xFFFFu) : (hb | 0x8000u); }
 __device__ __forceinline__ unsigned f16_unordered(unsigned ok) { return (ok & 0x8000u) ? (ok & 0x7FFFu) : (~ok & 0xFFFFu); }
 
-template <int D, int E, int LIST>
-__global__ void __launch_bounds__(kWarpsPerBlock * 32, 4)
-refine_f16_kernel(const __nv_bfloat16* __restrict__ Q, const __nv_bfloat16* __restrict__ K,
-                  const int32_t* __restrict__ offs, int G, int N, int H, int k,
-                  const uint32_t* __restrict__ cand_word, const uint16_t* __restrict__ cand_half,
-                  const F16HeadStat* __restrict__ stat, int32_t* __restrict__ topk_idx, float* __restrict__ topk_score,
+// The query row in registers (bf16: two values to a register) and one key row of the stage against it.
+template <typename T, int D> struct QueryRow;
+template <int D> struct QueryRow<__nv_bfloat16, D> {
+    uint32_t qp[D / 2];
+    __device__ void load(const __nv_bfloat16* s) {
+#pragma unroll
+        for (int v = 0; v < D / 8; ++v) {
+            const uint4 t = *reinterpret_cast<const uint4*>(s + v * 8);
+            qp[v * 4 + 0] = t.x; qp[v * 4 + 1] = t.y; qp[v * 4 + 2] = t.z; qp[v * 4 + 3] = t.w;
+        }
+    }
+    __device__ float dot(const unsigned char* kr) const {
+        float s = 0.0f;
+#pragma unroll
+        for (int v = 0; v < D / 8; ++v) {
+            const uint4 rw = *reinterpret_cast<const uint4*>(kr + v * 16);
+            const uint32_t wv[4] = {rw.x, rw.y, rw.z, rw.w};
+#pragma unroll
+            for (int x = 0; x < 4; ++x) s = ptx::fma_bf16_pair(qp[v * 4 + x], wv[x], s);
+        }
+        return s;
+    }
+};
+template <int D> struct QueryRow<float, D> {
+    const float* q;  // shared memory, the same address in every lane
+    __device__ void load(const float* s) { q = s; }
+    __device__ float dot(const unsigned char* kr) const {
+        float s = 0.0f;
+#pragma unroll
+        for (int c = 0; c < D; c += 4) {
+            const float4 kv = *reinterpret_cast<const float4*>(kr + c * 4);
+            const float4 qv = *reinterpret_cast<const float4*>(q + c);
+            s = fmaf(qv.x, kv.x, s);
+            s = fmaf(qv.y, kv.y, s);
+            s = fmaf(qv.z, kv.z, s);
+            s = fmaf(qv.w, kv.w, s);
+        }
+        return s;
+    }
+};
+__device__ __forceinline__ float to_float(__nv_bfloat16 x) { return __bfloat162float(x); }
+__device__ __forceinline__ float to_float(float x) { return x; }
+
+// TOPK arrays and lists: with lists in the output arrays (`lists` points into topk_idx / topk_score) a row's list is read
+// before the same warp writes the row's answer over it.
+template <typename T, int D, int E, int LIST>
+__global__ void __launch_bounds__(kWarpsPerBlock * 32, D * sizeof(T) <= 64 ? 4 : D * sizeof(T) <= 128 ? 2 : 1)
+refine_f16_kernel(const T* __restrict__ Q, const T* __restrict__ K,
+                  const int32_t* __restrict__ offs, int G, int N, int H, int k, const GroupLists lists,
+                  const F16HeadStat* __restrict__ stat, int32_t* topk_idx, float* topk_score,
                   StatusBlock* __restrict__ sb, int* __restrict__ redo_list) {
     if (sb->status != KMIP_OK) return;
-    using T = __nv_bfloat16;
+    constexpr bool kLossy = sizeof(T) == 4;
+    constexpr int QE = (D + 31) / 32;  // query elements per lane
     constexpr int CAP = 32 * E;
     constexpr int EPL = (LIST + 31) / 32;  // list entries per lane
     constexpr int KSTEPS = D / 16;
-    static_assert(E <= 4 && LIST <= 64 && D <= 32, "k <= 32, head widths 16 and 32");
+    static_assert(E <= 4 && LIST <= 64, "k <= 32");
     __shared__ cand_t s_rows[kWarpsPerBlock][CAP];
-    __shared__ __align__(16) unsigned short s_qb[kWarpsPerBlock][D];  // the query row, bf16 bits
+    __shared__ __align__(16) T s_qb[kWarpsPerBlock][D];  // the query row
     __shared__ uint32_t s_words[kWarpsPerBlock][LIST];
     __shared__ int s_offs[kOffsCached];
     if (offs != nullptr && G < kOffsCached) {
@@ -83,37 +130,41 @@ refine_f16_kernel(const __nv_bfloat16* __restrict__ Q, const __nv_bfloat16* __re
     const long long n_rows = (long long)N * H;
     const long long stride = (long long)gridDim.x * kWarpsPerBlock;
     const int room = CAP - k;
-    constexpr int P = D / 8;                   // 16-byte pieces of a key row
-    constexpr int kRowStride = D * 2 + 16;     // padded: a lane per row reads 16-byte pieces without bank conflicts
+    constexpr int P = D * (int)sizeof(T) / 16;                 // 16-byte pieces of a key row
+    constexpr int kRowStride = D * (int)sizeof(T) + 16;        // padded: a lane per row reads 16-byte pieces without bank conflicts
     constexpr int kStageBytes = 32 * kRowStride;
     extern __shared__ __align__(16) unsigned char s_stage[];  // [warp][2 stages][32 rows]
     unsigned char* stage = s_stage + wib * 2 * kStageBytes;
     const int pl = lane % P;
     const unsigned row_bytes = (unsigned)(H * D * (int)sizeof(T));
 
-    // a row's list (entry t in lane t % 32, register t / 32) and query element are fetched one row ahead
+    // a row's list (entry t in lane t % 32, register t / 32) and query elements are fetched one row ahead
     uint32_t nx_word[EPL];
     unsigned nx_half[EPL];
-    float nx_q = 0.0f;
+    T nx_q[QE];
     auto fetch = [&](long long r) {
 #pragma unroll
         for (int e = 0; e < EPL; ++e) {
             const int t = e * 32 + lane;
             nx_half[e] = 0xFFFFu;
             nx_word[e] = 0xFFFFFFFFu;
-            if (r < n_rows && t < LIST) {
-                nx_half[e] = __ldg(cand_half + (size_t)r * LIST + t);
-                nx_word[e] = __ldg(cand_word + (size_t)r * LIST + t);  // never written for an empty slot: ignored below
+            if (r < n_rows && t < lists.slots) {
+                nx_half[e] = *reinterpret_cast<const uint16_t*>(lists.half + r * lists.half_pitch + 2 * t);
+                // never written for an empty slot: ignored below
+                const unsigned char* wp = lists.word + r * lists.word_pitch;
+                nx_word[e] = lists.compact ? (uint32_t)reinterpret_cast<const uint16_t*>(wp)[t] : reinterpret_cast<const uint32_t*>(wp)[t];
             }
         }
-        nx_q = (r < n_rows && lane < D) ? Elem<T>::load(Q + (size_t)r * D + lane) : 0.0f;
+#pragma unroll
+        for (int e = 0; e < QE; ++e) nx_q[e] = (r < n_rows && e * 32 + lane < D) ? Q[(size_t)r * D + e * 32 + lane] : T(0.0f);
     };
     long long r = (long long)blockIdx.x * kWarpsPerBlock + wib;
     fetch(r);
 
     for (; r < n_rows; r += stride) {
         const int i = (int)(r / H), h = (int)(r % H);
-        const int hi = graph_end_of(offs, s_offs, G, N, i);
+        int lo, hi;
+        graph_range_of(offs, s_offs, G, N, i, lo, hi);
 
         // empty slots: the four-pipeline sweep marks them by the half 0xFFFF and never writes their group word,
         // the ring sweep writes an all-ones word
@@ -123,34 +174,56 @@ refine_f16_kernel(const __nv_bfloat16* __restrict__ Q, const __nv_bfloat16* __re
         unsigned ok_min = 0xFFFFu;
 #pragma unroll
         for (int e = 0; e < EPL; ++e) {
-            word[e] = nx_word[e];
-            const bool valid = nx_half[e] != 0xFFFFu && word[e] != 0xFFFFFFFFu;
+            word[e] = lists.compact ? (uint32_t)(lo + (int)(nx_word[e] >> 1) * 16) | (nx_word[e] << 31) : nx_word[e];
+            const bool valid = nx_half[e] != 0xFFFFu && (lists.compact || word[e] != 0xFFFFFFFFu);
             okey[e] = valid ? f16_ordered(nx_half[e]) : 0u;
             n_valid += __popc(__ballot_sync(FULL, valid));
             ok_min = min(ok_min, valid ? okey[e] : 0xFFFFu);
         }
-        const float qc = nx_q;
-        __syncwarp();
-        if (lane < D) s_qb[wib][lane] = (unsigned short)(__float_as_uint(qc) >> 16);  // exact: the value came from bf16
-        for (int t = lane; t < k; t += 32) row[t] = 0ull;
-        fetch(r + stride);
-
-        // the query's norms; error bound of the fp16 scores in the scaled units of the sweep
-        float q2 = qc * qc, qa2 = lane < 16 ? qc * qc : 0.0f;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            q2 += __shfl_xor_sync(FULL, q2, o);
-            qa2 += __shfl_xor_sync(FULL, qa2, o);
-            ok_min = min(ok_min, __shfl_xor_sync(FULL, ok_min, o));
-        }
         const F16HeadStat hs = stat[h];
         const float sq = f16_scale_from_n2max(hs.q_n2max), sk = f16_scale_from_n2max(hs.k_n2max);
         const float sc = sq * sk;  // scaled score = sc * score, a power of two
-        const float nq = sqrtf(q2) * sq * 1.00001f, nqa = sqrtf(qa2) * sq * 1.00001f;
+        __syncwarp();
+        // the query's norms: of the whole row, of its first 16, 32 and 48 elements (the tensor cores' partial sums), and
+        // of what its conversion to fp16 lost
+        float q2 = 0.0f, qlost2 = 0.0f, qpart2[3] = {0.0f, 0.0f, 0.0f};
+#pragma unroll
+        for (int e = 0; e < QE; ++e) {
+            const int c = e * 32 + lane;
+            if (c < D) s_qb[wib][c] = nx_q[e];
+            const float x = to_float(nx_q[e]);
+            q2 = fmaf(x, x, q2);
+#pragma unroll
+            for (int p = 0; p < 3; ++p)
+                if (c < 16 * (p + 1)) qpart2[p] = fmaf(x, x, qpart2[p]);
+            if (kLossy) {
+                const float dx = x * sq - __half2float(__float2half_rn(x * sq));
+                qlost2 = fmaf(dx, dx, qlost2);
+            }
+        }
+        for (int t = lane; t < k; t += 32) row[t] = 0ull;
+        fetch(r + stride);
+
+        // error bound of the fp16 scores in the scaled units of the sweep
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            q2 += __shfl_xor_sync(FULL, q2, o);
+#pragma unroll
+            for (int p = 0; p < KSTEPS - 1 && p < 3; ++p) qpart2[p] += __shfl_xor_sync(FULL, qpart2[p], o);
+            if (kLossy) qlost2 += __shfl_xor_sync(FULL, qlost2, o);
+            ok_min = min(ok_min, __shfl_xor_sync(FULL, ok_min, o));
+        }
+        const float nq = sqrtf(q2) * sq * 1.00001f;
         const float nk = sqrtf(hs.k_n2max) * sk, nka = sqrtf(hs.k_first16_n2max) * sk;
-        const float ea = f16_abs_err(KSTEPS, nqa, nka, nq, nk) * 1.0001f;
+        float partial = 0.0f;  // |q[0:16 s]| |k[0:16 s]| over the steps before the last
+#pragma unroll
+        for (int p = 0; p < KSTEPS - 1 && p < 3; ++p) partial += sqrtf(qpart2[p]) * sq * 1.00001f * (p == 0 ? nka : nk);
+        const float nk_lost = sqrtf(hs.k_lost_n2max), nq_lost = sqrtf(qlost2) * 1.00001f;
+        const float lost = kLossy ? (nq * nk_lost + nq_lost * (nk + nk_lost)) * 1.0001f : 0.0f;
+        const float ea = f16_abs_err(partial, nq, nk, lost) * 1.0001f;
         const float er = kF16RelErr;
-        const float fp32_err = 4e-6f * nq * nk;  // of the fp32 rescoring below, in scaled units
+        // of the fp32 rescoring below, in scaled units: D roundings of at most 2^-24 |q||k| each, twice that
+        const float fp32_err = (D <= 32 ? 4e-6f : D * 1.2e-7f) * nq * nk;
         const float g_min = __half2float(__ushort_as_half((unsigned short)f16_unordered(ok_min)));
 
         // m_k, the k-th largest group maximum: the largest 16-bit key that at least k entries reach, bit by bit
@@ -185,13 +258,13 @@ refine_f16_kernel(const __nv_bfloat16* __restrict__ Q, const __nv_bfloat16* __re
         const float floor_tau = n_valid >= k ? (lowS - fp32_err) / sc - 1e-30f : -CUDART_INF_F;
         float tau = floor_tau;
         int cnt = 0;
-        // Rescoring, 32 keys (4 groups) per step.  A key row is P = D / 8 pieces of 16 bytes.  The rows come in by
+        // Rescoring, 32 keys (4 groups) per step.  A key row is P pieces of 16 bytes.  The rows come in by
         // asynchronous 16-byte copies in which P neighbouring lanes fetch one row, so one copy instruction touches
         // 32 / P cache lines instead of 32 (the kernel is bound by these line accesses); they land in a per-warp
         // stage of padded rows, one step ahead of the arithmetic.  Then each lane reads one whole row back and
         // scores it with the same chain of fused multiply-adds in index order as every other kernel.
         const int nsteps = (n_kept + 3) / 4;
-        const unsigned char* kb = reinterpret_cast<const unsigned char*>(K) + ((size_t)h * D + pl * 8) * sizeof(T);
+        const unsigned char* kb = reinterpret_cast<const unsigned char*>(K) + (size_t)h * D * sizeof(T) + pl * 16;
         auto issue = [&](int step) {
             if (step < nsteps) {
                 unsigned char* buf = stage + (step & 1) * kStageBytes;
@@ -209,13 +282,9 @@ refine_f16_kernel(const __nv_bfloat16* __restrict__ Q, const __nv_bfloat16* __re
             }
             ptx::cp_async_commit();  // an empty group when there is nothing left, so that the count below holds
         };
-        uint32_t qp[D / 2];  // the query row, two bf16 values to a register
         __syncwarp();
-#pragma unroll
-        for (int v = 0; v < D / 8; ++v) {
-            const uint4 t4 = *reinterpret_cast<const uint4*>(&s_qb[wib][v * 8]);
-            qp[v * 4 + 0] = t4.x; qp[v * 4 + 1] = t4.y; qp[v * 4 + 2] = t4.z; qp[v * 4 + 3] = t4.w;
-        }
+        QueryRow<T, D> qrow;
+        qrow.load(s_qb[wib]);
         issue(0);
         for (int step = 0; step < nsteps; ++step) {
             issue(step + 1);
@@ -226,16 +295,7 @@ refine_f16_kernel(const __nv_bfloat16* __restrict__ Q, const __nv_bfloat16* __re
             const int jj = (int)(wd & 0x7FFFFFFFu) + (int)(wd >> 31) + 2 * (lane & 7);
             const bool kv = t < n_kept && jj < hi;
             float s = 0.0f;
-            if (kv) {
-                const unsigned char* kr = stage + (step & 1) * kStageBytes + lane * kRowStride;
-#pragma unroll
-                for (int v = 0; v < P; ++v) {
-                    const uint4 rw = *reinterpret_cast<const uint4*>(kr + v * 16);
-                    const uint32_t wv[4] = {rw.x, rw.y, rw.z, rw.w};
-#pragma unroll
-                    for (int x = 0; x < 4; ++x) s = ptx::fma_bf16_pair(qp[v * 4 + x], wv[x], s);
-                }
-            }
+            if (kv) s = qrow.dot(stage + (step & 1) * kStageBytes + lane * kRowStride);
             const bool pass = kv && (s > tau);
             const unsigned m = __ballot_sync(FULL, pass);
             if (m) {
@@ -254,7 +314,7 @@ refine_f16_kernel(const __nv_bfloat16* __restrict__ Q, const __nv_bfloat16* __re
         const float kth = warp_merge_row_chunks(row, k, cnt, lane);
         // a dropped group scores at most g_min + err(g_min) exactly (scaled); it matters if that reaches the
         // k-th best score found
-        if (n_valid == LIST && g_min + ea + er * fabsf(g_min) >= kth * sc - fp32_err) {
+        if (n_valid == lists.slots && g_min + ea + er * fabsf(g_min) >= kth * sc - fp32_err) {
             if (lane == 0) {
                 const int pos = atomicAdd(&sb->n_redo, 1);
                 if (kmip_check(pos >= 0 && pos < n_rows, sb, 102)) redo_list[pos] = (int)r;  // checks builds: inside the list
@@ -265,20 +325,18 @@ refine_f16_kernel(const __nv_bfloat16* __restrict__ Q, const __nv_bfloat16* __re
     }
 }
 
-template <int D>
+template <typename T, int D>
 cudaError_t launch_d(const FwdArgs& a, const FwdWorkspace& w) {
     const long long n_rows = (long long)a.N * a.H;
     const int blocks = (int)std::min<long long>((n_rows + kWarpsPerBlock - 1) / kWarpsPerBlock, (long long)sm_count() * 32);
-    constexpr int kSmem = kWarpsPerBlock * 2 * 32 * (D * 2 + 16);  // the rescoring stages
+    constexpr int kSmem = kWarpsPerBlock * 2 * 32 * (D * (int)sizeof(T) + 16);  // the rescoring stages
+    const F16Buffers b = f16_buffers(a, w);
 #define KMIP_LAUNCH_REFINE16(E_, LIST_) \
-    if ((err = cudaFuncSetAttribute(refine_f16_kernel<D, E_, LIST_>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem)) != cudaSuccess) return err; \
-    refine_f16_kernel<D, E_, LIST_><<<blocks, kWarpsPerBlock * 32, kSmem, a.stream>>>( \
-        static_cast<const __nv_bfloat16*>(a.Q), static_cast<const __nv_bfloat16*>(a.K), a.graph_offsets, a.G, (int)a.N, \
-        a.H, a.k, reinterpret_cast<const uint32_t*>(a.ws + w.cand_word_off), \
-        reinterpret_cast<const uint16_t*>(a.ws + w.cand_half_off), reinterpret_cast<const F16HeadStat*>(a.ws + w.f16stat_off), \
-        a.topk_idx, a.topk_score, reinterpret_cast<StatusBlock*>(a.ws), reinterpret_cast<int*>(a.ws + w.redo_off))
+    if ((err = cudaFuncSetAttribute(refine_f16_kernel<T, D, E_, LIST_>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem)) != cudaSuccess) return err; \
+    refine_f16_kernel<T, D, E_, LIST_><<<blocks, kWarpsPerBlock * 32, kSmem, a.stream>>>( \
+        static_cast<const T*>(a.Q), static_cast<const T*>(a.K), a.graph_offsets, a.G, (int)a.N, a.H, a.k, b.lists, \
+        reinterpret_cast<const F16HeadStat*>(a.ws + w.f16stat_off), a.topk_idx, a.topk_score, reinterpret_cast<StatusBlock*>(a.ws), b.redo)
     cudaError_t err;
-    // the list sizes are those of score_select_f16_list
     if (a.k <= 8) { KMIP_LAUNCH_REFINE16(2, 16); }
     else if (a.k <= 16) { KMIP_LAUNCH_REFINE16(2, 24); }
     else { KMIP_LAUNCH_REFINE16(4, kF16List32); }
@@ -286,10 +344,20 @@ cudaError_t launch_d(const FwdArgs& a, const FwdWorkspace& w) {
     return cudaGetLastError();
 }
 
+template <typename T>
+cudaError_t launch_t(const FwdArgs& a, const FwdWorkspace& w) {
+    switch (a.d) {
+        case 16: return launch_d<T, 16>(a, w);
+        case 32: return launch_d<T, 32>(a, w);
+        case 64: return launch_d<T, 64>(a, w);
+        default: return cudaErrorInvalidValue;
+    }
+}
+
 }  // namespace
 
 cudaError_t launch_refine_f16(const FwdArgs& a, const FwdWorkspace& w) {
-    return a.d == 16 ? launch_d<16>(a, w) : launch_d<32>(a, w);
+    return a.mode == KMIP_FP32_EXACT ? launch_t<float>(a, w) : launch_t<__nv_bfloat16>(a, w);
 }
 
 }  // namespace kmip

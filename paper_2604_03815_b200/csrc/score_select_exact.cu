@@ -258,26 +258,42 @@ cudaError_t launch_t(const FwdArgs& a) {
     }
 }
 
+
+template <typename T, int D>
+void launch_redo_d(const FwdArgs& a, const F16Buffers& b) {
+    const int blocks = sm_count() * kRedoBlocksPerSm;
+    const long long lists = b.scratch_words / a.k;
+#define KMIP_LAUNCH_REDO(E_) \
+    score_select_redo_kernel<T, D, E_><<<blocks, kRedoWarps * 32, 0, a.stream>>>( \
+        static_cast<const T*>(a.Q), static_cast<const T*>(a.K), a.graph_offsets, a.G, (int)a.N, a.H, a.k, \
+        a.topk_idx, a.topk_score, reinterpret_cast<StatusBlock*>(a.ws), b.redo, static_cast<cand_t*>(b.scratch), lists)
+    if (a.k <= 16) KMIP_LAUNCH_REDO(2);
+    else KMIP_LAUNCH_REDO(4);
+#undef KMIP_LAUNCH_REDO
+}
+
+template <typename T>
+cudaError_t launch_redo_t(const FwdArgs& a, const F16Buffers& b) {
+    switch (a.d) {
+        case 16: launch_redo_d<T, 16>(a, b); break;
+        case 32: launch_redo_d<T, 32>(a, b); break;
+        case 64: launch_redo_d<T, 64>(a, b); break;
+        default: return cudaErrorInvalidValue;
+    }
+    return cudaGetLastError();
+}
+
 }  // namespace
 
 cudaError_t launch_score_select_exact(const FwdArgs& a) {
     return a.mode == KMIP_FP32_EXACT ? launch_t<float>(a) : launch_t<__nv_bfloat16>(a);
 }
 
-// The rows the half-precision prefilter could not decide (bf16 storage, head widths 16 and 32, k <= 32), again from
-// all keys of their graph; overwrites their topk_idx / topk_score.
+// The rows the half-precision prefilter could not decide (k <= 32), again from all keys of their graph; overwrites
+// their topk_idx / topk_score.
 cudaError_t launch_score_select_exact_redo(const FwdArgs& a, const FwdWorkspace& w) {
-    const int blocks = sm_count() * kRedoBlocksPerSm;
-    const long long lists = (long long)a.N * a.H * a.d * 2 / ((long long)a.k * (long long)sizeof(cand_t));
-#define KMIP_LAUNCH_REDO(D_, E_) \
-    score_select_redo_kernel<__nv_bfloat16, D_, E_><<<blocks, kRedoWarps * 32, 0, a.stream>>>( \
-        static_cast<const __nv_bfloat16*>(a.Q), static_cast<const __nv_bfloat16*>(a.K), a.graph_offsets, a.G, (int)a.N, a.H, a.k, \
-        a.topk_idx, a.topk_score, reinterpret_cast<StatusBlock*>(a.ws), reinterpret_cast<const int*>(a.ws + w.redo_off), \
-        static_cast<cand_t*>(a.out), lists)
-    if (a.d == 16) { if (a.k <= 16) KMIP_LAUNCH_REDO(16, 2); else KMIP_LAUNCH_REDO(16, 4); }
-    else { if (a.k <= 16) KMIP_LAUNCH_REDO(32, 2); else KMIP_LAUNCH_REDO(32, 4); }
-#undef KMIP_LAUNCH_REDO
-    return cudaGetLastError();
+    const F16Buffers b = f16_buffers(a, w);
+    return a.mode == KMIP_FP32_EXACT ? launch_redo_t<float>(a, b) : launch_redo_t<__nv_bfloat16>(a, b);
 }
 
 }  // namespace kmip

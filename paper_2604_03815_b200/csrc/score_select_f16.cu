@@ -1,5 +1,5 @@
-// Half-precision prefilter sweep of the tensor-core mode (Algorithm 1 lines 2-3) for head widths
-// 16 and 32 and 16 < k <= 32 (k <= 16: score_select_f16x4.cu, the same filter on another pipeline).
+// Half-precision prefilter sweep (Algorithm 1 lines 2-3) of the tensor-core mode for head widths 16 and 32
+// and 16 < k <= 32 (other shapes and fp32 storage: score_select_f16x4.cu, the same filter on another pipeline).
 //
 // The paper lists half-precision arithmetic and tensor-core support as the engineering it left open
 // (Sec. 6; closing remark of the FlashAttention comparison in the appendix).  The sweep of
@@ -584,13 +584,25 @@ cudaError_t launch_d(const FwdArgs& a, const FwdWorkspace& w, float* dump) {
 
 }  // namespace
 
+// Lists in the workspace (bf16 storage).
 bool score_select_f16_supported(int32_t d, int32_t k) { return (d == 16 || d == 32) && k <= 32; }
 int score_select_f16_list(int32_t k) { return k <= 8 ? 16 : k <= 16 ? 24 : kF16List32; }
-// lists of up to 24 groups (k <= 16) run the four-pipeline kernel of score_select_f16x4.cu with 512-row work items
-int score_select_f16_rows_per_item(int32_t k) { return k <= 16 ? score_select_f16x4_rows_per_item() : 3 * BM; }
+
+// Lists in the output arrays: a row's topk_idx and topk_score hold 2 k entries of two 16-bit numbers, so the groups are
+// numbered inside their graph (up to 2^16 of 8 keys) and k + slack <= 2 k, which wants k >= 4.
+int score_select_f16_list_in_outputs(int32_t k) { return std::min(2 * k, k <= 8 ? 16 : k <= 16 ? 24 : kF16List32); }
+bool score_select_f16_in_outputs_supported(int64_t N, int32_t H, int32_t d, int32_t k, int mode) {
+    if (k < 4 || k > 32 || N > (1 << 19)) return false;
+    return mode == KMIP_FP32_EXACT && (d == 16 || d == 32 || d == 64) && N * H >= kF16MinRowsFp32;
+}
+
+// k in 17..32 with lists in the workspace runs the ring above with 384-row work items; everything else the kernel of
+// score_select_f16x4.cu with 512-row work items (384 for 64-wide heads: shared memory)
+static bool ring(const FwdWorkspace& w, int32_t k) { return !w.in_outputs && k > 16; }
+int score_select_f16_rows_per_item(const FwdWorkspace& w, int32_t d, int32_t k) { return ring(w, k) || d == 64 ? 3 * BM : 4 * BM; }
 
 cudaError_t launch_score_select_f16(const FwdArgs& a, const FwdWorkspace& w) {
-    if (a.k <= 16) return launch_score_select_f16x4(a, w);
+    if (!ring(w, a.k)) return launch_score_select_f16x4(a, w);
     return a.d == 16 ? launch_d<16, false>(a, w, nullptr) : launch_d<32, false>(a, w, nullptr);
 }
 

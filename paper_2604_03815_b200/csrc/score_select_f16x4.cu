@@ -1,15 +1,17 @@
-// Half-precision prefilter sweep of the tensor-core mode (Algorithm 1 lines 2-3) for head widths 16
-// and 32 and k <= 16: the filter of score_select_f16.cu (fp16 operands and accumulators, packed
-// three-input maxima over 16-key windows, the k + slack best 8-key groups per row, exact rescoring in
-// refine_f16.cu) on a pipeline cut for short lists.
-//   * Four 128-row query tiles per CTA (512 rows per work item, 16 selection warps: four per SM
+// Half-precision prefilter sweep (Algorithm 1 lines 2-3): the filter of score_select_f16.cu (fp16 operands and
+// accumulators, packed three-input maxima over 16-key windows, the k + slack best 8-key groups per row, exact rescoring
+// in refine_f16.cu) on a pipeline cut for short lists.  It serves the tensor-core mode with k <= 16 and head widths 16
+// and 32 (lists in the workspace), head width 64, and fp32 storage (both with their lists in the output arrays).
+//   * Up to four 128-row query tiles per CTA (512 rows per work item, 16 selection warps: four per SM
 //     sub-partition to hide each other's tensor-memory loads and dependent instruction chains), each with
 //     an accumulator buffer and an MMA issuer of its own: four independent pipelines that meet only at
 //     the key stages.  A selection warp hands its buffer back as soon as the scores are in registers and
-//     its issuer multiplies the next key tile while the warp reduces the current one.
+//     its issuer multiplies the next key tile while the warp reduces the current one.  64-wide heads have three
+//     (the operand tiles take four times the shared memory of 16-wide ones, and the MMA, 256 clocks a tile,
+//     bounds them anyway).
 //   * The group words of the lists live in global memory (each row's place in the output array: they
 //     are only ever written, and a work item's rows stay in L2 while it runs), which leaves the shared
-//     memory to the 16-bit score plane and to 32 pending entries per row, so the CTA-wide lock-step
+//     memory to the 16-bit score plane and to ~30 pending entries per row, so the CTA-wide lock-step
 //     flushes are rarer and better filled.
 // With lists of 24 groups (k = 16) this layout is faster than the four-buffer ring of
 // score_select_f16.cu (200k-node hub graphs, d = 16: 93 against 108 ms); with 48 groups (k = 32) it is
@@ -19,6 +21,7 @@
 #include <algorithm>
 
 #include "common.cuh"
+#include "f16_filter.cuh"
 #include "ptx.cuh"
 
 #include <cuda_fp16.h>
@@ -34,20 +37,19 @@ constexpr int NBUF = 4;  // accumulator buffers of BN columns: all 512 columns o
 constexpr int kRelaxedPollNs = 100;
 // MMA issuer threads (one warp each).  An issuer spends about 390 clocks per pair on top of the pair's own
 // MMAs between a buffer's release and its next commit (measured in isolation), so two of them cap the
-// pipeline at one pair per ~260 clocks, four at ~180; with four, issuer i always fills buffer i.
-constexpr int NISS = 4;
+// pipeline at one pair per ~260 clocks, four at ~180; there is one per query tile, and issuer i always fills buffer i.
 // 16 selection warps and 4 service warps: the register file of an SM holds 96 registers for 640 threads (it is
 // handed out in units of four warps), so the five single-thread roles share four warps: lane 0 of the service
 // warps 1..3 runs issuers 0..2, and service warp 0 runs the TMA producer in lane 0 and issuer 3 in lane 16
 // (two divergent single-lane paths of one warp; neither uses a warp-level operation, and both only ever wait
 // with bounded waits).
-constexpr int kThreads16 = 4 * 128 + 4 * 32;
+constexpr int threads16(int nqt) { return nqt * 128 + 4 * 32; }
 
 template <int D>
 struct Shape16 {
-    static_assert(D == 16 || D == 32, "the fp16 prefilter covers head widths 16 and 32");
+    static_assert(D == 16 || D == 32 || D == 64, "head widths of the fp16 prefilter");
     static constexpr int RB = D * 2;                       // bytes per operand row = swizzle span
-    static constexpr uint32_t LAYOUT = RB == 64 ? 4u : 6u;  // UMMA swizzle code (64-byte / 32-byte)
+    static constexpr uint32_t LAYOUT = RB == 128 ? 2u : RB == 64 ? 4u : 6u;  // UMMA swizzle code (128 / 64 / 32 bytes)
     static constexpr int KSTEPS = D / 16;                  // one tcgen05.mma covers 16 halves of depth
     static constexpr int TILE_BYTES = 128 * RB;
 };
@@ -118,11 +120,12 @@ struct RowSel16 {
 };
 
 template <int KG>
-__device__ __forceinline__ void row_init16(RowSel16<KG>& r, uint16_t* wl, int lane, bool rvalid) {
+__device__ __forceinline__ void row_init16(RowSel16<KG>& r, uint16_t* wl, int lane, bool rvalid, int slots) {
+    // slots past the list's length hold the largest value and are never the minimum
 #pragma unroll 1
-    for (int s = 0; s < 8 * KG; ++s) wl[s * 32 + lane] = 0;
+    for (int s = 0; s < 8 * KG; ++s) wl[s * 32 + lane] = s < slots ? 0 : 0xFFFFu;
 #pragma unroll
-    for (int g = 0; g < KG; ++g) r.gmin[g] = 0u;
+    for (int g = 0; g < KG; ++g) r.gmin[g] = 8 * g < slots ? 0u : 0xFFFFu;
     r.lmin = 0u;
     r.tau2 = rvalid ? kHalfNegInf2 : kHalfPosInf2;
     r.cnt = 0;
@@ -131,7 +134,7 @@ __device__ __forceinline__ void row_init16(RowSel16<KG>& r, uint16_t* wl, int la
 // All 32 lanes insert their pending groups into their own lists, in lock step.  A pending entry is
 // {group word, packed register}: bit 31 of the word says which half of the register is the group's score.
 template <int KG>
-__device__ __forceinline__ void flush_pending16(RowSel16<KG>& r, uint32_t wl_s, uint32_t* __restrict__ wk_g, uint32_t wp_s, bool rvalid) {
+__device__ __forceinline__ void flush_pending16(RowSel16<KG>& r, uint32_t wl_s, unsigned char* wk_g, int compact, uint32_t wp_s, bool rvalid) {
     const int maxc = __reduce_max_sync(FULL, r.cnt);
     __syncwarp();
 #pragma unroll 1
@@ -154,7 +157,8 @@ __device__ __forceinline__ void flush_pending16(RowSel16<KG>& r, uint32_t wl_s, 
                     if (y == m && pos < 0) pos = s; else nm = min(nm, y);
                 }
                 ptx::sts_u16(grp + (uint32_t)pos * 64u, x);
-                wk_g[g * 8 + pos] = raw.x;
+                if (compact) reinterpret_cast<uint16_t*>(wk_g)[g * 8 + pos] = (uint16_t)((raw.x >> 3) | (raw.x >> 31));  // 2 * window + odd
+                else reinterpret_cast<uint32_t*>(wk_g)[g * 8 + pos] = raw.x;
 #pragma unroll
                 for (int q = 0; q < KG; ++q)
                     if (q == g) r.gmin[q] = nm;
@@ -231,18 +235,17 @@ __device__ __forceinline__ void append_groups16(const uint32_t (&w)[8], const ui
 }
 
 template <int D, int KG, int NQT, int S, int ROOM, bool DUMP>
-__global__ void __launch_bounds__(kThreads16, 1)
+__global__ void __launch_bounds__(threads16(NQT), 1)
 score_select_f16x4_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                         const WorkItem* __restrict__ items, StatusBlock* __restrict__ sb, int H,
-                        uint32_t* __restrict__ cand_word, uint16_t* __restrict__ cand_half,
-                        float* __restrict__ dump, int n_total /* = N */, long long wait_limit, int drop_first_tile,
+                        const GroupLists lists, float* __restrict__ dump, int n_total /* = N */, long long wait_limit, int drop_first_tile,
                         const int* __restrict__ perm) {
     using Sh = Shape16<D>;
     using Sp = Plan16<KG, NQT, S, ROOM>;
     constexpr int NEPI = 4 * NQT;
-    constexpr int LIST = Sp::LIST;
+    constexpr int LIST = Sp::LIST, NISS = NQT;
     constexpr uint32_t TMEM_COLS = NBUF * BN;
-    static_assert(NQT == NISS && NQT == NBUF && kThreads16 == 32 * (4 * NQT + NISS), "one issuer and one accumulator buffer per query tile");
+    static_assert(NQT <= NBUF, "one issuer and one accumulator buffer per query tile");
 
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -307,7 +310,8 @@ score_select_f16x4_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_
     };
 
     const bool is_producer = warp == NEPI && lane == 0;
-    const int issuer = (warp > NEPI && warp < NEPI + NISS && lane == 0) ? warp - NEPI - 1 : (warp == NEPI && lane == 16) ? NISS - 1 : -1;
+    const int issuer = (warp > NEPI && warp < NEPI + 4 && lane == 0 && warp - NEPI - 1 < NISS) ? warp - NEPI - 1
+                       : (NISS == 4 && warp == NEPI && lane == 16)                                       ? 3 : -1;
     if (is_producer) {
         // ------------------------------------------------------------------ TMA producer
         {
@@ -409,14 +413,14 @@ score_select_f16x4_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_
             const bool active = qt * BM < it.nrows;
             const int local = qt * BM + quarter * 32 + lane;
             const bool rvalid = local < it.nrows;
-            if (active) row_init16<KG>(rs, wl, lane, rvalid);
+            if (active) row_init16<KG>(rs, wl, lane, rvalid, lists.slots);
             // the row's LIST group words in the output array: sweep order in, the row's own place out
-            uint32_t* wk_g = cand_word;
+            unsigned char* wk_g = lists.word;
             if (!DUMP && rvalid) {
                 const int srow = it.row0 + local;
                 const int orow = perm ? __ldg(perm + srow) : srow;
                 // checks builds: a row of the batch (a row that fails keeps writing to row 0's slots of the scratch list)
-                if (kmip_check(orow >= 0 && orow < n_total, sb, 103)) wk_g = cand_word + ((size_t)orow * H + h) * LIST;
+                if (kmip_check(orow >= 0 && orow < n_total, sb, 103)) wk_g = lists.word + ((long long)orow * H + h) * lists.word_pitch;
             }
             __syncwarp();
             const int ntiles = (it.key_hi - it.key_lo + BN - 1) / BN;
@@ -447,12 +451,13 @@ score_select_f16x4_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_
                 }
             } else {
                 const int ragged_j = ((it.key_hi - it.key_lo) & (BN - 1)) ? ntiles - 1 : -1;
-                int key0 = it.key_lo;
+                const int n_keys = it.key_hi - it.key_lo;
+                int key0 = lists.compact ? 0 : it.key_lo;  // how the group words count: inside the graph, or over the batch
                 for (int j = 0; j < ntiles; ++j, ++tcnt, key0 += BN) {
                     const uint32_t full_par = (uint32_t)tcnt & 1u;
                     if (!__all_sync(FULL, ptx::mbar_try_wait(full_bar, full_par))) {
                         // scores not there yet: merge pending groups meanwhile, then block
-                        if (__any_sync(FULL, rs.cnt > 0)) flush_pending16<KG>(rs, wl_s, wk_g, wp_addr, rvalid);
+                        if (__any_sync(FULL, rs.cnt > 0)) flush_pending16<KG>(rs, wl_s, wk_g, lists.compact, wp_addr, rvalid);
                         ok = wait_or_abort(full_bar, full_par, sAbort, sb, 6, wait_limit);
                         ok = __all_sync(FULL, ok);
                         if (!ok) break;
@@ -464,7 +469,7 @@ score_select_f16x4_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_
                     ptx::tc_fence_before();
                     __syncwarp();
                     if (lane == 0) ptx::mbar_arrive(empty_bar);  // the buffer goes straight back to its issuer
-                    if (j == ragged_j) tile_maxima16<true>(v, it.key_hi - key0, wm, qm, m);
+                    if (j == ragged_j) tile_maxima16<true>(v, n_keys - j * BN, wm, qm, m);
                     else tile_maxima16<false>(v, BN, wm, qm, m);
                     const int req = (int)ptx::lds_u32(flush_req_s);
                     bool do_flush = req != flush_seen;
@@ -478,7 +483,7 @@ score_select_f16x4_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_
                         }
                     }
                     if (do_flush) {
-                        flush_pending16<KG>(rs, wl_s, wk_g, wp_addr, rvalid);
+                        flush_pending16<KG>(rs, wl_s, wk_g, lists.compact, wp_addr, rvalid);
                         flush_seen = req + ((req == flush_seen) ? 1 : 0);
                     }
                 }
@@ -487,15 +492,16 @@ score_select_f16x4_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_
             if (!DUMP && active) {
                 // finalise: drain the pending slots, then store the fp16 maxima of each row's LIST groups beside
                 // the group words that are in place already (unsorted; an empty slot is marked by the half 0xFFFF)
-                flush_pending16<KG>(rs, wl_s, wk_g, wp_addr, rvalid);
+                flush_pending16<KG>(rs, wl_s, wk_g, lists.compact, wp_addr, rvalid);
                 __syncwarp();
                 const int nloc = min(32, it.nrows - (qt * BM + quarter * 32));
                 for (int r = 0; r < nloc; ++r) {
                     const int srow = it.row0 + qt * BM + quarter * 32 + r;  // sweep order; the result goes to the row's own place
-                    const size_t o = ((size_t)(perm ? __ldg(perm + srow) : srow) * H + h) * LIST;
-                    for (int t = lane; t < LIST; t += 32) {
+                    const int orow = perm ? __ldg(perm + srow) : srow;
+                    uint16_t* half = reinterpret_cast<uint16_t*>(lists.half + ((long long)orow * H + h) * lists.half_pitch);
+                    for (int t = lane; t < lists.slots; t += 32) {
                         const uint32_t c = wl[t * 32 + r];
-                        cand_half[o + t] = (uint16_t)(c ? unorder16(c) : 0xFFFFu);
+                        half[t] = (uint16_t)(c ? unorder16(c) : 0xFFFFu);
                     }
                 }
                 __syncwarp();
@@ -537,7 +543,7 @@ bool make_tensor_map16(CUtensorMap* tm, const void* base, int64_t rows, int64_t 
     const cuuint64_t gstride[1] = {(cuuint64_t)row_elems * 2};
     const cuuint32_t box[2] = {(cuuint32_t)D, 128u};
     const cuuint32_t estr[2] = {1u, 1u};
-    const CUtensorMapSwizzle sw = D == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B;
+    const CUtensorMapSwizzle sw = D == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : D == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B;
     return enc(tm, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, const_cast<void*>(base), gdim, gstride, box, estr,
                CU_TENSOR_MAP_INTERLEAVE_NONE, sw, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
@@ -551,35 +557,40 @@ cudaError_t launch_cfg(const FwdArgs& a, const FwdWorkspace& w, float* dump) {
                                   (size_t)Sp::NBARS * 8 + 64;
     static_assert(smem_bytes <= 232448, "shared memory budget of one CTA");
     CUtensorMap tmQ, tmK;
-    if (!make_tensor_map16<D>(&tmQ, a.ws + w.qperm_off, a.N, (int64_t)a.H * D) ||
-        !make_tensor_map16<D>(&tmK, a.ws + w.kpack_off, a.N * a.H, D))
+    const F16Buffers buf = f16_buffers(a, w);
+    if (!make_tensor_map16<D>(&tmQ, buf.q16, a.N, (int64_t)a.H * D) || !make_tensor_map16<D>(&tmK, buf.k16, a.N * a.H, D))
         return cudaErrorInvalidValue;
     auto kern = score_select_f16x4_kernel<D, KG, NQT, S, ROOM, DUMP>;
     cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
     if (err != cudaSuccess) return err;
     const long long max_total = (long long)w.max_items * a.H;
     const int grid = (int)std::min<long long>(sm_count(), max_total);
-    kern<<<grid, kThreads16, smem_bytes, a.stream>>>(
+    kern<<<grid, threads16(NQT), smem_bytes, a.stream>>>(
         tmQ, tmK, reinterpret_cast<const WorkItem*>(a.ws + w.items_off), reinterpret_cast<StatusBlock*>(a.ws), a.H,
-        reinterpret_cast<uint32_t*>(a.ws + w.cand_word_off), reinterpret_cast<uint16_t*>(a.ws + w.cand_half_off), dump,
-        (int)a.N, a.wait_limit_cycles > 0 ? a.wait_limit_cycles : kDefaultWaitLimitCycles, a.drop_first_tile,
+        buf.lists, dump, (int)a.N, a.wait_limit_cycles > 0 ? a.wait_limit_cycles : kDefaultWaitLimitCycles, a.drop_first_tile,
         (w.reorder && !DUMP) ? reinterpret_cast<const int*>(a.ws + w.perm_off) : nullptr);
     return cudaGetLastError();
 }
 
 template <int D, bool DUMP>
 cudaError_t launch_d(const FwdArgs& a, const FwdWorkspace& w, float* dump) {
-    // (list blocks, query tiles per CTA, key stages, pending slots per row) by k; shared memory decides
-    if (a.k <= 8) return launch_cfg<D, 2, 4, 4, 32, DUMP>(a, w, dump);
-    return launch_cfg<D, 3, 4, 4, 32, DUMP>(a, w, dump);
+    // (list blocks, query tiles per CTA, key stages, pending slots per row) by list length; shared memory decides
+    constexpr int NQ = D == 64 ? 3 : 4, S = D == 64 ? 3 : 4, ROOM = D == 64 ? 30 : 32;
+    if (w.list <= 16) return launch_cfg<D, 2, NQ, S, ROOM, DUMP>(a, w, dump);
+    if (DUMP) return cudaErrorInvalidValue;
+    if (w.list <= 24) return launch_cfg<D, 3, NQ, S, ROOM, false>(a, w, dump);
+    return launch_cfg<D, kF16List32 / 8, NQ, S, D == 16 ? 32 : 28, false>(a, w, dump);
 }
 
 }  // namespace
 
-int score_select_f16x4_rows_per_item() { return 4 * BM; }
-
 cudaError_t launch_score_select_f16x4(const FwdArgs& a, const FwdWorkspace& w) {
-    return a.d == 16 ? launch_d<16, false>(a, w, nullptr) : launch_d<32, false>(a, w, nullptr);
+    switch (a.d) {
+        case 16: return launch_d<16, false>(a, w, nullptr);
+        case 32: return launch_d<32, false>(a, w, nullptr);
+        case 64: return launch_d<64, false>(a, w, nullptr);
+        default: return cudaErrorInvalidValue;
+    }
 }
 
 // Test entry: the fp16 scores themselves (scaled as the converted operands are), dump[h][i][j], ld = N.

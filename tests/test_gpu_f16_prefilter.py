@@ -132,3 +132,32 @@ def test_few_undecidable_rows(n_tied, k):
     w.Q[rows] = 0.0
     st = _check(w, 0.98)
     assert st["redo"] == n_tied
+
+
+@pytest.mark.parametrize("sizes,H,d,k", [([1536], 1, 16, 4), ([1537, 3, 0, 700], 1, 32, 5), ([2500], 2, 16, 12), ([127, 129, 2000], 2, 64, 9),
+                                         ([5000], 1, 64, 32), ([3000], 1, 32, 17), ([9001], 1, 32, 31), ([40, 1, 700] * 3, 1, 16, 8)])
+def test_fp32_through_the_filter_is_the_same_bit_for_bit(sizes, H, d, k):
+    """fp32 storage, values that fp16 cannot hold exactly: the filter path (operand copies and lists in the output arrays)
+    against the one-warp-per-row kernel, which scores every key in fp32 - the same keys in the same order and the same
+    scores, bit for bit."""
+    N = sum(sizes)
+    g = torch.Generator().manual_seed(N + d + k)
+    Q, K, V = (torch.randn(N, H, d, generator=g).cuda() for _ in range(3))
+    Q[N // 2] *= 1e-3
+    offs = torch.tensor(np.concatenate([[0], np.cumsum(sizes)]), dtype=torch.int32, device="cuda")
+    a = kb.forward(Q, K, V, offs, k, kb.KMIP_FP32_EXACT)
+    b = kb.forward(Q, K, V, offs, k, kb.KMIP_FP32_EXACT, fp32_path=1)
+    assert torch.equal(a.topk_idx, b.topk_idx) and torch.equal(a.topk_score, b.topk_score) and torch.equal(a.out, b.out)
+
+
+def test_fp32_near_ties_beyond_half_precision():
+    """Keys that differ by a few fp32 ulps only: no fp16 score can tell them apart, the rows go to the exact kernel."""
+    g = torch.Generator().manual_seed(5)
+    N, d, k = 3000, 32, 16
+    Q = torch.randn(N, 1, d, generator=g)
+    K = torch.randn(5, 1, d, generator=g)[torch.arange(N) % 5] * (1 + 1e-6 * torch.randn(N, 1, 1, generator=g))
+    Q, K, V = Q.cuda(), K.cuda(), torch.randn(N, 1, d, generator=g).cuda()
+    a = kb.forward(Q, K, V, None, k, kb.KMIP_FP32_EXACT)
+    assert kb.kmip_attn_sweep_counters(a.workspace)[4] > 0
+    b = kb.forward(Q, K, V, None, k, kb.KMIP_FP32_EXACT, fp32_path=1)
+    assert torch.equal(a.topk_idx, b.topk_idx) and torch.equal(a.topk_score, b.topk_score) and torch.equal(a.out, b.out)
