@@ -80,7 +80,7 @@ int kmip_test_gemm_tn(const void *A, const void *B, void *C, int32_t M, int32_t 
  *   order[s]       = row number of the node the sweep handled at position s, s = 0 .. N-1
  *                    (the identity where the library keeps the row order: small problems, fp32 mode,
  *                    graphs below 8192 nodes);
- *   *rows_per_item = query rows per work item (128 x the query tiles a CTA owns; 128 in fp32 mode).
+ *   *rows_per_item = query rows per work item (128 x the query tiles a CTA owns).
  * N, G, H, d, k, mode: as passed to that forward call.  Errors as for kmip_attn_workspace_bytes,
  * KMIP_ERR_CUDA if the synchronisation or the copy fails.
  */

@@ -101,7 +101,7 @@ struct FwdWorkspace {
 constexpr int64_t kReorderMinNodes = 32768;  // below this the extra launches cost more than they can save
 
 bool score_select_tc_supported(int32_t d, int32_t k);
-bool score_select_f16_supported(int32_t d, int32_t k);
+bool score_select_f16_supported(int64_t N, int32_t d, int32_t k);
 bool score_select_f16_in_outputs_supported(int64_t N, int32_t H, int32_t d, int32_t k, int mode);
 int score_select_f16_list(int32_t k);
 int score_select_f16_list_in_outputs(int32_t k);
@@ -122,7 +122,7 @@ inline FwdWorkspace plan_fwd_workspace(int64_t N, int32_t G, int32_t H, int32_t 
     const int32_t g = G > 0 ? G : 1;
     w.tc = variant == kPlanByMode ? (mode != KMIP_FP32_EXACT && score_select_tc_supported(d, k))
                                   : variant != kPlanNoTensorCore;
-    w.f16 = variant == kPlanByMode ? (w.tc && mode == KMIP_BF16_TC && score_select_f16_supported(d, k))
+    w.f16 = variant == kPlanByMode ? (w.tc && mode == KMIP_BF16_TC && score_select_f16_supported(N, d, k))
                                    : variant == kPlanTcFp16Acc;
     w.in_outputs = variant == kPlanByMode && !w.f16 && score_select_f16_in_outputs_supported(N, H, d, k, mode);
     w.f16 = w.f16 || w.in_outputs;
@@ -333,6 +333,7 @@ constexpr int kMinRowsToSort = 8192;  // smaller graphs keep their row and key o
 // fp32 mode: smallest N * H that runs the half-precision prefilter.  Its launches cost about 100 us, and one warp per row
 // takes 58 us at 1024 rows (one graph, d = 32), 167 at 2048 (filter: 114) and 601 at 4096 (150).
 constexpr int64_t kF16MinRowsFp32 = 1536;
+constexpr int64_t kF16MinRowsWide = 2048;
 // score_select_exact.cu: CUDA-core scores + running top-k, any supported (d, k), fp32 or bf16 storage
 cudaError_t launch_score_select_exact(const FwdArgs& a);
 int sm_count();  // multiprocessors of the current device (cached per device)
@@ -342,7 +343,7 @@ int score_select_tc_rows_per_item(int32_t d, int32_t k);
 cudaError_t launch_score_select_tc(const FwdArgs& a, const FwdWorkspace& w);
 cudaError_t launch_score_dump_tc(const FwdArgs& a, const FwdWorkspace& w, float* dump);
 // Half-precision prefilter (k <= 32; bf16 storage: head widths 16, 32, 64, fp32 storage: the same on large problems):
-// f16_convert.cu (norm maxima, scaled fp16 copies of K and Q), score_select_f16.cu / score_select_f16x4.cu (sweeps),
+// f16_convert.cu (norm maxima, scaled fp16 copies of K and Q), score_select_f16.cu (sweep),
 // refine_f16.cu (exact rescoring, redo list), score_select_exact.cu (the listed rows again, from all keys)
 
 // The groups a row kept: `slots` entries per (node, head) row, the group and the fp16 maximum of its scores.
@@ -382,10 +383,9 @@ inline F16Buffers f16_buffers(const FwdArgs& a, const FwdWorkspace& w) {
     b.scratch_words = out_bytes > used ? (long long)((out_bytes - used) / 8) : 0;
     return b;
 }
-int score_select_f16_rows_per_item(const FwdWorkspace& w, int32_t d, int32_t k);
+int score_select_f16_rows_per_item(int32_t d);
 cudaError_t launch_f16_convert(const FwdArgs& a, const FwdWorkspace& w);
 cudaError_t launch_score_select_f16(const FwdArgs& a, const FwdWorkspace& w);
-cudaError_t launch_score_select_f16x4(const FwdArgs& a, const FwdWorkspace& w);  // called by the above
 cudaError_t launch_score_dump_f16(const FwdArgs& a, const FwdWorkspace& w, float* dump);
 cudaError_t launch_refine_f16(const FwdArgs& a, const FwdWorkspace& w);
 cudaError_t launch_score_select_exact_redo(const FwdArgs& a, const FwdWorkspace& w);

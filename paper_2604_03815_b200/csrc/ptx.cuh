@@ -18,6 +18,13 @@ __device__ __forceinline__ uint64_t globaltimer_ns() {
     return t;
 }
 
+// One lane of a converged warp.
+__device__ __forceinline__ bool elect_one() {
+    uint32_t r;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(r));
+    return r != 0;
+}
+
 // ------------------------------------------------------------------------------------ mbarrier
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
@@ -30,6 +37,9 @@ __device__ __forceinline__ void fence_proxy_async() {
 }
 __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void mbar_arrive_if(uint32_t bar, bool cond) {
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %1, 0;\n\t@p mbarrier.arrive.shared::cta.b64 _, [%0];\n\t}" ::"r"(bar), "r"((uint32_t)cond) : "memory");
 }
 __device__ __forceinline__ void mbar_arrive_expect_tx(uint32_t bar, uint32_t bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
@@ -221,6 +231,12 @@ __device__ __forceinline__ uint32_t lds_u32(uint32_t addr) {
     asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
     return v;
 }
+// counter in shared memory: what was written before an increment is seen by whoever reads a later count
+__device__ __forceinline__ uint32_t atom_add_shared(uint32_t addr, uint32_t v) {
+    uint32_t old;
+    asm volatile("atom.acq_rel.cta.shared::cta.add.u32 %0, [%1], %2;" : "=r"(old) : "r"(addr), "r"(v) : "memory");
+    return old;
+}
 __device__ __forceinline__ uint2 lds_v2(uint32_t addr) {
     uint2 v;
     asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(addr) : "memory");
@@ -268,7 +284,47 @@ __device__ __forceinline__ uint32_t hmax2(uint32_t a, uint32_t b) {
     asm("max.f16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
     return d;
 }
+__device__ __forceinline__ uint32_t hmin2(uint32_t a, uint32_t b) {
+    uint32_t d;
+    asm("min.f16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
+    return d;
+}
 __device__ __forceinline__ uint32_t hmax3(uint32_t a, uint32_t b, uint32_t c) { return hmax2(hmax2(a, b), c); }
+
+// Packed fp16 sums, and comparisons that give 1.0 or 0.0 in each half (false for not-a-number).
+__device__ __forceinline__ uint32_t hadd2(uint32_t a, uint32_t b) {
+    uint32_t d;
+    asm("add.rn.f16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
+    return d;
+}
+__device__ __forceinline__ uint32_t hge2(uint32_t a, uint32_t b) {
+    uint32_t d;
+    asm("set.ge.f16x2.f16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
+    return d;
+}
+__device__ __forceinline__ uint32_t hgt2(uint32_t a, uint32_t b) {
+    uint32_t d;
+    asm("set.gt.f16x2.f16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
+    return d;
+}
+// All ones in each half of the result where the half of `a` is above the half of `b`.
+__device__ __forceinline__ uint32_t hgt_mask2(uint32_t a, uint32_t b) {
+    uint32_t d;
+    asm("set.gt.u32.f16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
+    return d;
+}
+// The sum of both halves (small integers).
+__device__ __forceinline__ float half_sum(uint32_t a) {
+    float lo, hi;
+    asm("{\n\t.reg .b16 l, h;\n\tmov.b32 {l, h}, %2;\n\tcvt.f32.f16 %0, l;\n\tcvt.f32.f16 %1, h;\n\t}" : "=f"(lo), "=f"(hi) : "r"(a));
+    return lo + hi;
+}
+// fp16 comparison of the low halves (false for not-a-number)
+__device__ __forceinline__ bool half_ge(uint32_t a, uint32_t b) {
+    uint32_t r;
+    asm("{\n\t.reg .pred p;\n\tsetp.ge.f16 p, %1, %2;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(r) : "h"((uint16_t)a), "h"((uint16_t)b));
+    return r != 0;
+}
 
 // Does any lane of the warp hold a half of `m` above the same half of `t`?
 __device__ __forceinline__ bool warp_any_half_gt(uint32_t m, uint32_t t) {
@@ -283,6 +339,22 @@ __device__ __forceinline__ bool warp_any_half_gt(uint32_t m, uint32_t t) {
         "}"
         : "=r"(r)
         : "r"(m), "r"(t));
+    return r != 0;
+}
+// The same, or is `also` true in any lane?
+__device__ __forceinline__ bool warp_any_half_gt_or(uint32_t m, uint32_t t, bool also) {
+    uint32_t r;
+    asm volatile(
+        "{\n\t"
+        ".reg .pred p, q;\n\t"
+        "setp.gt.f16x2 p|q, %1, %2;\n\t"
+        "or.pred p, p, q;\n\t"
+        "setp.ne.or.u32 p, %3, 0, p;\n\t"
+        "vote.sync.any.pred p, p, 0xffffffff;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t"
+        "}"
+        : "=r"(r)
+        : "r"(m), "r"(t), "r"((uint32_t)also));
     return r != 0;
 }
 // Lanes of the warp that hold a half of `m` above the same half of `t`.

@@ -9,8 +9,7 @@
 //   2. The keys of the other groups are scored again - fp32 fused multiply-adds in index order (over bf16 values the
 //      mixed-precision instruction: exact product, one rounding, the same bits as convert + fmaf), read from K in place - and the k best under (score desc, key asc) are kept with the
 //      running top-k buffer of the CUDA-core kernel.
-//   3. If the sweep's list was full, groups it dropped have maxima at most g_min, the smallest one
-//      kept.  When g_min + err(g_min) reaches the k-th best exact score found, a dropped group could
+//   3. If the sweep dropped groups, these have maxima at most g_min, the smallest one kept.  When g_min + err(g_min) reaches the k-th best exact score found, a dropped group could
 //      still hold a better key: the row goes to the redo list and the exact CUDA-core kernel
 //      recomputes it from all keys.  That needs more than L groups within the error bound of the
 //      k-th best score, which well-separated scores never produce; rows whose keys tie massively do.
@@ -166,8 +165,7 @@ refine_f16_kernel(const T* __restrict__ Q, const T* __restrict__ K,
         int lo, hi;
         graph_range_of(offs, s_offs, G, N, i, lo, hi);
 
-        // empty slots: the four-pipeline sweep marks them by the half 0xFFFF and never writes their group word,
-        // the ring sweep writes an all-ones word
+        // empty slots: the sweep marks them by the half 0xFFFF and never writes their group word
         uint32_t word[EPL];
         unsigned okey[EPL];  // ordered 16-bit key of the group maximum; 0 for an empty slot (below every value)
         int n_valid = 0;
@@ -175,7 +173,7 @@ refine_f16_kernel(const T* __restrict__ Q, const T* __restrict__ K,
 #pragma unroll
         for (int e = 0; e < EPL; ++e) {
             word[e] = lists.compact ? (uint32_t)(lo + (int)(nx_word[e] >> 1) * 16) | (nx_word[e] << 31) : nx_word[e];
-            const bool valid = nx_half[e] != 0xFFFFu && (lists.compact || word[e] != 0xFFFFFFFFu);
+            const bool valid = nx_half[e] != 0xFFFFu;
             okey[e] = valid ? f16_ordered(nx_half[e]) : 0u;
             n_valid += __popc(__ballot_sync(FULL, valid));
             ok_min = min(ok_min, valid ? okey[e] : 0xFFFFu);
@@ -312,9 +310,10 @@ refine_f16_kernel(const T* __restrict__ Q, const T* __restrict__ K,
         }
         ptx::cp_async_wait<0>();
         const float kth = warp_merge_row_chunks(row, k, cnt, lane);
-        // a dropped group scores at most g_min + err(g_min) exactly (scaled); it matters if that reaches the
-        // k-th best score found
-        if (n_valid == lists.slots && g_min + ea + er * fabsf(g_min) >= kth * sc - fp32_err) {
+        // the sweep dropped a group unless the list holds every group of the graph; a dropped one scores at most
+        // g_min + err(g_min) exactly (scaled), and it matters if that reaches the k-th best score found
+        const int n_groups = 2 * ((hi - lo) / 16) + min((hi - lo) % 16, 2);
+        if (n_valid < n_groups && g_min + ea + er * fabsf(g_min) >= kth * sc - fp32_err) {
             if (lane == 0) {
                 const int pos = atomicAdd(&sb->n_redo, 1);
                 if (kmip_check(pos >= 0 && pos < n_rows, sb, 102)) redo_list[pos] = (int)r;  // checks builds: inside the list

@@ -1,5 +1,4 @@
-// Half-precision prefilter sweep (Algorithm 1 lines 2-3) of the tensor-core mode for head widths 16 and 32
-// and 16 < k <= 32 (other shapes and fp32 storage: score_select_f16x4.cu, the same filter on another pipeline).
+// Half-precision prefilter sweep (Algorithm 1 lines 2-3): k <= 32, head widths 16, 32 and 64, bf16 and fp32 storage.
 //
 // The paper lists half-precision arithmetic and tensor-core support as the engineering it left open
 // (Sec. 6; closing remark of the FlashAttention comparison in the appendix).  The sweep of
@@ -10,22 +9,39 @@
 // two to a register and reduces them with packed three-input maxima - half the registers and half the
 // instructions per score.  What it computes is a FILTER, not the answer:
 //   * Q and K are converted to fp16 after a power-of-two scaling per head that puts the largest row
-//     norm into [32, 64) (f16_convert.cu), so nothing overflows and the conversion is exact except for
+//     norm into [32, 64) (f16_convert.cu), so nothing overflows and a bf16 value converts exactly except for
 //     elements below 2^-14 of that;
 //   * a candidate is a group of 8 keys - the even or the odd keys of a window of 16 consecutive keys,
 //     which is what one packed register chain covers - ranked by the fp16 maximum of its scores;
-//   * every row keeps the L best groups, L = k + slack (16, 24, 48 for k <= 8, 16, 32), in an unsorted
-//     list in shared memory; a group that ties with the list's minimum is dropped;
+//   * every row keeps at least k + slack of its best groups (select_rows below); whatever it drops has a
+//     maximum at most the smallest one kept;
 //   * refine_f16.cu rescoring decides: it computes the exact fp32 scores of the kept groups' keys, proves
 //     from the error bound of the fp16 scores that no dropped group can hold one of the k best keys, and
-//     sends the rare row for which it cannot (more than L groups within the error bound of the k-th
-//     best) to the exact CUDA-core kernel.
+//     sends the rare row for which it cannot to the exact CUDA-core kernel.
 // The tensor cores round an fp16 accumulator to nearest after each 16-deep step (checked against the
-// exact sums on the device), so |fp16 score - exact scaled score| <= 2^-11 (|partial sum| + |result|)
-// for d = 32 and 2^-11 |result| for d = 16, plus the conversion's underflow terms.
+// exact sums on the device); f16_filter.cuh has the bound.
 //
-// Warp roles, barriers, the ring of four 128-column accumulator buffers, the CTA-wide flush counter,
-// the split tail of the persistent schedule and the bounded waits are those of score_select_tc.cu.
+// Pipeline.  Up to four 128-row query tiles per CTA (512 rows per work item, 16 selection warps: four per SM
+// sub-partition to hide each other's tensor-memory loads and dependent instruction chains), each with an accumulator
+// buffer and an MMA issuer of its own: four independent pipelines that meet only at the key stages.  A selection warp
+// hands its buffer back as soon as the scores are in registers and its issuer multiplies the next key tile while the
+// warp reduces the current one.  64-wide heads have three query tiles: the operand tiles take four times the shared
+// memory of 16-wide ones, and the MMA, 256 clocks a tile, bounds them anyway.
+//
+// Selection.  A row's entries (fp16 maximum, group number) sit in one column of shared memory.  A group that beats the
+// row's threshold is appended, nothing else; when a row runs out of room, all rows of the CTA raise their thresholds and
+// drop what falls below, each lane for its own row (all together: a query tile that stalls alone stalls the others
+// later, at the key stages).  Appending costs a few instructions, and the expected number of such rounds is the
+// logarithm of the number of tiles (a row of random scores appends L per e-fold of keys seen).
+//
+// Measured (us; before: an always exact list with one insertion at a time, issuers that were single lanes, one of them in
+// the producer's warp): 100k nodes, H 4, d 32, k 16 4160 -> 3650, k 30 5880 -> 4820; 31 623 nodes, H 1, d 16, k 10
+// 290 -> 243; point cloud of 300k nodes, k 32 29 900 -> 26 800; 64-wide heads (fp32-accumulate sweep before), 50 001
+// nodes, k 20 1975 -> 1445.  With thresholds that nothing beats the same loop takes 1090 to 1190 clocks per four tiles;
+// selection warps (37 packed maxima at half rate and ~25 other instructions per tile and warp) bound it, not the MMA.
+//
+// Persistent CTAs, head-major visiting order, the split tail of the schedule and the bounded waits are those of
+// score_select_tc.cu.
 #include <cuda.h>
 
 #include <algorithm>
@@ -43,14 +59,20 @@ namespace {
 constexpr int BM = 128;  // query rows per tile = TMEM lanes
 constexpr int BN = 128;  // keys per tile = accumulator columns
 constexpr unsigned FULL = 0xFFFFFFFFu;
-constexpr int NBUF = 4;  // accumulator buffers of BN columns: all 512 columns of tensor memory, used as a ring
+constexpr int NBUF = 4;  // accumulator buffers of BN columns: all 512 columns of tensor memory, one per query tile
 constexpr int kRelaxedPollNs = 100;
+// 16 selection warps and 4 service warps (the register file of an SM holds 96 registers for 640 threads; it is handed
+// out in units of four warps).  Service warp i issues the MMAs of query tile i, and service warp 0 the TMA loads as well.
+// The time from a buffer's release to the next commit is on every pipeline's critical path, so a service warp runs its
+// loop as one (operands in uniform registers, an elected lane issues) and has everything ready before it waits.
+constexpr int kServiceWarps = 4;
+constexpr int threads16(int nqt) { return (4 * nqt + kServiceWarps) * 32; }
 
 template <int D>
 struct Shape16 {
-    static_assert(D == 16 || D == 32, "the fp16 prefilter covers head widths 16 and 32");
+    static_assert(D == 16 || D == 32 || D == 64, "head widths of the fp16 prefilter");
     static constexpr int RB = D * 2;                       // bytes per operand row = swizzle span
-    static constexpr uint32_t LAYOUT = RB == 64 ? 4u : 6u;  // UMMA swizzle code (64-byte / 32-byte)
+    static constexpr uint32_t LAYOUT = RB == 128 ? 2u : RB == 64 ? 4u : 6u;  // UMMA swizzle code (128 / 64 / 32 bytes)
     static constexpr int KSTEPS = D / 16;                  // one tcgen05.mma covers 16 halves of depth
     static constexpr int TILE_BYTES = 128 * RB;
 };
@@ -70,13 +92,12 @@ __device__ __forceinline__ uint64_t make_desc16(uint32_t saddr) {
 // Instruction descriptor: fp16 accumulate (format 0), fp16 A and B (format 0), both K-major, M = 128, N = BN.
 constexpr uint32_t kInstrDesc16 = ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
 
-template <int KG, int NQT, int S, int ROOM>
+// CAP entries of 4 bytes per row: a warp's block of shared memory is slot-major (entry s of lane l at s * 128 + 4 l), so
+// that no access conflicts.
+template <int CAP, int NQT, int S>
 struct Plan16 {
-    static constexpr int LIST = 8 * KG;  // groups kept per row
-    // per row: LIST 16-bit scores, LIST 32-bit group words, ROOM pending 8-byte entries
-    static constexpr int ROW_BYTES = 6 * LIST + 8 * ROOM;
-    static constexpr int WARP_BYTES = 32 * ROW_BYTES;
-    static constexpr int NBARS = 3 + 2 * S + NBUF * NQT + NBUF;
+    static constexpr int WARP_BYTES = CAP * 128;
+    static constexpr int NBARS = 3 + 2 * S + 2 * NQT;
 };
 
 struct Bars {
@@ -87,8 +108,8 @@ struct Bars {
     __device__ uint32_t done() const { return base + 16; }
     __device__ uint32_t k_full(int s) const { return base + 8 * (3 + s); }
     __device__ uint32_t k_empty(int s) const { return base + 8 * (3 + S + s); }
-    __device__ uint32_t t_full(int b, int qt) const { return base + 8 * (3 + 2 * S + b * NQT + qt); }
-    __device__ uint32_t t_empty(int b) const { return base + 8 * (3 + 2 * S + NBUF * NQT + b); }
+    __device__ uint32_t t_full(int qt) const { return base + 8 * (3 + 2 * S + qt); }
+    __device__ uint32_t t_empty(int qt) const { return base + 8 * (3 + 2 * S + NQT + qt); }
 };
 
 template <int SLEEP_NS = 0>
@@ -104,86 +125,140 @@ __device__ __forceinline__ uint32_t order16(uint32_t h) { return (h ^ ((h & 0x80
 __device__ __forceinline__ uint32_t unorder16(uint32_t x) { return (x ^ ((x & 0x8000u) ? 0x8000u : 0xFFFFu)) & 0xFFFFu; }
 constexpr uint32_t kHalfNegInf2 = 0xFC00FC00u, kHalfPosInf2 = 0x7C007C00u;
 
-// Per-row selection state.  A warp's block of shared memory holds, slot-major so that lock-step loops
-// are bank-conflict free: the score plane (slot s of lane l: 16 bits at s*64 + 2l), the group-word plane
-// (32 bits at s*128 + 4l) and the pending entries (8 bytes at s*256 + 8l).  gmin caches the minimum of
-// each 8-slot block of the list and lmin the minimum of the list, which stays 0 (empty) until LIST
-// groups exist, so tau stays -inf until then.
-template <int KG>
+constexpr uint32_t kEmptyEntry = 0x7FFF0000u;  // not a number: no comparison keeps it, no maximum returns it
+
+// Groups of a graph are numbered 2 * (16-key window) + (odd keys); an entry holds the low 16 bits.  Graphs of more than
+// 2^19 keys have 2^16 groups per segment: the high bits of a KEPT entry wait in the row's own list in global memory (one
+// byte each), and rows are selected at every segment's end, so that all entries behind the kept ones are of the
+// current segment.
+constexpr int kSegTiles = (1 << 19) / BN;
+
 struct RowSel16 {
-    uint32_t gmin[KG];
-    uint32_t lmin;
-    uint32_t tau2;  // the row's threshold in both halves: fp16 maximum of the LIST-th best group so far
-    int cnt;
+    uint32_t pend;   // shared address of the row's next free entry
+    uint32_t tau2;   // the row's threshold in both halves
 };
 
-template <int KG>
-__device__ __forceinline__ void row_init16(RowSel16<KG>& r, uint16_t* wl, int lane, bool rvalid) {
-#pragma unroll 1
-    for (int s = 0; s < 8 * KG; ++s) wl[s * 32 + lane] = 0;
-#pragma unroll
-    for (int g = 0; g < KG; ++g) r.gmin[g] = 0u;
-    r.lmin = 0u;
-    r.tau2 = rvalid ? kHalfNegInf2 : kHalfPosInf2;
-    r.cnt = 0;
-}
+struct SelectTargets {
+    int lo, hi;  // entries a row should be left with: at least lo, at most hi (all, where it has fewer)
+};
 
-// All 32 lanes insert their pending groups into their own lists, in lock step.  A pending entry is
-// {group word, packed register}: bit 31 of the word says which half of the register is the group's score.
-template <int KG>
-__device__ __forceinline__ void flush_pending16(RowSel16<KG>& r, uint32_t wl_s, uint32_t wk_s, uint32_t wp_s, bool rvalid) {
-    const int maxc = __reduce_max_sync(FULL, r.cnt);
-    __syncwarp();
+// All lanes raise their rows' thresholds such that between lo and hi entries reach them, and drop the others.  The
+// threshold of a row is searched between its smallest and its largest entry, counting packed halves in registers: three
+// steps that interpolate (the entries above a threshold thin out exponentially), then bisection over the ordered 16-bit
+// values.  Where many entries tie and no threshold leaves a number in range, the smallest tied ones past `hi` are
+// dropped too.  `seg` >= 0: also keeps the high bytes at `hi_bytes` (`n_old` kept entries have one).
+// About 900 instructions a warp at CAP = 80.
+template <int CAP>
+__device__ __forceinline__ void select_rows(RowSel16& r, uint32_t base, SelectTargets t, bool raise, unsigned char* hi_bytes,
+                                            int seg, int& n_old) {
+    constexpr int NP = CAP / 2;
+    static_assert(CAP % 8 == 0, "entries are moved eight at a time");
+    const int cnt = (int)((r.pend - base) >> 7);
+    const int maxcnt = __reduce_max_sync(FULL, cnt);
+    uint32_t pk[NP];  // the maxima, two entries to a register
+    uint32_t top = kHalfNegInf2, bot = kHalfPosInf2;
+#pragma unroll
+    for (int i = 0; i < NP; ++i) {
+        uint32_t a = kEmptyEntry, b = kEmptyEntry;
+        if (2 * i < cnt) a = ptx::lds_u32(base + (uint32_t)(2 * i) * 128u);
+        if (2 * i + 1 < cnt) b = ptx::lds_u32(base + (uint32_t)(2 * i + 1) * 128u);
+        pk[i] = __byte_perm(a, b, 0x7632);
+        top = ptx::hmax2(top, pk[i]);
+        bot = ptx::hmin2(bot, pk[i]);
+    }
+    auto value = [](uint32_t ordered) { return __half2float(__ushort_as_half((unsigned short)unorder16(ordered))); };
+    // invariants of the search: c_lo > t.hi entries reach `lo`, c_hi < t.lo reach `hi`
+    uint32_t lo = min(order16(bot & 0xFFFFu), order16(bot >> 16)), hi = max(order16(top & 0xFFFFu), order16(top >> 16)) + 1u;
+    float c_lo = (float)cnt, c_hi = 0.0f;
+    uint32_t thr = lo;
+    const bool keep_all = cnt <= t.hi && !(raise && cnt >= t.lo);
+    bool done = cnt <= t.hi, tie = false;  // a row with lo .. hi entries only raises its threshold to the smallest
+    const float want = 0.5f * (float)(t.lo + t.hi);
 #pragma unroll 1
-    for (int t = 0; t < maxc; ++t) {
-        if (t < r.cnt) {
-            const uint2 raw = ptx::lds_v2(wp_s + (uint32_t)t * 256u);
-            const uint32_t x = order16((raw.x >> 31) ? (raw.y >> 16) : (raw.y & 0xFFFFu));
-            if (x > r.lmin) {
-                int g = 0;
-                uint32_t m = r.gmin[0];
+    for (int step = 0; !__all_sync(FULL, done); ++step) {
+        uint32_t mid = (lo + hi) >> 1;
+        if (step < 3) {
+            const float f = __logf(c_lo / want) / __logf(c_lo / fmaxf(c_hi, 0.7f));
+            const float x = value(lo), g = x + f * (value(hi) - x);
+            mid = min(max(order16(__half_as_ushort(__float2half_rn(g))), lo + 1u), hi - 1u);
+        }
+        const uint32_t h = unorder16(mid), h2 = h | (h << 16);
+        uint32_t c2 = 0u, d2 = 0u;  // counts as packed fp16 numbers: exact up to 2048
 #pragma unroll
-                for (int q = 1; q < KG; ++q)
-                    if (r.gmin[q] < m) { m = r.gmin[q]; g = q; }
-                const uint32_t grp = wl_s + (uint32_t)g * (8u * 64u);
-                uint32_t nm = x;
-                int pos = -1;
+        for (int i = 0; i < NP; i += 2) {
+            c2 = ptx::hadd2(c2, ptx::hge2(pk[i], h2));
+            d2 = ptx::hadd2(d2, ptx::hge2(pk[i + 1], h2));
+        }
+        const float c = ptx::half_sum(ptx::hadd2(c2, d2));
+        if (!done) {
+            if (c >= (float)t.lo && c <= (float)t.hi) { thr = mid; done = true; }
+            else if (c > (float)t.hi) { lo = mid; c_lo = c; }
+            else { hi = mid; c_hi = c; }
+            if (!done && hi - lo <= 1u) { thr = lo; done = tie = true; }
+        }
+    }
+    const uint32_t th = keep_all ? 0xFC00u : unorder16(thr), th2 = th | (th << 16);
+    uint32_t out = base;
+    if (seg < 0 && !__any_sync(FULL, tie)) {
 #pragma unroll
-                for (int s = 0; s < 8; ++s) {
-                    const uint32_t y = ptx::lds_u16(grp + s * 64);
-                    if (y == m && pos < 0) pos = s; else nm = min(nm, y);
-                }
-                ptx::sts_u16(grp + (uint32_t)pos * 64u, x);
-                ptx::sts_u32(wk_s + (uint32_t)(g * 8 + pos) * 128u, raw.x);
+        for (int i = 0; i < NP; i += 4) {
+            if (2 * i < maxcnt) {  // warp-uniform
+                uint32_t e[8];
 #pragma unroll
-                for (int q = 0; q < KG; ++q)
-                    if (q == g) r.gmin[q] = nm;
-                uint32_t lm = r.gmin[0];
+                for (int x = 0; x < 8; ++x) e[x] = ptx::lds_u32(base + (uint32_t)(2 * i + x) * 128u);
 #pragma unroll
-                for (int q = 1; q < KG; ++q) lm = min(lm, r.gmin[q]);
-                r.lmin = lm;
+                for (int x = 0; x < 4; ++x)
+                    asm volatile(
+                        "{\n\t"
+                        ".reg .pred p, q;\n\t"
+                        "setp.ge.f16x2 p|q, %1, %2;\n\t"
+                        "@p st.shared.b32 [%0], %3;\n\t"
+                        "@p add.u32 %0, %0, 128;\n\t"
+                        "@q st.shared.b32 [%0], %4;\n\t"
+                        "@q add.u32 %0, %0, 128;\n\t"
+                        "}"
+                        : "+r"(out)
+                        : "r"(pk[i + x]), "r"(th2), "r"(e[2 * x]), "r"(e[2 * x + 1])
+                        : "memory");
             }
         }
+    } else {
+        // rare: ties, or a graph of several segments
+        uint32_t c2 = 0u;
+#pragma unroll
+        for (int i = 0; i < NP; ++i) c2 = ptx::hadd2(c2, ptx::hgt2(pk[i], th2));
+        int budget = tie ? t.hi - (int)ptx::half_sum(c2) : CAP;  // of entries equal to the threshold (zeros of either sign too)
+        int n_new = 0;
+#pragma unroll 1
+        for (int s = 0; s < cnt; ++s) {
+            const uint32_t e = ptx::lds_u32(base + (uint32_t)s * 128u);
+            bool keep = ptx::half_ge(e >> 16, th);
+            if (keep && ptx::half_ge(th, e >> 16) && budget-- <= 0) keep = false;
+            if (keep) {
+                ptx::sts_u32(out, e);
+                if (seg >= 0) hi_bytes[n_new] = s < n_old ? hi_bytes[s] : (unsigned char)seg;
+                out += 128u;
+                ++n_new;
+            }
+        }
+        n_old = n_new;
+        __syncwarp();
     }
-    r.cnt = 0;
-    if (rvalid) {
-        const uint32_t t = r.lmin ? unorder16(r.lmin) : 0xFC00u;
-        r.tau2 = t | (t << 16);
-    }
+    r.pend = out;
+    if (!keep_all) r.tau2 = th2;
 }
 
-// Packed maxima of a row's 128 scores: w[j] covers the 16-key window j (low half: its even keys, high
-// half: its odd keys), q[c] the 32 keys of quad c, m the tile.  RAGGED: columns at or past `nvalid`
-// do not exist (end of the key range).
-template <bool RAGGED>
-__device__ __forceinline__ void tile_maxima16(uint32_t (&v)[64], int nvalid, uint32_t (&w)[8], uint32_t (&q)[4], uint32_t& m) {
-    if (RAGGED) {
+// Columns at or past `nvalid` do not exist (end of the key range).
+__device__ __forceinline__ void mask_ragged16(uint32_t (&v)[64], int nvalid) {
 #pragma unroll
-        for (int x = 0; x < 64; ++x) {
-            if (2 * x >= nvalid) v[x] = kHalfNegInf2;
-            else if (2 * x + 1 >= nvalid) v[x] = (v[x] & 0xFFFFu) | 0xFC000000u;
-        }
+    for (int x = 0; x < 64; ++x) {
+        if (2 * x >= nvalid) v[x] = kHalfNegInf2;
+        else if (2 * x + 1 >= nvalid) v[x] = (v[x] & 0xFFFFu) | 0xFC000000u;
     }
+}
+// Packed maxima of a row's 128 scores: w[j] covers the 16-key window j (low half: its even keys, high half: its odd
+// keys), m the tile.
+__device__ __forceinline__ void tile_maxima16(const uint32_t (&v)[64], uint32_t (&w)[8], uint32_t& m) {
     uint32_t a[8], b[8];
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
@@ -195,54 +270,45 @@ __device__ __forceinline__ void tile_maxima16(uint32_t (&v)[64], int nvalid, uin
     for (int j = 0; j < 8; ++j) a[j] = ptx::hmax3(v[8 * j + 6], v[8 * j + 7], a[j]);
 #pragma unroll
     for (int j = 0; j < 8; ++j) w[j] = ptx::hmax2(a[j], b[j]);
-#pragma unroll
-    for (int c = 0; c < 4; ++c) q[c] = ptx::hmax2(w[2 * c], w[2 * c + 1]);
-    m = ptx::hmax2(ptx::hmax3(q[0], q[1], q[2]), q[3]);
+    m = ptx::hmax2(ptx::hmax3(ptx::hmax3(w[0], w[1], w[2]), w[3], w[4]), ptx::hmax3(w[5], w[6], w[7]));
 }
 
-// Lists the groups of a row's tile whose maximum beats tau.  Control flow is warp-uniform: a quad is
-// visited when any lane has a hit in it (one vote); inside it each window costs one packed compare and
-// two predicated (8-byte store, pointer bump) pairs.  `pend`: shared address of the lane's next free slot.
-__device__ __forceinline__ void append_groups16(const uint32_t (&w)[8], const uint32_t (&q)[4], uint32_t tau2, int key0,
-                                                uint32_t& pend) {
-    unsigned hit[4];
+// Appends the groups of a row's tile whose maximum beats tau (at most 16): per window one packed compare and two
+// predicated (4-byte store, pointer bump) pairs, without branches.  `id`: number of the tile's first group (its low 16
+// bits count).
+__device__ __forceinline__ void append_groups16(const uint32_t (&w)[8], uint32_t tau2, uint32_t id, uint32_t& pend) {
+    uint32_t ids = (id & 0xFFFFu) | ((id + 1u) << 16);  // of the even and the odd keys of a window
 #pragma unroll
-    for (int c = 0; c < 4; ++c) hit[c] = ptx::warp_ballot_half_gt(q[c], tau2);
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-        if (hit[c]) {
-#pragma unroll
-            for (int j = 2 * c; j < 2 * c + 2; ++j) {
-                asm volatile(
-                    "{\n\t"
-                    ".reg .pred p, q;\n\t"
-                    "setp.gt.f16x2 p|q, %1, %2;\n\t"
-                    "@p st.shared.v2.b32 [%0], {%3, %1};\n\t"
-                    "@p add.u32 %0, %0, 256;\n\t"
-                    "@q st.shared.v2.b32 [%0], {%4, %1};\n\t"
-                    "@q add.u32 %0, %0, 256;\n\t"
-                    "}"
-                    : "+r"(pend)
-                    : "r"(w[j]), "r"(tau2), "r"(key0 + 16 * j), "r"((key0 + 16 * j) | 0x80000000u)
-                    : "memory");
-            }
-        }
+    for (int j = 0; j < 8; ++j) {
+        asm volatile(
+            "{\n\t"
+            ".reg .pred p, q;\n\t"
+            ".reg .b32 a, b;\n\t"
+            "setp.gt.f16x2 p|q, %1, %2;\n\t"
+            "prmt.b32 a, %3, %1, 0x5410;\n\t"
+            "prmt.b32 b, %3, %1, 0x7632;\n\t"
+            "@p st.shared.b32 [%0], a;\n\t"
+            "@p add.u32 %0, %0, 128;\n\t"
+            "@q st.shared.b32 [%0], b;\n\t"
+            "@q add.u32 %0, %0, 128;\n\t"
+            "}"
+            : "+r"(pend)
+            : "r"(w[j]), "r"(tau2), "r"(ids + (uint32_t)j * 0x00020002u)
+            : "memory");
     }
 }
 
-template <int D, int KG, int NQT, int S, int ROOM, bool DUMP>
-__global__ void __launch_bounds__(NQT * 128 + 96, 1)
+template <int D, int CAP, int NQT, int S, bool DUMP>
+__global__ void __launch_bounds__(threads16(NQT), 1)
 score_select_f16_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                         const WorkItem* __restrict__ items, StatusBlock* __restrict__ sb, int H,
-                        uint32_t* __restrict__ cand_word, uint16_t* __restrict__ cand_half,
-                        float* __restrict__ dump, int n_total /* = N */, long long wait_limit, int drop_first_tile,
+                        const GroupLists lists, SelectTargets target, float* __restrict__ dump, int n_total /* = N */, long long wait_limit, int drop_first_tile,
                         const int* __restrict__ perm) {
     using Sh = Shape16<D>;
-    using Sp = Plan16<KG, NQT, S, ROOM>;
+    using Sp = Plan16<CAP, NQT, S>;
     constexpr int NEPI = 4 * NQT;
-    constexpr int NISS = 2;
-    constexpr int LIST = Sp::LIST;
     constexpr uint32_t TMEM_COLS = NBUF * BN;
+    static_assert(NQT <= NBUF && NQT <= kServiceWarps && S >= 3, "an accumulator buffer and an issuer per query tile");
 
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -252,25 +318,25 @@ score_select_f16_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
     uint64_t* sBars = reinterpret_cast<uint64_t*>(sRows + NEPI * Sp::WARP_BYTES);
     uint32_t* sTmem = reinterpret_cast<uint32_t*>(sBars + Sp::NBARS);
     volatile int* sAbort = reinterpret_cast<volatile int*>(sTmem + 1);
-    volatile int* sFlushReq = reinterpret_cast<volatile int*>(sTmem + 2);
+    volatile int* sSelectReq = reinterpret_cast<volatile int*>(sTmem + 2);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     Bars bars{ptx::smem_u32(sBars), S, NQT};
 
     if (threadIdx.x == 0) {
         ptx::mbar_init(bars.q_full(), 1);
-        ptx::mbar_init(bars.q_empty(), NISS);
-        ptx::mbar_init(bars.done(), NISS);
+        ptx::mbar_init(bars.q_empty(), NQT);
+        ptx::mbar_init(bars.done(), NQT);
         for (int s = 0; s < S; ++s) {
             ptx::mbar_init(bars.k_full(s), 1);
             ptx::mbar_init(bars.k_empty(s), NQT);
         }
-        for (int b = 0; b < NBUF; ++b) {
-            for (int q = 0; q < NQT; ++q) ptx::mbar_init(bars.t_full(b, q), 1);
-            ptx::mbar_init(bars.t_empty(b), 4);
+        for (int q = 0; q < NQT; ++q) {
+            ptx::mbar_init(bars.t_full(q), 1);
+            ptx::mbar_init(bars.t_empty(q), 4);  // the four selection warps of the query tile
         }
         *sAbort = 0;
-        *sFlushReq = 0;
+        *sSelectReq = 0;
         ptx::fence_barrier_init();
         ptx::fence_proxy_async();
     }
@@ -306,108 +372,116 @@ score_select_f16_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
         return it.nrows > 0;
     };
 
-    if (warp == NEPI) {
-        // ------------------------------------------------------------------ TMA producer
-        if (lane == 0) {
-            int kt = 0, ic = 0;
+    if (warp >= NEPI) {
+        // ------------------------------------------------------------------ service warps
+        // Issuer `mine` multiplies every key tile against query tile `mine` into accumulator buffer `mine` and commits to
+        // that tile's barrier; its four selection warps hand the buffer back as soon as the scores are in their
+        // registers.  Every issuer waits for every key tile (a parity wait is sound only on a barrier whose every phase
+        // the waiter observes).  Warp 0 loads key tiles S - 1 ahead of the one it multiplies, so the stage it refills was
+        // last read two tiles ago and is free as a rule; the query tiles are loaded when the unit before is done.
+        const int mine = warp - NEPI;
+        if (mine < NQT) {
+            const bool producer = mine == 0;
             bool ok = true;
+            // producer's place in the sequence of all key tiles of this CTA
+            long long pw = blockIdx.x;
+            int ph = 0, pj = 0, pn = 0, pkt = 0, ps = 0;
+            WorkItem pit{};
+            auto next_unit = [&] {  // the producer's next unit with any tiles
+                for (pn = 0; pn == 0 && pw < n_units; pw += gridDim.x)
+                    if (unit(pw, ph, pit)) { pn = (pit.key_hi - pit.key_lo + BN - 1) / BN; pj = 0; }
+            };
+            auto produce_up_to = [&](int kt_end) {  // key tiles of the CTA before number kt_end are loaded or on their way
+                while (ok && pn > 0 && pkt < kt_end) {
+                    ok = wait_or_abort<kRelaxedPollNs>(bars.k_empty(ps), ((pkt / S) & 1) ^ 1, sAbort, sb, 2, wait_limit);
+                    ok = __all_sync(FULL, ok);
+                    if (!ok) break;
+                    // failure-detection test option: CTA 0 never loads its first key tile
+                    if (!(drop_first_tile && blockIdx.x == 0 && pkt == 0) && ptx::elect_one()) {
+                        ptx::mbar_arrive_expect_tx(bars.k_full(ps), Sh::TILE_BYTES);
+                        ptx::tma_load_2d(ptx::smem_u32(sK + ps * Sh::TILE_BYTES), &tmK, 0, ph * n_total + pit.key_lo + pj * BN, bars.k_full(ps));
+                    }
+                    __syncwarp();
+                    ++pkt;
+                    ps = ps + 1 == S ? 0 : ps + 1;
+                    if (++pj == pn) next_unit();
+                }
+            };
+            if (producer) next_unit();
+            const uint64_t desc_q = make_desc16<D>(ptx::smem_u32(sQ + mine * Sh::TILE_BYTES));
+            const uint32_t d_tmem = tmem_base + (uint32_t)(mine * BN), full_bar = bars.t_full(mine), empty_bar = bars.t_empty(mine);
+            int kt = 0, s = 0, ic = 0;
+            uint32_t k_par = 0;  // parity of the tile's pass through the ring
             for (long long w = blockIdx.x; ok && w < n_units; w += gridDim.x) {
                 int h;
                 WorkItem it;
                 if (!unit(w, h, it)) continue;
-                if (!(ok = wait_or_abort<kRelaxedPollNs>(bars.q_empty(), (ic & 1) ^ 1, sAbort, sb, 1, wait_limit))) break;
-                ptx::mbar_arrive_expect_tx(bars.q_full(), NQT * Sh::TILE_BYTES);
-                for (int qt = 0; qt < NQT; ++qt)
-                    ptx::tma_load_2d(ptx::smem_u32(sQ + qt * Sh::TILE_BYTES), &tmQ, h * D, it.row0 + qt * BM, bars.q_full());
-                const int ntiles = (it.key_hi - it.key_lo + BN - 1) / BN;
-                for (int j = 0; j < ntiles; ++j, ++kt) {
-                    const int s = kt % S;
-                    if (!(ok = wait_or_abort<kRelaxedPollNs>(bars.k_empty(s), ((kt / S) & 1) ^ 1, sAbort, sb, 2, wait_limit))) break;
-                    // failure-detection test option: CTA 0 never loads its first key tile
-                    if (drop_first_tile && blockIdx.x == 0 && kt == 0) continue;
-                    ptx::mbar_arrive_expect_tx(bars.k_full(s), Sh::TILE_BYTES);
-                    ptx::tma_load_2d(ptx::smem_u32(sK + s * Sh::TILE_BYTES), &tmK, 0, h * n_total + it.key_lo + j * BN,
-                                     bars.k_full(s));
-                }
-                ++ic;
-            }
-            if (!ok) {
-                // give copies that are still in flight a bounded time to land before the CTA exits
-                const long long t0 = clock64();
-                for (int s = 0; s < S && kt > 0; ++s) {
-                    const int last = kt - 1 - ((kt - 1 - s) % S + S) % S;
-                    if (last < 0) continue;
-                    while (!ptx::mbar_try_wait(bars.k_full(s), (last / S) & 1) && clock64() - t0 < 40000000ll) {}
-                }
-            }
-        }
-    } else if (warp >= NEPI + 1 && warp <= NEPI + NISS) {
-        // ------------------------------------------------------------------ MMA issuers
-        // Pair number q of the CTA's (key tile, query tile) sequence uses accumulator buffer q mod 4; two
-        // threads take the pairs alternately; the commit goes to a barrier per (buffer, query tile); both
-        // issuers wait for every key tile (a parity wait is sound only on a barrier whose every phase the
-        // waiter observes).
-        if (lane == 0) {
-            const int mine = warp - (NEPI + 1);
-            uint64_t desc_q[NQT][Sh::KSTEPS], desc_k0[Sh::KSTEPS];
-#pragma unroll
-            for (int ks = 0; ks < Sh::KSTEPS; ++ks) {
-#pragma unroll
-                for (int qt = 0; qt < NQT; ++qt) desc_q[qt][ks] = make_desc16<D>(ptx::smem_u32(sQ + qt * Sh::TILE_BYTES + ks * 32));
-                desc_k0[ks] = make_desc16<D>(ptx::smem_u32(sK + ks * 32));
-            }
-            int kt = 0, ic = 0;
-            bool ok = true;
-            for (long long w = blockIdx.x; ok && w < n_units; w += gridDim.x) {
-                int h_unused;
-                WorkItem it;
-                if (!unit(w, h_unused, it)) continue;
-                const int nq = (it.nrows + BM - 1) / BM;
-                if (!(ok = wait_or_abort<0>(bars.q_full(), ic & 1, sAbort, sb, 3, wait_limit))) break;
-                ptx::tc_fence_after();
-                const int ntiles = (it.key_hi - it.key_lo + BN - 1) / BN;
-                for (int j = 0; ok && j < ntiles; ++j, ++kt) {
-                    const int s = kt % S;
-                    const uint64_t stage_off = (uint64_t)((s * Sh::TILE_BYTES) >> 4);
-                    if (!(ok = wait_or_abort<0>(bars.k_full(s), (kt / S) & 1, sAbort, sb, 4, wait_limit))) break;
-#pragma unroll
-                    for (int qt = 0; qt < NQT; ++qt) {
-                        const int seq = kt * NQT + qt;
-                        if ((seq & 1) != mine) continue;
-                        const int b = seq & (NBUF - 1);
-                        if (!(ok = wait_or_abort<0>(bars.t_empty(b), ((seq >> 2) & 1) ^ 1, sAbort, sb, 5, wait_limit))) break;
-                        ptx::tc_fence_after();
-                        if (qt < nq) {
-                            const uint32_t d_tmem = tmem_base + (uint32_t)(b * BN);
-#pragma unroll
-                            for (int ks = 0; ks < Sh::KSTEPS; ++ks)
-                                ptx::mma_f16_ss(d_tmem, desc_q[qt][ks], desc_k0[ks] + stage_off, kInstrDesc16, ks > 0 ? 1u : 0u);
-                        }
-                        ptx::mma_commit(bars.t_full(b, qt));
+                const bool active = mine * BM < it.nrows;
+                if (producer) {
+                    ok = wait_or_abort<0>(bars.q_empty(), (ic & 1) ^ 1, sAbort, sb, 1, wait_limit);
+                    ok = __all_sync(FULL, ok);
+                    if (!ok) break;
+                    if (ptx::elect_one()) {
+                        ptx::mbar_arrive_expect_tx(bars.q_full(), NQT * Sh::TILE_BYTES);
+                        for (int qt = 0; qt < NQT; ++qt)
+                            ptx::tma_load_2d(ptx::smem_u32(sQ + qt * Sh::TILE_BYTES), &tmQ, h * D, it.row0 + qt * BM, bars.q_full());
                     }
+                    __syncwarp();
+                }
+                const int ntiles = (it.key_hi - it.key_lo + BN - 1) / BN;
+                if (producer) produce_up_to(kt + S - 1);
+                ok = ok && wait_or_abort<0>(bars.q_full(), ic & 1, sAbort, sb, 3, wait_limit);
+                ok = __all_sync(FULL, ok);
+                for (int j = 0; ok && j < ntiles; ++j, ++kt) {
+                    if (producer) produce_up_to(kt + S - 1);
+                    const uint64_t desc_k = make_desc16<D>(ptx::smem_u32(sK) + (uint32_t)(s * Sh::TILE_BYTES));
+                    ok = ok && wait_or_abort<0>(bars.k_full(s), k_par, sAbort, sb, 4, wait_limit) &&
+                         wait_or_abort<0>(empty_bar, (kt & 1) ^ 1, sAbort, sb, 5, wait_limit);
+                    ok = __all_sync(FULL, ok);
+                    if (!ok) break;
+                    ptx::tc_fence_after();
+                    if (ptx::elect_one()) {
+                        if (active) {
+#pragma unroll
+                            for (int ks = 0; ks < Sh::KSTEPS; ++ks)  // 16 values of depth = 32 bytes of a row
+                                ptx::mma_f16_ss(d_tmem, desc_q + (uint64_t)(2 * ks), desc_k + (uint64_t)(2 * ks), kInstrDesc16, ks > 0 ? 1u : 0u);
+                        }
+                        ptx::mma_commit(full_bar);
+                        // the scores of the tile before have been read, so its stage has been read too
+                        if (kt > 0) ptx::mbar_arrive(bars.k_empty(s == 0 ? S - 1 : s - 1));
+                    }
+                    __syncwarp();
+                    if (++s == S) { s = 0; k_par ^= 1u; }
                 }
                 if (!ok) break;
-                ptx::mma_commit(bars.q_empty());
+                if (ptx::elect_one()) ptx::mma_commit(bars.q_empty());
+                __syncwarp();
                 ++ic;
             }
-            ptx::mma_commit(bars.done());
-            const long long t0 = clock64();
-            while (!ptx::mbar_try_wait(bars.done(), 0) && clock64() - t0 < 2000000000ll) {}
+            if (ptx::elect_one()) {
+                ptx::mma_commit(bars.done());
+                // bounded, like every wait: MMAs, and after a failed wait also copies that are still in flight
+                const long long t0 = clock64();
+                while (!ptx::mbar_try_wait(bars.done(), 0) && clock64() - t0 < 2000000000ll) {}
+                if (producer && !ok) {
+                    for (int x = 0; x < S && pkt > 0; ++x) {
+                        const int last = pkt - 1 - ((pkt - 1 - x) % S + S) % S;
+                        if (last < 0) continue;
+                        while (!ptx::mbar_try_wait(bars.k_full(x), (last / S) & 1) && clock64() - t0 < 2000000000ll) {}
+                    }
+                }
+            }
+            __syncwarp();
         }
-    } else if (warp < NEPI) {
+    } else {
         // ------------------------------------------------------------------ selection warps
         const int qt = warp >> 2, quarter = warp & 3;
-        uint8_t* wblock = sRows + (size_t)warp * Sp::WARP_BYTES;
-        uint16_t* wl = reinterpret_cast<uint16_t*>(wblock);                    // score plane
-        uint32_t* wk = reinterpret_cast<uint32_t*>(wblock + LIST * 64);        // group-word plane
-        const uint32_t wl_s = ptx::smem_u32(wl + lane);
-        const uint32_t wk_s = ptx::smem_u32(wk + lane);
-        const uint32_t wp_addr = ptx::smem_u32(wblock + LIST * 192) + 8u * lane;  // this lane's first pending slot
-        const uint32_t flush_req_s = ptx::smem_u32(const_cast<int*>(sFlushReq));
-        const uint32_t full_bar0 = bars.t_full(0, qt);
-        const uint32_t taddr0 = tmem_base + ((uint32_t)(quarter * 32) << 16);
-        RowSel16<KG> rs;
-        int flush_seen = 0;
+        const uint32_t row_base = ptx::smem_u32(sRows + (size_t)warp * Sp::WARP_BYTES) + 4u * lane;  // the row's first entry
+        const uint32_t full_bar = bars.t_full(qt), empty_bar = bars.t_empty(qt);
+        const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(qt * BN);
+        const uint32_t select_req_s = ptx::smem_u32(const_cast<int*>(sSelectReq));
+        RowSel16 rs;
+        int select_seen = 0;
         int tcnt = 0;
         bool ok = true;
         for (long long w = blockIdx.x; ok && w < n_units; w += gridDim.x) {
@@ -417,24 +491,30 @@ score_select_f16_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
             const bool active = qt * BM < it.nrows;
             const int local = qt * BM + quarter * 32 + lane;
             const bool rvalid = local < it.nrows;
-            if (active) row_init16<KG>(rs, wl, lane, rvalid);
+            // the row's place in the list arrays: sweep order in, the row's own place out
+            long long list_row = 0;
+            if (!DUMP && rvalid) {
+                const int srow = it.row0 + local;
+                const int orow = perm ? __ldg(perm + srow) : srow;
+                // checks builds: a row of the batch (a row that fails keeps to row 0's slots of the scratch list)
+                if (kmip_check(orow >= 0 && orow < n_total, sb, 103)) list_row = (long long)orow * H + h;
+            }
+            unsigned char* const list_word = lists.word + list_row * lists.word_pitch;
+            rs.pend = row_base;
+            rs.tau2 = rvalid ? kHalfNegInf2 : kHalfPosInf2;
             __syncwarp();
             const int ntiles = (it.key_hi - it.key_lo + BN - 1) / BN;
-            constexpr int kUseShift = NQT == 2 ? 1 : 2;
             if (DUMP || !active) {
                 for (int j = 0; j < ntiles; ++j, ++tcnt) {
-                    const int b = (tcnt * NQT + qt) & (NBUF - 1);
-                    ok = wait_or_abort(full_bar0 + (uint32_t)b * (8u * NQT), (uint32_t)(tcnt >> kUseShift) & 1u, sAbort, sb,
-                                       6, wait_limit);
+                    ok = wait_or_abort(full_bar, (uint32_t)tcnt & 1u, sAbort, sb, 6, wait_limit);
                     ok = __all_sync(FULL, ok);
                     if (!ok) break;
-                    if (quarter == 0 && lane == 0) ptx::mbar_arrive(bars.k_empty(tcnt % S));
                     ptx::tc_fence_after();
                     if (DUMP && active) {
                         const int key0 = it.key_lo + j * BN;
                         const int ncol = min(BN, it.key_hi - key0);
                         uint32_t v[64];
-                        ptx::tmem_ld_32x128_pack16_sync(taddr0 + (uint32_t)(b * BN), v);
+                        ptx::tmem_ld_32x128_pack16_sync(taddr, v);
                         if (rvalid) {
 #pragma unroll
                             for (int x = 0; x < 64; ++x) {
@@ -446,68 +526,81 @@ score_select_f16_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                     }
                     ptx::tc_fence_before();
                     __syncwarp();
-                    if (lane == 0) ptx::mbar_arrive(bars.t_empty(b));
+                    if (lane == 0) ptx::mbar_arrive(empty_bar);
                 }
             } else {
-                const int ragged_j = ((it.key_hi - it.key_lo) & (BN - 1)) ? ntiles - 1 : -1;
-                int key0 = it.key_lo;
-                for (int j = 0; j < ntiles; ++j, ++tcnt, key0 += BN) {
-                    const int b = (tcnt * NQT + qt) & (NBUF - 1);
-                    const uint32_t full_bar = full_bar0 + (uint32_t)b * (8u * NQT);
-                    const uint32_t full_par = (uint32_t)(tcnt >> kUseShift) & 1u;
-                    if (!__all_sync(FULL, ptx::mbar_try_wait(full_bar, full_par))) {
-                        // scores not there yet: merge pending groups meanwhile, then block
-                        if (__any_sync(FULL, rs.cnt > 0)) flush_pending16<KG>(rs, wl_s, wk_s, wp_addr, rvalid);
-                        ok = wait_or_abort(full_bar, full_par, sAbort, sb, 6, wait_limit);
+                const int n_keys = it.key_hi - it.key_lo;
+                const int ragged_j = (n_keys & (BN - 1)) ? ntiles - 1 : -1;
+                const bool segmented = ntiles > kSegTiles;
+                // next tile that is not like the others: a segment's last, or the last of all, which may be ragged
+                int special_j = segmented ? kSegTiles - 1 : ntiles - 1;
+                int n_old = 0;
+                uint32_t par = (uint32_t)tcnt & 1u;
+                for (int j = 0; j < ntiles; ++j, par ^= 1u) {
+                    if (!__all_sync(FULL, ptx::mbar_try_wait(full_bar, par))) {
+                        ok = wait_or_abort(full_bar, par, sAbort, sb, 6, wait_limit);
                         ok = __all_sync(FULL, ok);
                         if (!ok) break;
                     }
-                    if (quarter == 0 && lane == 0) ptx::mbar_arrive(bars.k_empty(tcnt % S));
                     ptx::tc_fence_after();
-                    uint32_t v[64], wm[8], qm[4], m;
-                    ptx::tmem_ld_32x128_pack16_sync(taddr0 + (uint32_t)(b * BN), v);
+                    uint32_t v[64], wm[8], m;
+                    ptx::tmem_ld_32x128_pack16_sync(taddr, v);
                     ptx::tc_fence_before();
                     __syncwarp();
-                    if (lane == 0) ptx::mbar_arrive(bars.t_empty(b));  // the buffer goes straight back to the issuers
-                    if (j == ragged_j) tile_maxima16<true>(v, it.key_hi - key0, wm, qm, m);
-                    else tile_maxima16<false>(v, BN, wm, qm, m);
-                    const int req = (int)ptx::lds_u32(flush_req_s);
-                    bool do_flush = req != flush_seen;
-                    if (ptx::warp_any_half_gt(m, rs.tau2)) {  // some lane of the warp has a hit in this tile
-                        uint32_t pend = wp_addr + (uint32_t)rs.cnt * 256u;
-                        append_groups16(wm, qm, rs.tau2, key0, pend);
-                        rs.cnt = (int)((pend - wp_addr) >> 8);
-                        if (__any_sync(FULL, rs.cnt > ROOM - 16)) {  // a tile adds at most 16 groups per row
-                            do_flush = true;
-                            if (lane == 0 && req == flush_seen) atomicAdd(const_cast<int*>(sFlushReq), 1);
+                    ptx::mbar_arrive_if(empty_bar, lane == 0);  // the buffer goes straight back to its issuer
+                    const int req = (int)ptx::lds_u32(select_req_s);
+                    if (j == special_j && j == ragged_j) mask_ragged16(v, n_keys - j * BN);
+                    tile_maxima16(v, wm, m);
+                    // some lane of the warp has a hit in this tile, or it is time to select
+                    if (!ptx::warp_any_half_gt_or(m, rs.tau2, req != select_seen || j == special_j)) continue;
+                    append_groups16(wm, rs.tau2, (uint32_t)j * 16u, rs.pend);
+                    bool select = j == special_j || req != select_seen;
+                    if (__any_sync(FULL, rs.pend > row_base + (uint32_t)(CAP - 16) * 128u)) {  // a row may have no room for the next tile
+                        select = true;
+                        if (req == select_seen) {  // the whole CTA selects now: the pipelines stall together, not in turn
+                            if (lane == 0) atomicAdd(const_cast<int*>(sSelectReq), 1);
+                            ++select_seen;
                         }
                     }
-                    if (do_flush) {
-                        flush_pending16<KG>(rs, wl_s, wk_s, wp_addr, rvalid);
-                        flush_seen = req + ((req == flush_seen) ? 1 : 0);
+                    if (select) {
+                        // at the end a row keeps all that its list can hold
+                        const bool last = j == ntiles - 1;
+                        const SelectTargets t = last ? SelectTargets{lists.slots - 2, lists.slots} : target;
+                        select_rows<CAP>(rs, row_base, t, !last, list_word, segmented ? j / kSegTiles : -1, n_old);
+                        select_seen = max(select_seen, req);
+                        if (j == special_j) special_j = min(special_j + kSegTiles, ntiles - 1);
                     }
                 }
+                tcnt += ntiles;
+                if (ok && rvalid) {
+                    // each lane stores its row's groups and maxima, two at a time (unsorted; an empty slot is marked by the
+                    // half 0xFFFF and its group is not written)
+                    unsigned char* const list_half = lists.half + list_row * lists.half_pitch;
+                    const int cnt = (int)((rs.pend - row_base) >> 7);
+                    // high bytes first: they lie where the words go, and word s only covers bytes 4 s and up
+                    for (int s = (lists.slots - 1) & ~1; s >= 0; s -= 2) {
+                        uint32_t e[2];
+#pragma unroll
+                        for (int x = 0; x < 2; ++x) e[x] = s + x < cnt ? ptx::lds_u32(row_base + (uint32_t)(s + x) * 128u) : 0xFFFF0000u;
+                        *reinterpret_cast<uint32_t*>(list_half + 2 * s) = __byte_perm(e[0], e[1], 0x7632);
+                        if (s >= cnt) continue;
+                        if (lists.compact) {
+                            *reinterpret_cast<uint32_t*>(list_word + 2 * s) = __byte_perm(e[0], e[1], 0x5410);
+                        } else {
+                            uint32_t word[2];
+#pragma unroll
+                            for (int x = 0; x < 2; ++x) {
+                                uint32_t id = e[x] & 0xFFFFu;
+                                if (segmented && s + x < cnt) id |= (uint32_t)list_word[s + x] << 16;
+                                word[x] = ((uint32_t)it.key_lo + (id >> 1) * 16u) | (id << 31);
+                            }
+                            *reinterpret_cast<uint2*>(list_word + 4 * s) = make_uint2(word[0], word[1]);
+                        }
+                    }
+                }
+                __syncwarp();
             }
             if (!ok) break;
-            if (!DUMP && active) {
-                // finalise: drain the pending slots, then store each row's LIST groups (group word and fp16
-                // maximum, unsorted; empty slots as all-ones / -inf) for the rescoring kernel
-                flush_pending16<KG>(rs, wl_s, wk_s, wp_addr, rvalid);
-                __syncwarp();
-                const int nloc = min(32, it.nrows - (qt * BM + quarter * 32));
-                for (int r = 0; r < nloc; ++r) {
-                    const int srow = it.row0 + qt * BM + quarter * 32 + r;  // sweep order; the result goes to the row's own place
-                    const int orow = perm ? __ldg(perm + srow) : srow;
-                    if (!kmip_check(orow >= 0 && orow < n_total, sb, 103)) continue;  // checks builds: a row of the batch
-                    const size_t o = ((size_t)orow * H + h) * LIST;
-                    for (int t = lane; t < LIST; t += 32) {
-                        const uint32_t c = wl[t * 32 + r];
-                        cand_word[o + t] = c ? wk[t * 32 + r] : 0xFFFFFFFFu;
-                        cand_half[o + t] = (uint16_t)(c ? unorder16(c) : 0xFC00u);
-                    }
-                }
-                __syncwarp();
-            }
         }
     }
 
@@ -545,65 +638,76 @@ bool make_tensor_map16(CUtensorMap* tm, const void* base, int64_t rows, int64_t 
     const cuuint64_t gstride[1] = {(cuuint64_t)row_elems * 2};
     const cuuint32_t box[2] = {(cuuint32_t)D, 128u};
     const cuuint32_t estr[2] = {1u, 1u};
-    const CUtensorMapSwizzle sw = D == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B;
+    const CUtensorMapSwizzle sw = D == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : D == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B;
     return enc(tm, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, const_cast<void*>(base), gdim, gstride, box, estr,
                CU_TENSOR_MAP_INTERLEAVE_NONE, sw, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <int D, int KG, int NQT, int S, int ROOM, bool DUMP>
+// Entries a row is left with before the end: about as many as its list holds at the end (k + slack: fewer would send
+// more rows to the exact kernel, more would be appended more often).  The width of the range saves search steps.
+SelectTargets select_targets(int slots) { return {slots - 2, slots + 6}; }
+
+template <int D, int CAP, int NQT, int S, bool DUMP>
 cudaError_t launch_cfg(const FwdArgs& a, const FwdWorkspace& w, float* dump) {
     using Sh = Shape16<D>;
-    using Sp = Plan16<KG, NQT, S, ROOM>;
+    using Sp = Plan16<CAP, NQT, S>;
     constexpr size_t smem_bytes = 1024 + (size_t)(NQT + S) * Sh::TILE_BYTES + (size_t)4 * NQT * Sp::WARP_BYTES +
                                   (size_t)Sp::NBARS * 8 + 64;
     static_assert(smem_bytes <= 232448, "shared memory budget of one CTA");
     CUtensorMap tmQ, tmK;
-    if (!make_tensor_map16<D>(&tmQ, a.ws + w.qperm_off, a.N, (int64_t)a.H * D) ||
-        !make_tensor_map16<D>(&tmK, a.ws + w.kpack_off, a.N * a.H, D))
+    const F16Buffers buf = f16_buffers(a, w);
+    if (!make_tensor_map16<D>(&tmQ, buf.q16, a.N, (int64_t)a.H * D) || !make_tensor_map16<D>(&tmK, buf.k16, a.N * a.H, D))
         return cudaErrorInvalidValue;
-    auto kern = score_select_f16_kernel<D, KG, NQT, S, ROOM, DUMP>;
+    auto kern = score_select_f16_kernel<D, CAP, NQT, S, DUMP>;
     cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
     if (err != cudaSuccess) return err;
     const long long max_total = (long long)w.max_items * a.H;
     const int grid = (int)std::min<long long>(sm_count(), max_total);
-    kern<<<grid, NQT * 128 + 96, smem_bytes, a.stream>>>(
+    kern<<<grid, threads16(NQT), smem_bytes, a.stream>>>(
         tmQ, tmK, reinterpret_cast<const WorkItem*>(a.ws + w.items_off), reinterpret_cast<StatusBlock*>(a.ws), a.H,
-        reinterpret_cast<uint32_t*>(a.ws + w.cand_word_off), reinterpret_cast<uint16_t*>(a.ws + w.cand_half_off), dump,
-        (int)a.N, a.wait_limit_cycles > 0 ? a.wait_limit_cycles : kDefaultWaitLimitCycles, a.drop_first_tile,
+        buf.lists, select_targets(w.list), dump, (int)a.N, a.wait_limit_cycles > 0 ? a.wait_limit_cycles : kDefaultWaitLimitCycles, a.drop_first_tile,
         (w.reorder && !DUMP) ? reinterpret_cast<const int*>(a.ws + w.perm_off) : nullptr);
     return cudaGetLastError();
 }
 
-template <int D, bool DUMP>
-cudaError_t launch_d(const FwdArgs& a, const FwdWorkspace& w, float* dump) {
-    // (list blocks, query tiles per CTA, key stages, pending slots per row); shared memory decides
-    // the per-warp block of shared memory stays at 14848 bytes: 192 per list slot, 256 per pending slot
-    return launch_cfg<D, kF16List32 / 8, 3, 3, (14848 - kF16List32 * 192) / 256, DUMP>(a, w, dump);
+template <int D>
+cudaError_t launch_d(const FwdArgs& a, const FwdWorkspace& w) {
+    // entries per row by list length, as far as shared memory goes
+    constexpr int NQ = D == 64 ? 3 : 4, S = D == 16 ? 4 : 3;
+    if (w.list <= 24) return launch_cfg<D, 72, NQ, S, false>(a, w, nullptr);
+    return launch_cfg<D, D == 16 ? 96 : 80, NQ, S, false>(a, w, nullptr);
 }
 
 }  // namespace
 
-// Lists in the workspace (bf16 storage).
-bool score_select_f16_supported(int32_t d, int32_t k) { return (d == 16 || d == 32) && k <= 32; }
+// Lists in the workspace (bf16 storage); a graph has at most 256 segments.
+bool score_select_f16_supported(int64_t N, int32_t d, int32_t k) { return (d == 16 || d == 32) && k <= 32 && N <= 256ll * kSegTiles * BN; }
 int score_select_f16_list(int32_t k) { return k <= 8 ? 16 : k <= 16 ? 24 : kF16List32; }
 
 // Lists in the output arrays: a row's topk_idx and topk_score hold 2 k entries of two 16-bit numbers, so the groups are
 // numbered inside their graph (up to 2^16 of 8 keys) and k + slack <= 2 k, which wants k >= 4.
 int score_select_f16_list_in_outputs(int32_t k) { return std::min(2 * k, k <= 8 ? 16 : k <= 16 ? 24 : kF16List32); }
 bool score_select_f16_in_outputs_supported(int64_t N, int32_t H, int32_t d, int32_t k, int mode) {
-    if (k < 4 || k > 32 || N > (1 << 19)) return false;
-    return mode == KMIP_FP32_EXACT && (d == 16 || d == 32 || d == 64) && N * H >= kF16MinRowsFp32;
+    if (k < 4 || k > 32 || N > (1 << 19) || (d != 16 && d != 32 && d != 64)) return false;
+    if (mode == KMIP_FP32_EXACT) return N * H >= kF16MinRowsFp32;
+    return mode == KMIP_BF16_TC && d == 64 && N * H >= kF16MinRowsWide;
 }
 
-// k in 17..32 with lists in the workspace runs the ring above with 384-row work items; everything else the kernel of
-// score_select_f16x4.cu with 512-row work items (384 for 64-wide heads: shared memory)
-static bool ring(const FwdWorkspace& w, int32_t k) { return !w.in_outputs && k > 16; }
-int score_select_f16_rows_per_item(const FwdWorkspace& w, int32_t d, int32_t k) { return ring(w, k) || d == 64 ? 3 * BM : 4 * BM; }
+int score_select_f16_rows_per_item(int32_t d) { return (d == 64 ? 3 : 4) * BM; }
 
 cudaError_t launch_score_select_f16(const FwdArgs& a, const FwdWorkspace& w) {
-    if (!ring(w, a.k)) return launch_score_select_f16x4(a, w);
-    return a.d == 16 ? launch_d<16, false>(a, w, nullptr) : launch_d<32, false>(a, w, nullptr);
+    switch (a.d) {
+        case 16: return launch_d<16>(a, w);
+        case 32: return launch_d<32>(a, w);
+        case 64: return launch_d<64>(a, w);
+        default: return cudaErrorInvalidValue;
+    }
+}
+
+// Test entry: the fp16 scores themselves (scaled as the converted operands are), dump[h][i][j], ld = N.
+cudaError_t launch_score_dump_f16(const FwdArgs& a, const FwdWorkspace& w, float* dump) {
+    return a.d == 16 ? launch_cfg<16, 64, 4, 4, true>(a, w, dump) : launch_cfg<32, 64, 4, 3, true>(a, w, dump);
 }
 
 }  // namespace kmip

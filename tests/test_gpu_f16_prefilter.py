@@ -161,3 +161,20 @@ def test_fp32_near_ties_beyond_half_precision():
     assert kb.kmip_attn_sweep_counters(a.workspace)[4] > 0
     b = kb.forward(Q, K, V, None, k, kb.KMIP_FP32_EXACT, fp32_path=1)
     assert torch.equal(a.topk_idx, b.topk_idx) and torch.equal(a.topk_score, b.topk_score) and torch.equal(a.out, b.out)
+
+
+def test_graph_of_several_segments():
+    """More than 2^19 keys: the entries of a row number their groups inside a segment, the kept ones carry its number along.
+    Against dense fp32 scores of sampled rows; the best keys of every row are planted in the first and the last segment."""
+    N, d, k = (1 << 19) + 70_001, 16, 6
+    g = torch.Generator(device="cuda").manual_seed(11)
+    Q, K, V = (torch.randn(N, 1, d, device="cuda", generator=g).to(torch.bfloat16) for _ in range(3))
+    for j in (3, (1 << 19) - 1, 1 << 19, N - 1):
+        K[j] = K[j] * 4
+    fb = kb.forward(Q, K, V, None, k, kb.KMIP_BF16_TC)
+    rows = torch.randint(0, N, (256,), device="cuda", generator=g)
+    dense = Q[rows, 0].float() @ K[:, 0].float().T
+    best = dense.topk(k, dim=1).values
+    got = dense.gather(1, fb.topk_idx[rows, 0].long())
+    assert torch.all((got - best).abs() <= 1e-4 * best.abs() + 1e-4)
+    assert all(len(set(r)) == k for r in fb.topk_idx[rows, 0].tolist())
