@@ -114,6 +114,7 @@ int forward_impl(const void* Q, const void* K, const void* V, const int32_t* gra
     if (mode == KMIP_FP32_EXACT && opt && opt->fp32_path != 0) w.f16 = w.in_outputs = false;  // a test picks the CUDA-core sweep
     const bool tc = w.tc;
     if (workspace_bytes < w.total) return KMIP_ERR_WORKSPACE;
+    if (w.f16) w.item_tiles = score_select_f16_item_tiles(N, graph_offsets ? G : 1, H, d);
 
     FwdArgs a{Q, K, V, graph_offsets, graph_offsets ? G : 1, N, H, d, k, mode, out, topk_idx, topk_score,
               static_cast<unsigned char*>(workspace), static_cast<cudaStream_t>(stream)};
@@ -134,7 +135,7 @@ int forward_impl(const void* Q, const void* K, const void* V, const int32_t* gra
     // 0.70 ms at 64 blocks, 1.7 against 8.4 ms at 247), slower below (0.25 against 0.19 ms at 32)
     const bool tiled32 = mode == KMIP_FP32_EXACT && !w.f16 && score_select_fp32_tiled_supported(d, k) &&
                          (a.fp32_path == 0 ? (N / 128) * H >= 48 : a.fp32_path == 2);
-    if (launch_plan(a, w, w.f16 ? score_select_f16_rows_per_item(d) : tc ? score_select_tc_rows_per_item(d, k) : 128) !=
+    if (launch_plan(a, w, w.f16 ? 128 * w.item_tiles : tc ? score_select_tc_rows_per_item(d, k) : 128) !=
         cudaSuccess)
         return KMIP_ERR_CUDA;
     if (w.reorder && launch_reorder_queries(a, w) != cudaSuccess) return KMIP_ERR_CUDA;
@@ -379,8 +380,9 @@ int kmip_test_sweep_order(const void* workspace, int64_t N, int32_t G, int32_t H
     const int rc = check_shape(N, H, d, k, mode);
     if (rc != KMIP_OK) return rc;
     if (!workspace || !order || !rows_per_item || G < 0) return KMIP_ERR_INVALID_ARG;
-    const FwdWorkspace w = plan_fwd_workspace(N, G > 0 ? G : 1, H, d, k, mode);
-    *rows_per_item = w.f16 ? score_select_f16_rows_per_item(d) : w.tc ? score_select_tc_rows_per_item(d, k) : 128;
+    FwdWorkspace w = plan_fwd_workspace(N, G > 0 ? G : 1, H, d, k, mode);
+    if (w.f16) w.item_tiles = score_select_f16_item_tiles(N, G > 0 ? G : 1, H, d);
+    *rows_per_item = w.f16 ? 128 * w.item_tiles : w.tc ? score_select_tc_rows_per_item(d, k) : 128;
     if (cudaStreamSynchronize(static_cast<cudaStream_t>(stream)) != cudaSuccess) return KMIP_ERR_CUDA;
     if (w.reorder) {
         if (cudaMemcpy(order, static_cast<const unsigned char*>(workspace) + w.perm_off, (size_t)N * 4,
@@ -415,12 +417,13 @@ int kmip_test_f16_scores(const void* Q, const void* K, int64_t N, int32_t H, int
     if (rc != KMIP_OK) return rc;
     if (d > 32) return KMIP_ERR_UNSUPPORTED;
     if (!Q || !K || !scores || !scales || !workspace || N < 1 || N > 8192) return KMIP_ERR_INVALID_ARG;
-    const FwdWorkspace w = plan_fwd_workspace(N, 1, H, d, 1, KMIP_BF16_TC, kPlanTcFp16Acc);
+    FwdWorkspace w = plan_fwd_workspace(N, 1, H, d, 1, KMIP_BF16_TC, kPlanTcFp16Acc);
+    w.item_tiles = score_select_f16_item_tiles(N, 1, H, d);
     if (workspace_bytes < w.total) return KMIP_ERR_WORKSPACE;
     FwdArgs a{Q, K, nullptr, nullptr, 1, N, H, d, 1, KMIP_BF16_TC, nullptr, nullptr, nullptr,
               static_cast<unsigned char*>(workspace), static_cast<cudaStream_t>(stream)};
     if (cudaMemsetAsync(a.ws, 0, kStatusBytes, a.stream) != cudaSuccess) return KMIP_ERR_CUDA;
-    if (launch_plan(a, w, score_select_f16_rows_per_item(d)) != cudaSuccess) return KMIP_ERR_CUDA;
+    if (launch_plan(a, w, 128 * w.item_tiles) != cudaSuccess) return KMIP_ERR_CUDA;
     if (launch_f16_convert(a, w) != cudaSuccess) return KMIP_ERR_CUDA;
     if (launch_score_dump_f16(a, w, scores) != cudaSuccess) return KMIP_ERR_CUDA;
     // per head: {q_n2max, k_n2max, k_first16_n2max, 0} as the conversion measured them

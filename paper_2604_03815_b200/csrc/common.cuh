@@ -88,6 +88,8 @@ struct FwdWorkspace {
     size_t total;
     int max_items;
     int max_tiles;
+    int item_tiles;    // 128-row query tiles per work item of the half-precision prefilter (set where the plan is used:
+                       // sizing a workspace makes no CUDA call)
     int list;          // groups kept per row by the half-precision prefilter
     bool tc;           // a tensor-core sweep runs (bf16 storage and a supported (d, k))
     bool f16;          // the half-precision prefilter runs (bf16: instead of that sweep; fp32: instead of the CUDA-core ones)
@@ -105,6 +107,7 @@ bool score_select_f16_supported(int64_t N, int32_t d, int32_t k);
 bool score_select_f16_in_outputs_supported(int64_t N, int32_t H, int32_t d, int32_t k, int mode);
 int score_select_f16_list(int32_t k);
 int score_select_f16_list_in_outputs(int32_t k);
+int score_select_f16_item_tiles(int64_t N, int32_t G, int32_t H, int32_t d);
 
 // Which sweep the plan is for: the one the mode selects, or one a test entry point asks for.
 enum PlanVariant { kPlanByMode = 0, kPlanNoTensorCore = 1, kPlanTcFp32Acc = 2, kPlanTcFp16Acc = 3,
@@ -127,6 +130,7 @@ inline FwdWorkspace plan_fwd_workspace(int64_t N, int32_t G, int32_t H, int32_t 
     w.in_outputs = variant == kPlanByMode && !w.f16 && score_select_f16_in_outputs_supported(N, H, d, k, mode);
     w.f16 = w.f16 || w.in_outputs;
     w.list = w.in_outputs ? score_select_f16_list_in_outputs(k) : w.f16 ? score_select_f16_list(k) : 0;
+    w.item_tiles = 0;
     w.max_items = (int)(N / 128 + g + 1);
     w.items_off = region(kStatusBytes);
     w.kpack_off = region(w.items_off + sizeof(WorkItem) * (size_t)w.max_items);
@@ -383,7 +387,6 @@ inline F16Buffers f16_buffers(const FwdArgs& a, const FwdWorkspace& w) {
     b.scratch_words = out_bytes > used ? (long long)((out_bytes - used) / 8) : 0;
     return b;
 }
-int score_select_f16_rows_per_item(int32_t d);
 cudaError_t launch_f16_convert(const FwdArgs& a, const FwdWorkspace& w);
 cudaError_t launch_score_select_f16(const FwdArgs& a, const FwdWorkspace& w);
 cudaError_t launch_score_dump_f16(const FwdArgs& a, const FwdWorkspace& w, float* dump);

@@ -85,7 +85,7 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar, uint32_t parity,
     if (mbar_try_wait(bar, parity)) return true;
     uint32_t spins = 0;
     long long t0 = 0;
-    while (!mbar_try_wait_suspend(bar, parity, 20000u)) {
+    while (!mbar_try_wait(bar, parity)) {
         if (SLEEP_NS > 0) __nanosleep(SLEEP_NS);
         if ((++spins & 15u) == 0u) {
             if (*abort_flag) return false;

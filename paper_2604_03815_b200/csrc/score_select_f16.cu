@@ -23,7 +23,7 @@
 //
 // Pipeline.  Up to four 128-row query tiles per CTA (512 rows per work item, 16 selection warps: four per SM
 // sub-partition to hide each other's tensor-memory loads and dependent instruction chains), each with an accumulator
-// buffer and an MMA issuer of its own: four independent pipelines that meet only at the key stages.  A selection warp
+// buffer of its own: four independent pipelines that meet only at the key stages.  A selection warp
 // hands its buffer back as soon as the scores are in registers and its issuer multiplies the next key tile while the
 // warp reduces the current one.  64-wide heads have three query tiles: the operand tiles take four times the shared
 // memory of 16-wide ones, and the MMA, 256 clocks a tile, bounds them anyway.
@@ -35,10 +35,11 @@
 // logarithm of the number of tiles (a row of random scores appends L per e-fold of keys seen).
 //
 // Measured (us; before: an always exact list with one insertion at a time, issuers that were single lanes, one of them in
-// the producer's warp): 100k nodes, H 4, d 32, k 16 4160 -> 3650, k 30 5880 -> 4820; 31 623 nodes, H 1, d 16, k 10
-// 290 -> 243; point cloud of 300k nodes, k 32 29 900 -> 26 800; 64-wide heads (fp32-accumulate sweep before), 50 001
-// nodes, k 20 1975 -> 1445.  With thresholds that nothing beats the same loop takes 1090 to 1190 clocks per four tiles;
-// selection warps (37 packed maxima at half rate and ~25 other instructions per tile and warp) bound it, not the MMA.
+// the producer's warp): 303 104 nodes, H 1, d 32, k 16 7250 -> 6020, d 16, k 8 6220 -> 5580; 100k nodes, H 4, d 32, k 30
+// 5880 -> 4480; 31 623 nodes, H 1, d 16, k 10 291 -> 236; 64-wide heads (fp32-accumulate sweep before), 151 552 nodes,
+// k 16 2990 -> 2100.  With thresholds that nothing beats the loop takes 850 to 980 clocks per four tiles (540 to 580 in
+// isolation, 1100 when the producer was one of the issuers); the hits of unstructured inputs add a quarter at 300k
+// nodes and as much again at 100k with k = 30.
 //
 // Persistent CTAs, head-major visiting order, the split tail of the schedule and the bounded waits are those of
 // score_select_tc.cu.
@@ -62,10 +63,11 @@ constexpr unsigned FULL = 0xFFFFFFFFu;
 constexpr int NBUF = 4;  // accumulator buffers of BN columns: all 512 columns of tensor memory, one per query tile
 constexpr int kRelaxedPollNs = 100;
 // 16 selection warps and 4 service warps (the register file of an SM holds 96 registers for 640 threads; it is handed
-// out in units of four warps).  Service warp i issues the MMAs of query tile i, and service warp 0 the TMA loads as well.
-// The time from a buffer's release to the next commit is on every pipeline's critical path, so a service warp runs its
-// loop as one (operands in uniform registers, an elected lane issues) and has everything ready before it waits.
-constexpr int kServiceWarps = 4;
+// out in units of four warps): the TMA producer, and three issuers, of which the first has query tiles 0 and 3.
+// The time from a buffer's release to the next commit is on every pipeline's critical path, so an issuer runs its loop
+// as a whole warp (operands in uniform registers, an elected lane issues), has everything ready before it waits, and
+// does nothing else.
+constexpr int kServiceWarps = 4, kIssuers = kServiceWarps - 1;
 constexpr int threads16(int nqt) { return (4 * nqt + kServiceWarps) * 32; }
 
 template <int D>
@@ -136,6 +138,7 @@ constexpr int kSegTiles = (1 << 19) / BN;
 struct RowSel16 {
     uint32_t pend;   // shared address of the row's next free entry
     uint32_t tau2;   // the row's threshold in both halves
+    uint32_t n_old;  // entries that were there after the last selection (segmented graphs)
 };
 
 struct SelectTargets {
@@ -146,11 +149,11 @@ struct SelectTargets {
 // threshold of a row is searched between its smallest and its largest entry, counting packed halves in registers: three
 // steps that interpolate (the entries above a threshold thin out exponentially), then bisection over the ordered 16-bit
 // values.  Where many entries tie and no threshold leaves a number in range, the smallest tied ones past `hi` are
-// dropped too.  `seg` >= 0: also keeps the high bytes at `hi_bytes` (`n_old` kept entries have one).
+// dropped too.  `seg` >= 0: also keeps the high bytes at `hi_bytes` (the first n_old entries have one).
 // About 900 instructions a warp at CAP = 80.
+// Out of line: the loop that calls it rarely keeps its registers.
 template <int CAP>
-__device__ __forceinline__ void select_rows(RowSel16& r, uint32_t base, SelectTargets t, bool raise, unsigned char* hi_bytes,
-                                            int seg, int& n_old) {
+__device__ __noinline__ RowSel16 select_rows(RowSel16 r, uint32_t base, SelectTargets t, bool raise, unsigned char* hi_bytes, int seg) {
     constexpr int NP = CAP / 2;
     static_assert(CAP % 8 == 0, "entries are moved eight at a time");
     const int cnt = (int)((r.pend - base) >> 7);
@@ -236,16 +239,17 @@ __device__ __forceinline__ void select_rows(RowSel16& r, uint32_t base, SelectTa
             if (keep && ptx::half_ge(th, e >> 16) && budget-- <= 0) keep = false;
             if (keep) {
                 ptx::sts_u32(out, e);
-                if (seg >= 0) hi_bytes[n_new] = s < n_old ? hi_bytes[s] : (unsigned char)seg;
+                if (seg >= 0) hi_bytes[n_new] = s < (int)r.n_old ? hi_bytes[s] : (unsigned char)seg;
                 out += 128u;
                 ++n_new;
             }
         }
-        n_old = n_new;
         __syncwarp();
     }
     r.pend = out;
+    r.n_old = (out - base) >> 7;
     if (!keep_all) r.tau2 = th2;
+    return r;
 }
 
 // Columns at or past `nvalid` do not exist (end of the key range).
@@ -302,13 +306,13 @@ template <int D, int CAP, int NQT, int S, bool DUMP>
 __global__ void __launch_bounds__(threads16(NQT), 1)
 score_select_f16_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                         const WorkItem* __restrict__ items, StatusBlock* __restrict__ sb, int H,
-                        const GroupLists lists, SelectTargets target, float* __restrict__ dump, int n_total /* = N */, long long wait_limit, int drop_first_tile,
+                        const GroupLists lists, SelectTargets target, int item_tiles, float* __restrict__ dump, int n_total /* = N */, long long wait_limit, int drop_first_tile,
                         const int* __restrict__ perm) {
     using Sh = Shape16<D>;
     using Sp = Plan16<CAP, NQT, S>;
     constexpr int NEPI = 4 * NQT;
     constexpr uint32_t TMEM_COLS = NBUF * BN;
-    static_assert(NQT <= NBUF && NQT <= kServiceWarps && S >= 3, "an accumulator buffer and an issuer per query tile");
+    static_assert(NQT <= NBUF && NQT <= kIssuers + 1, "an accumulator buffer per query tile");
 
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -325,8 +329,8 @@ score_select_f16_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
 
     if (threadIdx.x == 0) {
         ptx::mbar_init(bars.q_full(), 1);
-        ptx::mbar_init(bars.q_empty(), NQT);
-        ptx::mbar_init(bars.done(), NQT);
+        ptx::mbar_init(bars.q_empty(), NQT < kIssuers ? NQT : kIssuers);
+        ptx::mbar_init(bars.done(), NQT < kIssuers ? NQT : kIssuers);
         for (int s = 0; s < S; ++s) {
             ptx::mbar_init(bars.k_full(s), 1);
             ptx::mbar_init(bars.k_empty(s), NQT);
@@ -355,124 +359,126 @@ score_select_f16_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
 
     const int n_items = sb->n_items;
     const long long total = (long long)n_items * H;
-    // Tail of the persistent schedule: the units (work item, head) past the last full wave of CTAs are cut
-    // into their 128-row query tiles, one CTA each, provided the pieces fit one wave (see score_select_tc.cu).
+    // Tail of the persistent schedule: the units (work item, head) past the last full wave of CTAs are cut into pieces of
+    // fewer query tiles, one CTA each, as far as the pieces fit one wave.
     long long n_whole = total, n_units = total;
-    if (!DUMP && NQT > 1 && total > (long long)gridDim.x) {
-        const long long left = total % gridDim.x;
-        if (left * NQT <= (long long)gridDim.x) { n_whole = total - left; n_units = n_whole + left * NQT; }
+    int pieces = 1, piece_rows = item_tiles * BM;
+    if (!DUMP && total > (long long)gridDim.x) {
+        const int left = (int)(total % gridDim.x);
+        if (left > 0) {
+            const int tiles = (item_tiles + min(item_tiles, (int)gridDim.x / left) - 1) / min(item_tiles, (int)gridDim.x / left);
+            pieces = (item_tiles + tiles - 1) / tiles;
+            piece_rows = tiles * BM;
+            n_whole = total - left;
+            n_units = n_whole + (long long)left * pieces;
+        }
     }
     auto unit = [&](long long w, int& h, WorkItem& it) -> bool {
         long long base = w;
         int piece = -1;
-        if (w >= n_whole) { base = n_whole + (w - n_whole) / NQT; piece = (int)((w - n_whole) % NQT); }
+        if (w >= n_whole && pieces > 1) { base = n_whole + (w - n_whole) / pieces; piece = (int)((w - n_whole) % pieces); }
         h = (int)(base / n_items);
         it = items[base % n_items];
-        if (piece >= 0) { it.row0 += piece * BM; it.nrows = min(BM, it.nrows - piece * BM); }
+        if (piece >= 0) { it.row0 += piece * piece_rows; it.nrows = min(piece_rows, it.nrows - piece * piece_rows); }
         return it.nrows > 0;
     };
 
-    if (warp >= NEPI) {
-        // ------------------------------------------------------------------ service warps
-        // Issuer `mine` multiplies every key tile against query tile `mine` into accumulator buffer `mine` and commits to
-        // that tile's barrier; its four selection warps hand the buffer back as soon as the scores are in their
-        // registers.  Every issuer waits for every key tile (a parity wait is sound only on a barrier whose every phase
-        // the waiter observes).  Warp 0 loads key tiles S - 1 ahead of the one it multiplies, so the stage it refills was
-        // last read two tiles ago and is free as a rule; the query tiles are loaded when the unit before is done.
-        const int mine = warp - NEPI;
-        if (mine < NQT) {
-            const bool producer = mine == 0;
-            bool ok = true;
-            // producer's place in the sequence of all key tiles of this CTA
-            long long pw = blockIdx.x;
-            int ph = 0, pj = 0, pn = 0, pkt = 0, ps = 0;
-            WorkItem pit{};
-            auto next_unit = [&] {  // the producer's next unit with any tiles
-                for (pn = 0; pn == 0 && pw < n_units; pw += gridDim.x)
-                    if (unit(pw, ph, pit)) { pn = (pit.key_hi - pit.key_lo + BN - 1) / BN; pj = 0; }
-            };
-            auto produce_up_to = [&](int kt_end) {  // key tiles of the CTA before number kt_end are loaded or on their way
-                while (ok && pn > 0 && pkt < kt_end) {
-                    ok = wait_or_abort<kRelaxedPollNs>(bars.k_empty(ps), ((pkt / S) & 1) ^ 1, sAbort, sb, 2, wait_limit);
-                    ok = __all_sync(FULL, ok);
-                    if (!ok) break;
-                    // failure-detection test option: CTA 0 never loads its first key tile
-                    if (!(drop_first_tile && blockIdx.x == 0 && pkt == 0) && ptx::elect_one()) {
-                        ptx::mbar_arrive_expect_tx(bars.k_full(ps), Sh::TILE_BYTES);
-                        ptx::tma_load_2d(ptx::smem_u32(sK + ps * Sh::TILE_BYTES), &tmK, 0, ph * n_total + pit.key_lo + pj * BN, bars.k_full(ps));
-                    }
-                    __syncwarp();
-                    ++pkt;
-                    ps = ps + 1 == S ? 0 : ps + 1;
-                    if (++pj == pn) next_unit();
+    if (warp == NEPI) {
+        // ------------------------------------------------------------------ TMA producer
+        int kt = 0, ic = 0;
+        bool ok = true;
+        for (long long w = blockIdx.x; ok && w < n_units; w += gridDim.x) {
+            int h;
+            WorkItem it;
+            if (!unit(w, h, it)) continue;
+            ok = __all_sync(FULL, wait_or_abort<kRelaxedPollNs>(bars.q_empty(), (ic & 1) ^ 1, sAbort, sb, 1, wait_limit));
+            if (!ok) break;
+            if (ptx::elect_one()) {
+                ptx::mbar_arrive_expect_tx(bars.q_full(), NQT * Sh::TILE_BYTES);
+                for (int qt = 0; qt < NQT; ++qt)
+                    ptx::tma_load_2d(ptx::smem_u32(sQ + qt * Sh::TILE_BYTES), &tmQ, h * D, it.row0 + qt * BM, bars.q_full());
+            }
+            __syncwarp();
+            const int ntiles = (it.key_hi - it.key_lo + BN - 1) / BN;
+            for (int j = 0; j < ntiles; ++j, ++kt) {
+                const int s = kt % S;
+                ok = __all_sync(FULL, wait_or_abort<kRelaxedPollNs>(bars.k_empty(s), ((kt / S) & 1) ^ 1, sAbort, sb, 2, wait_limit));
+                if (!ok) break;
+                // failure-detection test option: CTA 0 never loads its first key tile
+                if (drop_first_tile && blockIdx.x == 0 && kt == 0) continue;
+                if (ptx::elect_one()) {
+                    ptx::mbar_arrive_expect_tx(bars.k_full(s), Sh::TILE_BYTES);
+                    ptx::tma_load_2d(ptx::smem_u32(sK + s * Sh::TILE_BYTES), &tmK, 0, h * n_total + it.key_lo + j * BN, bars.k_full(s));
                 }
-            };
-            if (producer) next_unit();
-            const uint64_t desc_q = make_desc16<D>(ptx::smem_u32(sQ + mine * Sh::TILE_BYTES));
-            const uint32_t d_tmem = tmem_base + (uint32_t)(mine * BN), full_bar = bars.t_full(mine), empty_bar = bars.t_empty(mine);
-            int kt = 0, s = 0, ic = 0;
-            uint32_t k_par = 0;  // parity of the tile's pass through the ring
-            for (long long w = blockIdx.x; ok && w < n_units; w += gridDim.x) {
-                int h;
-                WorkItem it;
-                if (!unit(w, h, it)) continue;
-                const bool active = mine * BM < it.nrows;
-                if (producer) {
-                    ok = wait_or_abort<0>(bars.q_empty(), (ic & 1) ^ 1, sAbort, sb, 1, wait_limit);
-                    ok = __all_sync(FULL, ok);
-                    if (!ok) break;
-                    if (ptx::elect_one()) {
-                        ptx::mbar_arrive_expect_tx(bars.q_full(), NQT * Sh::TILE_BYTES);
-                        for (int qt = 0; qt < NQT; ++qt)
-                            ptx::tma_load_2d(ptx::smem_u32(sQ + qt * Sh::TILE_BYTES), &tmQ, h * D, it.row0 + qt * BM, bars.q_full());
-                    }
-                    __syncwarp();
-                }
-                const int ntiles = (it.key_hi - it.key_lo + BN - 1) / BN;
-                if (producer) produce_up_to(kt + S - 1);
-                ok = ok && wait_or_abort<0>(bars.q_full(), ic & 1, sAbort, sb, 3, wait_limit);
-                ok = __all_sync(FULL, ok);
-                for (int j = 0; ok && j < ntiles; ++j, ++kt) {
-                    if (producer) produce_up_to(kt + S - 1);
-                    const uint64_t desc_k = make_desc16<D>(ptx::smem_u32(sK) + (uint32_t)(s * Sh::TILE_BYTES));
-                    ok = ok && wait_or_abort<0>(bars.k_full(s), k_par, sAbort, sb, 4, wait_limit) &&
-                         wait_or_abort<0>(empty_bar, (kt & 1) ^ 1, sAbort, sb, 5, wait_limit);
-                    ok = __all_sync(FULL, ok);
+                __syncwarp();
+            }
+            ++ic;
+        }
+        if (!ok && lane == 0) {
+            // give copies that are still in flight a bounded time to land before the CTA exits
+            const long long t0 = clock64();
+            for (int s = 0; s < S && kt > 0; ++s) {
+                const int last = kt - 1 - ((kt - 1 - s) % S + S) % S;
+                if (last < 0) continue;
+                while (!ptx::mbar_try_wait(bars.k_full(s), (last / S) & 1) && clock64() - t0 < 40000000ll) {}
+            }
+        }
+        __syncwarp();
+    } else if (warp > NEPI) {
+        // ------------------------------------------------------------------ MMA issuers
+        // Query tile qt is multiplied with every key tile into accumulator buffer qt, committed to a barrier of its own,
+        // and its four selection warps hand the buffer back as soon as the scores are in their registers.  Every issuer
+        // waits for every key tile (a parity wait is sound only on a barrier whose every phase the waiter observes).
+        const int first = warp - NEPI - 1;
+        constexpr int PER = (NQT + kIssuers - 1) / kIssuers;  // query tiles of an issuer, at most
+        int kt = 0, s = 0, ic = 0;
+        uint32_t k_par = 0;  // parity of the tile's pass through the ring
+        bool ok = true;
+        const uint64_t desc_q0 = make_desc16<D>(ptx::smem_u32(sQ)), desc_k0 = make_desc16<D>(ptx::smem_u32(sK));
+        for (long long w = blockIdx.x; ok && w < n_units; w += gridDim.x) {
+            int h_unused;
+            WorkItem it;
+            if (!unit(w, h_unused, it)) continue;
+            ok = __all_sync(FULL, wait_or_abort<0>(bars.q_full(), ic & 1, sAbort, sb, 3, wait_limit));
+            const int ntiles = (it.key_hi - it.key_lo + BN - 1) / BN;
+            for (int j = 0; ok && j < ntiles; ++j, ++kt) {
+                const uint64_t desc_k = desc_k0 + (uint64_t)((s * Sh::TILE_BYTES) >> 4);
+                ok = __all_sync(FULL, wait_or_abort<0>(bars.k_full(s), k_par, sAbort, sb, 4, wait_limit));
+                if (!ok) break;
+#pragma unroll
+                for (int x = 0; x < PER; ++x) {
+                    const int qt = first + x * kIssuers;
+                    if (qt >= NQT) break;
+                    ok = ok && __all_sync(FULL, wait_or_abort<0>(bars.t_empty(qt), (kt & 1) ^ 1, sAbort, sb, 5, wait_limit));
                     if (!ok) break;
                     ptx::tc_fence_after();
                     if (ptx::elect_one()) {
-                        if (active) {
+                        if (qt * BM < it.nrows) {
+                            const uint64_t desc_q = desc_q0 + (uint64_t)((qt * Sh::TILE_BYTES) >> 4);
 #pragma unroll
                             for (int ks = 0; ks < Sh::KSTEPS; ++ks)  // 16 values of depth = 32 bytes of a row
-                                ptx::mma_f16_ss(d_tmem, desc_q + (uint64_t)(2 * ks), desc_k + (uint64_t)(2 * ks), kInstrDesc16, ks > 0 ? 1u : 0u);
+                                ptx::mma_f16_ss(tmem_base + (uint32_t)(qt * BN), desc_q + (uint64_t)(2 * ks), desc_k + (uint64_t)(2 * ks),
+                                                kInstrDesc16, ks > 0 ? 1u : 0u);
                         }
-                        ptx::mma_commit(full_bar);
+                        ptx::mma_commit(bars.t_full(qt));
                         // the scores of the tile before have been read, so its stage has been read too
                         if (kt > 0) ptx::mbar_arrive(bars.k_empty(s == 0 ? S - 1 : s - 1));
                     }
                     __syncwarp();
-                    if (++s == S) { s = 0; k_par ^= 1u; }
                 }
-                if (!ok) break;
-                if (ptx::elect_one()) ptx::mma_commit(bars.q_empty());
-                __syncwarp();
-                ++ic;
+                if (++s == S) { s = 0; k_par ^= 1u; }
             }
-            if (ptx::elect_one()) {
-                ptx::mma_commit(bars.done());
-                // bounded, like every wait: MMAs, and after a failed wait also copies that are still in flight
-                const long long t0 = clock64();
-                while (!ptx::mbar_try_wait(bars.done(), 0) && clock64() - t0 < 2000000000ll) {}
-                if (producer && !ok) {
-                    for (int x = 0; x < S && pkt > 0; ++x) {
-                        const int last = pkt - 1 - ((pkt - 1 - x) % S + S) % S;
-                        if (last < 0) continue;
-                        while (!ptx::mbar_try_wait(bars.k_full(x), (last / S) & 1) && clock64() - t0 < 2000000000ll) {}
-                    }
-                }
-            }
+            if (!ok) break;
+            if (first < NQT && ptx::elect_one()) ptx::mma_commit(bars.q_empty());
             __syncwarp();
+            ++ic;
         }
+        if (first < NQT && ptx::elect_one()) {
+            ptx::mma_commit(bars.done());
+            const long long t0 = clock64();
+            while (!ptx::mbar_try_wait(bars.done(), 0) && clock64() - t0 < 2000000000ll) {}
+        }
+        __syncwarp();
     } else {
         // ------------------------------------------------------------------ selection warps
         const int qt = warp >> 2, quarter = warp & 3;
@@ -534,7 +540,7 @@ score_select_f16_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                 const bool segmented = ntiles > kSegTiles;
                 // next tile that is not like the others: a segment's last, or the last of all, which may be ragged
                 int special_j = segmented ? kSegTiles - 1 : ntiles - 1;
-                int n_old = 0;
+                rs.n_old = 0u;
                 uint32_t par = (uint32_t)tcnt & 1u;
                 for (int j = 0; j < ntiles; ++j, par ^= 1u) {
                     if (!__all_sync(FULL, ptx::mbar_try_wait(full_bar, par))) {
@@ -566,7 +572,7 @@ score_select_f16_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                         // at the end a row keeps all that its list can hold
                         const bool last = j == ntiles - 1;
                         const SelectTargets t = last ? SelectTargets{lists.slots - 2, lists.slots} : target;
-                        select_rows<CAP>(rs, row_base, t, !last, list_word, segmented ? j / kSegTiles : -1, n_old);
+                        rs = select_rows<CAP>(rs, row_base, t, !last, list_word, segmented ? j / kSegTiles : -1);
                         select_seen = max(select_seen, req);
                         if (j == special_j) special_j = min(special_j + kSegTiles, ntiles - 1);
                     }
@@ -666,7 +672,7 @@ cudaError_t launch_cfg(const FwdArgs& a, const FwdWorkspace& w, float* dump) {
     const int grid = (int)std::min<long long>(sm_count(), max_total);
     kern<<<grid, threads16(NQT), smem_bytes, a.stream>>>(
         tmQ, tmK, reinterpret_cast<const WorkItem*>(a.ws + w.items_off), reinterpret_cast<StatusBlock*>(a.ws), a.H,
-        buf.lists, select_targets(w.list), dump, (int)a.N, a.wait_limit_cycles > 0 ? a.wait_limit_cycles : kDefaultWaitLimitCycles, a.drop_first_tile,
+        buf.lists, select_targets(w.list), w.item_tiles, dump, (int)a.N, a.wait_limit_cycles > 0 ? a.wait_limit_cycles : kDefaultWaitLimitCycles, a.drop_first_tile,
         (w.reorder && !DUMP) ? reinterpret_cast<const int*>(a.ws + w.perm_off) : nullptr);
     return cudaGetLastError();
 }
@@ -694,7 +700,27 @@ bool score_select_f16_in_outputs_supported(int64_t N, int32_t H, int32_t d, int3
     return mode == KMIP_BF16_TC && d == 64 && N * H >= kF16MinRowsWide;
 }
 
-int score_select_f16_rows_per_item(int32_t d) { return (d == 64 ? 3 : 4) * BM; }
+// Query tiles per work item.  A round (one key tile against all query tiles of a CTA) takes about as long with one
+// query tile as with four (measured, clocks at d = 16, k = 8, 75 776 nodes: 1150, 1220, 1265, 1460 - the chain of one
+// pipeline, not its work, is what takes the time), so fewer tiles per item pay only where they fill idle SMs: the
+// smallest number of rounds, weighted with their length, wins.  Graphs of one size are assumed.
+int score_select_f16_item_tiles(int64_t N, int32_t G, int32_t H, int32_t d) {
+    constexpr double kRound[5] = {0.0, 0.80, 0.84, 0.88, 1.0};
+    const int most = d == 64 ? 3 : 4;
+    const int64_t grid = sm_count(), tiles = (N / std::max(G, 1) + BM - 1) / BM;  // query tiles of a graph
+    int best = most;
+    double best_cost = 0.0;
+    for (int t = most; t >= 1; --t) {
+        const int64_t units = (tiles + t - 1) / t * G * H, left = units % grid;
+        double cost = (double)(units / grid) * kRound[t];
+        if (left > 0) {
+            const int64_t pieces = units > grid ? std::min<int64_t>(t, grid / left) : 1;  // the kernel cuts the tail
+            cost += kRound[(t + pieces - 1) / pieces];
+        }
+        if (t == most || cost < best_cost) { best = t; best_cost = cost; }
+    }
+    return best;
+}
 
 cudaError_t launch_score_select_f16(const FwdArgs& a, const FwdWorkspace& w) {
     switch (a.d) {
