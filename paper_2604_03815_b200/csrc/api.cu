@@ -129,6 +129,15 @@ int forward_impl(const void* Q, const void* K, const void* V, const int32_t* gra
     if (launch_canary_fill(a.ws, w.canaries, a.stream) != cudaSuccess) return KMIP_ERR_CUDA;
     cudaEvent_t* ev = (g_prof.on && g_prof.n_fwd < g_prof.max_calls) ? g_prof.fwd[g_prof.n_fwd++] : nullptr;
     if (ev) cudaEventRecord(ev[0], a.stream);
+    const bool test_sweep = opt && (opt->fp32_path != 0 || opt->drop_first_tile != 0);  // a test wants one of the sweeps below
+    if (!test_sweep && small_graphs_preferred(N, a.G, H, d, k)) {
+        if (launch_plan(a, w, 128) != cudaSuccess) return KMIP_ERR_CUDA;
+        if (ev) cudaEventRecord(ev[1], a.stream);
+        if (launch_small_graphs(a) != cudaSuccess) return KMIP_ERR_CUDA;
+        for (int e = 2; ev && e <= 4; ++e) cudaEventRecord(ev[e], a.stream);
+        if (launch_canary_check(a.ws, w.canaries, a.stream) != cudaSuccess) return KMIP_ERR_CUDA;
+        return KMIP_OK;
+    }
     if (tc && !w.prune && !w.f16 && launch_pack_keys(a, w) != cudaSuccess) return KMIP_ERR_CUDA;
     // the tiled fp32 sweep runs one block per 128 query rows and head and reads a key once per block instead of
     // once per row: measured faster than the one-warp-per-row kernel from about 48 blocks on (0.43 against

@@ -402,6 +402,10 @@ cudaError_t launch_topk_mass_tc(const FwdArgs& a, const FwdWorkspace& w, float* 
 // tiled CUDA-core sweep of fp32 mode (score_select_fp32.cu): 128-row work items, then launch_refine_topk_fp32
 bool score_select_fp32_tiled_supported(int32_t d, int32_t k);
 cudaError_t launch_score_select_fp32_tiled(const FwdArgs& a, const FwdWorkspace& w);
+// small_graphs.cu: the whole forward pass of batches of small graphs (any graph size, k <= 32, d <= 64); after the plan
+// kernel, which validates the offsets
+bool small_graphs_preferred(int64_t N, int32_t G, int32_t H, int32_t d, int32_t k);
+cudaError_t launch_small_graphs(const FwdArgs& a);
 // epilogue.cu: softmax over the k kept scores fused with the gather-V weighted sum
 cudaError_t launch_softmax_gather(const FwdArgs& a);
 // backward.cu

@@ -303,3 +303,20 @@ def test_kth_score_near_zero_keeps_k_keys(d):
     idx = fb.topk_idx.cpu().numpy()
     assert np.all(idx >= 0), f"{int((idx < 0).sum())} padded slots although every graph has more than k nodes"
     pu.check_forward(w, fb)
+
+
+@pytest.mark.parametrize("sizes,H,d,k,mode", [([1, 2, 0, 33, 31], 2, 16, 32, wl.MODE_BF16_TC), ([255, 256, 257, 64, 1], 1, 32, 7, wl.MODE_BF16_TC),
+                                              ([511, 513, 40], 3, 64, 31, wl.MODE_BF16_TC), ([1500], 1, 16, 1, wl.MODE_BF16_TC),
+                                              ([255, 256, 257, 3], 2, 16, 9, wl.MODE_FP32_EXACT), ([700, 0, 5], 1, 64, 32, wl.MODE_FP32_EXACT),
+                                              ([1030], 1, 32, 16, wl.MODE_FP32_EXACT)])
+def test_small_graphs_in_one_kernel(sizes, H, d, k, mode):
+    """Batches whose forward pass is one kernel: chunk edges (256 keys), graphs smaller than k and than a warp, several
+    graphs in a block, several chunks against the running list; with ties, which the list order must break by key."""
+    w = wl.iid_workload("s", 6300 + sum(sizes) + k, sizes, H, d, k, mode, backward=False)
+    pu.check_forward(w, pu.run_forward(w))
+    w.K[::2] = w.K[1]                                    # half of the keys tie
+    Q, K, V, dO, offs = pu.to_device(w)
+    a = kb.forward(Q, K, V, offs, k, w.mode)
+    # one warp per row in fp32: of bf16 values the same exact products and the same order of sums
+    b = kb.forward(Q.float(), K.float(), V.float(), offs, k, kb.KMIP_FP32_EXACT, fp32_path=1)
+    assert torch.equal(a.topk_idx, b.topk_idx) and torch.equal(a.topk_score, b.topk_score)
