@@ -114,7 +114,7 @@ int forward_impl(const void* Q, const void* K, const void* V, const int32_t* gra
     if (mode == KMIP_FP32_EXACT && opt && opt->fp32_path != 0) w.f16 = w.in_outputs = false;  // a test picks the CUDA-core sweep
     const bool tc = w.tc;
     if (workspace_bytes < w.total) return KMIP_ERR_WORKSPACE;
-    if (w.f16) w.item_tiles = score_select_f16_item_tiles(N, graph_offsets ? G : 1, H, d);
+    if (w.f16) w.item_tiles = score_select_f16_item_tiles(N, graph_offsets ? G : 1, H, d, w.list);
 
     FwdArgs a{Q, K, V, graph_offsets, graph_offsets ? G : 1, N, H, d, k, mode, out, topk_idx, topk_score,
               static_cast<unsigned char*>(workspace), static_cast<cudaStream_t>(stream)};
@@ -390,7 +390,7 @@ int kmip_test_sweep_order(const void* workspace, int64_t N, int32_t G, int32_t H
     if (rc != KMIP_OK) return rc;
     if (!workspace || !order || !rows_per_item || G < 0) return KMIP_ERR_INVALID_ARG;
     FwdWorkspace w = plan_fwd_workspace(N, G > 0 ? G : 1, H, d, k, mode);
-    if (w.f16) w.item_tiles = score_select_f16_item_tiles(N, G > 0 ? G : 1, H, d);
+    if (w.f16) w.item_tiles = score_select_f16_item_tiles(N, G > 0 ? G : 1, H, d, w.list);
     *rows_per_item = w.f16 ? 128 * w.item_tiles : w.tc ? score_select_tc_rows_per_item(d, k) : 128;
     if (cudaStreamSynchronize(static_cast<cudaStream_t>(stream)) != cudaSuccess) return KMIP_ERR_CUDA;
     if (w.reorder) {
@@ -427,7 +427,7 @@ int kmip_test_f16_scores(const void* Q, const void* K, int64_t N, int32_t H, int
     if (d > 32) return KMIP_ERR_UNSUPPORTED;
     if (!Q || !K || !scores || !scales || !workspace || N < 1 || N > 8192) return KMIP_ERR_INVALID_ARG;
     FwdWorkspace w = plan_fwd_workspace(N, 1, H, d, 1, KMIP_BF16_TC, kPlanTcFp16Acc);
-    w.item_tiles = score_select_f16_item_tiles(N, 1, H, d);
+    w.item_tiles = score_select_f16_item_tiles(N, 1, H, d, w.list);
     if (workspace_bytes < w.total) return KMIP_ERR_WORKSPACE;
     FwdArgs a{Q, K, nullptr, nullptr, 1, N, H, d, 1, KMIP_BF16_TC, nullptr, nullptr, nullptr,
               static_cast<unsigned char*>(workspace), static_cast<cudaStream_t>(stream)};

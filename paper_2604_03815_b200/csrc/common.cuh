@@ -107,7 +107,7 @@ bool score_select_f16_supported(int64_t N, int32_t d, int32_t k);
 bool score_select_f16_in_outputs_supported(int64_t N, int32_t H, int32_t d, int32_t k, int mode);
 int score_select_f16_list(int32_t k);
 int score_select_f16_list_in_outputs(int32_t k);
-int score_select_f16_item_tiles(int64_t N, int32_t G, int32_t H, int32_t d);
+int score_select_f16_item_tiles(int64_t N, int32_t G, int32_t H, int32_t d, int list);
 
 // Which sweep the plan is for: the one the mode selects, or one a test entry point asks for.
 enum PlanVariant { kPlanByMode = 0, kPlanNoTensorCore = 1, kPlanTcFp32Acc = 2, kPlanTcFp16Acc = 3,
@@ -338,6 +338,9 @@ constexpr int kMinRowsToSort = 8192;  // smaller graphs keep their row and key o
 // takes 58 us at 1024 rows (one graph, d = 32), 167 at 2048 (filter: 114) and 601 at 4096 (150).
 constexpr int64_t kF16MinRowsFp32 = 1536;
 constexpr int64_t kF16MinRowsWide = 2048;
+// Smallest N * H with 32 < k <= 103 that does (us for the forward pass, fp32-accumulate sweep / filter): 1024 rows, d 16, k 45:
+// 165 / 113; d 32, k 80: 171 / 139; 10 000 rows, d 16, k 45: 348 / 218; smaller calls were not measured.
+constexpr int64_t kF16MinRowsLong = 1024;
 // score_select_exact.cu: CUDA-core scores + running top-k, any supported (d, k), fp32 or bf16 storage
 cudaError_t launch_score_select_exact(const FwdArgs& a);
 int sm_count();  // multiprocessors of the current device (cached per device)

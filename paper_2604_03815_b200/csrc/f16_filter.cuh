@@ -11,6 +11,8 @@ namespace kmip {
 
 // Groups kept per row by the prefilter sweep for 16 < k <= 32 (k + slack, a multiple of 8).
 constexpr int kF16List32 = 48;
+// ... and for 32 < k <= 103.
+constexpr int kF16ListMost = 120;
 
 // Per head: largest squared norm of a query row, of a key row, and of the first 16 elements of a key
 // row (the partial sum after the first tensor-core step of a wider head); largest squared norm of what the conversion

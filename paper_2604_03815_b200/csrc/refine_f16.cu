@@ -114,7 +114,7 @@ refine_f16_kernel(const T* __restrict__ Q, const T* __restrict__ K,
     constexpr int CAP = 32 * E;
     constexpr int EPL = (LIST + 31) / 32;  // list entries per lane
     constexpr int KSTEPS = D / 16;
-    static_assert(E <= 4 && LIST <= 64, "k <= 32");
+    constexpr bool kLong = LIST > kF16List32;  // k > 32: more than one kept key per lane
     __shared__ cand_t s_rows[kWarpsPerBlock][CAP];
     __shared__ __align__(16) T s_qb[kWarpsPerBlock][D];  // the query row
     __shared__ uint32_t s_words[kWarpsPerBlock][LIST];
@@ -128,7 +128,6 @@ refine_f16_kernel(const T* __restrict__ Q, const T* __restrict__ K,
     uint32_t* words = s_words[wib];
     const long long n_rows = (long long)N * H;
     const long long stride = (long long)gridDim.x * kWarpsPerBlock;
-    const int room = CAP - k;
     constexpr int P = D * (int)sizeof(T) / 16;                 // 16-byte pieces of a key row
     constexpr int kRowStride = D * (int)sizeof(T) + 16;        // padded: a lane per row reads 16-byte pieces without bank conflicts
     constexpr int kStageBytes = 32 * kRowStride;
@@ -199,7 +198,8 @@ refine_f16_kernel(const T* __restrict__ Q, const T* __restrict__ K,
                 qlost2 = fmaf(dx, dx, qlost2);
             }
         }
-        for (int t = lane; t < k; t += 32) row[t] = 0ull;
+        if (!kLong)
+            for (int t = lane; t < k; t += 32) row[t] = 0ull;
         fetch(r + stride);
 
         // error bound of the fp16 scores in the scaled units of the sweep
@@ -255,7 +255,18 @@ refine_f16_kernel(const T* __restrict__ Q, const T* __restrict__ K,
         // every key of the answer scores at least lowS / sc exactly; keep a margin for the fp32 sums
         const float floor_tau = n_valid >= k ? (lowS - fp32_err) / sc - 1e-30f : -CUDART_INF_F;
         float tau = floor_tau;
-        int cnt = 0;
+        // Candidates wait behind the kept ones: behind the k slots of the sorted list (k <= 32), or, before the first
+        // compaction of a longer one, from slot 0 on.
+        int kept = kLong ? 0 : k, cnt = 0;
+        auto compact = [&]() -> float {
+            if (!kLong) return warp_merge_row_chunks(row, k, cnt, lane);
+            // the usual row passes few keys beyond its k best: sort no more than there are
+            const int n = max(kept + cnt, k), extra = kept + cnt - k;
+            kept = k;
+            if (n <= 64) return warp_compact_row<2>(row, k, extra, lane);
+            if (E > 4 && n <= 128) return warp_compact_row<4>(row, k, extra, lane);
+            return warp_compact_row<E>(row, k, extra, lane);
+        };
         // Rescoring, 32 keys (4 groups) per step.  A key row is P pieces of 16 bytes.  The rows come in by
         // asynchronous 16-byte copies in which P neighbouring lanes fetch one row, so one copy instruction touches
         // 32 / P cache lines instead of 32 (the kernel is bound by these line accesses); they land in a per-warp
@@ -297,19 +308,19 @@ refine_f16_kernel(const T* __restrict__ Q, const T* __restrict__ K,
             const bool pass = kv && (s > tau);
             const unsigned m = __ballot_sync(FULL, pass);
             if (m) {
-                if (pass) row[k + cnt + __popc(m & ((1u << lane) - 1u))] = make_cand(s, jj);
+                if (pass) row[kept + cnt + __popc(m & ((1u << lane) - 1u))] = make_cand(s, jj);
                 cnt += __popc(m);
-                if (cnt > room - 32) {
+                if (kept + cnt > CAP - 32) {
                     // the groups come in list order, not key order: a later key with the same score as the
                     // k-th best and a smaller index must still get in, so the threshold sits just below it
-                    tau = fmaxf(floor_tau, nextafterf(warp_merge_row_chunks(row, k, cnt, lane), -CUDART_INF_F));
+                    tau = fmaxf(floor_tau, nextafterf(compact(), -CUDART_INF_F));
                     cnt = 0;
                 }
             }
             __syncwarp();  // the stage is free for the copies of step + 2
         }
         ptx::cp_async_wait<0>();
-        const float kth = warp_merge_row_chunks(row, k, cnt, lane);
+        const float kth = compact();
         // the sweep dropped a group unless the list holds every group of the graph; a dropped one scores at most
         // g_min + err(g_min) exactly (scaled), and it matters if that reaches the k-th best score found
         const int n_groups = 2 * ((hi - lo) / 16) + min((hi - lo) % 16, 2);
@@ -338,7 +349,13 @@ cudaError_t launch_d(const FwdArgs& a, const FwdWorkspace& w) {
     cudaError_t err;
     if (a.k <= 8) { KMIP_LAUNCH_REFINE16(2, 16); }
     else if (a.k <= 16) { KMIP_LAUNCH_REFINE16(2, 24); }
-    else { KMIP_LAUNCH_REFINE16(4, kF16List32); }
+    else if (a.k <= 32) { KMIP_LAUNCH_REFINE16(4, kF16List32); }
+    else if constexpr (D <= 32) {
+        if (a.k <= 64) { KMIP_LAUNCH_REFINE16(4, 80); }
+        else { KMIP_LAUNCH_REFINE16(8, kF16ListMost); }
+    } else {
+        return cudaErrorInvalidValue;
+    }
 #undef KMIP_LAUNCH_REFINE16
     return cudaGetLastError();
 }

@@ -268,7 +268,8 @@ void launch_redo_d(const FwdArgs& a, const F16Buffers& b) {
         static_cast<const T*>(a.Q), static_cast<const T*>(a.K), a.graph_offsets, a.G, (int)a.N, a.H, a.k, \
         a.topk_idx, a.topk_score, reinterpret_cast<StatusBlock*>(a.ws), b.redo, static_cast<cand_t*>(b.scratch), lists)
     if (a.k <= 16) KMIP_LAUNCH_REDO(2);
-    else KMIP_LAUNCH_REDO(4);
+    else if (a.k <= 96) KMIP_LAUNCH_REDO(4);
+    else KMIP_LAUNCH_REDO(8);
 #undef KMIP_LAUNCH_REDO
 }
 
@@ -289,7 +290,7 @@ cudaError_t launch_score_select_exact(const FwdArgs& a) {
     return a.mode == KMIP_FP32_EXACT ? launch_t<float>(a) : launch_t<__nv_bfloat16>(a);
 }
 
-// The rows the half-precision prefilter could not decide (k <= 32), again from all keys of their graph; overwrites
+// The rows the half-precision prefilter could not decide, again from all keys of their graph; overwrites
 // their topk_idx / topk_score.
 cudaError_t launch_score_select_exact_redo(const FwdArgs& a, const FwdWorkspace& w) {
     const F16Buffers b = f16_buffers(a, w);

@@ -1,4 +1,4 @@
-// Half-precision prefilter sweep (Algorithm 1 lines 2-3): k <= 32, head widths 16, 32 and 64, bf16 and fp32 storage.
+// Half-precision prefilter sweep (Algorithm 1 lines 2-3): k <= 32, head widths 16, 32 and 64; k <= 103, widths 16 and 32; bf16 and fp32 storage.
 //
 // The paper lists half-precision arithmetic and tensor-core support as the engineering it left open
 // (Sec. 6; closing remark of the FlashAttention comparison in the appendix).  The sweep of
@@ -433,7 +433,7 @@ score_select_f16_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
         constexpr int PER = (NQT + kIssuers - 1) / kIssuers;  // query tiles of an issuer, at most
         int kt = 0, s = 0, ic = 0;
         uint32_t k_par = 0;  // parity of the tile's pass through the ring
-        bool ok = true;
+        bool ok = first < NQT;  // one without a query tile would not be waited for at the key stages: it stays out
         const uint64_t desc_q0 = make_desc16<D>(ptx::smem_u32(sQ)), desc_k0 = make_desc16<D>(ptx::smem_u32(sK));
         for (long long w = blockIdx.x; ok && w < n_units; w += gridDim.x) {
             int h_unused;
@@ -677,12 +677,25 @@ cudaError_t launch_cfg(const FwdArgs& a, const FwdWorkspace& w, float* dump) {
     return cudaGetLastError();
 }
 
+// Long lists, measured (us for the sweep, fp32-accumulate sweep / this one): 100k nodes, H 1, d 16, k 45 2098 / 1070, k 100
+// 5513 / 1859; 50k nodes, H 2, d 32, k 64 1627 / 939, k 100 3946 / 1180.
+// Query tiles per CTA by list length, as far as shared memory goes: a row needs room for a good number of groups beyond
+// its list, or the CTA selects too often.
+int query_tiles(int32_t d, int list) {
+    if (list <= kF16List32) return d == 64 ? 3 : 4;
+    return list <= (d == 16 ? 80 : 64) ? 3 : 2;
+}
+
 template <int D>
 cudaError_t launch_d(const FwdArgs& a, const FwdWorkspace& w) {
-    // entries per row by list length, as far as shared memory goes
     constexpr int NQ = D == 64 ? 3 : 4, S = D == 16 ? 4 : 3;
     if (w.list <= 24) return launch_cfg<D, 72, NQ, S, false>(a, w, nullptr);
-    return launch_cfg<D, D == 16 ? 96 : 80, NQ, S, false>(a, w, nullptr);
+    if (w.list <= kF16List32) return launch_cfg<D, D == 16 ? 96 : 80, NQ, S, false>(a, w, nullptr);
+    if constexpr (D <= 32) {
+        if (query_tiles(D, w.list) == 3) return launch_cfg<D, D == 16 ? 128 : 112, 3, S, false>(a, w, nullptr);
+        return launch_cfg<D, 184, 2, S, false>(a, w, nullptr);
+    }
+    return cudaErrorInvalidValue;
 }
 
 }  // namespace
@@ -693,9 +706,15 @@ int score_select_f16_list(int32_t k) { return k <= 8 ? 16 : k <= 16 ? 24 : kF16L
 
 // Lists in the output arrays: a row's topk_idx and topk_score hold 2 k entries of two 16-bit numbers, so the groups are
 // numbered inside their graph (up to 2^16 of 8 keys) and k + slack <= 2 k, which wants k >= 4.
-int score_select_f16_list_in_outputs(int32_t k) { return std::min(2 * k, k <= 8 ? 16 : k <= 16 ? 24 : kF16List32); }
+// Beyond 32 the slack grows slower than k: far down the list the scores lie close together, but L / k of them fit into
+// the error bound all the same.
+int score_select_f16_list_in_outputs(int32_t k) {
+    if (k > 32) return std::max(kF16List32, (k + k / 8 + 4 + 7) / 8 * 8);
+    return std::min(2 * k, k <= 8 ? 16 : k <= 16 ? 24 : kF16List32);
+}
 bool score_select_f16_in_outputs_supported(int64_t N, int32_t H, int32_t d, int32_t k, int mode) {
-    if (k < 4 || k > 32 || N > (1 << 19) || (d != 16 && d != 32 && d != 64)) return false;
+    if (k < 4 || N > (1 << 19) || (d != 16 && d != 32 && d != 64)) return false;
+    if (k > 32) return mode != KMIP_BF16_TC_PRUNED && d <= 32 && score_select_f16_list_in_outputs(k) <= kF16ListMost && N * H >= kF16MinRowsLong;
     if (mode == KMIP_FP32_EXACT) return N * H >= kF16MinRowsFp32;
     return mode == KMIP_BF16_TC && d == 64 && N * H >= kF16MinRowsWide;
 }
@@ -704,9 +723,9 @@ bool score_select_f16_in_outputs_supported(int64_t N, int32_t H, int32_t d, int3
 // query tile as with four (measured, clocks at d = 16, k = 8, 75 776 nodes: 1150, 1220, 1265, 1460 - the chain of one
 // pipeline, not its work, is what takes the time), so fewer tiles per item pay only where they fill idle SMs: the
 // smallest number of rounds, weighted with their length, wins.  Graphs of one size are assumed.
-int score_select_f16_item_tiles(int64_t N, int32_t G, int32_t H, int32_t d) {
+int score_select_f16_item_tiles(int64_t N, int32_t G, int32_t H, int32_t d, int list) {
     constexpr double kRound[5] = {0.0, 0.80, 0.84, 0.88, 1.0};
-    const int most = d == 64 ? 3 : 4;
+    const int most = query_tiles(d, list);
     const int64_t grid = sm_count(), tiles = (N / std::max(G, 1) + BM - 1) / BM;  // query tiles of a graph
     int best = most;
     double best_cost = 0.0;

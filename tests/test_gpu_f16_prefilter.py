@@ -178,3 +178,21 @@ def test_graph_of_several_segments():
     got = dense.gather(1, fb.topk_idx[rows, 0].long())
     assert torch.all((got - best).abs() <= 1e-4 * best.abs() + 1e-4)
     assert all(len(set(r)) == k for r in fb.topk_idx[rows, 0].tolist())
+
+
+@pytest.mark.parametrize("sizes,H,d,k,mode", [([2048], 1, 16, 33, wl.MODE_BF16_TC), ([2049, 3, 0, 700], 1, 32, 45, wl.MODE_BF16_TC),
+                                              ([1500, 1200], 2, 16, 64, wl.MODE_BF16_TC), ([127, 129, 2000], 1, 32, 72, wl.MODE_BF16_TC),
+                                              ([40, 2500], 1, 16, 103, wl.MODE_BF16_TC), ([1024], 2, 32, 65, wl.MODE_FP32_EXACT),
+                                              ([33000], 1, 16, 80, wl.MODE_BF16_TC)])
+def test_long_lists_through_the_filter(sizes, H, d, k, mode):
+    """32 < k <= 103: three and two query tiles per block, lists of more than one entry per lane, rows with fewer keys than
+    k, rows in locality order; then half of the keys tied, so that every row is undecidable.  Both must be what one warp
+    per row finds in fp32 (of bf16 values the same exact products in the same order)."""
+    w = wl.iid_workload("l", 7100 + sum(sizes) + k, sizes, H, d, k, mode, backward=False)
+    for tied in (False, True):
+        if tied:
+            w.K[::2] = w.K[1]
+        Q, K, V, _, offs = pu.to_device(w)
+        a = kb.forward(Q, K, V, offs, k, w.mode)
+        b = kb.forward(Q.float(), K.float(), V.float(), offs, k, kb.KMIP_FP32_EXACT, fp32_path=1)
+        assert torch.equal(a.topk_idx, b.topk_idx) and torch.equal(a.topk_score, b.topk_score)
