@@ -62,6 +62,7 @@ constexpr int BN = 128;  // keys per tile = accumulator columns
 constexpr unsigned FULL = 0xFFFFFFFFu;
 constexpr int NBUF = 4;  // accumulator buffers of BN columns: all 512 columns of tensor memory, one per query tile
 constexpr int kRelaxedPollNs = 100;
+constexpr int64_t kLargeGraph = 150000;
 // 16 selection warps and 4 service warps (the register file of an SM holds 96 registers for 640 threads; it is handed
 // out in units of four warps): the TMA producer, and three issuers, of which the first has query tiles 0 and 3.
 // The time from a buffer's release to the next commit is on every pipeline's critical path, so an issuer runs its loop
@@ -679,23 +680,27 @@ cudaError_t launch_cfg(const FwdArgs& a, const FwdWorkspace& w, float* dump) {
 
 // Long lists, measured (us for the sweep, fp32-accumulate sweep / this one): 100k nodes, H 1, d 16, k 45 2098 / 1070, k 100
 // 5513 / 1859; 50k nodes, H 2, d 32, k 64 1627 / 939, k 100 3946 / 1180.
-// Query tiles per CTA by list length, as far as shared memory goes: a row needs room for a good number of groups beyond
-// its list, or the CTA selects too often.
-int query_tiles(int32_t d, int list) {
-    if (list <= kF16List32) return d == 64 ? 3 : 4;
-    return list <= (d == 16 ? 80 : 64) ? 3 : 2;
+// Query tiles per CTA, at most, by list length: a row needs room for a good number of groups beyond its list, or the CTA
+// selects too often, and shared memory is shared by the tiles' rows.  n: keys per graph; the longer the graph, the
+// rarer the selections.  Measured for lists of 48, us with four / three tiles: 20k nodes, H 4, d 16 376 / 317, d 32
+// 475 / 331; 100k nodes, H 1, d 16 1235 / 1035; H 4, d 32 4506 / 4191; 300k nodes, H 2, d 32 14134 / 14832; H 1, d 16
+// 5997 / 6704.
+int most_query_tiles(int64_t n, int32_t d, int list) {
+    if (d == 64 || (list > 24 && n < kLargeGraph)) return list > (d == 16 ? 80 : 64) ? 2 : 3;
+    return list <= kF16List32 ? 4 : list <= (d == 16 ? 80 : 64) ? 3 : 2;
 }
 
+// The kernel for as many query tiles as the work items have; entries per row as far as shared memory goes.  An idle tile
+// costs its share of a round and of the memory: 31 623 nodes, d 16, k 10, two tiles, 236 us in the kernel for four,
+// 181 in its own; 100k nodes, three tiles, 1084 and 948.
 template <int D>
 cudaError_t launch_d(const FwdArgs& a, const FwdWorkspace& w) {
-    constexpr int NQ = D == 64 ? 3 : 4, S = D == 16 ? 4 : 3;
-    if (w.list <= 24) return launch_cfg<D, 72, NQ, S, false>(a, w, nullptr);
-    if (w.list <= kF16List32) return launch_cfg<D, D == 16 ? 96 : 80, NQ, S, false>(a, w, nullptr);
+    constexpr int S = D == 16 ? 4 : 3;
     if constexpr (D <= 32) {
-        if (query_tiles(D, w.list) == 3) return launch_cfg<D, D == 16 ? 128 : 112, 3, S, false>(a, w, nullptr);
-        return launch_cfg<D, 184, 2, S, false>(a, w, nullptr);
+        if (w.item_tiles == 4) return launch_cfg<D, D == 16 ? 96 : 80, 4, S, false>(a, w, nullptr);
     }
-    return cudaErrorInvalidValue;
+    if (w.item_tiles == 3) return launch_cfg<D, D == 16 ? 128 : D == 32 ? 112 : 80, 3, S, false>(a, w, nullptr);
+    return launch_cfg<D, D <= 32 ? 184 : 128, 2, S, false>(a, w, nullptr);
 }
 
 }  // namespace
@@ -720,12 +725,13 @@ bool score_select_f16_in_outputs_supported(int64_t N, int32_t H, int32_t d, int3
 }
 
 // Query tiles per work item.  A round (one key tile against all query tiles of a CTA) takes about as long with one
-// query tile as with four (measured, clocks at d = 16, k = 8, 75 776 nodes: 1150, 1220, 1265, 1460 - the chain of one
-// pipeline, not its work, is what takes the time), so fewer tiles per item pay only where they fill idle SMs: the
-// smallest number of rounds, weighted with their length, wins.  Graphs of one size are assumed.
+// query tile as with three, and little less than with four (measured, ns, one work item per CTA, each with the kernel of
+// its size, 1 / 2 / 3 / 4 tiles: d 16, k 8: 682 669 671 777; d 32, k 16: 716 689 743 858; d 64, k 16: 716 709 786 - the
+// chain of one pipeline, not its work, is what takes the time), so fewer tiles per item pay only where they fill idle
+// SMs: the smallest number of rounds, weighted with their length, wins.  Graphs of one size are assumed.
 int score_select_f16_item_tiles(int64_t N, int32_t G, int32_t H, int32_t d, int list) {
-    constexpr double kRound[5] = {0.0, 0.80, 0.84, 0.88, 1.0};
-    const int most = query_tiles(d, list);
+    const double kRound[5] = {0.0, 0.87, 0.86, d == 64 ? 0.97 : 0.87, 1.0};
+    const int most = most_query_tiles(N / std::max(G, 1), d, list);
     const int64_t grid = sm_count(), tiles = (N / std::max(G, 1) + BM - 1) / BM;  // query tiles of a graph
     int best = most;
     double best_cost = 0.0;
