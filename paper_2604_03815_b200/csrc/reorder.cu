@@ -29,62 +29,101 @@ __device__ __forceinline__ uint32_t mix32(uint32_t x) {
     return x;
 }
 
-// One warp per node: bit b of the code is the sign of sum_c s(b, c) * q_c over the H*d columns of
-// the node's query row, s(b, c) = +-1 from bit b of a hash of c.
-__global__ void query_code_kernel(const __nv_bfloat16* __restrict__ Q, int N, int HD, unsigned short* __restrict__ code,
-                                  const StatusBlock* __restrict__ sb) {
-    if (sb->status != KMIP_OK) return;
-    const int lane = threadIdx.x & 31;
-    const long long row = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (row >= N) return;
-    float acc[kCodeBits];
-#pragma unroll
-    for (int b = 0; b < kCodeBits; ++b) acc[b] = 0.0f;
-    for (int c = lane; c < HD; c += 32) {
-        const float x = Elem<__nv_bfloat16>::load(Q + (size_t)row * HD + c);
-        const uint32_t m = mix32((uint32_t)c + 0x9E3779B9u);
-#pragma unroll
-        for (int b = 0; b < kCodeBits; ++b) acc[b] += ((m >> b) & 1u) ? x : -x;
+__device__ inline int graph_of(const int32_t* offs, int G, int i) {
+    if (offs == nullptr) return 0;
+    int a = 0, b = G;
+    while (b - a > 1) {
+        const int m = (a + b) >> 1;
+        if (__ldg(offs + m) <= i) a = m; else b = m;
     }
-    unsigned bits = 0;
-#pragma unroll
-    for (int b = 0; b < kCodeBits; ++b) {
-        float v = acc[b];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
-        bits |= (v > 0.0f ? 1u : 0u) << b;
-    }
-    if (lane == 0) code[row] = (unsigned short)bits;
+    return a;
 }
 
-// One block per graph: counting sort of the graph's rows by code (any order inside a bucket).
-// perm[sorted position] = original row; both lie in the graph's own row range.
-template <int BITS>
-__global__ void __launch_bounds__(kSortThreads)
-graph_sort_kernel(const int32_t* __restrict__ offs, int G, int N, const unsigned short* __restrict__ code,
-                  int* __restrict__ perm, const StatusBlock* __restrict__ sb) {
-    if (sb->status != KMIP_OK) return;  // malformed offsets were reported by the plan kernel
-    constexpr int kBuckets = 1 << BITS;
-    constexpr int PER = kBuckets >= kSortThreads ? kBuckets / kSortThreads : 1;  // consecutive bins per thread in the scan
-    extern __shared__ int s_bin[];
-    __shared__ int s_warp[32];
-    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    const int n_graphs = offs ? G : 1;
-    for (int g = blockIdx.x; g < n_graphs; g += gridDim.x) {
-        const int lo = offs ? __ldg(offs + g) : 0, hi = offs ? __ldg(offs + g + 1) : N;
-        if (hi - lo < kMinRowsToSort) {
-            for (int r = lo + tid; r < hi; r += kSortThreads) perm[r] = r;
-            continue;
+// Counting sort of every large graph's rows by query code (any order inside a bucket), in two passes over all rows.
+// First pass: one thread per row computes the code - bit b is the sign of sum_c s(b, c) * q_c over the H*d columns of the
+// node's query row, s(b, c) = +-1 from bit b of a hash of c - and takes the row's number inside its bucket from a counter
+// in global memory, the lanes of a warp with the same code together.  Second pass: a block adds up the counters of its
+// rows' graph and writes perm[sorted position] = original row.  Counters and numbers wait in the call's score and index
+// arrays, which the sweep writes later: a graph of at least kMinRowsToSort rows that starts at row lo has the counters
+// lo / kMinRowsToSort, two bytes a row in all.
+// Measured (us for the codes and the sort; before: a warp per row and one block per graph): 100k nodes, H 1, d 16 98 -> 12; H 4, d 32
+// 113 -> 32; 300k nodes, H 2, d 32 285 -> 42.
+constexpr int kCodeThreads = 128, kScatterThreads = 512, kScatterRows = 2048;
+constexpr int kCodeBuckets = 1 << kCodeBits;
+static_assert(kCodeBuckets * 4 <= kMinRowsToSort * 4, "counters fit a float per row");
+static_assert(kScatterRows <= kMinRowsToSort, "a block's rows meet two large graphs at most");
+
+__global__ void __launch_bounds__(kCodeThreads)
+query_code_kernel(const __nv_bfloat16* __restrict__ Q, int N, int HD, const int32_t* __restrict__ offs, int G,
+                  unsigned short* __restrict__ code, int* __restrict__ counters, int* __restrict__ number,
+                  const StatusBlock* __restrict__ sb) {
+    if (sb->status != KMIP_OK) return;
+    const int lane = threadIdx.x & 31;
+    const int row = blockIdx.x * kCodeThreads + threadIdx.x;
+    int lo = 0;
+    bool large = row < N;
+    if (large && offs != nullptr) {
+        const int g = graph_of(offs, G, row);
+        lo = __ldg(offs + g);
+        large = __ldg(offs + g + 1) - lo >= kMinRowsToSort;
+    }
+    unsigned bits = 0xFFFFFFFFu;  // no code
+    if (large) {
+        float acc[kCodeBits];
+#pragma unroll
+        for (int b = 0; b < kCodeBits; ++b) acc[b] = 0.0f;
+        for (int c0 = 0; c0 < HD; c0 += 8) {
+            float x[8];
+            Elem<__nv_bfloat16>::load_vec(Q + (size_t)row * HD + c0, x);
+#pragma unroll
+            for (int c = 0; c < 8; ++c) {
+                const uint32_t m = mix32((uint32_t)(c0 + c) + 0x9E3779B9u);  // the same in every thread
+#pragma unroll
+                for (int b = 0; b < kCodeBits; ++b) acc[b] += ((m >> b) & 1u) ? x[c] : -x[c];
+            }
         }
-        __syncthreads();  // the previous graph's cursors are no longer needed
-        for (int b = tid; b < kBuckets; b += kSortThreads) s_bin[b] = 0;
-        __syncthreads();
-        for (int r = lo + tid; r < hi; r += kSortThreads) atomicAdd(&s_bin[code[r]], 1);
-        __syncthreads();
-        // exclusive scan of the counts: PER consecutive bins per thread
+        bits = 0u;
+#pragma unroll
+        for (int b = 0; b < kCodeBits; ++b) bits |= (acc[b] > 0.0f ? 1u : 0u) << b;
+    }
+    const int slot = lo / kMinRowsToSort;
+    // lanes of the same bucket (the rows of a warp belong to two large graphs at most)
+    const unsigned key = large ? (bits | ((unsigned)slot << kCodeBits)) : 0xFFFFFFFFu;
+    const unsigned same = __match_any_sync(0xFFFFFFFFu, key);
+    if (!large) return;
+    const int leader = __ffs(same) - 1;
+    int first = 0;
+    if (lane == leader) first = atomicAdd(counters + (size_t)slot * kCodeBuckets + bits, __popc(same));
+    first = __shfl_sync(same, first, leader);
+    code[row] = (unsigned short)bits;
+    number[row] = first + __popc(same & ((1u << lane) - 1u));
+}
+
+__global__ void __launch_bounds__(kScatterThreads)
+scatter_rows_kernel(const int32_t* __restrict__ offs, int G, int N, const unsigned short* __restrict__ code,
+                    const int* __restrict__ counters, const int* __restrict__ number, int* __restrict__ perm,
+                    const StatusBlock* __restrict__ sb) {
+    if (sb->status != KMIP_OK) return;  // malformed offsets were reported by the plan kernel
+    constexpr int PER = kCodeBuckets / kScatterThreads;  // consecutive buckets per thread in the scan
+    __shared__ int s_start[kCodeBuckets];
+    __shared__ int s_warp[kScatterThreads / 32];
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int row_lo = (int)blockIdx.x * kScatterRows, row_hi = min(N, row_lo + kScatterRows);
+    const int g_first = graph_of(offs, G, row_lo), g_last = graph_of(offs, G, row_hi - 1);
+    // graphs that stay in order: between two large ones, or one of the two
+    for (int r = row_lo + tid; r < row_hi; r += kScatterThreads) {
+        const int g = offs ? graph_of(offs, G, r) : 0;
+        if (offs && __ldg(offs + g + 1) - __ldg(offs + g) < kMinRowsToSort) perm[r] = r;
+    }
+    for (int pass = 0; pass < (g_last != g_first ? 2 : 1); ++pass) {
+        const int g = pass ? g_last : g_first;
+        const int lo = offs ? __ldg(offs + g) : 0, hi = offs ? __ldg(offs + g + 1) : N;
+        if (hi - lo < kMinRowsToSort) continue;  // block-uniform
+        __syncthreads();  // the starts of the pass before have been read
+        const int* cnt = counters + (size_t)(lo / kMinRowsToSort) * kCodeBuckets + tid * PER;
         int c[PER], sum = 0;
 #pragma unroll
-        for (int x = 0; x < PER; ++x) { c[x] = tid * PER + x < kBuckets ? s_bin[tid * PER + x] : 0; sum += c[x]; }
+        for (int x = 0; x < PER; ++x) { c[x] = cnt[x]; sum += c[x]; }
         int incl = sum;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
@@ -93,26 +132,17 @@ graph_sort_kernel(const int32_t* __restrict__ offs, int G, int N, const unsigned
         }
         if (lane == 31) s_warp[wid] = incl;
         __syncthreads();
-        if (wid == 0) {
-            int v = s_warp[lane];
+        int start = lo + incl - sum;
+        for (int w = 0; w < wid; ++w) start += s_warp[w];
 #pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int t = __shfl_up_sync(0xFFFFFFFFu, v, o);
-                if (lane >= o) v += t;
-            }
-            s_warp[lane] = v;  // inclusive over warps
-        }
+        for (int x = 0; x < PER; ++x) { s_start[tid * PER + x] = start; start += c[x]; }
         __syncthreads();
-        int start = lo + (wid ? s_warp[wid - 1] : 0) + incl - sum;
-#pragma unroll
-        for (int x = 0; x < PER; ++x)
-            if (tid * PER + x < kBuckets) { s_bin[tid * PER + x] = start; start += c[x]; }
-        __syncthreads();
-        for (int r = lo + tid; r < hi; r += kSortThreads) perm[atomicAdd(&s_bin[code[r]], 1)] = r;
+        const int a = max(row_lo, lo), b = min(row_hi, hi);
+        for (int r = a + tid; r < b; r += kScatterThreads) perm[s_start[code[r]] + number[r]] = r;
     }
 }
 
-// The same sort, but stable (rows of a bucket stay in row order), so that the order - and with it which of
+// A sort of the pruned sweep's codes in one block per graph, stable (rows of a bucket stay in row order), so that the order - and with it which of
 // several keys with exactly equal scores the pruned sweep meets first - does not depend on the timing of
 // atomics.  Each of the 32 warps owns a contiguous chunk of the graph's rows and a histogram row of its
 // own in shared memory; after the counts are turned into start positions per (warp, bucket), a warp places
@@ -204,16 +234,6 @@ __global__ void gather_rows_kernel(const uint4* __restrict__ Q, const int* __res
 
 
 // ---- keys of the pruned sweep -------------------------------------------------------------------
-__device__ inline int graph_of(const int32_t* offs, int G, int i) {
-    if (offs == nullptr) return 0;
-    int a = 0, b = G;
-    while (b - a > 1) {
-        const int m = (a + b) >> 1;
-        if (__ldg(offs + m) <= i) a = m; else b = m;
-    }
-    return a;
-}
-
 // One warp per node: squared norm of the whole key vector, and the largest of each graph.
 __global__ void key_norm_kernel(const __nv_bfloat16* __restrict__ K, int N, int HD, const int32_t* __restrict__ offs,
                                 int G, float* __restrict__ norm2, unsigned* __restrict__ gmax,
@@ -380,10 +400,13 @@ cudaError_t launch_reorder_queries(const FwdArgs& a, const FwdWorkspace& w) {
         graph_sort_stable_kernel<kPivotBits><<<std::min(n_graphs, sm_count() * 2), kSortThreads, (32 << kPivotBits) * 4, a.stream>>>(
             a.graph_offsets, a.G, (int)a.N, code, perm, sb);
     } else {
-        query_code_kernel<<<(unsigned)((a.N * 32 + 255) / 256), 256, 0, a.stream>>>(
-            static_cast<const __nv_bfloat16*>(a.Q), (int)a.N, HD, code, sb);
-        graph_sort_kernel<kCodeBits><<<std::min(n_graphs, sm_count() * 2), kSortThreads, (1 << kCodeBits) * 4, a.stream>>>(
-            a.graph_offsets, a.G, (int)a.N, code, perm, sb);
+        int* counters = reinterpret_cast<int*>(a.topk_score);
+        cudaError_t err = cudaMemsetAsync(counters, 0, (size_t)(a.N / kMinRowsToSort) * kCodeBuckets * 4, a.stream);
+        if (err != cudaSuccess) return err;
+        query_code_kernel<<<(unsigned)((a.N + kCodeThreads - 1) / kCodeThreads), kCodeThreads, 0, a.stream>>>(
+            static_cast<const __nv_bfloat16*>(a.Q), (int)a.N, HD, a.graph_offsets, a.G, code, counters, a.topk_idx, sb);
+        scatter_rows_kernel<<<(unsigned)((a.N + kScatterRows - 1) / kScatterRows), kScatterThreads, 0, a.stream>>>(
+            a.graph_offsets, a.G, (int)a.N, code, counters, a.topk_idx, perm, sb);
     }
     if (w.f16) return cudaGetLastError();  // the half-precision prefilter gathers while it converts (f16_convert.cu)
     const int vec_per_row = HD * 2 / 16;

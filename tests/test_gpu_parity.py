@@ -320,3 +320,28 @@ def test_small_graphs_in_one_kernel(sizes, H, d, k, mode):
     # one warp per row in fp32: of bf16 values the same exact products and the same order of sums
     b = kb.forward(Q.float(), K.float(), V.float(), offs, k, kb.KMIP_FP32_EXACT, fp32_path=1)
     assert torch.equal(a.topk_idx, b.topk_idx) and torch.equal(a.topk_score, b.topk_score)
+
+
+@pytest.mark.parametrize("sizes", [[8192, 8191, 24385], [100, 9000, 0, 1, 7, 16384, 40, 8200, 1], [33000]])
+def test_sweep_order_of_large_graphs(sizes):
+    """The rows of a graph of at least 8192 rows are grouped by query (equal queries lie together), all others stay in order."""
+    N, H, d, k = sum(sizes), 1, 16, 8
+    g = torch.Generator().manual_seed(N)
+    kind = torch.randint(0, 60, (N,), generator=g)
+    Q = torch.randn(60, H, d, generator=g)[kind].bfloat16().cuda()
+    K = torch.randn(N, H, d, generator=g).bfloat16().cuda()
+    offs = torch.tensor(np.concatenate([[0], np.cumsum(sizes)]), dtype=torch.int32, device="cuda")
+    fb = kb.forward(Q, K, K, offs, k, kb.KMIP_BF16_TC)
+    order, _ = kb.kmip_test_sweep_order(fb.workspace, N, len(sizes), H, d, k, kb.KMIP_BF16_TC)
+    order = np.asarray(order)
+    lo = 0
+    for n in sizes:
+        part = order[lo:lo + n]
+        if n < 8192:
+            assert (part == np.arange(lo, lo + n)).all()
+        else:
+            assert (np.sort(part) == np.arange(lo, lo + n)).all()
+            kinds = kind.numpy()[part]
+            assert (kinds[1:] != kinds[:-1]).sum() < 60 * 60  # kinds that share a bucket may mix
+            assert (kinds[1:] != kinds[:-1]).mean() < 0.25    # unsorted: 59 of 60 neighbours differ
+        lo += n
