@@ -30,7 +30,7 @@ UNIT = "scores/s"
 FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustained": 1400.0}
 FWD_LAUNCHES = 5            # regroup keys, plan, score+select sweep, rescoring, softmax+gather-V
 F16_FWD_LAUNCHES = 7        # plan, norm maxima, operand conversion, prefilter sweep, rescoring, redo pass, softmax+gather-V
-REORDER_LAUNCHES = 3        # tensor-core mode from 32768 nodes on: locality codes, per-graph sort, permuted copy of Q
+REORDER_LAUNCHES = 3        # tensor-core mode from 32768 nodes on: locality codes, row order, permuted copy of Q
 BWD_LAUNCHES = 9            # rows, partition (count, 3 scan kernels, scatter), bucket sort (writes the list offsets), 2 segment kernels
 
 
@@ -155,9 +155,11 @@ def run_reference(args, w):
 
 def fwd_launches(w):
     """Kernels one forward call of the library launches for this workload."""
+    small_n = w.N // w.G * (w.d + 16)
+    if w.k <= 32 and w.d <= 64 and (small_n <= 15000 or w.N * w.H * small_n <= 300000000):
+        return 2                          # plan, the whole forward pass of small graphs
     if w.mode != wl.MODE_BF16_TC:
-        tiled = w.d <= 64 and w.k <= 32 and (w.N // 128) * w.H >= 48
-        return 4 if tiled else 3          # plan, sweep, (rescoring), softmax+gather-V
+        return F16_FWD_LAUNCHES if 4 <= w.k <= 32 and w.d <= 64 and w.N <= 1 << 19 else 4
     tc = w.k <= 64 or (w.k <= 128 and w.d <= 64)
     if not tc:
         return 3

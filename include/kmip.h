@@ -56,7 +56,8 @@ typedef enum {
     /* Q, K, V, out, d_out, dQ, dK, dV hold bf16.  Scores are a dense bf16 contraction with fp32
        accumulation on the tcgen05 tensor cores; softmax, sums and gradients accumulate in fp32. */
     KMIP_BF16_TC = 0,
-    /* All of them hold fp32.  Scores are fp32 fused multiply-adds in index order c = 0..d-1. */
+    /* All of them hold fp32.  Scores are fp32 fused multiply-adds in index order c = 0..d-1 (a half-precision filter with
+       a proven error bound may decide which keys need one). */
     KMIP_FP32_EXACT = 1,
     /* KMIP_BF16_TC with an exact pruning of the search (the quadratic search is the first limitation the
        paper names, Sec. 6): in graphs of 8192 nodes or more the keys are swept in an order that puts heavy
@@ -269,8 +270,9 @@ int kmip_last_status(const void *workspace, void *stream, int *device_status);
  * `stream`, then reads from the status block of `workspace` into counters[8] (HOST memory, int64):
  *   [0..3]  KMIP_BF16_TC_PRUNED: key tiles of all work items, key tiles loaded (one end marker per work
  *           item included), (key tile, query tile) pairs, pairs scored, summed over the sweep's CTAs;
- *   [4]     KMIP_BF16_TC with d <= 32 and k <= 32: (query, head) pairs that the half-precision prefilter
- *           could not decide and the exact kernel recomputed from all keys;
+ *   [4]     where the half-precision prefilter ran (KMIP_BF16_TC and KMIP_FP32_EXACT, d <= 64 with k <= 32 and d <= 32
+ *           with k <= 103, not the smallest calls): (query, head) pairs that it could not decide and the exact
+ *           kernel recomputed from all keys;
  *   [5..7]  zero.
  * Counters of a path that did not run are zero.  Returns KMIP_ERR_CUDA if the synchronisation or the
  * copy fails.
