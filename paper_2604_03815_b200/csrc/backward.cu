@@ -20,43 +20,42 @@ constexpr int kWarpsPerBlock = 8;
 constexpr int kLongSeg = 512;
 
 // ------------------------------------------------------------------------------------------ rows
-template <typename T, int D>
+template <typename T, int D, int E>
 __global__ void __launch_bounds__(kWarpsPerBlock * 32)
 bwd_rows_kernel(const T* __restrict__ K, const T* __restrict__ V, const T* __restrict__ dOut,
                 const int32_t* __restrict__ topk_idx, const float* __restrict__ topk_score,
                 int N, int H, int k, float scale, float drop_p, unsigned long long seed,
                 float* __restrict__ ws_p, float* __restrict__ ws_ds, T* __restrict__ dQ) {
-    constexpr int VEC = Elem<T>::kVec;
-    constexpr int LPR = D / VEC;
     const int lane = threadIdx.x & 31;
     const long long n_rows = (long long)N * H;
+    RowWalk walk(blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5), gridDim.x * kWarpsPerBlock, H);
     for (long long r = (long long)blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5); r < n_rows;
-         r += (long long)gridDim.x * kWarpsPerBlock) {
-        const int h = (int)(r % H);
-        int j[kMaxEntriesPerLane];
-        float p[kMaxEntriesPerLane];
+         r += (long long)gridDim.x * kWarpsPerBlock, walk.next()) {
+        const int h = walk.h;
+        int j[E];
+        float p[E];
         load_row_softmax(topk_idx + (size_t)r * k, topk_score + (size_t)r * k, k, N, scale, lane, j, p);
 
         // dP_t = g_i . v_{j_t}
-        float dP[kMaxEntriesPerLane];
+        float dP[E];
         gather_dot<T, D>(V, H, h, k, lane, dOut + (size_t)r * D, j, dP);
         // with dropout the output was sum_t f_t p_t v_t (f constant here): dP_t = f_t (g . v_t), and the
         // weight that reaches dV is f_t p_t
-        float f[kMaxEntriesPerLane];
+        float f[E];
 #pragma unroll
-        for (int e = 0; e < kMaxEntriesPerLane; ++e) f[e] = 1.0f;
+        for (int e = 0; e < E; ++e) f[e] = 1.0f;
         if (drop_p > 0.0f) {
             dropout_factors(r, k, lane, drop_p, seed, f);
 #pragma unroll
-            for (int e = 0; e < kMaxEntriesPerLane; ++e) dP[e] *= f[e];
+            for (int e = 0; e < E; ++e) dP[e] *= f[e];
         }
         float dsum = 0.0f;
 #pragma unroll
-        for (int e = 0; e < kMaxEntriesPerLane; ++e) dsum = fmaf(p[e], dP[e], dsum);
+        for (int e = 0; e < E; ++e) dsum = fmaf(p[e], dP[e], dsum);
         dsum = warp_sum(dsum);
-        float dS[kMaxEntriesPerLane];
+        float dS[E];
 #pragma unroll
-        for (int e = 0; e < kMaxEntriesPerLane; ++e) {
+        for (int e = 0; e < E; ++e) {
             dS[e] = scale * p[e] * (dP[e] - dsum);
             const int t = e * 32 + lane;
             if (t < k) {
@@ -64,9 +63,7 @@ bwd_rows_kernel(const T* __restrict__ K, const T* __restrict__ V, const T* __res
                 ws_ds[(size_t)r * k + t] = dS[e];
             }
         }
-        float acc[VEC];
-        gather_weighted_sum<T, D>(K, H, h, k, lane, j, dS, acc);
-        if (lane < LPR) Elem<T>::store_vec(dQ + (size_t)r * D + lane * VEC, acc);
+        gather_weighted_sum<T, D>(K, H, h, k, lane, j, dS, dQ + (size_t)r * D);
     }
 }
 
@@ -574,26 +571,27 @@ bwd_segments_kernel(const T* __restrict__ Q, const T* __restrict__ dOut,
     constexpr int LPR = D / VEC;
     constexpr int EPW = 32 / LPR;
     const int lane = threadIdx.x & 31, part = lane % LPR, sub = lane / LPR;
+    RowWalk walk(blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5), gridDim.x * kWarpsPerBlock, H);
     for (long long x = (long long)blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5); x < n_segs;
-         x += (long long)gridDim.x * kWarpsPerBlock) {
+         x += (long long)gridDim.x * kWarpsPerBlock, walk.next()) {
         const int start = __ldg(seg_off + x), len = __ldg(seg_off + x + 1) - start;
         if (len > kLongSeg) continue;  // reduced by bwd_long_segments_kernel
-        const int h = (int)(x % H);
         float accV[VEC], accK[VEC];
 #pragma unroll
         for (int c = 0; c < VEC; ++c) { accV[c] = 0.0f; accK[c] = 0.0f; }
-        accumulate_list<T, D>(hits + start, sub, EPW, len, h, H, part, Q, dOut, accV, accK);
-#pragma unroll
-        for (int o = LPR; o < 32; o <<= 1) {
-#pragma unroll
-            for (int c = 0; c < VEC; ++c) {
-                accV[c] += __shfl_xor_sync(0xFFFFFFFFu, accV[c], o);
-                accK[c] += __shfl_xor_sync(0xFFFFFFFFu, accK[c], o);
-            }
-        }
-        if (lane < LPR) {
+        accumulate_list<T, D>(hits + start, sub, EPW, len, walk.h, H, part, Q, dOut, accV, accK);
+        if constexpr (LPR == 32) {
             Elem<T>::store_vec(dV + (size_t)x * D + lane * VEC, accV);
             Elem<T>::store_vec(dK + (size_t)x * D + lane * VEC, accK);
+        } else {
+            // both sums as one: after the first exchange a lane keeps dV or dK
+            float both[2 * VEC];
+#pragma unroll
+            for (int c = 0; c < VEC; ++c) { both[c] = accV[c]; both[VEC + c] = accK[c]; }
+            using Sums = ColumnSums<2 * VEC, LPR>;
+            const int col = column_sums<2 * VEC, LPR>(both, lane);
+            T* const to = (col < VEC ? dV : dK) + (size_t)x * D + part * VEC + col % VEC;
+            if (lane < Sums::kWriters) store_columns<Sums::kLeft>(to, both);
         }
     }
 }
@@ -678,7 +676,8 @@ cudaError_t launch_d(const BwdArgs& a, const BwdWorkspace& w, cudaEvent_t* ev) {
     cudaError_t err;
 
     const int row_blocks = (int)std::min<long long>((n_rows + kWarpsPerBlock - 1) / kWarpsPerBlock, (long long)sm_count() * 32);
-    bwd_rows_kernel<T, D><<<row_blocks, kWarpsPerBlock * 32, 0, a.stream>>>(
+    auto rows_kernel = a.k <= 32 ? bwd_rows_kernel<T, D, 1> : bwd_rows_kernel<T, D, kMaxEntriesPerLane>;
+    rows_kernel<<<row_blocks, kWarpsPerBlock * 32, 0, a.stream>>>(
         K, V, dOut, a.topk_idx, a.topk_score, (int)a.N, a.H, a.k, scale, a.drop_p, a.seed, ws_p, ws_ds,
         static_cast<T*>(a.dQ));
     if (ev) cudaEventRecord(ev[0], a.stream);

@@ -11,32 +11,29 @@ namespace {
 
 constexpr int kWarpsPerBlock = 8;
 
-template <typename T, int D>
+template <typename T, int D, int E>
 __global__ void __launch_bounds__(kWarpsPerBlock * 32)
 softmax_gather_kernel(const T* __restrict__ V, const int32_t* __restrict__ topk_idx,
                       const float* __restrict__ topk_score, int N, int H, int k, float scale,
                       float drop_p, unsigned long long seed, T* __restrict__ out,
                       const StatusBlock* __restrict__ sb) {
     if (sb->status != KMIP_OK) return;  // an earlier stage failed: topk_idx was not written
-    constexpr int VEC = Elem<T>::kVec;
-    constexpr int LPR = D / VEC;
     const int lane = threadIdx.x & 31;
     const long long n_rows = (long long)N * H;
+    RowWalk walk(blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5), gridDim.x * kWarpsPerBlock, H);
     for (long long r = (long long)blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5); r < n_rows;
-         r += (long long)gridDim.x * kWarpsPerBlock) {
-        const int h = (int)(r % H);
-        int j[kMaxEntriesPerLane];
-        float p[kMaxEntriesPerLane];
+         r += (long long)gridDim.x * kWarpsPerBlock, walk.next()) {
+        const int h = walk.h;
+        int j[E];
+        float p[E];
         load_row_softmax(topk_idx + (size_t)r * k, topk_score + (size_t)r * k, k, N, scale, lane, j, p);
         if (drop_p > 0.0f) {  // training only: the weights go through dropout before the weighted sum
-            float f[kMaxEntriesPerLane];
+            float f[E];
             dropout_factors(r, k, lane, drop_p, seed, f);
 #pragma unroll
-            for (int e = 0; e < kMaxEntriesPerLane; ++e) p[e] *= f[e];
+            for (int e = 0; e < E; ++e) p[e] *= f[e];
         }
-        float acc[VEC];
-        gather_weighted_sum<T, D>(V, H, h, k, lane, j, p, acc);
-        if (lane < LPR) Elem<T>::store_vec(out + (size_t)r * D + lane * VEC, acc);
+        gather_weighted_sum<T, D>(V, H, h, k, lane, j, p, out + (size_t)r * D);
     }
 }
 
@@ -44,7 +41,8 @@ template <typename T, int D>
 cudaError_t launch_d(const FwdArgs& a) {
     const long long n_rows = (long long)a.N * a.H;
     const int blocks = (int)std::min<long long>((n_rows + kWarpsPerBlock - 1) / kWarpsPerBlock, (long long)sm_count() * 32);
-    softmax_gather_kernel<T, D><<<blocks, kWarpsPerBlock * 32, 0, a.stream>>>(
+    auto kern = a.k <= 32 ? softmax_gather_kernel<T, D, 1> : softmax_gather_kernel<T, D, kMaxEntriesPerLane>;
+    kern<<<blocks, kWarpsPerBlock * 32, 0, a.stream>>>(
         static_cast<const T*>(a.V), a.topk_idx, a.topk_score, (int)a.N, a.H, a.k,
         1.0f / sqrtf((float)a.d), a.drop_p, a.seed, static_cast<T*>(a.out), reinterpret_cast<const StatusBlock*>(a.ws));
     return cudaGetLastError();

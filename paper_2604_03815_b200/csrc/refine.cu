@@ -9,6 +9,7 @@
 #include <algorithm>
 
 #include "common.cuh"
+#include "rowops.cuh"
 #include "topk_buffer.cuh"
 
 namespace kmip {
@@ -46,9 +47,10 @@ refine_topk_kernel(const T* __restrict__ Q, const T* __restrict__ Kp, const int3
     const long long n_rows = (long long)N * H;
     const int room = CAP - k;
 
+    RowWalk walk(blockIdx.x * kWarpsPerBlock + wib, gridDim.x * kWarpsPerBlock, H);
     for (long long r = (long long)blockIdx.x * kWarpsPerBlock + wib; r < n_rows;
-         r += (long long)gridDim.x * kWarpsPerBlock) {
-        const int i = (int)(r / H), h = (int)(r % H);
+         r += (long long)gridDim.x * kWarpsPerBlock, walk.next()) {
+        const int i = walk.i, h = walk.h;
         const int hi = graph_end(offs, G, N, i);
 
         // the row's groups: entry t in lane t%32, register t/32

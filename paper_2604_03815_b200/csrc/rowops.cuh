@@ -1,6 +1,10 @@
 // Warp-level building blocks for the gather stages (Algorithm 1 lines 4-6 and their backward):
 // softmax over the k kept scores of one (query, head) row, and the weighted sum of gathered rows
 // with 16-byte vector loads.
+// The kernels made of them are bound by instruction issue more than by their gathers.  With sums by halves instead of
+// butterflies, one entry per lane where k <= 32 and no 64-bit division per row (us, before / after): softmax_gather 100k
+// nodes H 4 d 32 k 16 160 / 114, 4 x 200k nodes H 8 d 16 k 16 2201 / 1423; bwd_rows 309 / 232, 3901 / 2702; bwd_segments
+// 4 x 200k nodes 1888 / 1061.
 #pragma once
 
 #include "common.cuh"
@@ -8,7 +12,7 @@
 
 namespace kmip {
 
-constexpr int kMaxEntriesPerLane = 4;  // k <= 128
+constexpr int kMaxEntriesPerLane = 4;  // k <= 128; kernels come with E = 1 (k <= 32) and E = 4 entries per lane
 
 __device__ __forceinline__ float warp_max(float v) {
 #pragma unroll
@@ -21,15 +25,87 @@ __device__ __forceinline__ float warp_sum(float v) {
     return v;
 }
 
+// The (query, head) rows first, first + step, ... of a warp: row = i * H + h, without a 64-bit division per row.
+struct RowWalk {
+    int i, h;
+    int H, di, dh;
+    __device__ __forceinline__ RowWalk(unsigned first, unsigned step, int H_)
+        : i((int)(first / (unsigned)H_)), h((int)(first % (unsigned)H_)), H(H_), di((int)(step / (unsigned)H_)), dh((int)(step % (unsigned)H_)) {}
+    __device__ __forceinline__ void next() {
+        i += di;
+        h += dh;
+        if (h >= H) { h -= H; ++i; }
+    }
+};
+
+// Column sums over the 32 / LPR lane groups of a warp.  Before: lane l holds W partial sums for part l % LPR.  A step
+// exchanges halves, so W + W / 2 + ... values move instead of W per step (the additions are those of a butterfly, bit for
+// bit).  After: v[0 .. kLeft) of lane l are the full sums of columns col .. col + kLeft of its part (`col` returned), and
+// the lanes below kWriters hold every column once.
+template <int W, int LPR>
+struct ColumnSums {
+    static constexpr int kGroups = 32 / LPR;
+    static constexpr int kLeft = W > kGroups ? W / kGroups : 1;
+    static constexpr int kWriters = W > kGroups ? 32 : LPR * W;
+};
+template <int W, int LPR>
+__device__ __forceinline__ int column_sums(float (&v)[W], int lane) {
+    int col = 0, w = W;
+#pragma unroll
+    for (int o = LPR; o < 32; o <<= 1) {
+        if (w > 1) {
+            const int half = w / 2;
+            const bool up = (lane & o) != 0;
+#pragma unroll
+            for (int c = 0; c < W / 2; ++c) {
+                if (c < half) {
+                    const float send = up ? v[c] : v[c + half], keep = up ? v[c + half] : v[c];
+                    v[c] = keep + __shfl_xor_sync(0xFFFFFFFFu, send, o);
+                }
+            }
+            col += up ? half : 0;
+            w = half;
+        } else {
+            v[0] += __shfl_xor_sync(0xFFFFFFFFu, v[0], o);
+        }
+    }
+    return col;
+}
+
+// n values to consecutive columns, n times the element size aligned.
+template <int n>
+__device__ __forceinline__ void store_columns(float* p, const float* v) {
+    if constexpr (n == 1) *p = v[0];
+    else if constexpr (n == 2) *reinterpret_cast<float2*>(p) = make_float2(v[0], v[1]);
+    else *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
+}
+template <int n>
+__device__ __forceinline__ void store_columns(__nv_bfloat16* p, const float* v) {
+    if constexpr (n == 1) {
+        *p = __float2bfloat16_rn(v[0]);
+    } else {
+        uint32_t w[n / 2];
+#pragma unroll
+        for (int i = 0; i < n / 2; ++i) {
+            const __nv_bfloat162 b = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
+            w[i] = *reinterpret_cast<const uint32_t*>(&b);
+        }
+        if constexpr (n == 2) *reinterpret_cast<uint32_t*>(p) = w[0];
+        else if constexpr (n == 4) *reinterpret_cast<uint2*>(p) = make_uint2(w[0], w[1]);
+        else *reinterpret_cast<uint4*>(p) = make_uint4(w[0], w[1], w[2], w[3]);
+    }
+}
+
 // Entry t of a row lives in lane t%32, register t/32.  Loads the row's indices and scores and
 // turns the scores into softmax weights p_t = exp((s_t - max)/sqrt(d)) / sum (Algorithm 1 line 5).
 // Empty slots (index < 0) and indices outside [0, N) get weight 0.
+template <int E>
 __device__ __forceinline__ void load_row_softmax(const int32_t* idx_row, const float* score_row, int k, int N,
                                                  float scale, int lane,
-                                                 int (&j)[kMaxEntriesPerLane], float (&p)[kMaxEntriesPerLane]) {
+                                                 int (&j)[E], float (&p)[E]) {
     float m = -CUDART_INF_F;
 #pragma unroll
-    for (int e = 0; e < kMaxEntriesPerLane; ++e) {
+    for (int e = 0; e < E; ++e) {
         const int t = e * 32 + lane;
         j[e] = -1;
         p[e] = -CUDART_INF_F;
@@ -44,24 +120,25 @@ __device__ __forceinline__ void load_row_softmax(const int32_t* idx_row, const f
     m = warp_max(m);
     float z = 0.0f;
 #pragma unroll
-    for (int e = 0; e < kMaxEntriesPerLane; ++e) {
+    for (int e = 0; e < E; ++e) {
         p[e] = (j[e] >= 0) ? __expf((p[e] - m) * scale) : 0.0f;
         z += p[e];
     }
     z = warp_sum(z);
     const float inv = z > 0.0f ? 1.0f / z : 0.0f;
 #pragma unroll
-    for (int e = 0; e < kMaxEntriesPerLane; ++e) p[e] *= inv;
+    for (int e = 0; e < E; ++e) p[e] *= inv;
 }
 
 // Attention dropout on the k weights of row r (= query * H + head): factor 1/(1-drop) when the slot's
 // counter-based uniform is >= drop, else 0.  The draw of slot t is the (r*k + t + 1)-th SplitMix64
 // output for `seed`, top 24 bits / 2^24.  f[e] belongs to entry t = e*32 + lane.
+template <int E>
 __device__ __forceinline__ void dropout_factors(long long r, int k, int lane, float drop, unsigned long long seed,
-                                                float (&f)[kMaxEntriesPerLane]) {
+                                                float (&f)[E]) {
     const float keep_scale = 1.0f / (1.0f - drop);
 #pragma unroll
-    for (int e = 0; e < kMaxEntriesPerLane; ++e) {
+    for (int e = 0; e < E; ++e) {
         const unsigned long long pair = (unsigned long long)r * (unsigned long long)k + (unsigned long long)(e * 32 + lane);
         unsigned long long z = seed + (pair + 1ull) * 0x9E3779B97F4A7C15ull;
         z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
@@ -72,23 +149,21 @@ __device__ __forceinline__ void dropout_factors(long long r, int k, int lane, fl
     }
 }
 
-// acc (per lane: VEC columns of the part this lane owns) = sum_t w_t * X[j_t, h, part*VEC ..].
+// out_row[0, D) = sum_t w_t * X[j_t, h, :].
 // LPR = D/VEC lanes share one gathered row (one 16-byte load each), 32/LPR rows per round.
-// After the call lanes 0..LPR-1 hold the full sums for their part.
-template <typename T, int D>
+template <typename T, int D, int E>
 __device__ __forceinline__ void gather_weighted_sum(const T* __restrict__ X, int H, int h, int k, int lane,
-                                                    const int (&j)[kMaxEntriesPerLane],
-                                                    const float (&w)[kMaxEntriesPerLane],
-                                                    float (&acc)[Elem<T>::kVec]) {
+                                                    const int (&j)[E], const float (&w)[E], T* __restrict__ out_row) {
     constexpr int VEC = Elem<T>::kVec;
     constexpr int LPR = D / VEC;
     constexpr int EPW = 32 / LPR;
     static_assert(LPR >= 1 && LPR <= 32, "row width");
     const int part = lane % LPR, sub = lane / LPR;
+    float acc[VEC];
 #pragma unroll
     for (int c = 0; c < VEC; ++c) acc[c] = 0.0f;
 #pragma unroll
-    for (int e = 0; e < kMaxEntriesPerLane; ++e) {
+    for (int e = 0; e < E; ++e) {
         if (e * 32 < k) {
 #pragma unroll
             for (int base = 0; base < 32; base += EPW) {
@@ -105,20 +180,18 @@ __device__ __forceinline__ void gather_weighted_sum(const T* __restrict__ X, int
             }
         }
     }
-#pragma unroll
-    for (int o = LPR; o < 32; o <<= 1) {
-#pragma unroll
-        for (int c = 0; c < VEC; ++c) acc[c] += __shfl_xor_sync(0xFFFFFFFFu, acc[c], o);
-    }
+    using Sums = ColumnSums<VEC, LPR>;
+    const int col = column_sums<VEC, LPR>(acc, lane);
+    if (lane < Sums::kWriters) store_columns<Sums::kLeft>(out_row + part * VEC + col, acc);
 }
 
 // dots[e] of lane l = g . X[j[e] of lane l, h, :] for the row's entries (entry t in lane t % 32, register t / 32), with
 // the same lane layout as gather_weighted_sum: LPR lanes share one gathered row, one 16-byte load each, so a load
 // instruction touches 32 / LPR rows instead of 32; the partial sums of a row are added across its lanes and handed
 // to the entry's own lane.  g is the row-major vector of D elements at `g_row`.
-template <typename T, int D>
+template <typename T, int D, int E>
 __device__ __forceinline__ void gather_dot(const T* __restrict__ X, int H, int h, int k, int lane, const T* __restrict__ g_row,
-                                           const int (&j)[kMaxEntriesPerLane], float (&dots)[kMaxEntriesPerLane]) {
+                                           const int (&j)[E], float (&dots)[E]) {
     constexpr int VEC = Elem<T>::kVec;
     constexpr int LPR = D / VEC;
     constexpr int EPW = 32 / LPR;
@@ -126,7 +199,7 @@ __device__ __forceinline__ void gather_dot(const T* __restrict__ X, int H, int h
     float gv[VEC];
     Elem<T>::load_vec(g_row + part * VEC, gv);
 #pragma unroll
-    for (int e = 0; e < kMaxEntriesPerLane; ++e) {
+    for (int e = 0; e < E; ++e) {
         dots[e] = 0.0f;
         if (e * 32 < k) {
 #pragma unroll

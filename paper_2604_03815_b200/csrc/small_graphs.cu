@@ -80,7 +80,7 @@ small_forward_kernel(const T* __restrict__ Q, const T* __restrict__ K, const T* 
                      int N, int H, int k, int rows_per_warp, float scale, float drop_p, unsigned long long seed, T* __restrict__ out,
                      int32_t* __restrict__ topk_idx, float* __restrict__ topk_score, StatusBlock* __restrict__ sb) {
     if (sb->status != KMIP_OK) return;
-    constexpr int VEC = Elem<T>::kVec, LPR = D / VEC, P = D * (int)sizeof(T) / 16, kStride = row_stride<T, D>();
+    constexpr int P = D * (int)sizeof(T) / 16, kStride = row_stride<T, D>();
     extern __shared__ __align__(16) unsigned char smem[];
     unsigned char* sK = smem;                                          // [kChunk] padded key rows
     cand_t* sList = reinterpret_cast<cand_t*>(sK + kChunk * kStride);  // [rows of the block][32] running lists
@@ -197,28 +197,24 @@ small_forward_kernel(const T* __restrict__ Q, const T* __restrict__ K, const T* 
                         continue;
                     }
                     // softmax over the kept scores and the weighted sum of their V rows
-                    int jj[kMaxEntriesPerLane];
-                    float p[kMaxEntriesPerLane];
+                    int jj[1];
+                    float p[1];
                     jj[0] = best ? cand_index(best) : -1;
                     const float sc = best ? cand_score(best) : -CUDART_INF_F;
                     const float mx = __shfl_sync(FULL, sc, 0);
                     p[0] = best ? __expf((sc - mx) * scale) : 0.0f;
                     const float z = warp_sum(p[0]);
                     p[0] *= z > 0.0f ? 1.0f / z : 0.0f;
-#pragma unroll
-                    for (int e = 1; e < kMaxEntriesPerLane; ++e) { jj[e] = -1; p[e] = 0.0f; }
                     if (lane < k) {
                         topk_idx[r * k + lane] = jj[0];
                         topk_score[r * k + lane] = sc;
                     }
                     if (drop_p > 0.0f) {
-                        float f[kMaxEntriesPerLane];
+                        float f[1];
                         dropout_factors((long long)r, k, lane, drop_p, seed, f);
                         p[0] *= f[0];
                     }
-                    float acc[VEC];
-                    gather_weighted_sum<T, D>(V, H, h, k, lane, jj, p, acc);
-                    if (lane < LPR) Elem<T>::store_vec(out + r * D + lane * VEC, acc);
+                    gather_weighted_sum<T, D>(V, H, h, k, lane, jj, p, out + r * D);
                 }
             }
             i0 = i1;
