@@ -27,17 +27,17 @@ __device__ __forceinline__ void load8(const float* p, float (&v)[8]) {
 constexpr int kNormThreads = 256;
 
 // One head per grid row, a thread per node and step; a block reduces its maxima in registers and shared
-// memory and issues three atomics.  Bound by DRAM: Q and K are read once.  One atomic per row into the three slots of
+// memory and issues an atomic for each that is not zero.  Bound by DRAM: Q and K are read once.  One atomic per row into the slots of
 // its head serialised instead: 31 us for 22 400 nodes (4 heads), 27 us for 31 623 (1 head); now 2 to 3 us.
 template <typename T, int D>
 __global__ void __launch_bounds__(kNormThreads)
 f16_norm_max_kernel(const T* __restrict__ Q, const T* __restrict__ K, int N, int H,
                     unsigned* __restrict__ stat, const StatusBlock* __restrict__ sb) {
     if (sb->status != KMIP_OK) return;
-    __shared__ unsigned s_max[3][kNormThreads / 32];
+    __shared__ unsigned s_max[4][kNormThreads / 32];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     for (int h = blockIdx.y; h < H; h += gridDim.y) {
-        unsigned vals[3] = {0u, 0u, 0u};
+        unsigned vals[4] = {0u, 0u, 0u, 0u};  // the fields of F16HeadStat
         for (long long j = (long long)blockIdx.x * kNormThreads + threadIdx.x; j < N; j += (long long)gridDim.x * kNormThreads) {
             const size_t r = (size_t)j * H + h;
             float q2 = 0.0f, k2 = 0.0f, ka2 = 0.0f;
@@ -54,21 +54,22 @@ f16_norm_max_kernel(const T* __restrict__ Q, const T* __restrict__ K, int N, int
                 if (c0 == 8) ka2 = k2;  // the first 16 elements
             }
             // rounded up a little so that the fp32 sums above never understate a norm; the bits of non-negative floats
-            // order like the numbers, and rows that are not finite do not count
-            const float up[3] = {q2 * 1.00001f, k2 * 1.00001f, ka2 * 1.00001f};
-#pragma unroll
-            for (int x = 0; x < 3; ++x) {
-                const unsigned v = __float_as_uint(up[x]);
-                if (v < 0x7F800000u) vals[x] = max(vals[x], v);
+            // order like the numbers
+            if (q2 < kF16RangeN2) vals[0] = max(vals[0], __float_as_uint(q2 * 1.00001f));
+            if (k2 < kF16RangeN2) {
+                vals[1] = max(vals[1], __float_as_uint(k2 * 1.00001f));
+                vals[2] = max(vals[2], __float_as_uint(ka2 * 1.00001f));
+            } else if (k2 == k2) {  // a key with a NaN scores NaN everywhere and is nobody's choice
+                vals[3] = 0x7F800000u;
             }
         }
 #pragma unroll
-        for (int x = 0; x < 3; ++x) {
+        for (int x = 0; x < 4; ++x) {
             const unsigned m = __reduce_max_sync(0xFFFFFFFFu, vals[x]);
             if (lane == 0) s_max[x][wid] = m;
         }
         __syncthreads();
-        if (wid < 3) {
+        if (wid < 4) {
             const unsigned m = __reduce_max_sync(0xFFFFFFFFu, lane < kNormThreads / 32 ? s_max[wid][lane] : 0u);
             if (lane == 0 && m) atomicMax(stat + h * 4 + wid, m);
         }

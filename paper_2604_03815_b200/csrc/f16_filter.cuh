@@ -14,6 +14,11 @@ constexpr int kF16List32 = 48;
 // ... and for 32 < k <= 103.
 constexpr int kF16ListMost = 120;
 
+// Rows whose squared norm reaches this (or is not finite) take no part in the maxima below: their fp16 copies overflow under
+// any scale that suits the others.  Such a query row, and every row of a head with such a key, is scored exactly
+// (refine_f16.cu).
+constexpr float kF16RangeN2 = 1.5e38f;
+
 // Per head: largest squared norm of a query row, of a key row, and of the first 16 elements of a key
 // row (the partial sum after the first tensor-core step of a wider head); largest squared norm of what the conversion
 // of a key row to fp16 lost (fp32 storage only; bf16 values convert exactly up to underflow).  Float bits, maxima taken
@@ -22,7 +27,7 @@ struct F16HeadStat {
     float q_n2max;
     float k_n2max;
     float k_first16_n2max;
-    float k_lost_n2max;  // of the SCALED row
+    float k_lost_n2max;  // of the SCALED row; +infinity: the head has a key beyond kF16RangeN2
 };
 
 // Power of two s such that s * sqrt(n2max) lies in [32, 64) (up to the rounding of the square root):

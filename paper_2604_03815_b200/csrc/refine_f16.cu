@@ -12,7 +12,8 @@
 //   3. If the sweep dropped groups, these have maxima at most g_min, the smallest one kept.  When g_min + err(g_min) reaches the k-th best exact score found, a dropped group could
 //      still hold a better key: the row goes to the redo list and the exact CUDA-core kernel
 //      recomputes it from all keys.  That needs more than L groups within the error bound of the
-//      k-th best score, which well-separated scores never produce; rows whose keys tie massively do.
+//      k-th best score, which well-separated scores never produce; rows whose keys tie massively do.  Rows
+//      whose fp16 scores are no scores (a query or a key of the head beyond kF16RangeN2) go there unseen.
 // One warp per (query, head); a candidate key's row is read by D / 8 neighbouring lanes.
 #include <algorithm>
 
@@ -211,6 +212,9 @@ refine_f16_kernel(const T* __restrict__ Q, const T* __restrict__ K,
             if (kLossy) qlost2 += __shfl_xor_sync(FULL, qlost2, o);
             ok_min = min(ok_min, __shfl_xor_sync(FULL, ok_min, o));
         }
+        // beyond the range of the copies the fp16 scores say nothing (the sum here runs in another order than the
+        // conversion's, hence the margin): straight to the exact kernel.  A query with a NaN scores NaN in either.
+        const bool blind = q2 >= 0.999f * kF16RangeN2 || !(hs.k_lost_n2max < CUDART_INF_F);
         const float nq = sqrtf(q2) * sq * 1.00001f;
         const float nk = sqrtf(hs.k_n2max) * sk, nka = sqrtf(hs.k_first16_n2max) * sk;
         float partial = 0.0f;  // |q[0:16 s]| |k[0:16 s]| over the steps before the last
@@ -245,7 +249,7 @@ refine_f16_kernel(const T* __restrict__ Q, const T* __restrict__ K,
 #pragma unroll
         for (int e = 0; e < EPL; ++e) {
             const float g = __half2float(__ushort_as_half((unsigned short)f16_unordered(okey[e])));
-            const bool keep = okey[e] != 0u && (g + ea + er * fabsf(g) >= lowS);
+            const bool keep = !blind && okey[e] != 0u && (g + ea + er * fabsf(g) >= lowS);
             const unsigned m = __ballot_sync(FULL, keep);
             if (keep) words[n_kept + __popc(m & ((1u << lane) - 1u))] = word[e];
             n_kept += __popc(m);
@@ -324,7 +328,7 @@ refine_f16_kernel(const T* __restrict__ Q, const T* __restrict__ K,
         // the sweep dropped a group unless the list holds every group of the graph; a dropped one scores at most
         // g_min + err(g_min) exactly (scaled), and it matters if that reaches the k-th best score found
         const int n_groups = 2 * ((hi - lo) / 16) + min((hi - lo) % 16, 2);
-        if (n_valid < n_groups && g_min + ea + er * fabsf(g_min) >= kth * sc - fp32_err) {
+        if (blind || (n_valid < n_groups && g_min + ea + er * fabsf(g_min) >= kth * sc - fp32_err)) {
             if (lane == 0) {
                 const int pos = atomicAdd(&sb->n_redo, 1);
                 if (kmip_check(pos >= 0 && pos < n_rows, sb, 102)) redo_list[pos] = (int)r;  // checks builds: inside the list

@@ -196,3 +196,26 @@ def test_long_lists_through_the_filter(sizes, H, d, k, mode):
         a = kb.forward(Q, K, V, offs, k, w.mode)
         b = kb.forward(Q.float(), K.float(), V.float(), offs, k, kb.KMIP_FP32_EXACT, fp32_path=1)
         assert torch.equal(a.topk_idx, b.topk_idx) and torch.equal(a.topk_score, b.topk_score)
+
+
+@pytest.mark.parametrize("mode,d,k", [("fp32", 16, 12), ("fp32", 64, 8), ("bf16", 64, 20), ("bf16", 32, 45), ("bf16", 16, 16)])
+@pytest.mark.parametrize("what", ["key", "key_inf", "key_nan", "query", "query_nan"])
+def test_rows_beyond_the_range_of_the_copies(mode, d, k, what):
+    """A key or query whose squared norm overflows has no half-precision copy under the scale that suits the others; its
+    scores are finite all the same (or infinite, or not numbers), and the answer is what one warp per row finds in fp32."""
+    N, H = 4000, 2
+    g = torch.Generator().manual_seed(d + k)
+    Q, K, V = (torch.randn(N, H, d, generator=g).to(torch.bfloat16).cuda() for _ in range(3))
+    if what == "key": K[1234, 0] *= 1e20
+    if what == "key_inf": K[1234, 0, 3] = float("inf")
+    if what == "key_nan": K[1234, 0, 3] = float("nan")
+    if what == "query": Q[77, 1] *= 1e20
+    if what == "query_nan": Q[77, 1, 5] = float("nan")
+    m = kb.KMIP_FP32_EXACT if mode == "fp32" else kb.KMIP_BF16_TC
+    a = kb.forward(*(t.to(kb.storage_dtype(m)) for t in (Q, K, V)), None, k, m)
+    redo = kb.kmip_attn_sweep_counters(a.workspace)[4]
+    assert redo >= {"key": N, "key_inf": N, "query": 1}.get(what, 0) and redo < N + 100
+    b = kb.forward(Q.float(), K.float(), V.float(), None, k, kb.KMIP_FP32_EXACT, fp32_path=1)
+    assert torch.equal(a.topk_idx, b.topk_idx) and torch.equal(a.topk_score, b.topk_score)
+    if what == "key":
+        assert int((a.topk_idx[:, 0, 0] == 1234).sum()) > N // 4
