@@ -97,7 +97,9 @@ int kmip_attn_workspace_bytes(int64_t N, int32_t G, int32_t H, int32_t d, int32_
  * graph_offsets may be NULL, meaning one graph [0, N) (G is then ignored).
  * N = 0 returns KMIP_OK and enqueues nothing.
  * Inputs: Q, K, V, graph_offsets.  Outputs (fully overwritten when the device status word stays
- * KMIP_OK, undefined otherwise): out, topk_idx, topk_score.
+ * KMIP_OK, undefined otherwise): out, topk_idx, topk_score.  All three serve as scratch before they are
+ * written, so they must not overlap the inputs or each other, with one exception: `out` may overlap Q or K
+ * (an in-place inference call; some sizes then take a slower sweep).
  * In KMIP_BF16_TC mode the selection uses tensor-core scores, so a key whose exact score
  * differs from the k-th best by less than the fp32 accumulation error may swap with it.
  */

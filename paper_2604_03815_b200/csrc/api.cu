@@ -97,6 +97,12 @@ int kmip_test_attn_forward(const void* Q, const void* K, const void* V, const in
 
 namespace {
 
+// Whether two arrays of `bytes` bytes share any.
+bool overlap(const void* a, const void* b, size_t bytes) {
+    const uintptr_t x = reinterpret_cast<uintptr_t>(a), y = reinterpret_cast<uintptr_t>(b);
+    return x < y + bytes && y < x + bytes;
+}
+
 int forward_impl(const void* Q, const void* K, const void* V, const int32_t* graph_offsets, int32_t G, int64_t N,
                  int32_t H, int32_t d, int32_t k, int mode, float drop_p, uint64_t seed, void* out,
                  int32_t* topk_idx, float* topk_score, void* workspace, size_t workspace_bytes, void* stream,
@@ -112,6 +118,9 @@ int forward_impl(const void* Q, const void* K, const void* V, const int32_t* gra
         return KMIP_ERR_INVALID_ARG;
     FwdWorkspace w = plan_fwd_workspace(N, graph_offsets ? G : 1, H, d, k, mode);
     if (mode == KMIP_FP32_EXACT && opt && opt->fp32_path != 0) w.f16 = w.in_outputs = false;  // a test picks the CUDA-core sweep
+    const size_t array_bytes = (size_t)N * H * d * (mode == KMIP_FP32_EXACT ? 4 : 2);
+    const bool in_place = overlap(out, Q, array_bytes) || overlap(out, K, array_bytes);
+    if (in_place && w.in_outputs) w.f16 = w.in_outputs = false;  // the sweep that keeps its lists in the index and score arrays
     const bool tc = w.tc;
     if (workspace_bytes < w.total) return KMIP_ERR_WORKSPACE;
     if (w.f16) w.item_tiles = score_select_f16_item_tiles(N, graph_offsets ? G : 1, H, d, w.list);
@@ -120,6 +129,7 @@ int forward_impl(const void* Q, const void* K, const void* V, const int32_t* gra
               static_cast<unsigned char*>(workspace), static_cast<cudaStream_t>(stream)};
     a.drop_p = drop_p;
     a.seed = seed;
+    a.in_place = in_place;
     if (opt) {
         a.wait_limit_cycles = opt->wait_limit_cycles;
         a.drop_first_tile = opt->drop_first_tile;
@@ -130,7 +140,7 @@ int forward_impl(const void* Q, const void* K, const void* V, const int32_t* gra
     cudaEvent_t* ev = (g_prof.on && g_prof.n_fwd < g_prof.max_calls) ? g_prof.fwd[g_prof.n_fwd++] : nullptr;
     if (ev) cudaEventRecord(ev[0], a.stream);
     const bool test_sweep = opt && (opt->fp32_path != 0 || opt->drop_first_tile != 0);  // a test wants one of the sweeps below
-    if (!test_sweep && small_graphs_preferred(N, a.G, H, d, k)) {
+    if (!test_sweep && !in_place && small_graphs_preferred(N, a.G, H, d, k)) {
         if (launch_plan(a, w, 128) != cudaSuccess) return KMIP_ERR_CUDA;
         if (ev) cudaEventRecord(ev[1], a.stream);
         if (launch_small_graphs(a) != cudaSuccess) return KMIP_ERR_CUDA;

@@ -300,6 +300,7 @@ struct FwdArgs {
     // per-call test options (kmip_test.h); the public entry points leave the defaults
     long long wait_limit_cycles = 0;  // bound of every device-side wait in SM clocks; <= 0: kDefaultWaitLimitCycles
     int drop_first_tile = 0;          // leave one key tile of CTA 0 unloaded, so that the waits on it run out
+    bool in_place = false;            // `out` overlaps Q or K: nothing may be written there before the last stage
     int fp32_path = 0;                // fp32 mode: 0 = sweep chosen by problem size, 1 = one warp per row, 2 = tiled
 };
 
@@ -387,7 +388,7 @@ inline F16Buffers f16_buffers(const FwdArgs& a, const FwdWorkspace& w) {
         used = align_up(rows * 4, 16);
     }
     b.scratch = out + used;
-    b.scratch_words = out_bytes > used ? (long long)((out_bytes - used) / 8) : 0;
+    b.scratch_words = out_bytes > used && !a.in_place ? (long long)((out_bytes - used) / 8) : 0;
     return b;
 }
 cudaError_t launch_f16_convert(const FwdArgs& a, const FwdWorkspace& w);

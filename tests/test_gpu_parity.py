@@ -345,3 +345,30 @@ def test_sweep_order_of_large_graphs(sizes):
             assert (kinds[1:] != kinds[:-1]).sum() < 60 * 60  # kinds that share a bucket may mix
             assert (kinds[1:] != kinds[:-1]).mean() < 0.25    # unsorted: 59 of 60 neighbours differ
         lo += n
+
+
+@pytest.mark.parametrize("over", ["Q", "K", "both, shifted"])
+@pytest.mark.parametrize("sizes,H,d,k,mode", [([3100], 1, 32, 16, wl.MODE_FP32_EXACT), ([200, 1, 300], 2, 16, 8, wl.MODE_FP32_EXACT),
+                                              ([7000], 1, 16, 8, wl.MODE_FP32_EXACT), ([2900], 2, 64, 9, wl.MODE_BF16_TC),
+                                              ([3000], 1, 32, 45, wl.MODE_BF16_TC), ([3100], 1, 32, 16, wl.MODE_BF16_TC),
+                                              ([200, 1, 300], 2, 16, 8, wl.MODE_BF16_TC), ([33000], 1, 16, 8, "pruned")])
+def test_out_may_lie_over_the_queries_or_keys(sizes, H, d, k, mode, over):
+    """An in-place call: the same keys and outputs as a call with an array of its own, on every sweep, with a few rows that
+    the filter cannot decide."""
+    w = wl.iid_workload("p", 6400 + sum(sizes) + k, sizes, H, d, k, wl.MODE_BF16_TC if mode == "pruned" else mode, backward=False)
+    if mode == "pruned":
+        w.mode = kb.KMIP_BF16_TC_PRUNED
+    w.Q[3] = 0.0
+    Q, K, V, dO, offs = pu.to_device(w)
+    ref = kb.forward(Q, K, V, offs, k, w.mode)
+    fb = kb.ForwardBuffers(w.N, w.G, H, d, k, w.mode)
+    n, gap = Q.numel(), 64                     # 64 elements: 16-byte aligned, not a row of every shape
+    mem = torch.empty(2 * n + gap, dtype=Q.dtype, device="cuda")
+    q_at, k_at = (gap, n + gap) if over != "K" else (n + gap, gap)
+    qv, kv = (mem[at:at + n].view(Q.shape) for at in (q_at, k_at))
+    qv.copy_(Q); kv.copy_(K)
+    fb.out = mem[:n].view(Q.shape) if over == "both, shifted" else qv if over == "Q" else kv
+    kb.forward(qv, kv, V, offs, k, w.mode, buffers=fb)
+    if mode == wl.MODE_FP32_EXACT:
+        assert torch.equal(fb.topk_idx, ref.topk_idx) and torch.equal(fb.topk_score, ref.topk_score) and torch.equal(fb.out, ref.out)
+    pu.check_forward(w, fb, None if w.N < 10000 else wl.sample_rows(w, 256))
