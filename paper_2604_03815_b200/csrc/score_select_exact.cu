@@ -117,13 +117,13 @@ __device__ __forceinline__ void merge_into_row(cand_t* row, int k, const cand_t*
             if (pass) row[k + cnt + __popc(m & ((1u << lane) - 1u))] = v;
             cnt += __popc(m);
             if (cnt > room - 32) {
-                warp_compact_row<E>(row, k, cnt, lane);
+                compact_row_outlined<E>(row, k, cnt);
                 kth = row[k - 1];
                 cnt = 0;
             }
         }
     }
-    warp_compact_row<E>(row, k, cnt, lane);
+    compact_row_outlined<E>(row, k, cnt);
 }
 
 template <typename T, int D, int E>
@@ -185,13 +185,13 @@ score_select_redo_kernel(const T* __restrict__ Q, const T* __restrict__ K, const
                     if (pass) row[k + cnt + __popc(m & ((1u << lane) - 1u))] = make_cand(s[u], (int)j);
                     cnt += __popc(m);
                     if (cnt > room - 32) {
-                        tau = warp_compact_row<E>(row, k, cnt, lane);
+                        tau = compact_row_outlined<E>(row, k, cnt);
                         cnt = 0;
                     }
                 }
             }
         }
-        warp_compact_row<E>(row, k, cnt, lane);
+        compact_row_outlined<E>(row, k, cnt);
         if (by_warp) {
             warp_store_row(row, k, lane, topk_idx + (size_t)r * k, topk_score + (size_t)r * k);
             continue;
