@@ -147,14 +147,16 @@ small_forward_kernel(const T* __restrict__ Q, const T* __restrict__ K, const T* 
                         }
                     }
                     const float bound = unorder_bits(__shfl_sync(FULL, w, k - 1));
-                    // a later key with the score of the list's last entry loses to it, one with the bound's may be it
+                    // a later key with the score of the list's last entry loses to it, one with the bound's may be it;
+                    // keys past the end have the score -infinity
                     const cand_t kth = __shfl_sync(FULL, best, k - 1);
                     const float tau = kth ? cand_score(kth) : -CUDART_INF_F;
                     int cnt = 0;
 #pragma unroll
                     for (int u = 0; u < kU; ++u) {
                         if (u * 32 < nk) {
-                            const bool pass = u * 32 + lane < nk && s[u] >= bound && (!kth || s[u] > tau);
+                            // a score of -infinity (or a NaN) is nobody's choice, as in the other kernels
+                            const bool pass = s[u] >= bound && s[u] > tau;
                             const unsigned m = __ballot_sync(FULL, pass);
                             if (m) {
                                 if (pass) pend[cnt + __popc(m & ((1u << lane) - 1u))] = make_cand(s[u], c0 + u * 32 + lane);

@@ -372,3 +372,19 @@ def test_out_may_lie_over_the_queries_or_keys(sizes, H, d, k, mode, over):
     if mode == wl.MODE_FP32_EXACT:
         assert torch.equal(fb.topk_idx, ref.topk_idx) and torch.equal(fb.topk_score, ref.topk_score) and torch.equal(fb.out, ref.out)
     pu.check_forward(w, fb, None if w.N < 10000 else wl.sample_rows(w, 256))
+
+
+@pytest.mark.parametrize("n,d,k", [(40, 16, 32), (300, 32, 32), (700, 64, 5)])
+def test_small_graphs_with_scores_that_overflow(n, d, k):
+    """Scores of -infinity keep their slots empty, those of +infinity come first: what one warp per row does."""
+    g = torch.Generator().manual_seed(n)
+    Q, K, V = (torch.randn(n, 1, d, generator=g).cuda() for _ in range(3))
+    Q[::3] = 1e20
+    Q[::6] = -1e20
+    K[1::2] = 1e20
+    K[2, 0, 0] = float("nan")
+    a = kb.forward(Q, K, V, None, k, kb.KMIP_FP32_EXACT)
+    b = kb.forward(Q, K, V, None, k, kb.KMIP_FP32_EXACT, fp32_path=1)
+    assert n > 40 or bool((b.topk_idx[::6, 0, -1] < 0).all())
+    assert torch.equal(a.topk_idx, b.topk_idx) and torch.equal(a.topk_score, b.topk_score)
+    assert torch.equal(a.out.nan_to_num(nan=7.0), b.out.nan_to_num(nan=7.0))
