@@ -42,6 +42,17 @@ int kmip_test_attn_forward(const void *Q, const void *K, const void *V,
                            const kmip_test_options_t *options);
 
 /*
+ * Which kernels the last forward call on `workspace` ran (synchronises `stream`); `route` is HOST memory.  Errors as for
+ * kmip_last_status.
+ */
+#define KMIP_ROUTE_SMALL 1        /* one kernel for the whole forward pass of small graphs */
+#define KMIP_ROUTE_FILTER 2       /* half-precision prefilter sweep, exact rescoring */
+#define KMIP_ROUTE_TENSOR_CORE 3  /* fp32-accumulate tensor-core sweep (pruned or not), rescoring */
+#define KMIP_ROUTE_TILED 4        /* fp32 mode: CUDA-core sweep of 128-row blocks, rescoring */
+#define KMIP_ROUTE_ROWS 5         /* CUDA cores, one warp per query row */
+int kmip_test_route(const void *workspace, void *stream, int32_t *route);
+
+/*
  * Dense scores S[h][i][j] = q_i^h . k_j^h (Algorithm 1 line 2) of ONE graph of 1 <= N <= 8192 nodes,
  * written as fp32 [H, N, N] to `scores` (device memory) through the same TMA / tcgen05 pipeline as
  * the KMIP_BF16_TC forward pass.  Q, K: bf16 [N, H, d] device memory.  workspace: at least
@@ -79,7 +90,7 @@ int kmip_test_gemm_tn(const void *A, const void *B, void *C, int32_t M, int32_t 
  * the schedule) and not only by their row number.  Synchronises `stream`, then writes to HOST memory
  *   order[s]       = row number of the node the sweep handled at position s, s = 0 .. N-1
  *                    (the identity where the library keeps the row order: small problems, fp32 mode,
- *                    graphs below 8192 nodes);
+ *                    graphs below 8192 nodes, and where the small-graph kernel ran);
  *   *rows_per_item = query rows per work item (128 x the query tiles a CTA owns).
  * N, G, H, d, k, mode: as passed to that forward call.  Errors as for kmip_attn_workspace_bytes,
  * KMIP_ERR_CUDA if the synchronisation or the copy fails.

@@ -101,6 +101,8 @@ def lib() -> ctypes.CDLL:
         L.kmip_test_f16_scores.argtypes = [P, P, i64, i32, i32, P, P, P, sz, P]
         L.kmip_test_gemm_tn.restype = ctypes.c_int
         L.kmip_test_gemm_tn.argtypes = [P, P, P, i32, i32, i32, ctypes.c_int, P, sz, P]
+        L.kmip_test_route.restype = ctypes.c_int
+        L.kmip_test_route.argtypes = [P, P, ctypes.POINTER(i32)]
         L.kmip_test_sweep_order.restype = ctypes.c_int
         L.kmip_test_sweep_order.argtypes = [P, i64, i32, i32, i32, i32, ctypes.c_int, P, ctypes.POINTER(i32), P]
         L.kmip_test_attn_forward.restype = ctypes.c_int
@@ -307,6 +309,18 @@ def kmip_test_sweep_order(workspace, N, G, H, d, k, mode, stream=None):
     if rc != KMIP_OK:
         raise KmipError(rc, "kmip_test_sweep_order")
     return order, int(rpi.value)
+
+
+ROUTE_SMALL, ROUTE_FILTER, ROUTE_TENSOR_CORE, ROUTE_TILED, ROUTE_ROWS = 1, 2, 3, 4, 5
+
+
+def kmip_test_route(workspace, stream=None) -> int:
+    """kmip_test.h: which kernels the last forward call on `workspace` ran (ROUTE_*)."""
+    route = ctypes.c_int32(0)
+    rc = lib().kmip_test_route(_ptr(workspace), _stream(stream), ctypes.byref(route))
+    if rc != KMIP_OK:
+        raise KmipError(rc, "kmip_test_route")
+    return int(route.value)
 
 
 def kmip_attn_sweep_counters(workspace, stream=None):

@@ -97,6 +97,17 @@ int kmip_test_attn_forward(const void* Q, const void* K, const void* V, const in
 
 namespace {
 
+// The workspace of a forward call and, for the half-precision sweep, its work items.
+FwdWorkspace plan_forward(int64_t N, int32_t G, int32_t H, int32_t d, int32_t k, int mode, int small) {
+    FwdWorkspace w = plan_fwd_workspace(N, G, H, d, k, mode);
+    // graphs of one size are assumed; where the small-graph kernel takes those, the sweep runs if some are large
+    if (w.f16) w.item_tiles = score_select_f16_item_tiles(N, small == kSmallDecide ? 1 : G, H, d, w.list);
+    return w;
+}
+int rows_per_item(const FwdWorkspace& w, int32_t d, int32_t k) {
+    return w.f16 ? 128 * w.item_tiles : w.tc ? score_select_tc_rows_per_item(d, k) : 128;
+}
+
 // Whether two arrays of `bytes` bytes share any.
 bool overlap(const void* a, const void* b, size_t bytes) {
     const uintptr_t x = reinterpret_cast<uintptr_t>(a), y = reinterpret_cast<uintptr_t>(b);
@@ -116,14 +127,15 @@ int forward_impl(const void* Q, const void* K, const void* V, const int32_t* gra
     if (!aligned16(Q) || !aligned16(K) || !aligned16(V) || !aligned16(out) || !aligned16(topk_idx) ||
         !aligned16(topk_score) || !aligned16(workspace) || (reinterpret_cast<uintptr_t>(graph_offsets) & 3u))
         return KMIP_ERR_INVALID_ARG;
-    FwdWorkspace w = plan_fwd_workspace(N, graph_offsets ? G : 1, H, d, k, mode);
+    const bool test_sweep = opt && (opt->fp32_path != 0 || opt->drop_first_tile != 0);  // a test wants one of the sweeps
+    const int small = test_sweep ? kSmallNever : small_graphs_use(N, graph_offsets ? G : 1, H, d, k);
+    FwdWorkspace w = plan_forward(N, graph_offsets ? G : 1, H, d, k, mode, small);
     if (mode == KMIP_FP32_EXACT && opt && opt->fp32_path != 0) w.f16 = w.in_outputs = false;  // a test picks the CUDA-core sweep
     const size_t array_bytes = (size_t)N * H * d * (mode == KMIP_FP32_EXACT ? 4 : 2);
     const bool in_place = overlap(out, Q, array_bytes) || overlap(out, K, array_bytes);
     if (in_place && w.in_outputs) w.f16 = w.in_outputs = false;  // the sweep that keeps its lists in the index and score arrays
     const bool tc = w.tc;
     if (workspace_bytes < w.total) return KMIP_ERR_WORKSPACE;
-    if (w.f16) w.item_tiles = score_select_f16_item_tiles(N, graph_offsets ? G : 1, H, d, w.list);
 
     FwdArgs a{Q, K, V, graph_offsets, graph_offsets ? G : 1, N, H, d, k, mode, out, topk_idx, topk_score,
               static_cast<unsigned char*>(workspace), static_cast<cudaStream_t>(stream)};
@@ -139,28 +151,32 @@ int forward_impl(const void* Q, const void* K, const void* V, const int32_t* gra
     if (launch_canary_fill(a.ws, w.canaries, a.stream) != cudaSuccess) return KMIP_ERR_CUDA;
     cudaEvent_t* ev = (g_prof.on && g_prof.n_fwd < g_prof.max_calls) ? g_prof.fwd[g_prof.n_fwd++] : nullptr;
     if (ev) cudaEventRecord(ev[0], a.stream);
-    const bool test_sweep = opt && (opt->fp32_path != 0 || opt->drop_first_tile != 0);  // a test wants one of the sweeps below
-    if (!test_sweep && !in_place && small_graphs_preferred(N, a.G, H, d, k)) {
-        if (launch_plan(a, w, 128) != cudaSuccess) return KMIP_ERR_CUDA;
+    if (small == kSmallAlways && !in_place) {
+        if (launch_plan(a, w, 128, kSmallAlways, 0) != cudaSuccess) return KMIP_ERR_CUDA;
         if (ev) cudaEventRecord(ev[1], a.stream);
         if (launch_small_graphs(a) != cudaSuccess) return KMIP_ERR_CUDA;
         for (int e = 2; ev && e <= 4; ++e) cudaEventRecord(ev[e], a.stream);
         if (launch_canary_check(a.ws, w.canaries, a.stream) != cudaSuccess) return KMIP_ERR_CUDA;
         return KMIP_OK;
     }
-    if (tc && !w.prune && !w.f16 && launch_pack_keys(a, w) != cudaSuccess) return KMIP_ERR_CUDA;
+    a.maybe_small = small == kSmallDecide && !in_place;
     // the tiled fp32 sweep runs one block per 128 query rows and head and reads a key once per block instead of
     // once per row: measured faster than the one-warp-per-row kernel from about 48 blocks on (0.43 against
     // 0.70 ms at 64 blocks, 1.7 against 8.4 ms at 247), slower below (0.25 against 0.19 ms at 32)
     const bool tiled32 = mode == KMIP_FP32_EXACT && !w.f16 && score_select_fp32_tiled_supported(d, k) &&
                          (a.fp32_path == 0 ? (N / 128) * H >= 48 : a.fp32_path == 2);
-    if (launch_plan(a, w, w.f16 ? 128 * w.item_tiles : tc ? score_select_tc_rows_per_item(d, k) : 128) !=
-        cudaSuccess)
-        return KMIP_ERR_CUDA;
+    const int route = w.f16 ? kRouteFilter : tc ? kRouteTensorCore : tiled32 ? kRouteTiled : kRouteRows;
+    if (w.reorder && launch_reorder_clear(a, w) != cudaSuccess) return KMIP_ERR_CUDA;
+    if (launch_plan(a, w, rows_per_item(w, d, k), a.maybe_small ? kSmallDecide : kSmallNever, route) != cudaSuccess) return KMIP_ERR_CUDA;
+    if (a.maybe_small) {  // before the sweep's kernels: they are enqueued while it runs
+        if (ev) cudaEventRecord(ev[1], a.stream);
+        if (launch_small_graphs(a) != cudaSuccess) return KMIP_ERR_CUDA;
+    }
+    if (tc && !w.prune && !w.f16 && launch_pack_keys(a, w) != cudaSuccess) return KMIP_ERR_CUDA;
     if (w.reorder && launch_reorder_queries(a, w) != cudaSuccess) return KMIP_ERR_CUDA;
     if (w.f16 && launch_f16_convert(a, w) != cudaSuccess) return KMIP_ERR_CUDA;
     if (w.prune && (launch_reorder_keys(a, w) != cudaSuccess || launch_prune_stats(a, w) != cudaSuccess)) return KMIP_ERR_CUDA;
-    if (ev) cudaEventRecord(ev[1], a.stream);
+    if (ev && !a.maybe_small) cudaEventRecord(ev[1], a.stream);
     const cudaError_t sweep = w.f16 ? launch_score_select_f16(a, w) : tc ? launch_score_select_tc(a, w)
                               : tiled32 ? launch_score_select_fp32_tiled(a, w) : launch_score_select_exact(a);
     if (sweep != cudaSuccess) return KMIP_ERR_CUDA;
@@ -237,12 +253,12 @@ int kmip_attn_topk_mass(const void* Q, const void* K, const int32_t* graph_offse
               const_cast<float*>(topk_score), static_cast<unsigned char*>(workspace), static_cast<cudaStream_t>(stream)};
     if (cudaMemsetAsync(a.ws, 0, kStatusBytes, a.stream) != cudaSuccess) return KMIP_ERR_CUDA;
     if (tensor) {
+        if (launch_plan(a, w, score_select_tc_rows_per_item(d, 1), kSmallNever, kRouteTensorCore) != cudaSuccess) return KMIP_ERR_CUDA;
         if (launch_pack_keys(a, w) != cudaSuccess) return KMIP_ERR_CUDA;
-        if (launch_plan(a, w, score_select_tc_rows_per_item(d, 1)) != cudaSuccess) return KMIP_ERR_CUDA;
         if (launch_topk_mass_tc(a, w, mass) != cudaSuccess) return KMIP_ERR_CUDA;
         return KMIP_OK;
     }
-    if (launch_plan(a, w, 128) != cudaSuccess) return KMIP_ERR_CUDA;
+    if (launch_plan(a, w, 128, kSmallNever, kRouteRows) != cudaSuccess) return KMIP_ERR_CUDA;
     if (launch_topk_mass(a, w, mass) != cudaSuccess) return KMIP_ERR_CUDA;
     return KMIP_OK;
 }
@@ -399,17 +415,29 @@ int kmip_test_sweep_order(const void* workspace, int64_t N, int32_t G, int32_t H
     const int rc = check_shape(N, H, d, k, mode);
     if (rc != KMIP_OK) return rc;
     if (!workspace || !order || !rows_per_item || G < 0) return KMIP_ERR_INVALID_ARG;
-    FwdWorkspace w = plan_fwd_workspace(N, G > 0 ? G : 1, H, d, k, mode);
-    if (w.f16) w.item_tiles = score_select_f16_item_tiles(N, G > 0 ? G : 1, H, d, w.list);
-    *rows_per_item = w.f16 ? 128 * w.item_tiles : w.tc ? score_select_tc_rows_per_item(d, k) : 128;
-    if (cudaStreamSynchronize(static_cast<cudaStream_t>(stream)) != cudaSuccess) return KMIP_ERR_CUDA;
-    if (w.reorder) {
+    const FwdWorkspace w = plan_forward(N, G > 0 ? G : 1, H, d, k, mode, small_graphs_use(N, G > 0 ? G : 1, H, d, k));
+    *rows_per_item = ::rows_per_item(w, d, k);
+    StatusBlock sb;
+    if (cudaStreamSynchronize(static_cast<cudaStream_t>(stream)) != cudaSuccess ||
+        cudaMemcpy(&sb, workspace, sizeof(sb), cudaMemcpyDeviceToHost) != cudaSuccess)
+        return KMIP_ERR_CUDA;
+    if (w.reorder && sb.route != kRouteSmall) {
         if (cudaMemcpy(order, static_cast<const unsigned char*>(workspace) + w.perm_off, (size_t)N * 4,
                        cudaMemcpyDeviceToHost) != cudaSuccess)
             return KMIP_ERR_CUDA;
     } else {
         for (int64_t i = 0; i < N; ++i) order[i] = (int32_t)i;
     }
+    return KMIP_OK;
+}
+
+int kmip_test_route(const void* workspace, void* stream, int32_t* route) {
+    if (!workspace || !route) return KMIP_ERR_INVALID_ARG;
+    StatusBlock sb;
+    if (cudaStreamSynchronize(static_cast<cudaStream_t>(stream)) != cudaSuccess ||
+        cudaMemcpy(&sb, workspace, sizeof(sb), cudaMemcpyDeviceToHost) != cudaSuccess)
+        return KMIP_ERR_CUDA;
+    *route = sb.route;
     return KMIP_OK;
 }
 
@@ -424,8 +452,8 @@ int kmip_test_tc_scores(const void* Q, const void* K, int64_t N, int32_t H, int3
     FwdArgs a{Q, K, nullptr, nullptr, 1, N, H, d, 1, KMIP_BF16_TC, nullptr, nullptr, nullptr,
               static_cast<unsigned char*>(workspace), static_cast<cudaStream_t>(stream)};
     if (cudaMemsetAsync(a.ws, 0, kStatusBytes, a.stream) != cudaSuccess) return KMIP_ERR_CUDA;
+    if (launch_plan(a, w, score_select_tc_rows_per_item(d, 1), kSmallNever, kRouteTensorCore) != cudaSuccess) return KMIP_ERR_CUDA;
     if (launch_pack_keys(a, w) != cudaSuccess) return KMIP_ERR_CUDA;
-    if (launch_plan(a, w, score_select_tc_rows_per_item(d, 1)) != cudaSuccess) return KMIP_ERR_CUDA;
     if (launch_score_dump_tc(a, w, scores) != cudaSuccess) return KMIP_ERR_CUDA;
     return KMIP_OK;
 }
@@ -442,7 +470,7 @@ int kmip_test_f16_scores(const void* Q, const void* K, int64_t N, int32_t H, int
     FwdArgs a{Q, K, nullptr, nullptr, 1, N, H, d, 1, KMIP_BF16_TC, nullptr, nullptr, nullptr,
               static_cast<unsigned char*>(workspace), static_cast<cudaStream_t>(stream)};
     if (cudaMemsetAsync(a.ws, 0, kStatusBytes, a.stream) != cudaSuccess) return KMIP_ERR_CUDA;
-    if (launch_plan(a, w, 128 * w.item_tiles) != cudaSuccess) return KMIP_ERR_CUDA;
+    if (launch_plan(a, w, 128 * w.item_tiles, kSmallNever, kRouteFilter) != cudaSuccess) return KMIP_ERR_CUDA;
     if (launch_f16_convert(a, w) != cudaSuccess) return KMIP_ERR_CUDA;
     if (launch_score_dump_f16(a, w, scores) != cudaSuccess) return KMIP_ERR_CUDA;
     // per head: {q_n2max, k_n2max, k_first16_n2max, 0} as the conversion measured them

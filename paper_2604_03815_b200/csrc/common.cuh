@@ -6,6 +6,7 @@
 #include <stdint.h>
 
 #include "kmip.h"
+#include "kmip_test.h"
 
 namespace kmip {
 
@@ -37,6 +38,12 @@ struct Canaries {
 
 constexpr int kRedoSplitMax = 48;
 
+// Which kernels a forward call ran (StatusBlock::route; the values of kmip_test.h).
+enum Route {
+    kRouteSmall = KMIP_ROUTE_SMALL, kRouteFilter = KMIP_ROUTE_FILTER, kRouteTensorCore = KMIP_ROUTE_TENSOR_CORE,
+    kRouteTiled = KMIP_ROUTE_TILED, kRouteRows = KMIP_ROUTE_ROWS
+};
+
 struct StatusBlock {
     int status;      // kmip_status_t recorded by the device (first error wins)
     int detail;      // where it happened (kernel-specific code)
@@ -47,15 +54,16 @@ struct StatusBlock {
     unsigned long long counters[4];
     int n_redo;      // forward, fp16 prefilter: rows the rescoring kernel sent to the exact kernel
     int redo_done[kRedoSplitMax];  // parts finished of each of the first redo rows (score_select_exact.cu)
-    int reserved[51 - kRedoSplitMax];
+    int route;       // forward: Route, written by the plan kernel
+    int reserved[50 - kRedoSplitMax];
 };
 static_assert(sizeof(StatusBlock) == kStatusBytes, "status block size");
 
-// One unit of work of the tensor-core score kernel: up to 384 consecutive query rows of one
+// One unit of work of a sweep: up to 512 consecutive query rows of one
 // graph and that graph's key range (Eq. 1 restricted to the graph by the CSR offsets).
 struct WorkItem {
     int row0;    // first query row
-    int nrows;   // 1..384 (128 x the query tiles per CTA of the launched configuration)
+    int nrows;   // 1..512 (128 x the query tiles per CTA of the launched configuration)
     int key_lo;  // graph's first row
     int key_hi;  // one past the graph's last row
     int tile0;   // number of the graph's first 128-key tile in the per-tile statistics (pruned sweep)
@@ -241,6 +249,16 @@ __device__ __forceinline__ bool kmip_check(bool cond, StatusBlock* sb, int code)
     return cond;
 }
 
+// First thing in every kernel of the sweeps' routes: true if the plan kernel gave the batch to the small-graph kernel, or if
+// the call failed before.  The wait is for launches that overlap the end of the kernel before them (launch_next).
+// Kernels that may record a problem while blocks of theirs still start ask for the first only (it does not change under
+// them) and find no work items when the plan failed.
+__device__ __forceinline__ bool small_route(const StatusBlock* sb) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    return sb->route == kRouteSmall;
+}
+__device__ __forceinline__ bool sweep_off(const StatusBlock* sb) { return small_route(sb) || sb->status != KMIP_OK; }
+
 template <typename T> struct Elem;
 template <> struct Elem<float> {
     static constexpr int kVec = 4;  // elements per 16-byte vector
@@ -300,6 +318,7 @@ struct FwdArgs {
     // per-call test options (kmip_test.h); the public entry points leave the defaults
     long long wait_limit_cycles = 0;  // bound of every device-side wait in SM clocks; <= 0: kDefaultWaitLimitCycles
     int drop_first_tile = 0;          // leave one key tile of CTA 0 unloaded, so that the waits on it run out
+    bool maybe_small = false;         // the plan kernel decides between the small-graph kernel and the sweep's kernels
     bool in_place = false;            // `out` overlaps Q or K: nothing may be written there before the last stage
     int fp32_path = 0;                // fp32 mode: 0 = sweep chosen by problem size, 1 = one warp per row, 2 = tiled
 };
@@ -320,14 +339,33 @@ struct BwdArgs {
     unsigned long long seed = 0ull;
 };
 
+// Launches a kernel of a sweep's route.  Where the plan kernel decides whether it has work (maybe_small), every launch
+// may begin while the one before it ends: returning at once then costs 1.3 us each instead of 2.5.
+template <typename... P, typename... A>
+inline cudaError_t launch_next(const FwdArgs& a, void (*kern)(P...), dim3 grid, int threads, size_t smem, A&&... args) {
+    cudaLaunchConfig_t c{};
+    c.gridDim = grid;
+    c.blockDim = dim3(threads);
+    c.dynamicSmemBytes = smem;
+    c.stream = a.stream;
+    cudaLaunchAttribute overlap{};
+    overlap.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    overlap.val.programmaticStreamSerializationAllowed = 1;
+    c.attrs = &overlap;
+    c.numAttrs = a.maybe_small ? 1 : 0;
+    return cudaLaunchKernelEx(&c, kern, static_cast<P>(args)...);
+}
 // plan.cu, checks builds: write the canary blocks of a workspace / verify them (detail = 900 + block number)
 cudaError_t launch_canary_fill(unsigned char* ws, const Canaries& c, cudaStream_t stream);
 cudaError_t launch_canary_check(unsigned char* ws, const Canaries& c, cudaStream_t stream);
 // plan.cu: validates the offsets and writes the work items of the tensor-core kernel
-cudaError_t launch_plan(const FwdArgs& a, const FwdWorkspace& w, int rows_per_item);
+enum SmallUse { kSmallNever = 0, kSmallAlways = 1, kSmallDecide = 2 };
+cudaError_t launch_plan(const FwdArgs& a, const FwdWorkspace& w, int rows_per_item, int small_use, int route);
 // plan.cu: K [N, H, d] -> [H, N, d] so that a head's key tile is one contiguous block for TMA
 cudaError_t launch_pack_keys(const FwdArgs& a, const FwdWorkspace& w);
-// reorder.cu: locality codes, per-graph bucket sort, row-permuted copy of Q (after launch_plan)
+// reorder.cu: counters of the bucket sort (before launch_plan: they lie in an output array); locality codes, per-graph
+// bucket sort, row-permuted copy of Q (after launch_plan)
+cudaError_t launch_reorder_clear(const FwdArgs& a, const FwdWorkspace& w);
 cudaError_t launch_reorder_queries(const FwdArgs& a, const FwdWorkspace& w);
 // reorder.cu, pruned sweep: keys of large graphs sorted by (norm class, locality code) and regrouped by
 // head in that order (replaces launch_pack_keys; after launch_reorder_queries, which owns the code buffer first)
@@ -345,6 +383,12 @@ constexpr int64_t kF16MinRowsLong = 1024;
 // score_select_exact.cu: CUDA-core scores + running top-k, any supported (d, k), fp32 or bf16 storage
 cudaError_t launch_score_select_exact(const FwdArgs& a);
 int sm_count();  // multiprocessors of the current device (cached per device)
+// Blocks of a grid-stride kernel with `want` blocks of work, of which `per_sm` fit an SM.
+inline int grid_blocks(const FwdArgs& a, long long want, int per_sm) {
+    // a launch that may have nothing to do has no more blocks than fit the chip at once
+    const long long most = (long long)sm_count() * (a.maybe_small ? per_sm : 32);
+    return (int)(want < most ? want : most);
+}
 // score_select_tc.cu: tcgen05 scores + running top-k (bf16 storage); returns cudaErrorNotSupported
 // when (d, k) is outside what the tensor-core kernel covers
 int score_select_tc_rows_per_item(int32_t d, int32_t k);
@@ -408,7 +452,11 @@ bool score_select_fp32_tiled_supported(int32_t d, int32_t k);
 cudaError_t launch_score_select_fp32_tiled(const FwdArgs& a, const FwdWorkspace& w);
 // small_graphs.cu: the whole forward pass of batches of small graphs (any graph size, k <= 32, d <= 64); after the plan
 // kernel, which validates the offsets
-bool small_graphs_preferred(int64_t N, int32_t G, int32_t H, int32_t d, int32_t k);
+int small_graphs_use(int64_t N, int32_t G, int32_t H, int32_t d, int32_t k);
+// The rule, for `squares` = the sum of the squared graph sizes (the scores of a head); see small_graphs.cu
+__host__ __device__ inline bool small_graphs_preferred(double squares, long long N, int H, int d) {
+    return squares * (d + 16) <= 15000.0 * (double)N || squares * H * (d + 16) <= 3.0e8;
+}
 cudaError_t launch_small_graphs(const FwdArgs& a);
 // epilogue.cu: softmax over the k kept scores fused with the gather-V weighted sum
 cudaError_t launch_softmax_gather(const FwdArgs& a);

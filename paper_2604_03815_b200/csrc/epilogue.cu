@@ -17,7 +17,7 @@ softmax_gather_kernel(const T* __restrict__ V, const int32_t* __restrict__ topk_
                       const float* __restrict__ topk_score, int N, int H, int k, float scale,
                       float drop_p, unsigned long long seed, T* __restrict__ out,
                       const StatusBlock* __restrict__ sb) {
-    if (sb->status != KMIP_OK) return;  // an earlier stage failed: topk_idx was not written
+    if (sweep_off(sb)) return;  // an earlier stage failed: topk_idx was not written
     const int lane = threadIdx.x & 31;
     const long long n_rows = (long long)N * H;
     RowWalk walk(blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5), gridDim.x * kWarpsPerBlock, H);
@@ -40,12 +40,11 @@ softmax_gather_kernel(const T* __restrict__ V, const int32_t* __restrict__ topk_
 template <typename T, int D>
 cudaError_t launch_d(const FwdArgs& a) {
     const long long n_rows = (long long)a.N * a.H;
-    const int blocks = (int)std::min<long long>((n_rows + kWarpsPerBlock - 1) / kWarpsPerBlock, (long long)sm_count() * 32);
+    const int blocks = grid_blocks(a, (n_rows + kWarpsPerBlock - 1) / kWarpsPerBlock, 8);
     auto kern = a.k <= 32 ? softmax_gather_kernel<T, D, 1> : softmax_gather_kernel<T, D, kMaxEntriesPerLane>;
-    kern<<<blocks, kWarpsPerBlock * 32, 0, a.stream>>>(
+    return launch_next(a, kern, dim3(blocks), kWarpsPerBlock * 32, 0,
         static_cast<const T*>(a.V), a.topk_idx, a.topk_score, (int)a.N, a.H, a.k,
         1.0f / sqrtf((float)a.d), a.drop_p, a.seed, static_cast<T*>(a.out), reinterpret_cast<const StatusBlock*>(a.ws));
-    return cudaGetLastError();
 }
 
 template <typename T>

@@ -33,7 +33,7 @@ template <typename T, int D>
 __global__ void __launch_bounds__(kNormThreads)
 f16_norm_max_kernel(const T* __restrict__ Q, const T* __restrict__ K, int N, int H,
                     unsigned* __restrict__ stat, const StatusBlock* __restrict__ sb) {
-    if (sb->status != KMIP_OK) return;
+    if (sweep_off(sb)) return;
     __shared__ unsigned s_max[4][kNormThreads / 32];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     for (int h = blockIdx.y; h < H; h += gridDim.y) {
@@ -85,42 +85,48 @@ template <typename T, int D>
 __global__ void __launch_bounds__(kConvThreads)
 f16_convert_kernel(const T* __restrict__ Q, const T* __restrict__ K, const int* __restrict__ perm, uint4* __restrict__ Qp,
                    uint4* __restrict__ Kp, int N, int H, F16HeadStat* __restrict__ stat, const StatusBlock* __restrict__ sb) {
-    if (sb->status != KMIP_OK) return;
+    if (sweep_off(sb)) return;
     constexpr int V = D / 8;  // threads per row
     constexpr bool kLossy = sizeof(T) == 4;
     __shared__ unsigned s_lost;
     const bool keys = blockIdx.z == 0;
-    const long long v = (long long)blockIdx.x * kConvThreads + threadIdx.x;
-    const int p = (int)(v / V), c = (int)(v % V);  // V divides 32: the threads of a row share a warp
-    const bool live = v < (long long)N * V;
+    const long long n_pieces = (long long)N * V, step = (long long)gridDim.x * kConvThreads;
     for (int h = blockIdx.y; h < H; h += gridDim.y) {
         const float s = f16_scale_from_n2max(keys ? stat[h].k_n2max : stat[h].q_n2max);
-        float lost = 0.0f;
-        if (live) {
-            const int src = !keys && perm ? __ldg(perm + p) : p;
-            float x[8];
-            load8((keys ? K : Q) + ((size_t)src * H + h) * D + c * 8, x);
-            uint32_t o[4];
+        unsigned worst = 0u;  // float bits
+        for (long long v0 = (long long)blockIdx.x * kConvThreads; v0 < n_pieces; v0 += step) {  // block-uniform
+            const long long v = v0 + threadIdx.x;
+            const int p = (int)(v / V), c = (int)(v % V);  // V divides 32: the threads of a row share a warp
+            float lost = 0.0f;
+            if (v < n_pieces) {
+                const int src = !keys && perm ? __ldg(perm + p) : p;
+                float x[8];
+                load8((keys ? K : Q) + ((size_t)src * H + h) * D + c * 8, x);
+                uint32_t o[4];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const __half2 hh = __floats2half2_rn(x[2 * i] * s, x[2 * i + 1] * s);
-                o[i] = *reinterpret_cast<const uint32_t*>(&hh);
-                if (kLossy) {
-                    const float2 back = __half22float2(hh);
-                    const float d0 = x[2 * i] * s - back.x, d1 = x[2 * i + 1] * s - back.y;  // both exact
-                    lost = fmaf(d0, d0, fmaf(d1, d1, lost));
+                for (int i = 0; i < 4; ++i) {
+                    const __half2 hh = __floats2half2_rn(x[2 * i] * s, x[2 * i + 1] * s);
+                    o[i] = *reinterpret_cast<const uint32_t*>(&hh);
+                    if (kLossy) {
+                        const float2 back = __half22float2(hh);
+                        const float d0 = x[2 * i] * s - back.x, d1 = x[2 * i + 1] * s - back.y;  // both exact
+                        lost = fmaf(d0, d0, fmaf(d1, d1, lost));
+                    }
                 }
+                uint4* dst = keys ? Kp + ((size_t)h * N + p) * V + c : Qp + ((size_t)p * H + h) * V + c;
+                *dst = make_uint4(o[0], o[1], o[2], o[3]);
             }
-            uint4* dst = keys ? Kp + ((size_t)h * N + p) * V + c : Qp + ((size_t)p * H + h) * V + c;
-            *dst = make_uint4(o[0], o[1], o[2], o[3]);
+            if (kLossy && keys) {
+#pragma unroll
+                for (int o = 1; o < V; o <<= 1) lost += __shfl_xor_sync(0xFFFFFFFFu, lost, o);
+                const unsigned bits = __float_as_uint(lost * 1.00001f);
+                if (bits < 0x7F800000u) worst = max(worst, bits);
+            }
         }
         if (kLossy && keys) {
-#pragma unroll
-            for (int o = 1; o < V; o <<= 1) lost += __shfl_xor_sync(0xFFFFFFFFu, lost, o);
             if (threadIdx.x == 0) s_lost = 0u;
             __syncthreads();
-            const unsigned bits = __float_as_uint(lost * 1.00001f);
-            const unsigned m = __reduce_max_sync(0xFFFFFFFFu, bits < 0x7F800000u ? bits : 0u);
+            const unsigned m = __reduce_max_sync(0xFFFFFFFFu, worst);
             if ((threadIdx.x & 31) == 0 && m) atomicMax(&s_lost, m);
             __syncthreads();
             if (threadIdx.x == 0 && s_lost) atomicMax(reinterpret_cast<unsigned*>(&stat[h].k_lost_n2max), s_lost);
@@ -137,14 +143,16 @@ cudaError_t launch_d(const FwdArgs& a, const FwdWorkspace& w) {
     const T* K = static_cast<const T*>(a.K);
     const unsigned rows_y = (unsigned)std::min(a.H, 65535);
     // two waves of resident blocks at most: a block walks its head's nodes
-    const unsigned per_head = (unsigned)std::max(1, sm_count() * 16 / a.H);
+    const unsigned per_head = (unsigned)std::max(1, sm_count() * (a.maybe_small ? 1 : 16) / a.H);
     const dim3 norm_grid(std::min((unsigned)((a.N + kNormThreads - 1) / kNormThreads), per_head), rows_y);
-    f16_norm_max_kernel<T, D><<<norm_grid, kNormThreads, 0, a.stream>>>(Q, K, (int)a.N, a.H, reinterpret_cast<unsigned*>(stat), sb);
-    const dim3 conv_grid((unsigned)((a.N * (D / 8) + kConvThreads - 1) / kConvThreads), rows_y, 2);
-    f16_convert_kernel<T, D><<<conv_grid, kConvThreads, 0, a.stream>>>(
+    cudaError_t err = launch_next(a, f16_norm_max_kernel<T, D>, norm_grid, kNormThreads, 0, Q, K, (int)a.N, a.H,
+                                  reinterpret_cast<unsigned*>(stat), sb);
+    if (err != cudaSuccess) return err;
+    const unsigned conv_all = (unsigned)((a.N * (D / 8) + kConvThreads - 1) / kConvThreads);
+    const dim3 conv_grid(a.maybe_small ? std::min(conv_all, per_head) : conv_all, rows_y, 2);
+    return launch_next(a, f16_convert_kernel<T, D>, conv_grid, kConvThreads, 0,
         Q, K, w.reorder ? reinterpret_cast<const int*>(a.ws + w.perm_off) : nullptr, static_cast<uint4*>(b.q16), static_cast<uint4*>(b.k16),
         (int)a.N, a.H, stat, sb);
-    return cudaGetLastError();
 }
 
 template <typename T>

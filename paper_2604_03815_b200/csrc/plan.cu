@@ -12,8 +12,10 @@ constexpr int kPlanThreads = 1024;
 
 __global__ void __launch_bounds__(kPlanThreads)
 plan_kernel(const int32_t* __restrict__ offs, int G, int N, int rows_per_item, int max_items,
-            WorkItem* __restrict__ items, StatusBlock* __restrict__ sb, float* __restrict__ clear, int n_clear) {
+            WorkItem* __restrict__ items, StatusBlock* __restrict__ sb, float* __restrict__ clear, int n_clear, int small_use, int route,
+            int H, int d) {
     __shared__ int s_warp[32];
+    __shared__ unsigned long long s_squares[32];
     __shared__ int s_carry;
     __shared__ int s_bad;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
@@ -35,6 +37,25 @@ plan_kernel(const int32_t* __restrict__ offs, int G, int N, int rows_per_item, i
     }
 
     const int n_graphs = offs ? G : 1;
+    if (small_use == kSmallDecide) {
+        // the host knows the mean graph size only; what the small-graph kernel takes grows with the squares
+        unsigned long long sq = 0ull;
+        for (int g = tid; g < n_graphs; g += kPlanThreads) {
+            const unsigned long long n = (unsigned long long)(offs ? __ldg(offs + g + 1) - __ldg(offs + g) : N);
+            sq += n * n;
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xFFFFFFFFu, sq, o);
+        if (lane == 0) s_squares[wid] = sq;
+        __syncthreads();
+        if (tid == 0) {
+            sq = 0ull;
+            for (int x = 0; x < kPlanThreads / 32; ++x) sq += s_squares[x];
+            sb->route = small_graphs_preferred((double)sq, N, H, d) ? kRouteSmall : route;
+        }
+    } else if (tid == 0) {
+        sb->route = small_use == kSmallAlways ? kRouteSmall : route;
+    }
     for (int g0 = 0; g0 < n_graphs; g0 += kPlanThreads) {
         const int g = g0 + tid;
         int lo = 0, hi = 0;
@@ -88,7 +109,8 @@ plan_kernel(const int32_t* __restrict__ offs, int G, int N, int rows_per_item, i
 
 // K [N, H, d] -> [H, N, d], 16 bytes per thread.
 __global__ void pack_keys_kernel(const uint4* __restrict__ K, uint4* __restrict__ Kp, long long n_vec, int N, int H,
-                                 int vec_per_row) {
+                                 int vec_per_row, const StatusBlock* __restrict__ sb) {
+    if (sweep_off(sb)) return;
     const long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (v >= n_vec) return;
     const long long rowh = v / vec_per_row;  // j * H + h
@@ -127,15 +149,16 @@ cudaError_t launch_pack_keys(const FwdArgs& a, const FwdWorkspace& w) {
     const int vec_per_row = a.d * 2 / 16;
     const long long n_vec = (long long)a.N * a.H * vec_per_row;
     pack_keys_kernel<<<(unsigned)((n_vec + 255) / 256), 256, 0, a.stream>>>(
-        static_cast<const uint4*>(a.K), reinterpret_cast<uint4*>(a.ws + w.kpack_off), n_vec, (int)a.N, a.H, vec_per_row);
+        static_cast<const uint4*>(a.K), reinterpret_cast<uint4*>(a.ws + w.kpack_off), n_vec, (int)a.N, a.H, vec_per_row,
+        reinterpret_cast<const StatusBlock*>(a.ws));
     return cudaGetLastError();
 }
 
-cudaError_t launch_plan(const FwdArgs& a, const FwdWorkspace& w, int rows_per_item) {
+cudaError_t launch_plan(const FwdArgs& a, const FwdWorkspace& w, int rows_per_item, int small_use, int route) {
     plan_kernel<<<1, kPlanThreads, 0, a.stream>>>(
         a.graph_offsets, a.G, (int)a.N, rows_per_item, w.max_items,
         reinterpret_cast<WorkItem*>(a.ws + w.items_off), reinterpret_cast<StatusBlock*>(a.ws),
-        reinterpret_cast<float*>(a.ws + w.f16stat_off), w.f16 ? 4 * a.H : 0);
+        reinterpret_cast<float*>(a.ws + w.f16stat_off), w.f16 ? 4 * a.H : 0, small_use, route, a.H, a.d);
     return cudaGetLastError();
 }
 

@@ -100,7 +100,7 @@ prune_stats_kernel(const __nv_bfloat16* __restrict__ Qs, const __nv_bfloat16* __
                    int rows_per_item, float* __restrict__ qnorm, float* __restrict__ qstat, float* __restrict__ kstat,
                    const unsigned short* __restrict__ qcode, const int* __restrict__ perm,
                    const unsigned short* __restrict__ kcode_sorted) {
-    if (sb->status != KMIP_OK) return;
+    if (sweep_off(sb)) return;
     const int item = blockIdx.x, h = blockIdx.y;
     if (item >= sb->n_items) return;
     const WorkItem it = items[item];
@@ -141,7 +141,7 @@ template <int D>
 __global__ void __launch_bounds__(kThreads)
 suffix_max_kernel(const int32_t* __restrict__ offs, int G, int N, int H, float* __restrict__ kstat,
                   const StatusBlock* __restrict__ sb) {
-    if (sb->status != KMIP_OK) return;
+    if (sweep_off(sb)) return;
     constexpr int REC = D + 4;
     const int g = blockIdx.x, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int lo = offs ? __ldg(offs + g) : 0, hi = offs ? __ldg(offs + g + 1) : N;

@@ -36,7 +36,7 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32)
 refine_topk_kernel(const T* __restrict__ Q, const T* __restrict__ Kp, const int32_t* __restrict__ offs, int G,
                    int N, int H, int k, int32_t* __restrict__ topk_idx, float* __restrict__ topk_score,
                    const StatusBlock* __restrict__ sb, const int* __restrict__ kperm) {
-    if (sb->status != KMIP_OK) return;
+    if (sweep_off(sb)) return;
     constexpr int CAP = 32 * E;
     static_assert((sizeof(T) == 2) == REGROUPED, "bf16 keys come regrouped, fp32 keys in place");
     __shared__ cand_t s_rows[kWarpsPerBlock][CAP];

@@ -109,7 +109,7 @@ refine_f16_kernel(const T* __restrict__ Q, const T* __restrict__ K,
                   const int32_t* __restrict__ offs, int G, int N, int H, int k, const GroupLists lists,
                   const F16HeadStat* __restrict__ stat, int32_t* topk_idx, float* topk_score,
                   StatusBlock* __restrict__ sb, int* __restrict__ redo_list) {
-    if (sb->status != KMIP_OK) return;
+    if (sweep_off(sb)) return;
     constexpr bool kLossy = sizeof(T) == 4;
     constexpr int QE = (D + 31) / 32;  // query elements per lane
     constexpr int CAP = 32 * E;
@@ -342,12 +342,12 @@ refine_f16_kernel(const T* __restrict__ Q, const T* __restrict__ K,
 template <typename T, int D>
 cudaError_t launch_d(const FwdArgs& a, const FwdWorkspace& w) {
     const long long n_rows = (long long)a.N * a.H;
-    const int blocks = (int)std::min<long long>((n_rows + kWarpsPerBlock - 1) / kWarpsPerBlock, (long long)sm_count() * 32);
+    const int blocks = grid_blocks(a, (n_rows + kWarpsPerBlock - 1) / kWarpsPerBlock, 4);
     constexpr int kSmem = kWarpsPerBlock * 2 * 32 * (D * (int)sizeof(T) + 16);  // the rescoring stages
     const F16Buffers b = f16_buffers(a, w);
 #define KMIP_LAUNCH_REFINE16(E_, LIST_) \
     if ((err = cudaFuncSetAttribute(refine_f16_kernel<T, D, E_, LIST_>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem)) != cudaSuccess) return err; \
-    refine_f16_kernel<T, D, E_, LIST_><<<blocks, kWarpsPerBlock * 32, kSmem, a.stream>>>( \
+    return launch_next(a, refine_f16_kernel<T, D, E_, LIST_>, dim3(blocks), kWarpsPerBlock * 32, kSmem, \
         static_cast<const T*>(a.Q), static_cast<const T*>(a.K), a.graph_offsets, a.G, (int)a.N, a.H, a.k, b.lists, \
         reinterpret_cast<const F16HeadStat*>(a.ws + w.f16stat_off), a.topk_idx, a.topk_score, reinterpret_cast<StatusBlock*>(a.ws), b.redo)
     cudaError_t err;
@@ -361,7 +361,6 @@ cudaError_t launch_d(const FwdArgs& a, const FwdWorkspace& w) {
         return cudaErrorInvalidValue;
     }
 #undef KMIP_LAUNCH_REFINE16
-    return cudaGetLastError();
 }
 
 template <typename T>

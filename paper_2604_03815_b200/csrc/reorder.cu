@@ -57,7 +57,7 @@ __global__ void __launch_bounds__(kCodeThreads)
 query_code_kernel(const __nv_bfloat16* __restrict__ Q, int N, int HD, const int32_t* __restrict__ offs, int G,
                   unsigned short* __restrict__ code, int* __restrict__ counters, int* __restrict__ number,
                   const StatusBlock* __restrict__ sb) {
-    if (sb->status != KMIP_OK) return;
+    if (sweep_off(sb)) return;
     const int lane = threadIdx.x & 31;
     const int row = blockIdx.x * kCodeThreads + threadIdx.x;
     int lo = 0;
@@ -103,7 +103,7 @@ __global__ void __launch_bounds__(kScatterThreads)
 scatter_rows_kernel(const int32_t* __restrict__ offs, int G, int N, const unsigned short* __restrict__ code,
                     const int* __restrict__ counters, const int* __restrict__ number, int* __restrict__ perm,
                     const StatusBlock* __restrict__ sb) {
-    if (sb->status != KMIP_OK) return;  // malformed offsets were reported by the plan kernel
+    if (sweep_off(sb)) return;  // malformed offsets were reported by the plan kernel
     constexpr int PER = kCodeBuckets / kScatterThreads;  // consecutive buckets per thread in the scan
     __shared__ int s_start[kCodeBuckets];
     __shared__ int s_warp[kScatterThreads / 32];
@@ -152,7 +152,7 @@ template <int BITS>
 __global__ void __launch_bounds__(kSortThreads)
 graph_sort_stable_kernel(const int32_t* __restrict__ offs, int G, int N, const unsigned short* __restrict__ code,
                          int* __restrict__ perm, const StatusBlock* __restrict__ sb) {
-    if (sb->status != KMIP_OK) return;
+    if (sweep_off(sb)) return;
     constexpr int kBuckets = 1 << BITS;
     constexpr int kWarpsS = kSortThreads / 32;
     static_assert(kBuckets <= kSortThreads, "one thread per bucket in the scan");
@@ -224,7 +224,7 @@ graph_sort_stable_kernel(const int32_t* __restrict__ offs, int G, int N, const u
 // Qp[p, :] = Q[perm[p], :], 16 bytes per thread.
 __global__ void gather_rows_kernel(const uint4* __restrict__ Q, const int* __restrict__ perm, uint4* __restrict__ Qp,
                                    long long n_vec, int vec_per_row, const StatusBlock* __restrict__ sb) {
-    if (sb->status != KMIP_OK) return;
+    if (sweep_off(sb)) return;
     const long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (v >= n_vec) return;
     const long long p = v / vec_per_row;
@@ -238,7 +238,7 @@ __global__ void gather_rows_kernel(const uint4* __restrict__ Q, const int* __res
 __global__ void key_norm_kernel(const __nv_bfloat16* __restrict__ K, int N, int HD, const int32_t* __restrict__ offs,
                                 int G, float* __restrict__ norm2, unsigned* __restrict__ gmax,
                                 const StatusBlock* __restrict__ sb) {
-    if (sb->status != KMIP_OK) return;
+    if (sweep_off(sb)) return;
     const int lane = threadIdx.x & 31;
     const long long row = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (row >= N) return;
@@ -277,7 +277,7 @@ pivot_code_kernel(const __nv_bfloat16* __restrict__ X, const __nv_bfloat16* __re
                   const WorkItem* __restrict__ items, const StatusBlock* __restrict__ sb,
                   const int32_t* __restrict__ offs, int G, const float* __restrict__ norm2,
                   const unsigned* __restrict__ gmax, unsigned short* __restrict__ code) {
-    if (sb->status != KMIP_OK) return;
+    if (sweep_off(sb)) return;
     if ((int)blockIdx.x >= sb->n_items) return;
     const WorkItem it = items[blockIdx.x];
     const int n = it.key_hi - it.key_lo;
@@ -366,7 +366,7 @@ pivot_code_kernel(const __nv_bfloat16* __restrict__ X, const __nv_bfloat16* __re
 __global__ void pack_keys_perm_kernel(const uint4* __restrict__ K, const int* __restrict__ kperm, uint4* __restrict__ Kp,
                                       long long n_vec, int N, int H, int vec_per_row, const StatusBlock* __restrict__ sb,
                                       const unsigned short* __restrict__ code, unsigned short* __restrict__ code_sorted) {
-    if (sb->status != KMIP_OK) return;
+    if (sweep_off(sb)) return;
     const long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (v >= n_vec) return;
     const long long ph = v / vec_per_row;  // p * H + h
@@ -381,6 +381,10 @@ __global__ void pack_keys_perm_kernel(const uint4* __restrict__ K, const int* __
 }  // namespace
 
 // After launch_plan (which validates the offsets): codes, per-graph bucket sort, permuted copy of Q.
+cudaError_t launch_reorder_clear(const FwdArgs& a, const FwdWorkspace& w) {
+    return w.prune ? cudaSuccess : cudaMemsetAsync(a.topk_score, 0, (size_t)(a.N / kMinRowsToSort) * kCodeBuckets * 4, a.stream);
+}
+
 cudaError_t launch_reorder_queries(const FwdArgs& a, const FwdWorkspace& w) {
     const StatusBlock* sb = reinterpret_cast<const StatusBlock*>(a.ws);
     unsigned short* code = reinterpret_cast<unsigned short*>(a.ws + w.code_off);
@@ -401,8 +405,6 @@ cudaError_t launch_reorder_queries(const FwdArgs& a, const FwdWorkspace& w) {
             a.graph_offsets, a.G, (int)a.N, code, perm, sb);
     } else {
         int* counters = reinterpret_cast<int*>(a.topk_score);
-        cudaError_t err = cudaMemsetAsync(counters, 0, (size_t)(a.N / kMinRowsToSort) * kCodeBuckets * 4, a.stream);
-        if (err != cudaSuccess) return err;
         query_code_kernel<<<(unsigned)((a.N + kCodeThreads - 1) / kCodeThreads), kCodeThreads, 0, a.stream>>>(
             static_cast<const __nv_bfloat16*>(a.Q), (int)a.N, HD, a.graph_offsets, a.G, code, counters, a.topk_idx, sb);
         scatter_rows_kernel<<<(unsigned)((a.N + kScatterRows - 1) / kScatterRows), kScatterThreads, 0, a.stream>>>(

@@ -33,7 +33,7 @@ score_select_exact_kernel(const T* __restrict__ Q, const T* __restrict__ K,
                           const int32_t* __restrict__ offs, int G, int N, int H, int k,
                           int32_t* __restrict__ topk_idx, float* __restrict__ topk_score,
                           const StatusBlock* __restrict__ sb) {
-    if (sb->status != KMIP_OK) return;  // the plan kernel rejected the offsets
+    if (sweep_off(sb)) return;  // the plan kernel rejected the offsets
     constexpr int CAP = 32 * E;
     constexpr int VEC = Elem<T>::kVec;
     __shared__ cand_t s_rows[kWarpsPerBlock][CAP];
@@ -131,8 +131,9 @@ __global__ void __launch_bounds__(kRedoWarps * 32)
 score_select_redo_kernel(const T* __restrict__ Q, const T* __restrict__ K, const int32_t* __restrict__ offs, int G, int N, int H,
                          int k, int32_t* __restrict__ topk_idx, float* __restrict__ topk_score, StatusBlock* __restrict__ sb,
                          const int* __restrict__ redo_list, cand_t* scratch, long long scratch_lists) {
+    if (sweep_off(sb)) return;
     const int n_rows = sb->n_redo;
-    if (sb->status != KMIP_OK || n_rows == 0) return;
+    if (n_rows == 0) return;
     constexpr int CAP = 32 * E, VEC = Elem<T>::kVec, U = 2;
     __shared__ cand_t s_rows[kRedoWarps][CAP];
     __shared__ float s_q[kRedoWarps][D];
@@ -260,11 +261,11 @@ cudaError_t launch_t(const FwdArgs& a) {
 
 
 template <typename T, int D>
-void launch_redo_d(const FwdArgs& a, const F16Buffers& b) {
-    const int blocks = sm_count() * kRedoBlocksPerSm;
+cudaError_t launch_redo_d(const FwdArgs& a, const F16Buffers& b) {
+    const int blocks = sm_count() * (a.maybe_small ? 1 : kRedoBlocksPerSm);
     const long long lists = b.scratch_words / a.k;
 #define KMIP_LAUNCH_REDO(E_) \
-    score_select_redo_kernel<T, D, E_><<<blocks, kRedoWarps * 32, 0, a.stream>>>( \
+    return launch_next(a, score_select_redo_kernel<T, D, E_>, dim3(blocks), kRedoWarps * 32, 0, \
         static_cast<const T*>(a.Q), static_cast<const T*>(a.K), a.graph_offsets, a.G, (int)a.N, a.H, a.k, \
         a.topk_idx, a.topk_score, reinterpret_cast<StatusBlock*>(a.ws), b.redo, static_cast<cand_t*>(b.scratch), lists)
     if (a.k <= 16) KMIP_LAUNCH_REDO(2);
@@ -276,12 +277,11 @@ void launch_redo_d(const FwdArgs& a, const F16Buffers& b) {
 template <typename T>
 cudaError_t launch_redo_t(const FwdArgs& a, const F16Buffers& b) {
     switch (a.d) {
-        case 16: launch_redo_d<T, 16>(a, b); break;
-        case 32: launch_redo_d<T, 32>(a, b); break;
-        case 64: launch_redo_d<T, 64>(a, b); break;
+        case 16: return launch_redo_d<T, 16>(a, b);
+        case 32: return launch_redo_d<T, 32>(a, b);
+        case 64: return launch_redo_d<T, 64>(a, b);
         default: return cudaErrorInvalidValue;
     }
-    return cudaGetLastError();
 }
 
 }  // namespace

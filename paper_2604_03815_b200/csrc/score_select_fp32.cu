@@ -89,7 +89,7 @@ __global__ void __launch_bounds__(ROWS)
 score_select_fp32_kernel(const float* __restrict__ Q, const float* __restrict__ K, const WorkItem* __restrict__ items,
                          const StatusBlock* __restrict__ sb, int H, int k, int32_t* __restrict__ topk_idx,
                          float* __restrict__ topk_score) {
-    if (sb->status != KMIP_OK) return;  // the plan kernel rejected the offsets
+    if (sweep_off(sb)) return;  // the plan kernel rejected the offsets
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float* sK = reinterpret_cast<float*>(smem_raw);                                // [2][TK][D]
     cand_t* sList = reinterpret_cast<cand_t*>(smem_raw + 2 * TK * D * sizeof(float));  // [LIST][ROWS]

@@ -289,6 +289,7 @@ score_select_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
     constexpr int NISS = 2;  // MMA issuer threads (see the issuer branch)
     constexpr int ROOM = Sp::ROOM;
     constexpr uint32_t TMEM_COLS = NBUF * BN;
+    if (small_route(sb)) return;
 
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);

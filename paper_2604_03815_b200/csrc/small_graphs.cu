@@ -79,7 +79,7 @@ __global__ void __launch_bounds__(kWarps * 32)
 small_forward_kernel(const T* __restrict__ Q, const T* __restrict__ K, const T* __restrict__ V, const int32_t* __restrict__ offs, int G,
                      int N, int H, int k, int rows_per_warp, float scale, float drop_p, unsigned long long seed, T* __restrict__ out,
                      int32_t* __restrict__ topk_idx, float* __restrict__ topk_score, StatusBlock* __restrict__ sb) {
-    if (sb->status != KMIP_OK) return;
+    if (sb->status != KMIP_OK || sb->route != kRouteSmall) return;
     constexpr int P = D * (int)sizeof(T) / 16, kStride = row_stride<T, D>();
     extern __shared__ __align__(16) unsigned char smem[];
     unsigned char* sK = smem;                                          // [kChunk] padded key rows
@@ -257,10 +257,13 @@ cudaError_t launch_t(const FwdArgs& a) {
 //   batches of small graphs  22 400 rows x 4 heads, n = 175, d 16, k 8: 139 / 249, k 24: 196 / 412; n = 156, d 64: 215 / 358;
 //                            but n = 500, d 16, one head: 125 / 119
 //   few rows                 one graph of 500: 33 / 61, 1024: 40 / 68, 2000: 60 / 83, 4000: 152 / 99; 2000 x 4 heads: 112 / 93
-bool small_graphs_preferred(int64_t N, int32_t G, int32_t H, int32_t d, int32_t k) {
-    if (k > 32 || d > 64) return false;
-    const int64_t n = N / std::max(G, 1);  // of graphs of one size
-    return n * (d + 16) <= 15000 || N * H * n * (d + 16) <= 300000000ll;
+// What it takes grows with the sum of the squared graph sizes, so n is that sum / N (one graph of 20 000 nodes among 255 of
+// 60, 4 heads, d 16, has a mean size of 138: 5755 us here, 1100 behind the filter).  The host knows the mean alone, which is
+// never above n: where that decides nothing, the plan kernel applies the rule and both routes are launched.
+int small_graphs_use(int64_t N, int32_t G, int32_t H, int32_t d, int32_t k) {
+    if (k > 32 || d > 64) return kSmallNever;
+    if (small_graphs_preferred((double)N * N, N, H, d)) return kSmallAlways;
+    return small_graphs_preferred((double)N * N / std::max(G, 1), N, H, d) ? kSmallDecide : kSmallNever;
 }
 
 cudaError_t launch_small_graphs(const FwdArgs& a) {

@@ -388,3 +388,27 @@ def test_small_graphs_with_scores_that_overflow(n, d, k):
     assert n > 40 or bool((b.topk_idx[::6, 0, -1] < 0).all())
     assert torch.equal(a.topk_idx, b.topk_idx) and torch.equal(a.topk_score, b.topk_score)
     assert torch.equal(a.out.nan_to_num(nan=7.0), b.out.nan_to_num(nan=7.0))
+
+
+@pytest.mark.parametrize("sizes,H,d,k,mode,small", [
+    ([60] * 255 + [20000], 1, 16, 8, "bf16", False), ([20000] + [60] * 255, 2, 16, 8, "fp32", False), ([60] * 100 + [9000] + [60] * 100, 1, 64, 8, "bf16", False),
+    ([60] * 100 + [9000] + [60] * 100, 1, 64, 2, "bf16", False), ([60] * 255 + [9000], 1, 32, 2, "fp32", False), ([3000] * 5 + [0] * 1000, 2, 16, 8, "bf16", False),
+    ([100] * 400 + [12000], 1, 32, 16, "bf16", False), ([100] * 400 + [12000], 1, 32, 16, "pruned", False),
+    ([175] * 128, 4, 16, 8, "bf16", True), ([175] * 300, 1, 32, 8, "pruned", True), ([100] * 200 + [0, 1, 1500], 2, 16, 24, "fp32", True),
+    ([468] * 60, 2, 16, 9, "bf16", True), ([469] * 60, 2, 16, 9, "bf16", False)])
+def test_batches_of_unequal_graphs(sizes, H, d, k, mode, small):
+    """The small-graph kernel takes a batch by the sum of the squared graph sizes, which the device alone knows, not by the mean
+    size: a large graph among many tiny (or empty) ones goes to the sweep.  Either way the answer is that of one warp per
+    row in fp32 (at k < 4 the tensor-core sweep's: the same keys up to scores within its rounding)."""
+    m = {"bf16": kb.KMIP_BF16_TC, "fp32": kb.KMIP_FP32_EXACT, "pruned": kb.KMIP_BF16_TC_PRUNED}[mode]
+    w = wl.iid_workload("u", 6500 + len(sizes) + d + k, sizes, H, d, k, wl.MODE_FP32_EXACT if mode == "fp32" else wl.MODE_BF16_TC, backward=False)
+    w.mode = m
+    Q, K, V, _, offs = pu.to_device(w)
+    a = kb.forward(Q, K, V, offs, k, m)
+    assert (kb.kmip_test_route(a.workspace) == kb.ROUTE_SMALL) == small
+    if mode != "pruned" and k >= 4 or small:
+        b = kb.forward(Q.float(), K.float(), V.float(), offs, k, kb.KMIP_FP32_EXACT, fp32_path=1)
+        assert torch.equal(a.topk_idx, b.topk_idx) and torch.equal(a.topk_score, b.topk_score)
+    pu.check_forward(w, a, wl.sample_rows(w, 200))
+    order, rows = kb.kmip_test_sweep_order(a.workspace, w.N, w.G, H, d, k, m)
+    assert rows % 128 == 0 and (np.sort(order) == np.arange(w.N)).all()
