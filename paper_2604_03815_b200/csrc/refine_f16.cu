@@ -15,6 +15,9 @@
 //      k-th best score, which well-separated scores never produce; rows whose keys tie massively do.  Rows
 //      whose fp16 scores are no scores (a query or a key of the head beyond kF16RangeN2) go there unseen.
 // One warp per (query, head); a candidate key's row is read by D / 8 neighbouring lanes.
+//
+// Bound by instruction issue: about 2600 a row at d = 32, k = 30 (3060 with the places of the lists as arguments and a
+// 64-bit division per row: 1275 -> 1083 us for 400 000 rows; point cloud of 200k nodes, H 4, k 32: 3100 -> 2660 us).
 #include <algorithm>
 
 #include "common.cuh"
@@ -116,6 +119,9 @@ refine_f16_kernel(const T* __restrict__ Q, const T* __restrict__ K,
     constexpr int EPL = (LIST + 31) / 32;  // list entries per lane
     constexpr int KSTEPS = D / 16;
     constexpr bool kLong = LIST > kF16List32;  // k > 32: more than one kept key per lane
+    constexpr bool kCompact = kLossy || D > 32 || kLong;  // where score_select_f16_in_outputs_supported puts the lists
+    const int slots = kCompact ? lists.slots : LIST;
+    const unsigned word_pitch = kCompact ? 4u * k : 4u * LIST, half_pitch = kCompact ? 4u * k : 2u * LIST;
     __shared__ cand_t s_rows[kWarpsPerBlock][CAP];
     __shared__ __align__(16) T s_qb[kWarpsPerBlock][D];  // the query row
     __shared__ uint32_t s_words[kWarpsPerBlock][LIST];
@@ -127,8 +133,7 @@ refine_f16_kernel(const T* __restrict__ Q, const T* __restrict__ K,
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     cand_t* row = s_rows[wib];
     uint32_t* words = s_words[wib];
-    const long long n_rows = (long long)N * H;
-    const long long stride = (long long)gridDim.x * kWarpsPerBlock;
+    const unsigned n_rows = (unsigned)N * (unsigned)H, stride = gridDim.x * kWarpsPerBlock;  // below 2^31
     constexpr int P = D * (int)sizeof(T) / 16;                 // 16-byte pieces of a key row
     constexpr int kRowStride = D * (int)sizeof(T) + 16;        // padded: a lane per row reads 16-byte pieces without bank conflicts
     constexpr int kStageBytes = 32 * kRowStride;
@@ -141,27 +146,27 @@ refine_f16_kernel(const T* __restrict__ Q, const T* __restrict__ K,
     uint32_t nx_word[EPL];
     unsigned nx_half[EPL];
     T nx_q[QE];
-    auto fetch = [&](long long r) {
+    auto fetch = [&](unsigned r) {
 #pragma unroll
         for (int e = 0; e < EPL; ++e) {
             const int t = e * 32 + lane;
             nx_half[e] = 0xFFFFu;
             nx_word[e] = 0xFFFFFFFFu;
-            if (r < n_rows && t < lists.slots) {
-                nx_half[e] = *reinterpret_cast<const uint16_t*>(lists.half + r * lists.half_pitch + 2 * t);
+            if (r < n_rows && t < slots) {
+                nx_half[e] = *reinterpret_cast<const uint16_t*>(lists.half + (size_t)r * half_pitch + 2 * t);
                 // never written for an empty slot: ignored below
-                const unsigned char* wp = lists.word + r * lists.word_pitch;
-                nx_word[e] = lists.compact ? (uint32_t)reinterpret_cast<const uint16_t*>(wp)[t] : reinterpret_cast<const uint32_t*>(wp)[t];
+                const unsigned char* wp = lists.word + (size_t)r * word_pitch;
+                nx_word[e] = kCompact ? (uint32_t)reinterpret_cast<const uint16_t*>(wp)[t] : reinterpret_cast<const uint32_t*>(wp)[t];
             }
         }
 #pragma unroll
         for (int e = 0; e < QE; ++e) nx_q[e] = (r < n_rows && e * 32 + lane < D) ? Q[(size_t)r * D + e * 32 + lane] : T(0.0f);
     };
-    long long r = (long long)blockIdx.x * kWarpsPerBlock + wib;
+    unsigned r = blockIdx.x * kWarpsPerBlock + wib;
     fetch(r);
 
     for (; r < n_rows; r += stride) {
-        const int i = (int)(r / H), h = (int)(r % H);
+        const int i = (int)(r / (unsigned)H), h = (int)(r - (unsigned)i * (unsigned)H);
         int lo, hi;
         graph_range_of(offs, s_offs, G, N, i, lo, hi);
 
@@ -172,7 +177,7 @@ refine_f16_kernel(const T* __restrict__ Q, const T* __restrict__ K,
         unsigned ok_min = 0xFFFFu;
 #pragma unroll
         for (int e = 0; e < EPL; ++e) {
-            word[e] = lists.compact ? (uint32_t)(lo + (int)(nx_word[e] >> 1) * 16) | (nx_word[e] << 31) : nx_word[e];
+            word[e] = kCompact ? (uint32_t)(lo + (int)(nx_word[e] >> 1) * 16) | (nx_word[e] << 31) : nx_word[e];
             const bool valid = nx_half[e] != 0xFFFFu;
             okey[e] = valid ? f16_ordered(nx_half[e]) : 0u;
             n_valid += __popc(__ballot_sync(FULL, valid));
@@ -331,7 +336,7 @@ refine_f16_kernel(const T* __restrict__ Q, const T* __restrict__ K,
         if (blind || (n_valid < n_groups && g_min + ea + er * fabsf(g_min) >= kth * sc - fp32_err)) {
             if (lane == 0) {
                 const int pos = atomicAdd(&sb->n_redo, 1);
-                if (kmip_check(pos >= 0 && pos < n_rows, sb, 102)) redo_list[pos] = (int)r;  // checks builds: inside the list
+                if (kmip_check(pos >= 0 && (unsigned)pos < n_rows, sb, 102)) redo_list[pos] = (int)r;  // checks builds: inside the list
             }
         }
         warp_store_row(row, k, lane, topk_idx + (size_t)r * k, topk_score + (size_t)r * k);
@@ -345,6 +350,7 @@ cudaError_t launch_d(const FwdArgs& a, const FwdWorkspace& w) {
     const int blocks = grid_blocks(a, (n_rows + kWarpsPerBlock - 1) / kWarpsPerBlock, 4);
     constexpr int kSmem = kWarpsPerBlock * 2 * 32 * (D * (int)sizeof(T) + 16);  // the rescoring stages
     const F16Buffers b = f16_buffers(a, w);
+    if ((b.lists.compact != 0) != (sizeof(T) == 4 || D > 32 || a.k > 32)) return cudaErrorInvalidValue;  // the kernel's kCompact
 #define KMIP_LAUNCH_REFINE16(E_, LIST_) \
     if ((err = cudaFuncSetAttribute(refine_f16_kernel<T, D, E_, LIST_>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem)) != cudaSuccess) return err; \
     return launch_next(a, refine_f16_kernel<T, D, E_, LIST_>, dim3(blocks), kWarpsPerBlock * 32, kSmem, \
