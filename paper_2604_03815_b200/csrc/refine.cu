@@ -137,7 +137,10 @@ refine_topk_kernel(const T* __restrict__ Q, const T* __restrict__ Kp, const int3
                     if (pass) row[k + cnt + __popc(m & ((1u << lane) - 1u))] = make_cand(s, kperm ? __ldg(kperm + jj[u]) : jj[u]);
                     cnt += __popc(m);
                     if (cnt > room - 32) {
-                        tau = fmaxf(floor_now, E <= 4 ? warp_merge_row_chunks(row, k, cnt, lane) : warp_compact_row<E>(row, k, cnt, lane));
+                        // the groups come in list order, not key order: a later key with the score of the k-th best and a
+                        // smaller index must still get in
+                        const float kth = E <= 4 ? warp_merge_row_chunks(row, k, cnt, lane) : warp_compact_row<E>(row, k, cnt, lane);
+                        tau = fmaxf(floor_now, nextafterf(kth, -CUDART_INF_F));
                         cnt = 0;
                     }
                 }

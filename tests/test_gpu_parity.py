@@ -412,3 +412,18 @@ def test_batches_of_unequal_graphs(sizes, H, d, k, mode, small):
     pu.check_forward(w, a, wl.sample_rows(w, 200))
     order, rows = kb.kmip_test_sweep_order(a.workspace, w.N, w.G, H, d, k, m)
     assert rows % 128 == 0 and (np.sort(order) == np.arange(w.N)).all()
+
+
+@pytest.mark.parametrize("mode,sizes,d,k", [("fp32", [3300, 40, 3000], 64, 16), ("fp32", [2000], 16, 32), ("fp32", [1500], 32, 5),
+                                            ("bf16", [3000], 128, 16)])
+def test_lower_key_wins_among_thousands_of_ties(mode, sizes, d, k):
+    """Keys that are copies of 50 vectors through the sweeps that rank groups of keys: the groups of a row are rescored in
+    list order, and a key that ties with the k-th best must still displace one with a larger number."""
+    fp32 = mode == "fp32"
+    w = wl.iid_workload("t", 6600 + sum(sizes) + k, sizes, 2, d, k, wl.MODE_FP32_EXACT if fp32 else wl.MODE_BF16_TC, backward=False)
+    w.K[:] = w.K[np.random.default_rng(5).integers(0, 50, w.N)]
+    Q, K, V, _, offs = pu.to_device(w)
+    a = kb.forward(Q, K, V, offs, k, w.mode, fp32_path=2 if fp32 else 0)
+    b = kb.forward(Q.float(), K.float(), V.float(), offs, k, kb.KMIP_FP32_EXACT, fp32_path=1)
+    same = (a.topk_idx == b.topk_idx).all(-1)
+    assert bool(same.all()) if fp32 else float(same.float().mean()) > 0.999   # bf16: sums in another order
