@@ -97,15 +97,37 @@ int kmip_test_attn_forward(const void* Q, const void* K, const void* V, const in
 
 namespace {
 
+// Where the plan kernel decides between the small-graph kernel and the sweeps, batches below this many (query, head) rows
+// have the sweep with the fewest launches behind it, since most find nothing to do: three instead of six to nine, forward
+// pass of 40 graphs of 120, H 2, d 64, 39 instead of 54 us.  What that costs a batch that does need a sweep (us, filter /
+// this; 255 graphs of 60 and one of 20 000): bf16 H 4, d 16 903 / 861, H 1, d 64 265 / 279, fp32 H 1, d 16 213 / 1099; with
+// 3000 of 100 and one of 100 000, d 32, 2609 / 2898.
+constexpr int64_t kDirectRows = 131072;
+
 // The workspace of a forward call and, for the half-precision sweep, its work items.
 FwdWorkspace plan_forward(int64_t N, int32_t G, int32_t H, int32_t d, int32_t k, int mode, int small) {
     FwdWorkspace w = plan_fwd_workspace(N, G, H, d, k, mode);
+    w.direct = small == kSmallDecide && N * H < kDirectRows;
+    if (w.direct) w.f16 = w.in_outputs = w.prune = w.reorder = false;
     // graphs of one size are assumed; where the small-graph kernel takes those, the sweep runs if some are large
     if (w.f16) w.item_tiles = score_select_f16_item_tiles(N, small == kSmallDecide ? 1 : G, H, d, w.list);
     return w;
 }
 int rows_per_item(const FwdWorkspace& w, int32_t d, int32_t k) {
     return w.f16 ? 128 * w.item_tiles : w.tc ? score_select_tc_rows_per_item(d, k) : 128;
+}
+
+// The sweep that scores everything where the filter (the one with its lists in the output arrays) leaves more than *limit
+// (query, head) rows undecided - keys that tie by the thousands, a few keys much larger than the rest; 0 = none, the exact
+// pass takes any number.  That pass reads a graph's keys once per row: measured (ms, all rows undecided / the sweep) fp32
+// n = 60 000, d 16 28 / 4.9, n = 30 000, d 64 54 / 5.2; bf16 n = 100 000, d 64 300 / 2.4, n = 60 000, d 32, k 45 30 / 1.6.
+// Below 48 blocks of 128 rows the sweeps gain little, and three launches that find nothing to do (4 us) weigh.
+int second_sweep(int64_t N, int32_t H, int32_t d, int32_t k, int mode, int* limit) {
+    if ((N / 128) * H < 48) return 0;
+    const bool fp32 = mode == KMIP_FP32_EXACT;
+    if (fp32 ? !score_select_fp32_tiled_supported(d, k) : !score_select_tc_supported(d, k)) return 0;
+    *limit = (int)std::max<int64_t>(kRedoSplitMax, N * H / (fp32 ? 16 : d == 64 ? 256 : 64));
+    return fp32 ? kRouteTiled : kRouteTensorCore;
 }
 
 // Whether two arrays of `bytes` bytes share any.
@@ -147,7 +169,6 @@ int forward_impl(const void* Q, const void* K, const void* V, const int32_t* gra
         a.drop_first_tile = opt->drop_first_tile;
         a.fp32_path = opt->fp32_path;
     }
-    if (cudaMemsetAsync(a.ws, 0, kStatusBytes, a.stream) != cudaSuccess) return KMIP_ERR_CUDA;
     if (launch_canary_fill(a.ws, w.canaries, a.stream) != cudaSuccess) return KMIP_ERR_CUDA;
     cudaEvent_t* ev = (g_prof.on && g_prof.n_fwd < g_prof.max_calls) ? g_prof.fwd[g_prof.n_fwd++] : nullptr;
     if (ev) cudaEventRecord(ev[0], a.stream);
@@ -165,6 +186,7 @@ int forward_impl(const void* Q, const void* K, const void* V, const int32_t* gra
     // 0.70 ms at 64 blocks, 1.7 against 8.4 ms at 247), slower below (0.25 against 0.19 ms at 32)
     const bool tiled32 = mode == KMIP_FP32_EXACT && !w.f16 && score_select_fp32_tiled_supported(d, k) &&
                          (a.fp32_path == 0 ? (N / 128) * H >= 48 : a.fp32_path == 2);
+    const int again = w.in_outputs ? second_sweep(N, H, d, k, mode, &a.redo_limit) : 0;
     const int route = w.f16 ? kRouteFilter : tc ? kRouteTensorCore : tiled32 ? kRouteTiled : kRouteRows;
     if (w.reorder && launch_reorder_clear(a, w) != cudaSuccess) return KMIP_ERR_CUDA;
     if (launch_plan(a, w, rows_per_item(w, d, k), a.maybe_small ? kSmallDecide : kSmallNever, route) != cudaSuccess) return KMIP_ERR_CUDA;
@@ -172,7 +194,8 @@ int forward_impl(const void* Q, const void* K, const void* V, const int32_t* gra
         if (ev) cudaEventRecord(ev[1], a.stream);
         if (launch_small_graphs(a) != cudaSuccess) return KMIP_ERR_CUDA;
     }
-    if (tc && !w.prune && !w.f16 && launch_pack_keys(a, w) != cudaSuccess) return KMIP_ERR_CUDA;
+    a.keys_in_place = tc && w.direct;
+    if (tc && !w.prune && !w.f16 && !a.keys_in_place && launch_pack_keys(a, w) != cudaSuccess) return KMIP_ERR_CUDA;
     if (w.reorder && launch_reorder_queries(a, w) != cudaSuccess) return KMIP_ERR_CUDA;
     if (w.f16 && launch_f16_convert(a, w) != cudaSuccess) return KMIP_ERR_CUDA;
     if (w.prune && (launch_reorder_keys(a, w) != cudaSuccess || launch_prune_stats(a, w) != cudaSuccess)) return KMIP_ERR_CUDA;
@@ -183,6 +206,16 @@ int forward_impl(const void* Q, const void* K, const void* V, const int32_t* gra
     if (ev) cudaEventRecord(ev[2], a.stream);
     if (w.f16 && (launch_refine_f16(a, w) != cudaSuccess || launch_score_select_exact_redo(a, w) != cudaSuccess))
         return KMIP_ERR_CUDA;
+    if (again != 0) {
+        FwdArgs b = a;
+        FwdWorkspace v = w;
+        b.min_redo = a.redo_limit;
+        b.keys_in_place = true;
+        v.f16 = v.in_outputs = v.reorder = false;
+        if (launch_resweep_plan(b, v, rows_per_item(v, d, k), again) != cudaSuccess) return KMIP_ERR_CUDA;
+        if ((again == kRouteTensorCore ? launch_score_select_tc(b, v) : launch_score_select_fp32_tiled(b, v)) != cudaSuccess) return KMIP_ERR_CUDA;
+        if ((again == kRouteTensorCore ? launch_refine_topk(b, v) : launch_refine_topk_fp32(b)) != cudaSuccess) return KMIP_ERR_CUDA;
+    }
     if (tc && !w.f16 && launch_refine_topk(a, w) != cudaSuccess) return KMIP_ERR_CUDA;
     if (tiled32 && launch_refine_topk_fp32(a) != cudaSuccess) return KMIP_ERR_CUDA;
     if (ev) cudaEventRecord(ev[3], a.stream);

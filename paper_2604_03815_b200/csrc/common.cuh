@@ -104,6 +104,7 @@ struct FwdWorkspace {
     bool in_outputs;   // ... with its lists, the redo list and the operand copies that have no place here in the call's
                        // output arrays, which nothing else uses until the last stages write them (f16_buffers)
     bool reorder;      // the sweep runs the rows of large graphs in locality order (reorder.cu)
+    bool direct = false;  // set by plan_forward (api.cu): a fallback of the small-graph kernel with few launches
     bool prune;        // the sweep skips key tiles that cannot hold a candidate (prune.cu)
     Canaries canaries;
 };
@@ -249,15 +250,18 @@ __device__ __forceinline__ bool kmip_check(bool cond, StatusBlock* sb, int code)
     return cond;
 }
 
-// First thing in every kernel of the sweeps' routes: true if the plan kernel gave the batch to the small-graph kernel, or if
+// First thing in the kernels of the sweeps' routes: true if the plan kernel gave the batch to the small-graph kernel, or if
 // the call failed before.  The wait is for launches that overlap the end of the kernel before them (launch_next).
-// Kernels that may record a problem while blocks of theirs still start ask for the first only (it does not change under
-// them) and find no work items when the plan failed.
+// The tensor-core sweeps may record a problem while blocks of theirs still start, so they don't ask for the second: they find
+// no work items when the plan failed.  The half-precision one asks for neither - its loop is sensitive to what the compiler
+// makes of a line up here (100k nodes, d 16, k 16: 924 us without, 960 with) - and finds no work items in both cases.
 __device__ __forceinline__ bool small_route(const StatusBlock* sb) {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     return sb->route == kRouteSmall;
 }
 __device__ __forceinline__ bool sweep_off(const StatusBlock* sb) { return small_route(sb) || sb->status != KMIP_OK; }
+// ... and, in those that serve as the second sweep (FwdArgs::min_redo), whether the filter decided enough rows.
+__device__ __forceinline__ bool decided(const StatusBlock* sb, int min_redo) { return min_redo >= 0 && sb->n_redo <= min_redo; }
 
 template <typename T> struct Elem;
 template <> struct Elem<float> {
@@ -319,6 +323,9 @@ struct FwdArgs {
     long long wait_limit_cycles = 0;  // bound of every device-side wait in SM clocks; <= 0: kDefaultWaitLimitCycles
     int drop_first_tile = 0;          // leave one key tile of CTA 0 unloaded, so that the waits on it run out
     bool maybe_small = false;         // the plan kernel decides between the small-graph kernel and the sweep's kernels
+    int redo_limit = 0x7FFFFFFF;      // undecided rows that the exact pass takes; beyond, everything is swept again
+    int min_redo = -1;                // >= 0: the kernels of that second sweep return unless more rows than this are undecided
+    bool keys_in_place = false;       // the fp32-accumulate sweep and its rescoring read K as it lies, without a copy by head
     bool in_place = false;            // `out` overlaps Q or K: nothing may be written there before the last stage
     int fp32_path = 0;                // fp32 mode: 0 = sweep chosen by problem size, 1 = one warp per row, 2 = tiled
 };
@@ -339,8 +346,8 @@ struct BwdArgs {
     unsigned long long seed = 0ull;
 };
 
-// Launches a kernel of a sweep's route.  Where the plan kernel decides whether it has work (maybe_small), every launch
-// may begin while the one before it ends: returning at once then costs 1.3 us each instead of 2.5.
+// Launches a kernel of a sweep's route that begins with sweep_off or small_route: it may start while the one before it ends.
+// One that finds nothing to do then costs 1.3 us instead of 2.5.
 template <typename... P, typename... A>
 inline cudaError_t launch_next(const FwdArgs& a, void (*kern)(P...), dim3 grid, int threads, size_t smem, A&&... args) {
     cudaLaunchConfig_t c{};
@@ -352,15 +359,17 @@ inline cudaError_t launch_next(const FwdArgs& a, void (*kern)(P...), dim3 grid, 
     overlap.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     overlap.val.programmaticStreamSerializationAllowed = 1;
     c.attrs = &overlap;
-    c.numAttrs = a.maybe_small ? 1 : 0;
+    c.numAttrs = 1;
     return cudaLaunchKernelEx(&c, kern, static_cast<P>(args)...);
 }
 // plan.cu, checks builds: write the canary blocks of a workspace / verify them (detail = 900 + block number)
 cudaError_t launch_canary_fill(unsigned char* ws, const Canaries& c, cudaStream_t stream);
 cudaError_t launch_canary_check(unsigned char* ws, const Canaries& c, cudaStream_t stream);
-// plan.cu: validates the offsets and writes the work items of the tensor-core kernel
+// plan.cu: clears the status block, validates the offsets and writes the work items of the sweep
 enum SmallUse { kSmallNever = 0, kSmallAlways = 1, kSmallDecide = 2 };
 cudaError_t launch_plan(const FwdArgs& a, const FwdWorkspace& w, int rows_per_item, int small_use, int route);
+// plan.cu, after the exact pass: items of the second sweep (min_redo; route: kRouteTensorCore or kRouteTiled)
+cudaError_t launch_resweep_plan(const FwdArgs& a, const FwdWorkspace& w, int rows_per_item, int route);
 // plan.cu: K [N, H, d] -> [H, N, d] so that a head's key tile is one contiguous block for TMA
 cudaError_t launch_pack_keys(const FwdArgs& a, const FwdWorkspace& w);
 // reorder.cu: counters of the bucket sort (before launch_plan: they lie in an output array); locality codes, per-graph
@@ -386,7 +395,7 @@ int sm_count();  // multiprocessors of the current device (cached per device)
 // Blocks of a grid-stride kernel with `want` blocks of work, of which `per_sm` fit an SM.
 inline int grid_blocks(const FwdArgs& a, long long want, int per_sm) {
     // a launch that may have nothing to do has no more blocks than fit the chip at once
-    const long long most = (long long)sm_count() * (a.maybe_small ? per_sm : 32);
+    const long long most = (long long)sm_count() * (a.maybe_small || a.min_redo >= 0 ? per_sm : 32);
     return (int)(want < most ? want : most);
 }
 // score_select_tc.cu: tcgen05 scores + running top-k (bf16 storage); returns cudaErrorNotSupported
@@ -454,8 +463,8 @@ cudaError_t launch_score_select_fp32_tiled(const FwdArgs& a, const FwdWorkspace&
 // kernel, which validates the offsets
 int small_graphs_use(int64_t N, int32_t G, int32_t H, int32_t d, int32_t k);
 // The rule, for `squares` = the sum of the squared graph sizes (the scores of a head); see small_graphs.cu
-__host__ __device__ inline bool small_graphs_preferred(double squares, long long N, int H, int d) {
-    return squares * (d + 16) <= 15000.0 * (double)N || squares * H * (d + 16) <= 3.0e8;
+__host__ __device__ inline bool small_graphs_preferred(double squares, long long N, int H, int d, bool direct = false) {
+    return squares * (d + 16) <= (direct && d > 16 ? 25000.0 : 15000.0) * (double)N || squares * H * (d + 16) <= 3.0e8;
 }
 cudaError_t launch_small_graphs(const FwdArgs& a);
 // epilogue.cu: softmax over the k kept scores fused with the gather-V weighted sum

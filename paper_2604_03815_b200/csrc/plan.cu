@@ -10,52 +10,14 @@ namespace {
 
 constexpr int kPlanThreads = 1024;
 
-__global__ void __launch_bounds__(kPlanThreads)
-plan_kernel(const int32_t* __restrict__ offs, int G, int N, int rows_per_item, int max_items,
-            WorkItem* __restrict__ items, StatusBlock* __restrict__ sb, float* __restrict__ clear, int n_clear, int small_use, int route,
-            int H, int d) {
+// The work items of every graph, by one block of kPlanThreads threads.
+__device__ void write_items(const int32_t* __restrict__ offs, int n_graphs, int N, int rows_per_item, int max_items,
+                            WorkItem* __restrict__ items, StatusBlock* __restrict__ sb) {
     __shared__ int s_warp[32];
-    __shared__ unsigned long long s_squares[32];
     __shared__ int s_carry;
-    __shared__ int s_bad;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    if (tid == 0) { s_carry = 0; s_bad = 0; }
-    for (int x = tid; x < n_clear; x += kPlanThreads) clear[x] = 0.0f;  // statistics that later kernels take maxima into
+    if (tid == 0) s_carry = 0;
     __syncthreads();
-
-    if (offs != nullptr) {
-        int bad = 0;
-        if (tid == 0 && (__ldg(offs) != 0 || __ldg(offs + G) != N)) bad = 1;
-        for (int g = tid; g < G; g += kPlanThreads)
-            if (__ldg(offs + g) > __ldg(offs + g + 1) || __ldg(offs + g) < 0) bad = 1;
-        if (bad) s_bad = 1;
-        __syncthreads();
-        if (s_bad) {
-            if (tid == 0) { record_status(sb, KMIP_ERR_BAD_OFFSETS, 1); sb->n_items = 0; }
-            return;
-        }
-    }
-
-    const int n_graphs = offs ? G : 1;
-    if (small_use == kSmallDecide) {
-        // the host knows the mean graph size only; what the small-graph kernel takes grows with the squares
-        unsigned long long sq = 0ull;
-        for (int g = tid; g < n_graphs; g += kPlanThreads) {
-            const unsigned long long n = (unsigned long long)(offs ? __ldg(offs + g + 1) - __ldg(offs + g) : N);
-            sq += n * n;
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xFFFFFFFFu, sq, o);
-        if (lane == 0) s_squares[wid] = sq;
-        __syncthreads();
-        if (tid == 0) {
-            sq = 0ull;
-            for (int x = 0; x < kPlanThreads / 32; ++x) sq += s_squares[x];
-            sb->route = small_graphs_preferred((double)sq, N, H, d) ? kRouteSmall : route;
-        }
-    } else if (tid == 0) {
-        sb->route = small_use == kSmallAlways ? kRouteSmall : route;
-    }
     for (int g0 = 0; g0 < n_graphs; g0 += kPlanThreads) {
         const int g = g0 + tid;
         int lo = 0, hi = 0;
@@ -107,6 +69,55 @@ plan_kernel(const int32_t* __restrict__ offs, int G, int N, int rows_per_item, i
     if (tid == 0) sb->n_items = min(s_carry, max_items);
 }
 
+__global__ void __launch_bounds__(kPlanThreads)
+plan_kernel(const int32_t* __restrict__ offs, int G, int N, int rows_per_item, int max_items,
+            WorkItem* __restrict__ items, StatusBlock* sb, float* __restrict__ clear, int n_clear, int small_use, int route,
+            int H, int d, bool direct) {
+    __shared__ unsigned long long s_squares[32];
+    __shared__ int s_bad;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    if (tid == 0) s_bad = 0;
+    if (tid < (int)(kStatusBytes / 4)) reinterpret_cast<int*>(sb)[tid] = 0;
+    for (int x = tid; x < n_clear; x += kPlanThreads) clear[x] = 0.0f;  // statistics that later kernels take maxima into
+    __syncthreads();
+
+    if (offs != nullptr) {
+        int bad = 0;
+        if (tid == 0 && (__ldg(offs) != 0 || __ldg(offs + G) != N)) bad = 1;
+        for (int g = tid; g < G; g += kPlanThreads)
+            if (__ldg(offs + g) > __ldg(offs + g + 1) || __ldg(offs + g) < 0) bad = 1;
+        if (bad) s_bad = 1;
+        __syncthreads();
+        if (s_bad) {
+            if (tid == 0) { record_status(sb, KMIP_ERR_BAD_OFFSETS, 1); sb->n_items = 0; }
+            return;
+        }
+    }
+
+    const int n_graphs = offs ? G : 1;
+    if (small_use == kSmallDecide) {
+        // the host knows the mean graph size only; what the small-graph kernel takes grows with the squares
+        unsigned long long sq = 0ull;
+        for (int g = tid; g < n_graphs; g += kPlanThreads) {
+            const unsigned long long n = (unsigned long long)(offs ? __ldg(offs + g + 1) - __ldg(offs + g) : N);
+            sq += n * n;
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xFFFFFFFFu, sq, o);
+        if (lane == 0) s_squares[wid] = sq;
+        __syncthreads();
+        if (tid == 0) {
+            sq = 0ull;
+            for (int x = 0; x < kPlanThreads / 32; ++x) sq += s_squares[x];
+            sb->route = small_graphs_preferred((double)sq, N, H, d, direct) ? kRouteSmall : route;
+        }
+    } else if (tid == 0) {
+        sb->route = small_use == kSmallAlways ? kRouteSmall : route;
+    }
+    write_items(offs, n_graphs, N, rows_per_item, max_items, items, sb);
+    if (tid == 0 && sb->route == kRouteSmall) sb->n_items = 0;  // nothing for a sweep
+}
+
 // K [N, H, d] -> [H, N, d], 16 bytes per thread.
 __global__ void pack_keys_kernel(const uint4* __restrict__ K, uint4* __restrict__ Kp, long long n_vec, int N, int H,
                                  int vec_per_row, const StatusBlock* __restrict__ sb) {
@@ -118,6 +129,15 @@ __global__ void pack_keys_kernel(const uint4* __restrict__ K, uint4* __restrict_
     const long long j = rowh / H;
     const int h = (int)(rowh % H);
     Kp[((long long)h * N + j) * vec_per_row + c] = __ldg(K + v);
+}
+
+// The work items of the sweep that scores everything, where the filter left more rows undecided than min_redo.
+__global__ void __launch_bounds__(kPlanThreads)
+resweep_plan_kernel(const int32_t* __restrict__ offs, int G, int N, int rows_per_item, int max_items, WorkItem* __restrict__ items,
+                    StatusBlock* __restrict__ sb, int min_redo, int route) {
+    if (sweep_off(sb) || decided(sb, min_redo)) return;
+    if (threadIdx.x == 0) sb->route = route;
+    write_items(offs, offs ? G : 1, N, rows_per_item, max_items, items, sb);
 }
 
 __global__ void canary_kernel(unsigned char* __restrict__ ws, const Canaries c, bool fill) {
@@ -154,11 +174,16 @@ cudaError_t launch_pack_keys(const FwdArgs& a, const FwdWorkspace& w) {
     return cudaGetLastError();
 }
 
+cudaError_t launch_resweep_plan(const FwdArgs& a, const FwdWorkspace& w, int rows_per_item, int route) {
+    return launch_next(a, resweep_plan_kernel, dim3(1), kPlanThreads, 0, a.graph_offsets, a.G, (int)a.N, rows_per_item, w.max_items,
+                       reinterpret_cast<WorkItem*>(a.ws + w.items_off), reinterpret_cast<StatusBlock*>(a.ws), a.min_redo, route);
+}
+
 cudaError_t launch_plan(const FwdArgs& a, const FwdWorkspace& w, int rows_per_item, int small_use, int route) {
     plan_kernel<<<1, kPlanThreads, 0, a.stream>>>(
         a.graph_offsets, a.G, (int)a.N, rows_per_item, w.max_items,
         reinterpret_cast<WorkItem*>(a.ws + w.items_off), reinterpret_cast<StatusBlock*>(a.ws),
-        reinterpret_cast<float*>(a.ws + w.f16stat_off), w.f16 ? 4 * a.H : 0, small_use, route, a.H, a.d);
+        reinterpret_cast<float*>(a.ws + w.f16stat_off), w.f16 ? 4 * a.H : 0, small_use, route, a.H, a.d, w.direct);
     return cudaGetLastError();
 }
 

@@ -29,16 +29,14 @@ __device__ inline int graph_end(const int32_t* offs, int G, int N, int i) {
     return max(0, min(N, __ldg(offs + a + 1)));
 }
 
-// REGROUPED: `Kp` is the bf16 copy of K regrouped by head, [H, N, D] (tensor-core mode); otherwise it is
-// K itself, [N, H, D] (fp32 mode, scores by fp32 FMA in index order as in the exact kernel).
-template <typename T, int D, int E, bool REGROUPED>
+// Key j of head h at Kp + j * key_stride + h * head_stride: K itself, [N, H, D], or the copy regrouped by head, [H, N, D].
+template <typename T, int D, int E>
 __global__ void __launch_bounds__(kWarpsPerBlock * 32)
 refine_topk_kernel(const T* __restrict__ Q, const T* __restrict__ Kp, const int32_t* __restrict__ offs, int G,
                    int N, int H, int k, int32_t* __restrict__ topk_idx, float* __restrict__ topk_score,
-                   const StatusBlock* __restrict__ sb, const int* __restrict__ kperm) {
-    if (sweep_off(sb)) return;
+                   const StatusBlock* __restrict__ sb, const int* __restrict__ kperm, int min_redo, int key_stride, long long head_stride) {
+    if (sweep_off(sb) || decided(sb, min_redo)) return;
     constexpr int CAP = 32 * E;
-    static_assert((sizeof(T) == 2) == REGROUPED, "bf16 keys come regrouped, fp32 keys in place");
     __shared__ cand_t s_rows[kWarpsPerBlock][CAP];
     __shared__ float s_q[kWarpsPerBlock][D];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
@@ -104,9 +102,7 @@ refine_topk_kernel(const T* __restrict__ Q, const T* __restrict__ Kp, const int3
                 valid[u] = t < k && g >= 0 && jj[u] < hi &&
                            kmip_check(jj[u] >= 0 && hi <= N, const_cast<StatusBlock*>(sb), 101);  // checks builds: key row inside K
                 if (valid[u]) {
-                    // regrouped by head, the 8 keys of a group are 8 consecutive rows
-                    const uint4* kr = reinterpret_cast<const uint4*>(
-                        REGROUPED ? Kp + ((size_t)h * N + jj[u]) * D : Kp + ((size_t)jj[u] * H + h) * D);
+                    const uint4* kr = reinterpret_cast<const uint4*>(Kp + (size_t)jj[u] * key_stride + h * head_stride);
 #pragma unroll
                     for (int v = 0; v < NV; ++v) raw[u][v] = __ldg(kr + v);
                 }
@@ -163,34 +159,34 @@ refine_topk_kernel(const T* __restrict__ Q, const T* __restrict__ Kp, const int3
 }
 
 template <typename T, int D>
-cudaError_t launch_d(const FwdArgs& a, const T* keys, const int* kperm = nullptr) {
-    constexpr bool REGROUPED = sizeof(T) == 2;
+cudaError_t launch_d(const FwdArgs& a, const T* keys, bool by_head, const int* kperm = nullptr) {
     const long long n_rows = (long long)a.N * a.H;
-    const int blocks = (int)std::min<long long>((n_rows + kWarpsPerBlock - 1) / kWarpsPerBlock, (long long)sm_count() * 32);
+    const int blocks = grid_blocks(a, (n_rows + kWarpsPerBlock - 1) / kWarpsPerBlock, 4);
 #define KMIP_LAUNCH_REFINE(E_) \
-    refine_topk_kernel<T, D, E_, REGROUPED><<<blocks, kWarpsPerBlock * 32, 0, a.stream>>>( \
+    return launch_next(a, refine_topk_kernel<T, D, E_>, dim3(blocks), kWarpsPerBlock * 32, 0, \
         static_cast<const T*>(a.Q), keys, a.graph_offsets, a.G, (int)a.N, a.H, a.k, \
-        a.topk_idx, a.topk_score, reinterpret_cast<const StatusBlock*>(a.ws), kperm)
+        a.topk_idx, a.topk_score, reinterpret_cast<const StatusBlock*>(a.ws), kperm, a.min_redo, \
+        by_head ? D : a.H * D, by_head ? (long long)a.N * D : (long long)D)
     // pending room CAP-k: the survivors of a row (rarely more than 2k) should fit without intermediate
     // compactions, and the final sort costs log^2(CAP) compare-exchange stages
     if (a.k <= 16) KMIP_LAUNCH_REFINE(2);
     else if (a.k <= 32) KMIP_LAUNCH_REFINE(4);
     else KMIP_LAUNCH_REFINE(8);
 #undef KMIP_LAUNCH_REFINE
-    return cudaGetLastError();
 }
 
 }  // namespace
 
 cudaError_t launch_refine_topk(const FwdArgs& a, const FwdWorkspace& w) {
     using T = __nv_bfloat16;
-    const T* keys = reinterpret_cast<const T*>(a.ws + w.kpack_off);
+    const bool by_head = !a.keys_in_place;
+    const T* keys = by_head ? reinterpret_cast<const T*>(a.ws + w.kpack_off) : static_cast<const T*>(a.K);
     const int* kperm = w.prune ? reinterpret_cast<const int*>(a.ws + w.kperm_off) : nullptr;
     switch (a.d) {
-        case 16: return launch_d<T, 16>(a, keys, kperm);
-        case 32: return launch_d<T, 32>(a, keys, kperm);
-        case 64: return launch_d<T, 64>(a, keys, kperm);
-        case 128: return launch_d<T, 128>(a, keys, kperm);
+        case 16: return launch_d<T, 16>(a, keys, by_head, kperm);
+        case 32: return launch_d<T, 32>(a, keys, by_head, kperm);
+        case 64: return launch_d<T, 64>(a, keys, by_head, kperm);
+        case 128: return launch_d<T, 128>(a, keys, by_head, kperm);
         default: return cudaErrorInvalidValue;
     }
 }
@@ -199,9 +195,9 @@ cudaError_t launch_refine_topk(const FwdArgs& a, const FwdWorkspace& w) {
 cudaError_t launch_refine_topk_fp32(const FwdArgs& a) {
     const float* keys = static_cast<const float*>(a.K);
     switch (a.d) {
-        case 16: return launch_d<float, 16>(a, keys);
-        case 32: return launch_d<float, 32>(a, keys);
-        case 64: return launch_d<float, 64>(a, keys);
+        case 16: return launch_d<float, 16>(a, keys, false);
+        case 32: return launch_d<float, 32>(a, keys, false);
+        case 64: return launch_d<float, 64>(a, keys, false);
         default: return cudaErrorInvalidValue;
     }
 }

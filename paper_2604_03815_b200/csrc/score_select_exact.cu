@@ -130,10 +130,10 @@ template <typename T, int D, int E>
 __global__ void __launch_bounds__(kRedoWarps * 32)
 score_select_redo_kernel(const T* __restrict__ Q, const T* __restrict__ K, const int32_t* __restrict__ offs, int G, int N, int H,
                          int k, int32_t* __restrict__ topk_idx, float* __restrict__ topk_score, StatusBlock* __restrict__ sb,
-                         const int* __restrict__ redo_list, cand_t* scratch, long long scratch_lists) {
+                         const int* __restrict__ redo_list, cand_t* scratch, long long scratch_lists, int limit) {
     if (sweep_off(sb)) return;
     const int n_rows = sb->n_redo;
-    if (n_rows == 0) return;
+    if (n_rows == 0 || n_rows > limit) return;  // too many: all rows are swept again (api.cu)
     constexpr int CAP = 32 * E, VEC = Elem<T>::kVec, U = 2;
     __shared__ cand_t s_rows[kRedoWarps][CAP];
     __shared__ float s_q[kRedoWarps][D];
@@ -267,7 +267,7 @@ cudaError_t launch_redo_d(const FwdArgs& a, const F16Buffers& b) {
 #define KMIP_LAUNCH_REDO(E_) \
     return launch_next(a, score_select_redo_kernel<T, D, E_>, dim3(blocks), kRedoWarps * 32, 0, \
         static_cast<const T*>(a.Q), static_cast<const T*>(a.K), a.graph_offsets, a.G, (int)a.N, a.H, a.k, \
-        a.topk_idx, a.topk_score, reinterpret_cast<StatusBlock*>(a.ws), b.redo, static_cast<cand_t*>(b.scratch), lists)
+        a.topk_idx, a.topk_score, reinterpret_cast<StatusBlock*>(a.ws), b.redo, static_cast<cand_t*>(b.scratch), lists, a.redo_limit)
     if (a.k <= 16) KMIP_LAUNCH_REDO(2);
     else if (a.k <= 96) KMIP_LAUNCH_REDO(4);
     else KMIP_LAUNCH_REDO(8);

@@ -314,7 +314,6 @@ score_select_f16_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
     constexpr int NEPI = 4 * NQT;
     constexpr uint32_t TMEM_COLS = NBUF * BN;
     static_assert(NQT <= NBUF && NQT <= kIssuers + 1, "an accumulator buffer per query tile");
-    if (small_route(sb)) return;
 
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -675,10 +674,11 @@ cudaError_t launch_cfg(const FwdArgs& a, const FwdWorkspace& w, float* dump) {
     if (err != cudaSuccess) return err;
     const long long max_total = (long long)w.max_items * a.H;
     const int grid = (int)std::min<long long>(sm_count(), max_total);
-    return launch_next(a, kern, dim3(grid), threads16(NQT), smem_bytes,
+    kern<<<grid, threads16(NQT), smem_bytes, a.stream>>>(
         tmQ, tmK, reinterpret_cast<const WorkItem*>(a.ws + w.items_off), reinterpret_cast<StatusBlock*>(a.ws), a.H,
         buf.lists, select_targets(w.list), w.item_tiles, dump, (int)a.N, a.wait_limit_cycles > 0 ? a.wait_limit_cycles : kDefaultWaitLimitCycles, a.drop_first_tile,
         (w.reorder && !DUMP) ? reinterpret_cast<const int*>(a.ws + w.perm_off) : nullptr);
+    return cudaGetLastError();
 }
 
 // Long lists, measured (us for the sweep, fp32-accumulate sweep / this one): 100k nodes, H 1, d 16, k 45 2098 / 1070, k 100

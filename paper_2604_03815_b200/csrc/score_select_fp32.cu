@@ -88,8 +88,8 @@ template <int D>
 __global__ void __launch_bounds__(ROWS)
 score_select_fp32_kernel(const float* __restrict__ Q, const float* __restrict__ K, const WorkItem* __restrict__ items,
                          const StatusBlock* __restrict__ sb, int H, int k, int32_t* __restrict__ topk_idx,
-                         float* __restrict__ topk_score) {
-    if (sweep_off(sb)) return;  // the plan kernel rejected the offsets
+                         float* __restrict__ topk_score, int min_redo) {
+    if (sweep_off(sb) || decided(sb, min_redo)) return;  // the plan kernel rejected the offsets
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float* sK = reinterpret_cast<float*>(smem_raw);                                // [2][TK][D]
     cand_t* sList = reinterpret_cast<cand_t*>(smem_raw + 2 * TK * D * sizeof(float));  // [LIST][ROWS]
@@ -184,11 +184,10 @@ cudaError_t launch_d(const FwdArgs& a, const FwdWorkspace& w) {
     cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (err != cudaSuccess) return err;
     const long long total = (long long)w.max_items * a.H;
-    const int grid = (int)std::min<long long>(total, (long long)sm_count() * 16);
-    kern<<<grid, ROWS, smem, a.stream>>>(static_cast<const float*>(a.Q), static_cast<const float*>(a.K),
+    const int grid = (int)std::min<long long>(total, (long long)sm_count() * (a.min_redo >= 0 ? 4 : 16));
+    return launch_next(a, kern, dim3(grid), ROWS, smem, static_cast<const float*>(a.Q), static_cast<const float*>(a.K),
                                          reinterpret_cast<const WorkItem*>(a.ws + w.items_off),
-                                         reinterpret_cast<const StatusBlock*>(a.ws), a.H, a.k, a.topk_idx, a.topk_score);
-    return cudaGetLastError();
+                                         reinterpret_cast<const StatusBlock*>(a.ws), a.H, a.k, a.topk_idx, a.topk_score, a.min_redo);
 }
 
 }  // namespace

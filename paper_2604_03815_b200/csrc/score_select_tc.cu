@@ -18,7 +18,8 @@
 //               hold a key at least as good.  So the sweep only tracks groups: a lane whose tile
 //               maximum beats tau appends (group maximum, first key) for the groups above tau to
 //               its pending slots - no index search.  Groups with EQUAL maxima are not ordered
-//               further (a new one never displaces an equal old one); the rescoring kernel applies
+//               further (a new one never displaces an equal old one), except where this sweep stands in for the
+//               half-precision filter (min_redo); the rescoring kernel applies
 //               the (score desc, key asc) order to the keys it is given;
 //   flush       when a pending area fills up all 32 lanes insert their pending groups into their
 //               own unsorted k-entry lists in lock step (replace the list minimum, 8-slot blocks
@@ -137,12 +138,29 @@ __device__ __forceinline__ void row_init(RowSel<KG>& r, uint32_t* wl, int k, int
     r.cnt = 0;
 }
 
+// Of the list entries whose score is `m`, the slot of the one with the highest key; and the minimum of its 8-slot block once
+// `x` is in its place.
+__device__ __noinline__ uint2 last_of_equals(uint32_t wl_s, int n_slots, uint32_t m, uint32_t x) {
+    int at = 0;
+    uint32_t last = 0u;
+    for (int s = 0; s < n_slots; ++s) {
+        if (ptx::lds_u32(wl_s + (uint32_t)s * 128u) != m) continue;
+        const uint32_t key = ptx::lds_u32(wl_s + (uint32_t)(n_slots + s) * 128u);
+        if (key >= last) { last = key; at = s; }
+    }
+    uint32_t nm = x;
+    for (int s = at & ~7; s < (at & ~7) + 8; ++s)
+        if (s != at) nm = min(nm, ptx::lds_u32(wl_s + (uint32_t)s * 128u));
+    return make_uint2((uint32_t)at, nm);
+}
+
 // All 32 lanes insert their pending candidates into their own lists, in lock step.  `wl_s` is the
 // shared address of the lane's slot 0 in the score plane of the warp's lists (slots 128 bytes
 // apart, the key plane 8*KG*128 bytes further), `wp_s` that of the lane's first pending slot
-// (256 bytes apart).
+// (256 bytes apart).  `by_key`: of several entries with the smallest score the one with the highest key makes room, so that
+// the list is that of (score desc, key asc) whatever ties; costs the ordinary sweep 2 to 3 %.
 template <int KG>
-__device__ __forceinline__ void flush_pending(RowSel<KG>& r, uint32_t wl_s, uint32_t wp_s, bool rvalid) {
+__device__ __forceinline__ void flush_pending(RowSel<KG>& r, uint32_t wl_s, uint32_t wp_s, bool rvalid, bool by_key) {
     const int maxc = __reduce_max_sync(FULL, r.cnt);
     __syncwarp();
 #pragma unroll 1
@@ -156,13 +174,25 @@ __device__ __forceinline__ void flush_pending(RowSel<KG>& r, uint32_t wl_s, uint
 #pragma unroll
                 for (int q = 1; q < KG; ++q)
                     if (r.gmin[q] < m) { m = r.gmin[q]; g = q; }
-                const uint32_t grp = wl_s + (uint32_t)g * (8u * 128u);
+                uint32_t grp = wl_s + (uint32_t)g * (8u * 128u);
                 uint32_t nm = x;
                 int pos = -1;
 #pragma unroll
                 for (int s = 0; s < 8; ++s) {
                     const uint32_t y = ptx::lds_u32(grp + s * 128);
                     if (y == m && pos < 0) pos = s; else nm = min(nm, y);
+                }
+                if (by_key && m != 0u) {  // uniform; 0 = empty
+                    bool tie = nm == m;
+#pragma unroll
+                    for (int q = 0; q < KG; ++q) tie = tie || (q != g && r.gmin[q] == m);
+                    if (tie) {
+                        const uint2 p = last_of_equals(wl_s, 8 * KG, m, x);
+                        g = (int)p.x >> 3;
+                        pos = (int)p.x & 7;
+                        nm = p.y;
+                        grp = wl_s + (uint32_t)g * (8u * 128u);
+                    }
                 }
                 ptx::sts_u32(grp + (uint32_t)pos * 128u, x);
                 ptx::sts_u32(grp + (uint32_t)pos * 128u + 8u * KG * 128u, raw.x);
@@ -281,7 +311,8 @@ score_select_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
                        const WorkItem* __restrict__ items, StatusBlock* __restrict__ sb, int H, int k,
                        int32_t* __restrict__ topk_idx, float* __restrict__ topk_score,
                        float* __restrict__ dump, int dump_ld /* = N */, long long wait_limit, int drop_first_tile,
-                       const int* __restrict__ perm, const PruneArgs pr) {
+                       const int* __restrict__ perm, const PruneArgs pr, int min_redo, int key_col,
+                       int key_row /* head h's keys: column h * key_col, row h * key_row */) {
     static_assert(!(DUMP && PRUNE) && !(LSE && (DUMP || PRUNE)), "the score dump and the softmax-share pass sweep every tile");
     using Sh = TcShape<D>;
     using Sp = SmemPlan<KG, NQT, S>;
@@ -289,7 +320,7 @@ score_select_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
     constexpr int NISS = 2;  // MMA issuer threads (see the issuer branch)
     constexpr int ROOM = Sp::ROOM;
     constexpr uint32_t TMEM_COLS = NBUF * BN;
-    if (small_route(sb)) return;
+    if (small_route(sb) || decided(sb, min_redo)) return;
 
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -474,7 +505,7 @@ score_select_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
                             ptx::mbar_arrive_expect_tx(bars.k_full(s), Sh::TILE_BYTES);
                             for (int ch = 0; ch < Sh::KCH; ++ch)
                                 ptx::tma_load_2d(ptx::smem_u32(sK + s * Sh::TILE_BYTES + ch * Sh::CH_BYTES), &tmK,
-                                                 ch * 64, h * dump_ld + key0, bars.k_full(s));
+                                                 ch * 64, h * key_row + key0, bars.k_full(s));
                             ++kt;
                         }
                     }
@@ -540,7 +571,7 @@ score_select_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
                     ptx::mbar_arrive_expect_tx(bars.k_full(s), Sh::TILE_BYTES);
                     for (int ch = 0; ch < Sh::KCH; ++ch)
                         ptx::tma_load_2d(ptx::smem_u32(sK + s * Sh::TILE_BYTES + ch * Sh::CH_BYTES), &tmK,
-                                         ch * 64, h * dump_ld + it.key_lo + j * BN, bars.k_full(s));
+                                         ch * 64 + h * key_col, h * key_row + it.key_lo + j * BN, bars.k_full(s));
                 }
                 ++ic;
             }
@@ -780,7 +811,7 @@ score_select_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
                         // merge pending candidates into the lists meanwhile (always allowed, and it
                         // raises the thresholds early), then block.
                         if (__any_sync(FULL, rs.cnt > 0)) {
-                            flush_pending<KG>(rs, wl_s, wp_addr, rvalid);
+                            flush_pending<KG>(rs, wl_s, wp_addr, rvalid, !PRUNE && min_redo >= 0);
                             if constexpr (PRUNE) publish_thresholds(rs.tau, inv_qn, ic, warp_stat_s + 16u * warp, lane);
                         }
                         ok = wait_or_abort(full_bar, full_par, sAbort, sb, 6, wait_limit);
@@ -831,7 +862,7 @@ score_select_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
                         }
                     }
                     if (do_flush) {
-                        flush_pending<KG>(rs, wl_s, wp_addr, rvalid);
+                        flush_pending<KG>(rs, wl_s, wp_addr, rvalid, !PRUNE && min_redo >= 0);
                         if constexpr (PRUNE) publish_thresholds(rs.tau, inv_qn, ic, warp_stat_s + 16u * warp, lane);
                         flush_seen = req + ((req == flush_seen) ? 1 : 0);
                     }
@@ -841,7 +872,7 @@ score_select_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
             if (!DUMP && !LSE && active) {
                 // finalise: drain the pending slots, then store each row's k groups (first key and
                 // group maximum, unsorted; empty slots as -1 / -inf) for the rescoring kernel
-                flush_pending<KG>(rs, wl_s, wp_addr, rvalid);
+                flush_pending<KG>(rs, wl_s, wp_addr, rvalid, !PRUNE && min_redo >= 0);
                 __syncwarp();
                 const int nloc = min(32, it.nrows - (qt * BM + quarter * 32));
                 for (int r = 0; r < nloc; ++r) {
@@ -912,7 +943,7 @@ cudaError_t launch_cfg(const FwdArgs& a, const FwdWorkspace& w, float* dump) {
     static_assert(smem_bytes <= 232448, "shared memory budget of one CTA");
     CUtensorMap tmQ, tmK;
     if (!make_tensor_map<D>(&tmQ, w.reorder ? static_cast<const void*>(a.ws + w.qperm_off) : a.Q, a.N, (int64_t)a.H * D) ||
-        !make_tensor_map<D>(&tmK, a.ws + w.kpack_off, a.N * a.H, D))
+        !(a.keys_in_place ? make_tensor_map<D>(&tmK, a.K, a.N, (int64_t)a.H * D) : make_tensor_map<D>(&tmK, a.ws + w.kpack_off, a.N * a.H, D)))
         return cudaErrorInvalidValue;
     auto kern = score_select_tc_kernel<D, KG, NQT, S, DUMP, PRUNE, LSE>;
     PruneArgs pr{nullptr, nullptr, nullptr};
@@ -923,11 +954,11 @@ cudaError_t launch_cfg(const FwdArgs& a, const FwdWorkspace& w, float* dump) {
     if (err != cudaSuccess) return err;
     const long long max_total = (long long)w.max_items * a.H;
     const int grid = (int)std::min<long long>(sm_count(), max_total);
-    kern<<<grid, NQT * 128 + 96, smem_bytes, a.stream>>>(
+    return launch_next(a, kern, dim3(grid), NQT * 128 + 96, smem_bytes,
         tmQ, tmK, reinterpret_cast<const WorkItem*>(a.ws + w.items_off), reinterpret_cast<StatusBlock*>(a.ws),
         a.H, a.k, a.topk_idx, a.topk_score, dump, (int)a.N, a.wait_limit_cycles > 0 ? a.wait_limit_cycles : kDefaultWaitLimitCycles,
-        a.drop_first_tile, (w.reorder && !DUMP) ? reinterpret_cast<const int*>(a.ws + w.perm_off) : nullptr, pr);
-    return cudaGetLastError();
+        a.drop_first_tile, (w.reorder && !DUMP) ? reinterpret_cast<const int*>(a.ws + w.perm_off) : nullptr, pr, a.min_redo,
+        a.keys_in_place ? D : 0, a.keys_in_place ? 0 : (int)a.N);
 }
 
 template <int D, bool DUMP, bool PRUNE>

@@ -79,7 +79,7 @@ __global__ void __launch_bounds__(kWarps * 32)
 small_forward_kernel(const T* __restrict__ Q, const T* __restrict__ K, const T* __restrict__ V, const int32_t* __restrict__ offs, int G,
                      int N, int H, int k, int rows_per_warp, float scale, float drop_p, unsigned long long seed, T* __restrict__ out,
                      int32_t* __restrict__ topk_idx, float* __restrict__ topk_score, StatusBlock* __restrict__ sb) {
-    if (sb->status != KMIP_OK || sb->route != kRouteSmall) return;
+    if (!small_route(sb) || sb->status != KMIP_OK) return;
     constexpr int P = D * (int)sizeof(T) / 16, kStride = row_stride<T, D>();
     extern __shared__ __align__(16) unsigned char smem[];
     unsigned char* sK = smem;                                          // [kChunk] padded key rows
@@ -234,10 +234,9 @@ cudaError_t launch_d(const FwdArgs& a) {
     cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (err != cudaSuccess) return err;
     const dim3 grid((unsigned)((a.N + kWarps * rows_per_warp - 1) / (kWarps * rows_per_warp)), (unsigned)std::min(a.H, 65535));
-    kern<<<grid, kWarps * 32, smem, a.stream>>>(static_cast<const T*>(a.Q), static_cast<const T*>(a.K), static_cast<const T*>(a.V),
+    return launch_next(a, kern, grid, kWarps * 32, smem, static_cast<const T*>(a.Q), static_cast<const T*>(a.K), static_cast<const T*>(a.V),
                                                 a.graph_offsets, a.G, (int)a.N, a.H, a.k, rows_per_warp, 1.0f / sqrtf((float)a.d), a.drop_p,
                                                 a.seed, static_cast<T*>(a.out), a.topk_idx, a.topk_score, reinterpret_cast<StatusBlock*>(a.ws));
-    return cudaGetLastError();
 }
 
 template <typename T>
@@ -259,7 +258,10 @@ cudaError_t launch_t(const FwdArgs& a) {
 //   few rows                 one graph of 500: 33 / 61, 1024: 40 / 68, 2000: 60 / 83, 4000: 152 / 99; 2000 x 4 heads: 112 / 93
 // What it takes grows with the sum of the squared graph sizes, so n is that sum / N (one graph of 20 000 nodes among 255 of
 // 60, 4 heads, d 16, has a mean size of 138: 5755 us here, 1100 behind the filter).  The host knows the mean alone, which is
-// never above n: where that decides nothing, the plan kernel applies the rule and both routes are launched.
+// never above n: where that decides nothing, the plan kernel applies the rule and both routes are launched.  Smaller batches
+// then have the fp32-accumulate or the tiled sweep behind them (plan_forward, api.cu), which at d = 16 meet this kernel on
+// the same line (100 graphs of 460: 120 / 124 us bf16, 131 / 153 fp32), wider heads later: 100 of 300, d 32 182 / 306 bf16
+// and 254 / 409 fp32, 100 of 185, d 64 105 / 161 and 151 / 267.
 int small_graphs_use(int64_t N, int32_t G, int32_t H, int32_t d, int32_t k) {
     if (k > 32 || d > 64) return kSmallNever;
     if (small_graphs_preferred((double)N * N, N, H, d)) return kSmallAlways;

@@ -219,3 +219,34 @@ def test_rows_beyond_the_range_of_the_copies(mode, d, k, what):
     assert torch.equal(a.topk_idx, b.topk_idx) and torch.equal(a.topk_score, b.topk_score)
     if what == "key":
         assert int((a.topk_idx[:, 0, 0] == 1234).sum()) > N // 4
+
+
+@pytest.mark.parametrize("sizes,H,d,k,mode,route", [
+    ([7000], 1, 16, 12, "fp32", "ROUTE_TILED"), ([3300, 40, 3000], 2, 64, 16, "fp32", "ROUTE_TILED"), ([6500], 1, 64, 20, "bf16", "ROUTE_TENSOR_CORE"),
+    ([3300, 40, 3000], 2, 32, 45, "bf16", "ROUTE_TENSOR_CORE"), ([6400], 1, 32, 100, "bf16", "ROUTE_TENSOR_CORE"), ([33000], 1, 64, 8, "bf16", "ROUTE_TENSOR_CORE"),
+    ([6200], 1, 32, 80, "fp32", "ROUTE_FILTER"), ([5000], 1, 64, 20, "bf16", "ROUTE_FILTER")])
+@pytest.mark.parametrize("what", ["ties", "heavy"])
+def test_many_undecidable_rows_are_swept_again(sizes, H, d, k, mode, route, what):
+    """Keys that are copies of 50 vectors, or one key a thousand times the others' size: the filter decides next to no row.
+    From 48 blocks of rows on the sweep that scores everything takes over; smaller calls and those without such a sweep
+    stay with the exact pass.  Equal scores go to the lower key in all of them."""
+    fp32 = mode == "fp32"
+    w = wl.iid_workload("t", 5600 + sum(sizes) + k, sizes, H, d, k, wl.MODE_FP32_EXACT if fp32 else wl.MODE_BF16_TC, backward=False)
+    if fp32:                       # values that fp16 cannot hold exactly
+        w.Q[:], w.K[:] = w.Q * np.float32(1.1), w.K * np.float32(1.1)
+    if what == "ties":
+        w.K[:] = w.K[np.random.default_rng(5).integers(0, 50, w.N)]
+    else:
+        w.K[w.N // 2] = w.K[w.N // 2] * 1024
+    Q, K, V, _, offs = pu.to_device(w)
+    a = kb.forward(Q, K, V, offs, k, w.mode)
+    assert kb.kmip_attn_sweep_counters(a.workspace)[4] > w.N * H // 4
+    assert kb.kmip_test_route(a.workspace) == getattr(kb, route)
+    b = kb.forward(Q.float(), K.float(), V.float(), offs, k, kb.KMIP_FP32_EXACT, fp32_path=1)
+    same = (a.topk_idx == b.topk_idx).all(-1)
+    if route == "ROUTE_TENSOR_CORE":   # scores summed in another order: a tie within their rounding may go the other way
+        assert float(same.float().mean()) > 0.999 and torch.allclose(a.topk_score, b.topk_score, rtol=1e-5, atol=1e-5)
+    else:
+        assert bool(same.all()) and torch.equal(a.topk_score, b.topk_score)
+    if w.N < 10000:
+        pu.check_forward(w, a, wl.sample_rows(w, 200))
