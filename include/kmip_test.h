@@ -27,6 +27,9 @@ typedef struct {
     /* KMIP_FP32_EXACT only: 0 = the sweep is chosen by problem size, 1 = one warp per query row,
        2 = the tiled sweep whenever it supports (d, k). */
     int32_t fp32_path;
+    /* 0 = chosen as for kmip_attn_forward, otherwise one of KMIP_ROUTE_SMALL, KMIP_ROUTE_FILTER and KMIP_ROUTE_TENSOR_CORE
+       (below), whatever the problem size; KMIP_ERR_UNSUPPORTED where it does not serve (mode, d, k). */
+    int32_t route;
 } kmip_test_options_t;
 
 /*

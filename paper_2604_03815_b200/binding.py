@@ -35,7 +35,7 @@ _lib = None
 class TestOptions(ctypes.Structure):
     """kmip_test_options_t of include/kmip_test.h."""
     _fields_ = [("wait_limit_cycles", ctypes.c_int64), ("drop_first_tile", ctypes.c_int32),
-                ("fp32_path", ctypes.c_int32)]
+                ("fp32_path", ctypes.c_int32), ("route", ctypes.c_int32)]
 
 
 class LayerTensors(ctypes.Structure):
@@ -287,11 +287,11 @@ def kmip_test_gemm_tn(A, B, C, workspace, stream=None) -> int:
 
 
 def kmip_test_attn_forward(Q, K, V, graph_offsets, k, mode, out, topk_idx, topk_score, workspace, stream=None,
-                           wait_limit_cycles=0, drop_first_tile=0, fp32_path=0) -> int:
+                           wait_limit_cycles=0, drop_first_tile=0, fp32_path=0, route=0) -> int:
     """kmip_test.h: the forward pass with per-call test options; returns the library's status code."""
     N, H, d = Q.shape
     G = 0 if graph_offsets is None else int(graph_offsets.numel()) - 1
-    opt = TestOptions(int(wait_limit_cycles), int(drop_first_tile), int(fp32_path))
+    opt = TestOptions(int(wait_limit_cycles), int(drop_first_tile), int(fp32_path), int(route))
     return int(lib().kmip_test_attn_forward(_ptr(Q), _ptr(K), _ptr(V), _ptr(graph_offsets), G, N, H, d, k, mode,
                                             _ptr(out), _ptr(topk_idx), _ptr(topk_score), _ptr(workspace),
                                             0 if workspace is None else workspace.numel() * workspace.element_size(),
@@ -366,15 +366,15 @@ class BackwardBuffers:
 
 
 def forward(Q, K, V, graph_offsets, k, mode, buffers: ForwardBuffers | None = None, stream=None, check=True,
-            fp32_path=0):
-    """Allocate (unless given) and run the forward pass; returns the buffers.  fp32_path != 0 goes through
-    kmip_test_attn_forward to pin which fp32-mode sweep runs (tests only)."""
+            fp32_path=0, route=0):
+    """Allocate (unless given) and run the forward pass; returns the buffers.  fp32_path != 0 or route != 0 goes
+    through kmip_test_attn_forward to pin which kernels run (tests only)."""
     N, H, d = Q.shape
     G = 1 if graph_offsets is None else int(graph_offsets.numel()) - 1
     b = buffers or ForwardBuffers(N, G, H, d, k, mode, Q.device)
-    if fp32_path:
+    if fp32_path or route:
         rc = kmip_test_attn_forward(Q, K, V, graph_offsets, k, mode, b.out, b.topk_idx, b.topk_score, b.workspace,
-                                    stream, fp32_path=fp32_path)
+                                    stream, fp32_path=fp32_path, route=route)
     else:
         rc = kmip_attn_forward(Q, K, V, graph_offsets, k, mode, b.out, b.topk_idx, b.topk_score, b.workspace, stream)
     if rc != KMIP_OK:

@@ -149,9 +149,14 @@ int forward_impl(const void* Q, const void* K, const void* V, const int32_t* gra
     if (!aligned16(Q) || !aligned16(K) || !aligned16(V) || !aligned16(out) || !aligned16(topk_idx) ||
         !aligned16(topk_score) || !aligned16(workspace) || (reinterpret_cast<uintptr_t>(graph_offsets) & 3u))
         return KMIP_ERR_INVALID_ARG;
-    const bool test_sweep = opt && (opt->fp32_path != 0 || opt->drop_first_tile != 0);  // a test wants one of the sweeps
-    const int small = test_sweep ? kSmallNever : small_graphs_use(N, graph_offsets ? G : 1, H, d, k);
+    const int wanted = opt ? opt->route : 0;
+    const bool test_sweep = opt && (opt->fp32_path != 0 || opt->drop_first_tile != 0 || wanted > KMIP_ROUTE_SMALL);  // a test wants one of the sweeps
+    const int small = wanted == KMIP_ROUTE_SMALL ? kSmallAlways : test_sweep ? kSmallNever : small_graphs_use(N, graph_offsets ? G : 1, H, d, k);
     FwdWorkspace w = plan_forward(N, graph_offsets ? G : 1, H, d, k, mode, small);
+    if (wanted == KMIP_ROUTE_TENSOR_CORE) w.f16 = w.in_outputs = false;
+    if (wanted < 0 || wanted > KMIP_ROUTE_TENSOR_CORE || (wanted == KMIP_ROUTE_SMALL && (k > 32 || d > 64)) ||
+        (wanted == KMIP_ROUTE_FILTER && !w.f16) || (wanted == KMIP_ROUTE_TENSOR_CORE && !w.tc))
+        return KMIP_ERR_UNSUPPORTED;
     if (mode == KMIP_FP32_EXACT && opt && opt->fp32_path != 0) w.f16 = w.in_outputs = false;  // a test picks the CUDA-core sweep
     const size_t array_bytes = (size_t)N * H * d * (mode == KMIP_FP32_EXACT ? 4 : 2);
     const bool in_place = overlap(out, Q, array_bytes) || overlap(out, K, array_bytes);

@@ -382,11 +382,7 @@ cudaError_t launch_reorder_keys(const FwdArgs& a, const FwdWorkspace& w);
 // prune.cu: centroid / radius / norm statistics of every item's query rows and of every key tile
 cudaError_t launch_prune_stats(const FwdArgs& a, const FwdWorkspace& w);
 constexpr int kMinRowsToSort = 8192;  // smaller graphs keep their row and key order
-// fp32 mode: smallest N * H that runs the half-precision prefilter.  Its launches cost about 100 us, and one warp per row
-// takes 58 us at 1024 rows (one graph, d = 32), 167 at 2048 (filter: 114) and 601 at 4096 (150).
-constexpr int64_t kF16MinRowsFp32 = 1536;
-constexpr int64_t kF16MinRowsWide = 2048;
-// Smallest N * H with 32 < k <= 103 that does (us for the forward pass, fp32-accumulate sweep / filter): 1024 rows, d 16, k 45:
+// Smallest N * H with 32 < k <= 103 that runs the half-precision prefilter (us for the forward pass, fp32-accumulate sweep / filter): 1024 rows, d 16, k 45:
 // 165 / 113; d 32, k 80: 171 / 139; 10 000 rows, d 16, k 45: 348 / 218; smaller calls were not measured.
 constexpr int64_t kF16MinRowsLong = 1024;
 // score_select_exact.cu: CUDA-core scores + running top-k, any supported (d, k), fp32 or bf16 storage

@@ -723,8 +723,7 @@ int score_select_f16_list_in_outputs(int32_t k) {
 bool score_select_f16_in_outputs_supported(int64_t N, int32_t H, int32_t d, int32_t k, int mode) {
     if (k < 4 || N > (1 << 19) || (d != 16 && d != 32 && d != 64)) return false;
     if (k > 32) return mode != KMIP_BF16_TC_PRUNED && d <= 32 && score_select_f16_list_in_outputs(k) <= kF16ListMost && N * H >= kF16MinRowsLong;
-    if (mode == KMIP_FP32_EXACT) return N * H >= kF16MinRowsFp32;
-    return mode == KMIP_BF16_TC && d == 64 && N * H >= kF16MinRowsWide;
+    return mode == KMIP_FP32_EXACT || (mode == KMIP_BF16_TC && d == 64);  // the smallest calls are the small-graph kernel's
 }
 
 // Query tiles per work item.  A round (one key tile against all query tiles of a CTA) takes about as long with one

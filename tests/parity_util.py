@@ -35,10 +35,13 @@ def to_device(w):
     return t(w.Q), t(w.K), t(w.V), t(w.dOut), offs
 
 
-def run_forward(w, dev=None, fp32_path=0):
+def run_forward(w, dev=None, fp32_path=0, route=0):
+    """The forward pass; fp32_path and route (kb.ROUTE_*) pin the kernels that run, and the route is checked."""
     Q, K, V, dO, offs = dev or to_device(w)
-    fb = kb.forward(Q, K, V, offs, w.k, w.mode, fp32_path=fp32_path)
+    fb = kb.forward(Q, K, V, offs, w.k, w.mode, fp32_path=fp32_path, route=route)
     torch.cuda.synchronize()
+    expected = route or {1: kb.ROUTE_ROWS, 2: kb.ROUTE_TILED}.get(fp32_path, 0)
+    assert not expected or kb.kmip_test_route(fb.workspace) == expected
     return fb
 
 

@@ -59,7 +59,7 @@ def test_fp16_scores_stay_inside_the_error_bound(d, spread):
 
 def _check(w, min_identical=0.98):
     dev = pu.to_device(w)
-    fb = pu.run_forward(w, dev)
+    fb = pu.run_forward(w, dev, route=kb.ROUTE_FILTER)
     st = pu.check_forward(w, fb)
     st["redo"] = kb.kmip_attn_sweep_counters(fb.workspace)[4]
     if w.backward:
@@ -96,7 +96,7 @@ def test_extreme_magnitudes(scale_q, scale_k):
     w.K[:] = wl.round_to_bf16(w.K * np.float32(scale_k))
     w.K[:, 1] = wl.round_to_bf16(w.K[:, 1] * np.float32(64.0))       # heads on different scales
     dev = pu.to_device(w)
-    fb = pu.run_forward(w, dev)
+    fb = pu.run_forward(w, dev, route=kb.ROUTE_FILTER)
     # scores of this size are outside the absolute tolerances of check_forward: compare selections directly
     from oracle import kmip_oracle as oracle
     ref = oracle.forward(w.Q, w.K, w.V, w.graph_offsets, w.k)
@@ -135,7 +135,8 @@ def test_few_undecidable_rows(n_tied, k):
 
 
 @pytest.mark.parametrize("sizes,H,d,k", [([1536], 1, 16, 4), ([1537, 3, 0, 700], 1, 32, 5), ([2500], 2, 16, 12), ([127, 129, 2000], 2, 64, 9),
-                                         ([5000], 1, 64, 32), ([3000], 1, 32, 17), ([9001], 1, 32, 31), ([40, 1, 700] * 3, 1, 16, 8)])
+                                         ([5000], 1, 64, 32), ([3000], 1, 32, 17), ([9001], 1, 32, 31), ([40, 1, 700] * 3, 1, 16, 8),
+                                         ([7000, 0, 130, 4000], 1, 16, 4), ([300, 2500, 17] * 2, 2, 64, 5)])
 def test_fp32_through_the_filter_is_the_same_bit_for_bit(sizes, H, d, k):
     """fp32 storage, values that fp16 cannot hold exactly: the filter path (operand copies and lists in the output arrays)
     against the one-warp-per-row kernel, which scores every key in fp32 - the same keys in the same order and the same
@@ -145,7 +146,8 @@ def test_fp32_through_the_filter_is_the_same_bit_for_bit(sizes, H, d, k):
     Q, K, V = (torch.randn(N, H, d, generator=g).cuda() for _ in range(3))
     Q[N // 2] *= 1e-3
     offs = torch.tensor(np.concatenate([[0], np.cumsum(sizes)]), dtype=torch.int32, device="cuda")
-    a = kb.forward(Q, K, V, offs, k, kb.KMIP_FP32_EXACT)
+    a = kb.forward(Q, K, V, offs, k, kb.KMIP_FP32_EXACT, route=kb.ROUTE_FILTER)
+    assert kb.kmip_test_route(a.workspace) == kb.ROUTE_FILTER
     b = kb.forward(Q, K, V, offs, k, kb.KMIP_FP32_EXACT, fp32_path=1)
     assert torch.equal(a.topk_idx, b.topk_idx) and torch.equal(a.topk_score, b.topk_score) and torch.equal(a.out, b.out)
 
@@ -194,6 +196,7 @@ def test_long_lists_through_the_filter(sizes, H, d, k, mode):
             w.K[::2] = w.K[1]
         Q, K, V, _, offs = pu.to_device(w)
         a = kb.forward(Q, K, V, offs, k, w.mode)
+        assert kb.kmip_test_route(a.workspace) == kb.ROUTE_FILTER or (tied and w.N >= 33000)   # there all are swept again
         b = kb.forward(Q.float(), K.float(), V.float(), offs, k, kb.KMIP_FP32_EXACT, fp32_path=1)
         assert torch.equal(a.topk_idx, b.topk_idx) and torch.equal(a.topk_score, b.topk_score)
 

@@ -12,9 +12,15 @@ if torch.cuda.is_available():
     from tests import parity_util as pu
 
 
-def _fwd_bwd(w, rows=None, backward=True):
+# which kernels a call runs (kmip_test.h): 0 = the library's choice, the small-graph kernel, the prefilter, the fp32-accumulate sweep
+SMALL, FILTER, TENSOR_CORE = 1, 2, 3
+MODE_AND_ROUTE = [(wl.MODE_BF16_TC, SMALL), (wl.MODE_BF16_TC, FILTER), (wl.MODE_BF16_TC, TENSOR_CORE), (wl.MODE_FP32_EXACT, SMALL),
+                  (wl.MODE_FP32_EXACT, FILTER), (wl.MODE_FP32_EXACT, 0)]
+
+
+def _fwd_bwd(w, rows=None, backward=True, fp32_path=0, route=0):
     dev = pu.to_device(w)
-    fb = pu.run_forward(w, dev)
+    fb = pu.run_forward(w, dev, fp32_path=fp32_path, route=route)
     st = pu.check_forward(w, fb, rows)
     if backward:
         bb = pu.run_backward(w, fb, dev)
@@ -86,31 +92,32 @@ def test_small_hub_batch():
 
 
 # ------------------------------------------------------------------ edge cases
-@pytest.mark.parametrize("mode", [wl.MODE_BF16_TC, wl.MODE_FP32_EXACT])
-def test_ragged_batch_with_tiny_and_empty_graphs(mode):
+@pytest.mark.parametrize("mode,route", MODE_AND_ROUTE)
+def test_ragged_batch_with_tiny_and_empty_graphs(mode, route):
     sizes = [1, 0, 3, 129, 0, 7, 256, 2, 385, 16, 31, 33]
     w = wl.iid_workload("s", 77, sizes, 2, 32, 16, mode)
-    st = _fwd_bwd(w)
+    st = _fwd_bwd(w, route=route)
     assert st["rows"] == sum(sizes)
 
 
-def test_item_and_ring_boundaries():
+@pytest.mark.parametrize("route", [FILTER, TENSOR_CORE])
+def test_item_and_ring_boundaries(route):
     """Graphs around the 512-row and 384-row work-item sizes of the sweeps: one to four active query
     tiles, a short last key tile, and enough key tiles per item for the accumulator buffers and their
     barrier phases to wrap several times."""
     sizes = [383, 384, 385, 511, 512, 513, 769, 1025, 1153, 2000, 127, 128, 129]
     for d, k in ((32, 32), (16, 16)):
         w = wl.iid_workload("s", 90 + d, sizes, 2, d, k, wl.MODE_BF16_TC, input_scale=1.0 / np.sqrt(d))
-        st = _fwd_bwd(w)
+        st = _fwd_bwd(w, route=route)
         assert st["rows"] == sum(sizes)
 
 
-@pytest.mark.parametrize("mode", [wl.MODE_BF16_TC, wl.MODE_FP32_EXACT])
-def test_padded_head_width_of_the_paper_sweep(mode):
+@pytest.mark.parametrize("mode,route", MODE_AND_ROUTE)
+def test_padded_head_width_of_the_paper_sweep(mode, route):
     """d_K = 10 stored zero-padded to 16 columns, k = 10, one head (the shape of the paper's size
     sweep): same parity bar as every other shape, and the padded output and gradient columns stay zero."""
     w = wl.padded_workload("s", 91, 3000, 1, 10, 16, 10, mode)
-    _fwd_bwd(w)
+    _fwd_bwd(w, route=route)
 
 
 def test_single_node():
@@ -123,25 +130,24 @@ def test_single_node():
     pu.check_forward(w, fb)
 
 
-@pytest.mark.parametrize("mode", [wl.MODE_BF16_TC, wl.MODE_FP32_EXACT])
-def test_identical_keys_tie_break_by_index(mode):
+@pytest.mark.parametrize("mode,route", MODE_AND_ROUTE)
+def test_identical_keys_tie_break_by_index(mode, route):
     w = wl.iid_workload("s", 79, [200, 90], 2, 32, 8, mode)
     w.K[:] = w.K[5]
     dev = pu.to_device(w)
-    fb = pu.run_forward(w, dev)
+    fb = pu.run_forward(w, dev, route=route)
     idx = fb.topk_idx.cpu().numpy()
     assert np.all(idx[:200] == np.arange(8)) and np.all(idx[200:] == 200 + np.arange(8))
     pu.check_forward(w, fb)
 
 
-# fp32 problems with at least 48 blocks of 128 rows x heads run the tiled CUDA-core sweep and the
-# fp32 rescoring kernel instead of the one-warp-per-row kernel the small fp32 cases above exercise
+# fp32 problems with at least 48 blocks of 128 rows x heads have the tiled CUDA-core sweep and the
+# fp32 rescoring kernel behind the prefilter; here the two run by themselves
 @pytest.mark.parametrize("d,k", [(16, 10), (32, 32), (64, 17)])
 def test_fp32_tiled_sweep(d, k):
     sizes = [3000, 129, 5000, 1, 2000, 383, 0, 64]
     w = wl.iid_workload("s", 3000 + d, sizes, 4, d, k, wl.MODE_FP32_EXACT, input_scale=1.0 / np.sqrt(d))
-    assert (w.N // 128) * w.H >= 48
-    st = _fwd_bwd(w)
+    st = _fwd_bwd(w, fp32_path=2)
     assert st["identical_rows"] > 0.999   # all but rows where two neighbouring scores tie within fp32 rounding
     # of ~42 000 (row, head) pairs the rule could excuse up to 714 (oracle neighbours closer than the fp32
     # error bound); the pairs that really differ, and are let through, stay a handful
@@ -153,9 +159,8 @@ def test_fp32_tiled_sweep_tie_break_by_index():
     key indices of the graph, and equal group maxima must be ordered by their first key."""
     w = wl.iid_workload("s", 3100, [6000, 4500], 4, 16, 12, wl.MODE_FP32_EXACT)
     w.K[:] = w.K[7]
-    assert (w.N // 128) * w.H >= 48
     dev = pu.to_device(w)
-    fb = pu.run_forward(w, dev)
+    fb = pu.run_forward(w, dev, fp32_path=2)
     idx = fb.topk_idx.cpu().numpy()
     assert np.all(idx[:6000] == np.arange(12)) and np.all(idx[6000:] == 6000 + np.arange(12))
     pu.check_forward(w, fb)
@@ -179,11 +184,12 @@ def test_fp32_sweeps_agree_bit_for_bit(d, k):
     pu.check_forward(w, fb)
 
 
-def test_null_offsets_means_one_graph():
+@pytest.mark.parametrize("route", [SMALL, FILTER, TENSOR_CORE])
+def test_null_offsets_means_one_graph(route):
     w = wl.iid_workload("s", 80, [600], 2, 32, 8, wl.MODE_BF16_TC)
     Q, K, V, dO, offs = pu.to_device(w)
-    a = kb.forward(Q, K, V, offs, w.k, w.mode)
-    b = kb.forward(Q, K, V, None, w.k, w.mode)
+    a = kb.forward(Q, K, V, offs, w.k, w.mode, route=route)
+    b = kb.forward(Q, K, V, None, w.k, w.mode, route=route)
     torch.cuda.synchronize()
     assert torch.equal(a.topk_idx, b.topk_idx) and torch.equal(a.out, b.out)
 
@@ -223,7 +229,8 @@ def test_bounded_wait_runs_out_and_is_reported():
     pu.check_forward(w, pu.run_forward(w, dev))
 
 
-def test_forward_and_backward_replay_from_a_cuda_graph():
+@pytest.mark.parametrize("route", [0, SMALL, FILTER, TENSOR_CORE])
+def test_forward_and_backward_replay_from_a_cuda_graph(route):
     """Both calls only enqueue work on the caller's stream (no allocation, no synchronisation), so a
     forward + backward pair can be captured once and replayed on new input values."""
     w = wl.make_config(2)
@@ -233,7 +240,11 @@ def test_forward_and_backward_replay_from_a_cuda_graph():
     bb = kb.BackwardBuffers(w.N, G, w.H, w.d, w.k, w.mode)
 
     def step():
-        assert kb.kmip_attn_forward(Q, K, V, offs, w.k, w.mode, fb.out, fb.topk_idx, fb.topk_score, fb.workspace) == kb.KMIP_OK
+        if route:
+            assert kb.kmip_test_attn_forward(Q, K, V, offs, w.k, w.mode, fb.out, fb.topk_idx, fb.topk_score, fb.workspace,
+                                             route=route) == kb.KMIP_OK
+        else:
+            assert kb.kmip_attn_forward(Q, K, V, offs, w.k, w.mode, fb.out, fb.topk_idx, fb.topk_score, fb.workspace) == kb.KMIP_OK
         assert kb.kmip_attn_backward(Q, K, V, offs, w.k, w.mode, fb.out, dO, fb.topk_idx, fb.topk_score, bb.dQ, bb.dK,
                                      bb.dV, bb.workspace) == kb.KMIP_OK
 
@@ -280,8 +291,9 @@ def test_workspace_is_linear_in_n():
     assert kb.kmip_attn_workspace_bytes(1_000_000, 1, 4, 32, 16, kb.KMIP_BF16_TC, kb.PASS_FORWARD) < 2 * rows * 32 * 2 + rows * (24 * 6 + 4) + 8 * 1_000_000
 
 
+@pytest.mark.parametrize("route", [SMALL, FILTER, TENSOR_CORE])
 @pytest.mark.parametrize("d", [64, 32])
-def test_kth_score_near_zero_keeps_k_keys(d):
+def test_kth_score_near_zero_keeps_k_keys(d, route):
     """Rows whose k-th best score is a tiny remainder of large cancelling terms: the tensor-core score and
     the fp32 rescoring of the same key differ by far more than any margin RELATIVE to that score, and the
     key that defines the k-th place must still come back (Algorithm 1 line 3 returns k keys whenever the
@@ -299,7 +311,7 @@ def test_kth_score_near_zero_keeps_k_keys(d):
         K[near] = 4.0 * (u * alt)[None, None, :] + 2.0 ** -13 * rng.standard_normal((24, H, d)).astype(np.float32)
     w.K[:] = wl.round_to_bf16(K)
     dev = pu.to_device(w)
-    fb = pu.run_forward(w, dev)
+    fb = pu.run_forward(w, dev, route=route)
     idx = fb.topk_idx.cpu().numpy()
     assert np.all(idx >= 0), f"{int((idx < 0).sum())} padded slots although every graph has more than k nodes"
     pu.check_forward(w, fb)
