@@ -28,9 +28,13 @@ from paper_2604_03815_b200 import workloads as wl  # noqa: E402
 METRIC = "k-MIP fwd+bwd query-key scores/sec at N=500k"
 UNIT = "scores/s"
 FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustained": 1400.0}
-FWD_LAUNCHES = 5            # regroup keys, plan, score+select sweep, rescoring, softmax+gather-V
-F16_FWD_LAUNCHES = 7        # plan, norm maxima, operand conversion, prefilter sweep, rescoring, redo pass, softmax+gather-V
-REORDER_LAUNCHES = 3        # tensor-core mode from 32768 nodes on: locality codes, row order, permuted copy of Q
+# kernels of a forward call by the route the library reports (kmip_test_route)
+FWD_LAUNCHES = {1: 2,       # plan, the whole forward pass of small graphs
+                2: 7,       # plan, norm maxima, operand conversion, prefilter sweep, rescoring, exact pass, softmax+gather-V
+                3: 5,       # plan, keys by head, score+select sweep, rescoring, softmax+gather-V
+                4: 4,       # plan, sweep, rescoring, softmax+gather-V
+                5: 3}       # plan, sweep, softmax+gather-V
+REORDER_LAUNCHES = 2        # bf16 sweeps from 32768 nodes on: locality codes, row order; the fp32-accumulate one also copies Q
 BWD_LAUNCHES = 9            # rows, partition (count, 3 scan kernels, scatter), bucket sort (writes the list offsets), 2 segment kernels
 
 
@@ -153,19 +157,11 @@ def run_reference(args, w):
     }
 
 
-def fwd_launches(w):
-    """Kernels one forward call of the library launches for this workload."""
-    small_n = w.N // w.G * (w.d + 16)
-    if w.k <= 32 and w.d <= 64 and (small_n <= 15000 or w.N * w.H * small_n <= 300000000):
-        return 2                          # plan, the whole forward pass of small graphs
-    if w.mode != wl.MODE_BF16_TC:
-        return F16_FWD_LAUNCHES if 4 <= w.k <= 32 and w.d <= 64 and w.N <= 1 << 19 else 4
-    tc = w.k <= 64 or (w.k <= 128 and w.d <= 64)
-    if not tc:
-        return 3
-    if w.d <= 32 and w.k <= 32:      # half-precision prefilter; the permuted copy of Q is made by its conversion kernel
-        return F16_FWD_LAUNCHES + (REORDER_LAUNCHES - 1 if w.N >= 32768 else 0)
-    return FWD_LAUNCHES + (REORDER_LAUNCHES if w.N >= 32768 else 0)
+def fwd_launches(w, route):
+    """Kernels one forward call launches for this workload on the route the library took (launches that a choice made on
+    the device leaves without work are not counted)."""
+    reorder = w.mode == wl.MODE_BF16_TC and w.N >= 32768 and route in (2, 3)
+    return FWD_LAUNCHES[route] + (REORDER_LAUNCHES + (route == 3) if reorder else 0)
 
 
 def sweep_kernel_name(w):
@@ -458,7 +454,7 @@ def run_ours(args, w):
         "pruned": pruned,
         "redo_rows": kb.kmip_attn_sweep_counters(fb.workspace)[4],
         "other_configs": other,
-        "gpu_launches": (fwd_launches(w) + (BWD_LAUNCHES if w.backward else 0)) * args.steps,
+        "gpu_launches": (fwd_launches(w, kb.kmip_test_route(fb.workspace)) + (BWD_LAUNCHES if w.backward else 0)) * args.steps,
         "clocks": clocks,
     }
     if world == 1 and not args.no_cpu_baseline:
