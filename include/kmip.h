@@ -57,7 +57,8 @@ typedef enum {
        accumulation on the tcgen05 tensor cores; softmax, sums and gradients accumulate in fp32. */
     KMIP_BF16_TC = 0,
     /* All of them hold fp32.  Scores are fp32 fused multiply-adds in index order c = 0..d-1 (a half-precision filter with
-       a proven error bound may decide which keys need one). */
+       a proven error bound may decide which keys need one: N <= 2^19 and 4 <= k <= 32 with d <= 64, or k <= 103 with
+       d <= 32; other calls score every key, about ten times as long). */
     KMIP_FP32_EXACT = 1,
     /* KMIP_BF16_TC with an exact pruning of the search (the quadratic search is the first limitation the
        paper names, Sec. 6): in graphs of 8192 nodes or more the keys are swept in an order that puts heavy
@@ -100,8 +101,9 @@ int kmip_attn_workspace_bytes(int64_t N, int32_t G, int32_t H, int32_t d, int32_
  * KMIP_OK, undefined otherwise): out, topk_idx, topk_score.  All three serve as scratch before they are
  * written, so they must not overlap the inputs or each other, with one exception: `out` may overlap Q or K
  * (an in-place inference call; some sizes then take a slower sweep).
- * In KMIP_BF16_TC mode the selection uses tensor-core scores, so a key whose exact score
- * differs from the k-th best by less than the fp32 accumulation error may swap with it.
+ * In KMIP_BF16_TC mode the selection may use tensor-core scores (among others d = 128, k > 103, the pruned mode,
+ * large calls whose keys tie by the thousands), so a key whose exact score differs from the k-th best by less than the fp32 accumulation
+ * error may swap with it.
  */
 int kmip_attn_forward(const void *Q, const void *K, const void *V,
                       const int32_t *graph_offsets, int32_t G, int64_t N,
@@ -224,10 +226,10 @@ int kmip_layer_backward(const kmip_layer_tensors_t *t, const int32_t *graph_offs
 
 /*
  * Size in bytes of the scratch array that is built into the library for
- * kmip_attn_forward_static_scratch (8 MiB; each GPU that loads the library holds it until the
+ * kmip_attn_forward_static_scratch (8 MiB, and 4 KiB for the prefilter's statistics; each GPU that loads the library holds it until the
  * process exits).
  */
-#define KMIP_STATIC_SCRATCH_BYTES ((size_t)8 << 20)
+#define KMIP_STATIC_SCRATCH_BYTES (((size_t)8 << 20) + 4096)
 
 /*
  * The forward pass of kmip_attn_forward for callers that cannot provide a workspace because they
@@ -273,8 +275,8 @@ int kmip_last_status(const void *workspace, void *stream, int *device_status);
  *   [0..3]  KMIP_BF16_TC_PRUNED: key tiles of all work items, key tiles loaded (one end marker per work
  *           item included), (key tile, query tile) pairs, pairs scored, summed over the sweep's CTAs;
  *   [4]     where the half-precision prefilter ran (KMIP_BF16_TC and KMIP_FP32_EXACT, d <= 64 with k <= 32 and d <= 32
- *           with k <= 103, not the smallest calls): (query, head) pairs that it could not decide and the exact
- *           kernel recomputed from all keys;
+ *           with k <= 103, not the smallest calls): (query, head) pairs that it could not decide and that were
+ *           recomputed from all keys;
  *   [5..7]  zero.
  * Counters of a path that did not run are zero.  Returns KMIP_ERR_CUDA if the synchronisation or the
  * copy fails.

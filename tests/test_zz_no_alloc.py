@@ -26,6 +26,20 @@ def test_too_large_problem_is_refused_on_the_host():
     assert rc == kb.KMIP_ERR_UNSUPPORTED
 
 
+@pytest.mark.parametrize("H,d,k", [(2, 64, 16), (4, 64, 8), (3, 64, 31), (8, 32, 64), (16, 16, 100)])
+def test_statistics_of_the_prefilter_do_not_shrink_the_limit(H, d, k):
+    """Where the prefilter keeps its lists in the output arrays it needs 16 bytes per head of scratch beside the copy of K;
+    a problem whose other scratch fills 8 MiB to the last byte still fits the built-in array."""
+    from paper_2604_03815_b200 import build
+    build.build()
+    from paper_2604_03815_b200 import binding as kb
+    up = lambda n: (n + 255) // 256 * 256
+    fits = [N for N in range(1000, 32768) if 256 + up(20 * (N // 128 + 2)) + up(2 * N * H * d) <= 8 << 20]
+    N = fits[-1]
+    assert N == 32767 or kb.kmip_attn_workspace_bytes(N, 1, H, d, k, kb.KMIP_BF16_TC, kb.PASS_FORWARD) > (8 << 20) - 512
+    assert kb.kmip_attn_workspace_bytes(N, 1, H, d, k, kb.KMIP_BF16_TC, kb.PASS_FORWARD) <= (8 << 20) + 4096
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("mode", [wl.MODE_BF16_TC, wl.MODE_FP32_EXACT])
 def test_static_scratch_forward_matches_regular_forward_twice(mode):
