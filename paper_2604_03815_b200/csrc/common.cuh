@@ -399,7 +399,7 @@ inline int grid_blocks(const FwdArgs& a, long long want, int per_sm) {
 int score_select_tc_rows_per_item(int32_t d, int32_t k);
 cudaError_t launch_score_select_tc(const FwdArgs& a, const FwdWorkspace& w);
 cudaError_t launch_score_dump_tc(const FwdArgs& a, const FwdWorkspace& w, float* dump);
-// Half-precision prefilter (k <= 32; bf16 storage: head widths 16, 32, 64, fp32 storage: the same on large problems):
+// Half-precision prefilter (bf16 and fp32 storage; head widths 16, 32, 64 with k <= 32, 16 and 32 with k <= 103):
 // f16_convert.cu (norm maxima, scaled fp16 copies of K and Q), score_select_f16.cu (sweep),
 // refine_f16.cu (exact rescoring, redo list), score_select_exact.cu (the listed rows again, from all keys)
 

@@ -52,7 +52,7 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
     return ok != 0;
 }
 
-// Bounded wait: waits for the barrier phase in hardware-suspended slices of up to 20 us; gives up
+// Bounded wait: polls the barrier phase (each poll may suspend in hardware for a while); gives up
 // when `abort_flag` (shared memory) is set by another thread or after roughly `limit_cycles` SM
 // clocks (about 4 s by default), in which case it sets the flag itself and returns false.
 // Callers leave their loops on false; nothing waits forever.

@@ -687,7 +687,7 @@ cudaError_t launch_cfg(const FwdArgs& a, const FwdWorkspace& w, float* dump) {
 // selects too often, and shared memory is shared by the tiles' rows.  n: keys per graph; the longer the graph, the
 // rarer the selections.  Measured for lists of 48, us with four / three tiles: 20k nodes, H 4, d 16 376 / 317, d 32
 // 475 / 331; 100k nodes, H 1, d 16 1235 / 1035; H 4, d 32 4506 / 4191; 300k nodes, H 2, d 32 14134 / 14832; H 1, d 16
-// 5997 / 6704.
+// 5997 / 6704.  kLargeGraph lies between 100k and 300k; nothing in between was measured.
 int most_query_tiles(int64_t n, int32_t d, int list) {
     if (d == 64 || (list > 24 && n < kLargeGraph)) return list > (d == 16 ? 80 : 64) ? 2 : 3;
     return list <= kF16List32 ? 4 : list <= (d == 16 ? 80 : 64) ? 3 : 2;
@@ -729,7 +729,7 @@ bool score_select_f16_in_outputs_supported(int64_t N, int32_t H, int32_t d, int3
 // Query tiles per work item.  A round (one key tile against all query tiles of a CTA) takes about as long with one
 // query tile as with three, and little less than with four (measured, ns, one work item per CTA, each with the kernel of
 // its size, 1 / 2 / 3 / 4 tiles: d 16, k 8: 682 669 671 777; d 32, k 16: 716 689 743 858; d 64, k 16: 716 709 786 - the
-// chain of one pipeline, not its work, is what takes the time), so fewer tiles per item pay only where they fill idle
+// chain of one pipeline, not its work, is what takes the time; other list lengths are taken to be alike), so fewer tiles per item pay only where they fill idle
 // SMs: the smallest number of rounds, weighted with their length, wins.  Graphs of one size are assumed.
 int score_select_f16_item_tiles(int64_t N, int32_t G, int32_t H, int32_t d, int list) {
     const double kRound[5] = {0.0, 0.87, 0.86, d == 64 ? 0.97 : 0.87, 1.0};
