@@ -107,8 +107,8 @@ constexpr int64_t kDirectRows = 131072;
 // The workspace of a forward call and, for the half-precision sweep, its work items.
 FwdWorkspace plan_forward(int64_t N, int32_t G, int32_t H, int32_t d, int32_t k, int mode, int small) {
     FwdWorkspace w = plan_fwd_workspace(N, G, H, d, k, mode);
-    w.direct = small == kSmallDecide && N * H < kDirectRows;
-    if (w.direct) w.f16 = w.in_outputs = w.prune = w.reorder = false;
+    w.direct = small == kSmallDecide && N * H < kDirectRows && !w.prune;
+    if (w.direct) w.f16 = w.in_outputs = w.reorder = false;
     // graphs of one size are assumed; where the small-graph kernel takes those, the sweep runs if some are large
     if (w.f16) w.item_tiles = score_select_f16_item_tiles(N, small == kSmallDecide ? 1 : G, H, d, w.list);
     return w;
@@ -122,6 +122,8 @@ int rows_per_item(const FwdWorkspace& w, int32_t d, int32_t k) {
 // pass takes any number.  That pass reads a graph's keys once per row: measured (ms, all rows undecided / the sweep) fp32
 // n = 60 000, d 16 28 / 4.9, n = 30 000, d 64 54 / 5.2; bf16 n = 100 000, d 64 300 / 2.4, n = 60 000, d 32, k 45 30 / 1.6.
 // Below 48 blocks of 128 rows the sweeps gain little, and three launches that find nothing to do (4 us) weigh.
+// The limit is where the exact pass takes a third to two thirds of the sweep's time: 0.48 and 1.8 us a row in fp32 above, 3.0
+// at d = 64 and 0.5 at d = 32 in bf16.
 int second_sweep(int64_t N, int32_t H, int32_t d, int32_t k, int mode, int* limit) {
     if ((N / 128) * H < 48) return 0;
     const bool fp32 = mode == KMIP_FP32_EXACT;

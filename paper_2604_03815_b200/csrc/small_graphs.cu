@@ -231,8 +231,10 @@ cudaError_t launch_d(const FwdArgs& a) {
     const int rows_per_warp = (int)std::max<long long>(1, std::min<long long>(8, rows / ((long long)sm_count() * 4 * kWarps)));
     const size_t smem = (size_t)kChunk * row_stride<T, D>() + ((size_t)kWarps * rows_per_warp * 32 + (size_t)kWarps * kPend) * sizeof(cand_t);
     auto kern = small_forward_kernel<T, D>;
-    cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (err != cudaSuccess) return err;
+    if (smem > 48 * 1024) {  // what a kernel may have unasked
+        cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (err != cudaSuccess) return err;
+    }
     const dim3 grid((unsigned)((a.N + kWarps * rows_per_warp - 1) / (kWarps * rows_per_warp)), (unsigned)std::min(a.H, 65535));
     return launch_next(a, kern, grid, kWarps * 32, smem, static_cast<const T*>(a.Q), static_cast<const T*>(a.K), static_cast<const T*>(a.V),
                                                 a.graph_offsets, a.G, (int)a.N, a.H, a.k, rows_per_warp, 1.0f / sqrtf((float)a.d), a.drop_p,
