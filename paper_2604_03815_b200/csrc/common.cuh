@@ -255,8 +255,9 @@ __device__ __forceinline__ bool kmip_check(bool cond, StatusBlock* sb, int code)
 // The tensor-core sweeps may record a problem while blocks of theirs still start, so they don't ask for the second: they find
 // no work items when the plan failed.  The half-precision one asks for neither - its loop is sensitive to what the compiler
 // makes of a line up here (100k nodes, d 16, k 16: 924 us without, 960 with) - and finds no work items in both cases.
+__device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ bool small_route(const StatusBlock* sb) {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    wait_for_previous();
     return sb->route == kRouteSmall;
 }
 __device__ __forceinline__ bool sweep_off(const StatusBlock* sb) { return small_route(sb) || sb->status != KMIP_OK; }
@@ -346,7 +347,7 @@ struct BwdArgs {
     unsigned long long seed = 0ull;
 };
 
-// Launches a kernel of a sweep's route that begins with sweep_off or small_route: it may start while the one before it ends.
+// Launches a kernel that begins with sweep_off, small_route or wait_for_previous: it may start while the one before it ends.
 // One that finds nothing to do then costs 1.3 us instead of 2.5.
 template <typename... P, typename... A>
 inline cudaError_t launch_next(const FwdArgs& a, void (*kern)(P...), dim3 grid, int threads, size_t smem, A&&... args) {

@@ -73,6 +73,7 @@ __global__ void __launch_bounds__(kPlanThreads)
 plan_kernel(const int32_t* __restrict__ offs, int G, int N, int rows_per_item, int max_items,
             WorkItem* __restrict__ items, StatusBlock* sb, float* __restrict__ clear, int n_clear, int small_use, int route,
             int H, int d, bool direct) {
+    wait_for_previous();
     __shared__ unsigned long long s_squares[32];
     __shared__ int s_bad;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
@@ -180,11 +181,9 @@ cudaError_t launch_resweep_plan(const FwdArgs& a, const FwdWorkspace& w, int row
 }
 
 cudaError_t launch_plan(const FwdArgs& a, const FwdWorkspace& w, int rows_per_item, int small_use, int route) {
-    plan_kernel<<<1, kPlanThreads, 0, a.stream>>>(
-        a.graph_offsets, a.G, (int)a.N, rows_per_item, w.max_items,
-        reinterpret_cast<WorkItem*>(a.ws + w.items_off), reinterpret_cast<StatusBlock*>(a.ws),
-        reinterpret_cast<float*>(a.ws + w.f16stat_off), w.f16 ? 4 * a.H : 0, small_use, route, a.H, a.d, w.direct);
-    return cudaGetLastError();
+    return launch_next(a, plan_kernel, dim3(1), kPlanThreads, 0, a.graph_offsets, a.G, (int)a.N, rows_per_item, w.max_items,
+                       reinterpret_cast<WorkItem*>(a.ws + w.items_off), reinterpret_cast<StatusBlock*>(a.ws),
+                       reinterpret_cast<float*>(a.ws + w.f16stat_off), w.f16 ? 4 * a.H : 0, small_use, route, a.H, a.d, w.direct);
 }
 
 }  // namespace kmip
