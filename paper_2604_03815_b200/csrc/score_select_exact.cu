@@ -232,20 +232,18 @@ score_select_redo_kernel(const T* __restrict__ Q, const T* __restrict__ K, const
 template <typename T, int D>
 cudaError_t launch_d(const FwdArgs& a) {
     const long long n_rows = (long long)a.N * a.H;
-    const int blocks = (int)std::min<long long>((n_rows + kWarpsPerBlock - 1) / kWarpsPerBlock, (long long)sm_count() * 64);
+    const int blocks = (int)std::min<long long>((n_rows + kWarpsPerBlock - 1) / kWarpsPerBlock, (long long)sm_count() * (a.maybe_small ? 8 : 64));
     const T* Q = static_cast<const T*>(a.Q);
     const T* K = static_cast<const T*>(a.K);
-    const dim3 grid(blocks), block(kWarpsPerBlock * 32);
     // pending room CAP-k must hold one 32-key step beyond the compaction trigger
 #define KMIP_LAUNCH_EXACT(E_) \
-    score_select_exact_kernel<T, D, E_><<<grid, block, 0, a.stream>>>( \
+    return launch_next(a, score_select_exact_kernel<T, D, E_>, dim3(blocks), kWarpsPerBlock * 32, 0, \
         Q, K, a.graph_offsets, a.G, (int)a.N, a.H, a.k, a.topk_idx, a.topk_score, \
         reinterpret_cast<const StatusBlock*>(a.ws))
     if (a.k <= 16) KMIP_LAUNCH_EXACT(2);
     else if (a.k <= 96) KMIP_LAUNCH_EXACT(4);
     else KMIP_LAUNCH_EXACT(8);
 #undef KMIP_LAUNCH_EXACT
-    return cudaGetLastError();
 }
 
 template <typename T>

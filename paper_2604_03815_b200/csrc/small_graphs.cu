@@ -2,7 +2,7 @@
 // (query, head) row by one warp, against the graph's keys in shared memory.
 //
 // On graphs of a few hundred nodes the filter of score_select_f16.cu saves nothing: its rescoring alone takes about 900
-// instructions a row, and it needs eight launches.  Here a lane scores kU keys of a 256-key chunk (the same chains of
+// instructions a row, and it needs seven launches.  Here a lane scores kU keys of a 256-key chunk (the same chains of
 // fused multiply-adds in index order as every other kernel); the k-th largest of the 32 lane maxima is a lower bound of
 // the row's k-th best score (k <= 32), so only the few scores that reach it are sorted, as (score, key) words.  Graphs of
 // any size work, 256 keys at a time against the running list; small_graphs_preferred() has the line where the filter
@@ -259,7 +259,7 @@ cudaError_t launch_t(const FwdArgs& a) {
 //                            but n = 500, d 16, one head: 125 / 119
 //   few rows                 one graph of 500: 33 / 61, 1024: 40 / 68, 2000: 60 / 83, 4000: 152 / 99; 2000 x 4 heads: 112 / 93
 // What it takes grows with the sum of the squared graph sizes, so n is that sum / N (one graph of 20 000 nodes among 255 of
-// 60, 4 heads, d 16, has a mean size of 138: 5755 us here, 1100 behind the filter).  The host knows the mean alone, which is
+// 60, 4 heads, d 16, has a mean size of 138: 5755 us here, 915 behind the filter).  The host knows the mean alone, which is
 // never above n: where that decides nothing, the plan kernel applies the rule and both routes are launched.  Smaller batches
 // then have the fp32-accumulate or the tiled sweep behind them (plan_forward, api.cu), which at d = 16 meet this kernel on
 // the same line (100 graphs of 460: 120 / 124 us bf16, 131 / 153 fp32), wider heads later: 100 of 300, d 32 182 / 306 bf16
