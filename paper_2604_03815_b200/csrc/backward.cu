@@ -21,7 +21,7 @@ constexpr int kLongSeg = 512;
 
 // ------------------------------------------------------------------------------------------ rows
 template <typename T, int D, int E, int W>
-__global__ void __launch_bounds__(kWarpsPerBlock * 32)
+__global__ void __launch_bounds__(kWarpsPerBlock * 32, W == 32 ? 0 : 6)
 bwd_rows_kernel(const T* __restrict__ K, const T* __restrict__ V, const T* __restrict__ dOut,
                 const int32_t* __restrict__ topk_idx, const float* __restrict__ topk_score,
                 int N, int H, int k, float scale, float drop_p, unsigned long long seed,

@@ -12,7 +12,7 @@ namespace {
 constexpr int kWarpsPerBlock = 8;
 
 template <typename T, int D, int E, int W>
-__global__ void __launch_bounds__(kWarpsPerBlock * 32)
+__global__ void __launch_bounds__(kWarpsPerBlock * 32, W == 32 ? 0 : 8)
 softmax_gather_kernel(const T* __restrict__ V, const int32_t* __restrict__ topk_idx,
                       const float* __restrict__ topk_score, int N, int H, int k, float scale,
                       float drop_p, unsigned long long seed, T* __restrict__ out,

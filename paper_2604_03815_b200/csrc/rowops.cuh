@@ -16,8 +16,10 @@ constexpr int kMaxEntriesPerLane = 4;  // k <= 128; kernels come with E = 1 (k <
 
 // Lanes per row, W: a whole warp, or half of one for k <= 16, so that a warp does two rows at a time (the two halves run the
 // same instructions and must be converged).  Entry t of a row lives in lane t % W of its W lanes, register t / W.  Measured
-// (us, a warp per row / two rows per warp): softmax_gather 100k nodes H 4 d 32 k 16 119 / 76, 4 x 200k nodes H 8 d 16 k 16
-// 1431 / 847; bwd_rows 236 / 168, 2702 / 1723, 128 graphs of 175, H 4 d 16 k 8 42 / 25.
+// (us, a warp per row / two rows per warp): softmax_gather 100k nodes H 4 d 32 k 16 119 / 83, 4 x 40k nodes H 8 d 16 k 16
+// 295 / 177; bwd_rows 236 / 170, 545 / 333.  The second partial sum of a lane would cost the kernels of two rows a step of
+// occupancy (softmax_gather 40 registers instead of 32, bwd_rows 48 and more instead of 40: 100k nodes H 4 d 32 k 16 94 and
+// 206 us), so their launch bounds hold them to it.
 constexpr int kHalfWarp = 16;
 // Whether a gathered row is as wide as the vector loads of half a warp, or narrower.
 template <typename T, int D> __host__ __device__ constexpr bool half_warp_rows() { return D / Elem<T>::kVec <= kHalfWarp; }
@@ -48,9 +50,9 @@ struct RowWalk {
     }
 };
 
-// Column sums over the W / LPR lane groups of a row's lanes.  Before: lane l holds W partial sums for part l % LPR.  A step
+// Column sums over the W / LPR lane groups of a row's lanes.  Before: lane l holds N partial sums for part l % LPR.  A step
 // exchanges halves, so N + N / 2 + ... values move instead of N per step (the additions are those of a butterfly, bit for
-// bit).  Before: N partial sums a lane.  After: v[0 .. kLeft) of lane l are the full sums of columns col .. col + kLeft of its part (`col` returned), and
+// bit).  After: v[0 .. kLeft) of lane l are the full sums of columns col .. col + kLeft of its part (`col` returned), and
 // the lanes below kWriters hold every column once.
 template <int N, int LPR, int W = 32>
 struct ColumnSums {
@@ -161,38 +163,56 @@ __device__ __forceinline__ void dropout_factors(long long r, int k, int lane, fl
 
 // out_row[0, D) = sum_t w_t * X[j_t, h, :].
 // LPR = D/VEC lanes share one gathered row (one 16-byte load each), W/LPR rows per round.  `lane`: among the row's W lanes.
-template <typename T, int D, int E, int W = 32>
+// The order of the additions is that of 32 lanes whatever W is, so that every kernel gives the same bits: entry t goes to
+// partial sum t % (32 / LPR), and these are added as a tree of neighbours.  With half a warp a lane keeps two neighbours, so
+// the first step of the tree stays in the lane; up to W / LPR entries take one partial sum each, the other half are 0.
+// MIN_K: a k that the caller knows to be reached; rounds below it are not asked for.
+template <typename T, int D, int E, int W = 32, int MIN_K = 1>
 __device__ __forceinline__ void gather_weighted_sum(const T* __restrict__ X, int H, int h, int k, int lane,
                                                     const int (&j)[E], const float (&w)[E], T* __restrict__ out_row, bool live = true) {
     constexpr int VEC = Elem<T>::kVec;
     constexpr int LPR = D / VEC;
     constexpr int EPW = W / LPR;
+    constexpr int SETS = 32 / W;
     static_assert(LPR >= 1 && LPR <= W, "row width");
     const int part = lane % LPR, sub = lane / LPR;
-    float acc[VEC];
+    float acc[SETS][VEC];
 #pragma unroll
-    for (int c = 0; c < VEC; ++c) acc[c] = 0.0f;
+    for (int s = 0; s < SETS; ++s)
 #pragma unroll
-    for (int e = 0; e < E; ++e) {
-        if (e * W < k) {
+        for (int c = 0; c < VEC; ++c) acc[s][c] = 0.0f;
+    auto add = [&](int e, int src, float (&a)[VEC]) {
+        const int jj = __shfl_sync(0xFFFFFFFFu, j[e], src, W);
+        const float ww = __shfl_sync(0xFFFFFFFFu, w[e], src, W);
+        if (jj >= 0) {
+            float v[VEC];
+            Elem<T>::load_vec(X + ((size_t)jj * H + h) * D + part * VEC, v);
 #pragma unroll
-            for (int base = 0; base < W; base += EPW) {
-                if (e * W + base >= k) break;
-                const int src = base + sub;
-                const int jj = __shfl_sync(0xFFFFFFFFu, j[e], src, W);
-                const float ww = __shfl_sync(0xFFFFFFFFu, w[e], src, W);
-                if (jj >= 0) {
-                    float v[VEC];
-                    Elem<T>::load_vec(X + ((size_t)jj * H + h) * D + part * VEC, v);
+            for (int c = 0; c < VEC; ++c) a[c] = fmaf(ww, v[c], a[c]);
+        }
+    };
+    if (SETS == 2 && k <= EPW) {
+        add(0, sub, acc[0]);
+    } else {
 #pragma unroll
-                    for (int c = 0; c < VEC; ++c) acc[c] = fmaf(ww, v[c], acc[c]);
+        for (int e = 0; e < E; ++e) {
+            if (e * W < k) {
+#pragma unroll
+                for (int base = 0; base < W; base += SETS * EPW) {
+                    if (e * W + base >= MIN_K && e * W + base >= k) break;
+#pragma unroll
+                    for (int s = 0; s < SETS; ++s) add(e, base + SETS * sub + s, acc[s]);
                 }
             }
         }
+        if constexpr (SETS == 2) {
+#pragma unroll
+            for (int c = 0; c < VEC; ++c) acc[0][c] += acc[1][c];
+        }
     }
     using Sums = ColumnSums<VEC, LPR, W>;
-    const int col = column_sums<VEC, LPR, W>(acc, lane);
-    if (live && lane < Sums::kWriters) store_columns<Sums::kLeft>(out_row + part * VEC + col, acc);
+    const int col = column_sums<VEC, LPR, W>(acc[0], lane);
+    if (live && lane < Sums::kWriters) store_columns<Sums::kLeft>(out_row + part * VEC + col, acc[0]);
 }
 
 // dots[e] of lane l = g . X[j[e] of lane l, h, :] for the row's entries, with
