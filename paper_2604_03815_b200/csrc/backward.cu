@@ -514,91 +514,101 @@ radix_bucket_kernel(const int4* __restrict__ src, int4* __restrict__ dst, const 
 }
 
 // -------------------------------------------------------------------------------------- segments
-// Accumulate one hit into the lane's part of dV and dK.
-template <typename T, int D>
-__device__ __forceinline__ void accumulate_hit(int4 rec, int h, int H, int part,
-                                               const T* __restrict__ Q, const T* __restrict__ dOut,
-                                               float (&accV)[Elem<T>::kVec], float (&accK)[Elem<T>::kVec]) {
-    constexpr int VEC = Elem<T>::kVec;
-    const float pw = __int_as_float(rec.y), dsw = __int_as_float(rec.z);
-    const size_t off = ((size_t)rec.x * H + h) * D + part * VEC;
-    float gv[VEC], qv[VEC];
-    Elem<T>::load_vec(dOut + off, gv);
-    Elem<T>::load_vec(Q + off, qv);
-#pragma unroll
-    for (int c = 0; c < VEC; ++c) {
-        accV[c] = fmaf(pw, gv[c], accV[c]);
-        accK[c] = fmaf(dsw, qv[c], accK[c]);
-    }
-}
-
-// Accumulates the hits first, first+stride, ... (< len) of one list; four hits are in flight at a time
-// so that the dependent loads (record -> rows) of different hits overlap.
-template <typename T, int D>
+// Accumulates the hits first, ... first + SETS - 1 (one to each of the lane's SETS sums of its part of dV, then dK) and those
+// stride, 2 * stride, ... behind them (< len) of one list; several hits are in flight at a time so that the dependent loads
+// (record -> rows) of different hits overlap: four, or the SETS of a round (four more registers' worth would cost a block
+// per SM).
+template <typename T, int D, int SETS = 1>
 __device__ __forceinline__ void accumulate_list(const int4* __restrict__ list, int first, int stride, int len,
                                                 int h, int H, int part, const T* __restrict__ Q,
-                                                const T* __restrict__ dOut, float (&accV)[Elem<T>::kVec],
-                                                float (&accK)[Elem<T>::kVec]) {
+                                                const T* __restrict__ dOut, float (&acc)[SETS][2 * Elem<T>::kVec]) {
     constexpr int VEC = Elem<T>::kVec;
-    int t = first;
-    for (; t + 3 * stride < len; t += 4 * stride) {
-        int4 rec[4];
-        float gv[4][VEC], qv[4][VEC];
+    auto add = [&](const int4& rec, const float (&gv)[VEC], const float (&qv)[VEC], float (&a)[2 * VEC]) {
+        const float pw = __int_as_float(rec.y), dsw = __int_as_float(rec.z);
 #pragma unroll
-        for (int u = 0; u < 4; ++u) rec[u] = __ldg(list + t + u * stride);
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const size_t off = ((size_t)rec[u].x * H + h) * D + part * VEC;
-            Elem<T>::load_vec(dOut + off, gv[u]);
-            Elem<T>::load_vec(Q + off, qv[u]);
+        for (int c = 0; c < VEC; ++c) {
+            a[c] = fmaf(pw, gv[c], a[c]);
+            a[VEC + c] = fmaf(dsw, qv[c], a[VEC + c]);
         }
+    };
+    int t = first;
+    if constexpr (SETS == 1) {
+        for (; t + 3 * stride < len; t += 4 * stride) {
+            int4 rec[4];
+            float gv[4][VEC], qv[4][VEC];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const float pw = __int_as_float(rec[u].y), dsw = __int_as_float(rec[u].z);
+            for (int u = 0; u < 4; ++u) rec[u] = __ldg(list + t + u * stride);
 #pragma unroll
-            for (int c = 0; c < VEC; ++c) {
-                accV[c] = fmaf(pw, gv[u][c], accV[c]);
-                accK[c] = fmaf(dsw, qv[u][c], accK[c]);
+            for (int u = 0; u < 4; ++u) {
+                const size_t off = ((size_t)rec[u].x * H + h) * D + part * VEC;
+                Elem<T>::load_vec(dOut + off, gv[u]);
+                Elem<T>::load_vec(Q + off, qv[u]);
             }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) add(rec[u], gv[u], qv[u], acc[0]);
         }
     }
-    for (; t < len; t += stride) accumulate_hit<T, D>(__ldg(list + t), h, H, part, Q, dOut, accV, accK);
+    for (; t < len; t += stride) {
+        int4 rec[SETS];
+        float gv[SETS][VEC], qv[SETS][VEC];
+#pragma unroll
+        for (int s = 0; s < SETS; ++s) rec[s] = __ldg(list + (s > 0 ? min(t + s, len - 1) : t));
+#pragma unroll
+        for (int s = 0; s < SETS; ++s) {
+            const size_t off = ((size_t)rec[s].x * H + h) * D + part * VEC;
+            Elem<T>::load_vec(dOut + off, gv[s]);
+            Elem<T>::load_vec(Q + off, qv[s]);
+        }
+#pragma unroll
+        for (int s = 0; s < SETS; ++s)
+            if (s == 0 || t + s < len) add(rec[s], gv[s], qv[s], acc[s]);
+    }
 }
 
 // One list by W lanes (`lane`: among them): the sums of its part go to dV and dK.  `len` may differ between the two halves of
-// a warp (0: nothing to read); `live`: store.
+// a warp (0: nothing to read); `live`: store.  The order of the additions is that of 32 lanes whatever W is, as in
+// gather_weighted_sum, so that a list's sums are the same bits whatever lies beside it.
 template <typename T, int D, int W>
 __device__ __forceinline__ void reduce_list(const int4* __restrict__ list, int len, int h, int H, int lane, const T* __restrict__ Q,
                                             const T* __restrict__ dOut, T* __restrict__ dK_row, T* __restrict__ dV_row, bool live) {
     constexpr int VEC = Elem<T>::kVec;
     constexpr int LPR = D / VEC;
     constexpr int EPW = W / LPR;
+    constexpr int SETS = 32 / W;
     const int part = lane % LPR, sub = lane / LPR;
-    float accV[VEC], accK[VEC];
+    float acc[SETS][2 * VEC];  // dV, then dK
 #pragma unroll
-    for (int c = 0; c < VEC; ++c) { accV[c] = 0.0f; accK[c] = 0.0f; }
-    accumulate_list<T, D>(list, sub, EPW, len, h, H, part, Q, dOut, accV, accK);
+    for (int s = 0; s < SETS; ++s)
+#pragma unroll
+        for (int c = 0; c < 2 * VEC; ++c) acc[s][c] = 0.0f;
+    accumulate_list<T, D, SETS>(list, SETS * sub, SETS * EPW, len, h, H, part, Q, dOut, acc);
+    if constexpr (SETS == 2) {
+#pragma unroll
+        for (int c = 0; c < 2 * VEC; ++c) acc[0][c] += acc[1][c];
+    }
     if constexpr (EPW == 1) {
         if (!live) return;
-        Elem<T>::store_vec(dV_row + lane * VEC, accV);
-        Elem<T>::store_vec(dK_row + lane * VEC, accK);
+        store_columns<VEC>(dV_row + lane * VEC, acc[0]);
+        store_columns<VEC>(dK_row + lane * VEC, acc[0] + VEC);
     } else {
         // both sums as one: after the first exchange a lane keeps dV or dK
         __syncwarp();
-        float both[2 * VEC];
-#pragma unroll
-        for (int c = 0; c < VEC; ++c) { both[c] = accV[c]; both[VEC + c] = accK[c]; }
         using Sums = ColumnSums<2 * VEC, LPR, W>;
-        const int col = column_sums<2 * VEC, LPR, W>(both, lane);
+        const int col = column_sums<2 * VEC, LPR, W>(acc[0], lane);
         T* const to = (col < VEC ? dV_row : dK_row) + part * VEC + col % VEC;
-        if (live && lane < Sums::kWriters) store_columns<Sums::kLeft>(to, both);
+        if (live && lane < Sums::kWriters) store_columns<Sums::kLeft>(to, acc[0]);
     }
 }
 
 // A warp takes two lists at a time, half of it each, or one after the other where one is long (a half would wait for the
 // other): kPairedHits is four rounds of a half warp's hits.  W = 32: rows wider than a half warp's vector loads.
+// Bound by the gathers' latency and by issue.  Two hits of a lane in flight and four blocks per SM: with four hits and
+// three blocks (80 registers) 100k nodes, H 4, d 32, k 16 took 338 us.  Measured (us, a list / two lists per warp, where a
+// list has k hits on average): 100k nodes, H 4, d 32, k 16 318 / 265; 30k nodes, one head, d 16, k 10 37 / 31, k 100 69 / 64; 100k nodes, one
+// head, d 16, k 45 119 / 104, fp32 k 10 66 / 58, d 128, k 16 150 / 133; 50k nodes, H 4, fp32, d 32, k 16 191 / 191; 4 x 40k
+// nodes with hub keys, H 8, d 16, k 16 596 / 516.
 template <typename T, int D, int W>
-__global__ void __launch_bounds__(kWarpsPerBlock * 32)
+__global__ void __launch_bounds__(kWarpsPerBlock * 32, W == 32 ? 0 : 4)
 bwd_segments_kernel(const T* __restrict__ Q, const T* __restrict__ dOut,
                     const int* __restrict__ seg_off, const int4* __restrict__ hits,
                     long long n_segs, int H, int k, T* __restrict__ dK, T* __restrict__ dV) {
@@ -647,10 +657,13 @@ bwd_long_segments_kernel(const T* __restrict__ Q, const T* __restrict__ dOut,
         const int h = x % H;
         if (h != hp) continue;  // block-uniform
         const int start = __ldg(seg_off + x), len = __ldg(seg_off + x + 1) - start;
+        float acc[1][2 * VEC];
+#pragma unroll
+        for (int c = 0; c < 2 * VEC; ++c) acc[0][c] = 0.0f;
+        accumulate_list<T, D>(hits + start, wid * EPW + sub, kWarpsPerBlock * EPW, len, h, H, part, Q, dOut, acc);
         float accV[VEC], accK[VEC];
 #pragma unroll
-        for (int c = 0; c < VEC; ++c) { accV[c] = 0.0f; accK[c] = 0.0f; }
-        accumulate_list<T, D>(hits + start, wid * EPW + sub, kWarpsPerBlock * EPW, len, h, H, part, Q, dOut, accV, accK);
+        for (int c = 0; c < VEC; ++c) { accV[c] = acc[0][c]; accK[c] = acc[0][VEC + c]; }
 #pragma unroll
         for (int o = LPR; o < 32; o <<= 1) {
 #pragma unroll
@@ -754,19 +767,9 @@ cudaError_t launch_d(const BwdArgs& a, const BwdWorkspace& w, cudaEvent_t* ev) {
     }
     if (ev) cudaEventRecord(ev[1], a.stream);
 
-    // Two lists per warp where they are short, or where there are many of them: of few lists, the longest decide, and a warp
-    // may meet two (us, a list / two per warp: 89 600 lists of 8 on average, d 16 36 / 32; 400 000 of 16, d 32 296 / 275; 200 000 of
-    // 20, d 64 230 / 212; 6.4 million of 16, d 16 4405 / 4037; but 100 000 of 10, fp32 d 16 69 / 89, of 45, d 16 110 / 130).
-    bool pairs = false;
-    if constexpr (half_warp_rows<T, D>()) {
-        pairs = n_rows >= 150000 || a.k <= 2 * kHalfWarp / (D / Elem<T>::kVec);
-        if (pairs)
-            bwd_segments_kernel<T, D, kHalfWarp><<<(row_blocks + 1) / 2, kWarpsPerBlock * 32, 0, a.stream>>>(
-                Q, dOut, seg_off, hits, n_rows, a.H, a.k, static_cast<T*>(a.dK), static_cast<T*>(a.dV));
-    }
-    if (!pairs)
-        bwd_segments_kernel<T, D, 32><<<row_blocks, kWarpsPerBlock * 32, 0, a.stream>>>(
-            Q, dOut, seg_off, hits, n_rows, a.H, a.k, static_cast<T*>(a.dK), static_cast<T*>(a.dV));
+    constexpr int kLanes = half_warp_rows<T, D>() ? kHalfWarp : 32;
+    bwd_segments_kernel<T, D, kLanes><<<kLanes == 32 ? row_blocks : (row_blocks + 1) / 2, kWarpsPerBlock * 32, 0, a.stream>>>(
+        Q, dOut, seg_off, hits, n_rows, a.H, a.k, static_cast<T*>(a.dK), static_cast<T*>(a.dV));
     bwd_long_segments_kernel<T, D><<<sm_count() * 8, kWarpsPerBlock * 32, 0, a.stream>>>(
         Q, dOut, seg_off, hits, long_list, sb, a.H, a.k, static_cast<T*>(a.dK), static_cast<T*>(a.dV));
     if (ev) cudaEventRecord(ev[2], a.stream);

@@ -72,3 +72,25 @@ def test_weighted_sums_run_in_one_order(H, d, k, sizes, mode):
         w = np.where(idx >= 0, weight[:, None], np.float32(0))
         out = ordered_sums(w[..., None] * v[np.maximum(idx, 0), np.arange(H)], groups)
         assert torch.equal(fb.out, torch.from_numpy(out).to("cuda", V.dtype)), route
+
+
+@pytest.mark.parametrize("H,d,k,sizes,mode", CASES)
+def test_hit_lists_are_added_in_one_order(H, d, k, sizes, mode):
+    """dV of a key: its hits in the order of the queries."""
+    Q, K, V, dO, offs, m, weight, groups = problem(H, d, k, sizes, mode)
+    N = sum(sizes)
+    fb = kb.forward(Q, K, V, offs, k, m)
+    bb = kb.backward(Q, K, V, offs, k, m, fb, dO)
+    g, idx = dO.float().cpu().numpy(), fb.topk_idx.cpu().numpy()
+    q, h, t = np.nonzero(idx >= 0)
+    seg = idx[q, h, t].astype(np.int64) * H + h
+    by = np.argsort(seg, kind="stable")
+    q, h, seg = q[by], h[by], seg[by]
+    count = np.bincount(seg, minlength=N * H)
+    assert count.max() <= 512                                               # a longer list is a block's
+    rank = np.arange(len(seg)) - np.repeat(np.cumsum(count) - count, count)
+    part = np.zeros((groups, N * H, d), dtype=np.float32)
+    for r in range(count.max()):
+        at = rank == r
+        part[r % groups, seg[at]] += weight[q[at], None] * g[q[at], h[at]]
+    assert torch.equal(bb.dV, torch.from_numpy(tree(part).reshape(N, H, d)).to("cuda", V.dtype))

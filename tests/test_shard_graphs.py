@@ -145,3 +145,33 @@ def test_shards_through_the_library_equal_the_unsharded_call():
         assert torch.equal(pb.dQ, fb.dQ[lo:hi]) and torch.equal(pb.dK, fb.dK[lo:hi]) and torch.equal(pb.dV, fb.dV[lo:hi])
         covered += hi - lo
     assert covered == w.N
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("sizes,H,d,k", [([1001, 700, 333, 1, 900, 401], 1, 16, 8),        # shards that begin at an odd list
+                                         ([1001, 700, 333, 1, 900, 401], 1, 32, 8),
+                                         ([12001, 9000, 8000, 11111], 4, 32, 16),          # 160 000 lists cut into 53 000 and less
+                                         ([75001, 40000, 40001], 1, 16, 10)])
+def test_a_shards_lists_do_not_depend_on_their_neighbours(sizes, H, d, k):
+    """A shard's hit lists have other neighbours than in the whole batch, and there are fewer of them; some are long (a few large
+    keys per graph).  Gradients stay the slices of the whole batch's, bit for bit."""
+    import torch
+    from paper_2604_03815_b200 import binding as kb
+    w = wl.iid_workload("s", 79 + len(sizes), sizes, H, d, k, wl.MODE_BF16_TC)
+    w.K[::97] = wl.round_to_bf16(w.K[::97] * 4.0)
+    Q, K, V, dO = (torch.from_numpy(getattr(w, n)).to("cuda", torch.bfloat16) for n in ("Q", "K", "V", "dOut"))
+
+    def both(lo, hi, offs):
+        args = [x[lo:hi].contiguous() for x in (Q, K, V)] + [torch.as_tensor(offs, dtype=torch.int32, device="cuda"), k, w.mode]
+        f = kb.forward(*args)
+        return f, kb.backward(*args, f, dO[lo:hi].contiguous())
+
+    full, fb = both(0, w.N, w.graph_offsets)
+    for rank in range(3):
+        lo, hi, offs, _ = kdist.shard_of(w.graph_offsets, 3, rank)
+        if hi == lo:
+            continue
+        part, pb = both(lo, hi, offs)
+        assert torch.equal(part.topk_idx + lo * (part.topk_idx >= 0), full.topk_idx[lo:hi])
+        assert torch.equal(part.topk_score, full.topk_score[lo:hi]) and torch.equal(part.out, full.out[lo:hi])
+        assert torch.equal(pb.dQ, fb.dQ[lo:hi]) and torch.equal(pb.dK, fb.dK[lo:hi]) and torch.equal(pb.dV, fb.dV[lo:hi])
