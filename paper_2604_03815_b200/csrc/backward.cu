@@ -750,10 +750,14 @@ cudaError_t launch_d(const BwdArgs& a, const BwdWorkspace& w, cudaEvent_t* ev) {
             const long long n_tab = (long long)bins_hi * n_blocks;
             const int tab_blocks = (int)((n_tab + kScanItemsPerBlock - 1) / kScanItemsPerBlock);
             const size_t smem_cnt = (size_t)bins_hi * sizeof(unsigned);
-            const size_t smem_sct = (size_t)per_block * sizeof(int4) + (size_t)rp.warps * bins_hi * 2 + (size_t)bins_hi * 2 + (size_t)bins_hi * sizeof(int);
-            const size_t smem_lo = (size_t)kBucketWarps * bins_lo * sizeof(int);
-            if ((err = cudaFuncSetAttribute(radix_scatter_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_sct)) != cudaSuccess ||
-                (err = cudaFuncSetAttribute(radix_bucket_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_lo)) != cudaSuccess)
+            auto scatter_bytes = [](int warps, int bins) {
+                return (size_t)warps * kRadixPerWarp * sizeof(int4) + (size_t)warps * bins * 2 + (size_t)bins * 2 + (size_t)bins * sizeof(int);
+            };
+            auto bucket_bytes = [](int bins) { return (size_t)kBucketWarps * bins * sizeof(int); };
+            const size_t smem_sct = scatter_bytes(rp.warps, bins_hi), smem_lo = bucket_bytes(bins_lo);
+            if ((err = cudaFuncSetAttribute(radix_scatter_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                            (int)scatter_bytes(rp.warps, kRadixMaxBins))) != cudaSuccess ||
+                (err = cudaFuncSetAttribute(radix_bucket_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bucket_bytes(kRadixMaxBins))) != cudaSuccess)
                 return err;
             RadixSrc src{a.topk_idx, ws_p, ws_ds, (int)a.N, a.H, a.k, (int)n_rows};
             radix_count_kernel<<<n_blocks, 512, smem_cnt, a.stream>>>(src, n_pairs, per_block, rp.lo_bits, bins_hi, n_blocks, table, sb);

@@ -349,6 +349,8 @@ struct BwdArgs {
 
 // Launches a kernel that begins with sweep_off, small_route or wait_for_previous: it may start while the one before it ends.
 // One that finds nothing to do then costs 1.3 us instead of 2.5.
+// The shared memory that a kernel may ask for at a launch is set before, to the most that any call asks of it: it is state of
+// the kernel, and a call in another host thread may set it between this one's setting and its launch.
 template <typename... P, typename... A>
 inline cudaError_t launch_next(const FwdArgs& a, void (*kern)(P...), dim3 grid, int threads, size_t smem, A&&... args) {
     cudaLaunchConfig_t c{};

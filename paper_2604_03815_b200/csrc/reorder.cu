@@ -267,6 +267,7 @@ __global__ void key_norm_kernel(const __nv_bfloat16* __restrict__ K, int N, int 
 // than 64 are compared on 64 evenly spaced columns.
 constexpr int kPivots = 256;
 constexpr int kPivotDims = 64;  // columns compared (evenly spaced when the vector is wider)
+constexpr int pivot_smem(int dims) { return (kPivots * (dims + 1) + kPivots) * 4; }
 constexpr int kPivotBits = 8;
 constexpr int kKeyCodeBits2 = kPivotBits + 2;
 constexpr int kAssignThreads = 256;
@@ -394,9 +395,9 @@ cudaError_t launch_reorder_queries(const FwdArgs& a, const FwdWorkspace& w) {
     if (w.prune) {
         // pruned sweep: a query's code is the key pivot it scores highest against
         const int DP = std::min(HD, kPivotDims);
-        const int smem = (kPivots * (DP + 1) + kPivots) * 4;
+        const int smem = pivot_smem(DP);
         auto kern = pivot_code_kernel<false>;
-        cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, pivot_smem(kPivotDims));
         if (err != cudaSuccess) return err;
         kern<<<w.max_items, kAssignThreads, smem, a.stream>>>(
             static_cast<const __nv_bfloat16*>(a.Q), static_cast<const __nv_bfloat16*>(a.K), HD,
@@ -437,9 +438,9 @@ cudaError_t launch_reorder_keys(const FwdArgs& a, const FwdWorkspace& w) {
     key_norm_kernel<<<(unsigned)((a.N * 32 + 255) / 256), 256, 0, a.stream>>>(K, (int)a.N, HD, a.graph_offsets, a.G, norm2,
                                                                              gmax, sb);
     const int DP = std::min(HD, kPivotDims);
-    const int smem = (kPivots * (DP + 1) + kPivots) * 4;
+    const int smem = pivot_smem(DP);
     auto kern = pivot_code_kernel<true>;
-    err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, pivot_smem(kPivotDims));
     if (err != cudaSuccess) return err;
     kern<<<w.max_items, kAssignThreads, smem, a.stream>>>(K, K, HD, reinterpret_cast<const WorkItem*>(a.ws + w.items_off), sb,
                                                           a.graph_offsets, a.G, norm2, gmax, code);

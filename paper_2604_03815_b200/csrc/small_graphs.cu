@@ -21,6 +21,7 @@ namespace kmip {
 namespace {
 
 constexpr int kWarps = 8;
+constexpr int kMaxRowsPerWarp = 8;
 constexpr int kU = 8;               // keys per lane and chunk
 constexpr int kChunk = 32 * kU;     // keys per chunk
 constexpr int kPend = kChunk + 32;  // candidates of a chunk
@@ -459,13 +460,12 @@ template <typename T, int D>
 cudaError_t launch_d(const FwdArgs& a) {
     const long long rows = a.N * a.H;
     // one wave of rows per warp where they are few, eight rows per warp (and one load of the keys) where there are many
-    const int rows_per_warp = (int)std::max<long long>(1, std::min<long long>(8, rows / ((long long)sm_count() * 4 * kWarps)));
-    const size_t smem = (size_t)kChunk * row_stride<T, D>() + ((size_t)kWarps * rows_per_warp * 32 + (size_t)kWarps * kPend) * sizeof(cand_t);
+    const int rows_per_warp = (int)std::max<long long>(1, std::min<long long>(kMaxRowsPerWarp, rows / ((long long)sm_count() * 4 * kWarps)));
+    auto bytes = [](int rows_each) { return (size_t)kChunk * row_stride<T, D>() + ((size_t)kWarps * rows_each * 32 + (size_t)kWarps * kPend) * sizeof(cand_t); };
+    const size_t smem = bytes(rows_per_warp);
     auto kern = small_forward_kernel<T, D>;
-    if (smem > 48 * 1024) {  // what a kernel may have unasked
-        cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (err != cudaSuccess) return err;
-    }
+    cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes(kMaxRowsPerWarp));
+    if (err != cudaSuccess) return err;
     const dim3 grid((unsigned)((a.N + kWarps * rows_per_warp - 1) / (kWarps * rows_per_warp)), (unsigned)std::min(a.H, 65535));
     return launch_next(a, kern, grid, kWarps * 32, smem, static_cast<const T*>(a.Q), static_cast<const T*>(a.K), static_cast<const T*>(a.V),
                                                 a.graph_offsets, a.G, (int)a.N, a.H, a.k, rows_per_warp, 1.0f / sqrtf((float)a.d), a.drop_p,
@@ -476,7 +476,7 @@ template <typename T, int D, int R, int WR>
 cudaError_t launch_one(const FwdArgs& a) {
     const size_t smem = one_graph_smem((int)a.N, D * (int)sizeof(T), R, R * WR);
     auto kern = one_graph_forward_kernel<T, D, R, WR>;
-    cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem);
     if (err != cudaSuccess) return err;
     return launch_next(a, kern, dim3((unsigned)((a.N + R - 1) / R), (unsigned)a.H), R * WR * 32, smem, static_cast<const T*>(a.Q),
                        static_cast<const T*>(a.K), static_cast<const T*>(a.V), a.graph_offsets, (int)a.N, a.H, a.k, 1.0f / sqrtf((float)a.d),
