@@ -153,9 +153,10 @@ int forward_impl(const void* Q, const void* K, const void* V, const int32_t* gra
         return KMIP_ERR_INVALID_ARG;
     const int wanted = opt ? opt->route : 0;
     const bool test_sweep = opt && (opt->fp32_path != 0 || opt->drop_first_tile != 0 || wanted > KMIP_ROUTE_SMALL);  // a test wants one of the sweeps
-    const bool one_graph = one_graph_supported(N, graph_offsets ? G : 1, H, d, k, mode);
-    const int small = wanted == KMIP_ROUTE_SMALL ? kSmallAlways : test_sweep ? kSmallNever
-                      : one_graph ? (one_graph_preferred(N, H, d) ? kSmallAlways : kSmallNever) : small_graphs_use(N, graph_offsets ? G : 1, H, d, k);
+    const bool one_graph = one_graph_supported(N, graph_offsets ? G : 1, H, d, k, mode) &&
+                           (wanted == KMIP_ROUTE_SMALL || one_graph_preferred(N, H, d, k, mode));
+    const int small = wanted == KMIP_ROUTE_SMALL || (one_graph && !test_sweep) ? kSmallAlways
+                      : test_sweep ? kSmallNever : small_graphs_use(N, graph_offsets ? G : 1, H, d, k);
     FwdWorkspace w = plan_forward(N, graph_offsets ? G : 1, H, d, k, mode, small);
     if (wanted == KMIP_ROUTE_TENSOR_CORE) w.f16 = w.in_outputs = false;
     if (wanted < 0 || wanted > KMIP_ROUTE_TENSOR_CORE || (wanted == KMIP_ROUTE_SMALL && (k > 32 || d > 64)) ||

@@ -468,7 +468,7 @@ __host__ __device__ inline bool small_graphs_preferred(double squares, long long
 cudaError_t launch_small_graphs(const FwdArgs& a);
 // ... of one graph that fits its shared memory, without a plan kernel
 bool one_graph_supported(int64_t N, int32_t G, int32_t H, int32_t d, int32_t k, int mode);
-bool one_graph_preferred(int64_t N, int32_t H, int32_t d);
+bool one_graph_preferred(int64_t N, int32_t H, int32_t d, int32_t k, int mode);
 cudaError_t launch_one_graph(const FwdArgs& a);
 // epilogue.cu: softmax over the k kept scores fused with the gather-V weighted sum
 cudaError_t launch_softmax_gather(const FwdArgs& a);

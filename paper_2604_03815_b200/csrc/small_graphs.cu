@@ -483,16 +483,23 @@ cudaError_t launch_one(const FwdArgs& a) {
                        a.drop_p, a.seed, static_cast<T*>(a.out), a.topk_idx, a.topk_score, reinterpret_cast<StatusBlock*>(a.ws));
 }
 
+// Rows of a block and warps of a row: no more warps than there are keys for (100 nodes, d 16, H 1: 4.0 us with 8, 7.0 with
+// 32); half as many rows per block where that still is one wave of blocks (512 nodes, H 4: 12.3 us in two waves, 9.6 in one).
+struct OneGraphShape { int rows, warps; };
+OneGraphShape one_graph_shape(int64_t N, int32_t H, int row_bytes) {
+    if (N <= 256) return {8, 1};
+    const bool few = ((N + 7) / 8) * H <= sm_count();
+    if (few && N <= 512) return {8, 2};
+    if (few || one_graph_smem((int)N, row_bytes, 16, 32) > kMaxSmem) return {8, 4};
+    return {16, 2};
+}
+
 template <typename T, int D>
 cudaError_t launch_shape(const FwdArgs& a, bool one_graph) {
     if (!one_graph) return launch_d<T, D>(a);
-    // no more warps than there are keys for (100 nodes, d 16, H 1: 4.0 us with 8, 7.0 with 32); half as many rows per block
-    // where that still is one wave of blocks (512 nodes, H 4: 12.3 us in two waves, 9.6 in one)
-    if (a.N <= 256) return launch_one<T, D, 8, 1>(a);
-    const bool few = ((a.N + 7) / 8) * a.H <= sm_count();
-    if (few && a.N <= 512) return launch_one<T, D, 8, 2>(a);
-    if (few || one_graph_smem((int)a.N, D * (int)sizeof(T), 16, 32) > kMaxSmem) return launch_one<T, D, 8, 4>(a);
-    return launch_one<T, D, 16, 2>(a);
+    const OneGraphShape s = one_graph_shape(a.N, a.H, D * (int)sizeof(T));
+    if (s.rows == 16) return launch_one<T, D, 16, 2>(a);
+    return s.warps == 1 ? launch_one<T, D, 8, 1>(a) : s.warps == 2 ? launch_one<T, D, 8, 2>(a) : launch_one<T, D, 8, 4>(a);
 }
 
 template <typename T>
@@ -527,12 +534,23 @@ cudaError_t launch_small_graphs(const FwdArgs& a) {
     return a.mode == KMIP_FP32_EXACT ? launch_t<float>(a, false) : launch_t<__nv_bfloat16>(a, false);
 }
 
-// Where that beats the filter: its work grows with N^2 H d, the filter's mostly with its launches and its rows.  Measured (us,
-// CUDA graph, here / filter): fp32 d 16 H 1 n 2048 17 / 47, 2700 42 / 52, 4000 69 / 56, H 4 n 1536 42 / 57, 2048 66 / 64; d 32 H 1
-// 2048 26 / 53, 2700 63 / 63, H 4 1536 61 / 72, 2048 97 / 85; d 64 H 1 2048 39 / 76, 2700 95 / 84, H 4 1024 49 / 84, 2048
-// 151 / 138; bf16 d 16 H 1 2700 38 / 51, 4000 60 / 55, d 32 H 4 1536 50 / 57, 2048 78 / 65.
-bool one_graph_preferred(int64_t N, int32_t H, int32_t d) {
-    return (double)N * N * H * (d + 32) <= 4.2e8 + 3.0e4 * (double)N * H;
+// Where that beats what the call takes without it, the kernel for batches or the filter.  Its work grows with N^2 H d, the
+// filter's mostly with its launches and its rows, and its blocks of up to 32 warps want to come in one wave: from the second
+// on a warp per row fills the chip as well, without a block's barriers, unless key rows of 128 bytes and more are dear to
+// read a row at a time.  With k > 24 most of its time is selection; fp32 has no filter below k = 4.  Measured (us, CUDA graph,
+// here / batch kernel / filter), up to one wave: fp32 d 16 H 1 n 2048 17 / 36 / 47, d 32 H 1 1184 16 / 26 / 48; 1.2 to 5 waves:
+// bf16 d 16 H 8 n 351 k 16 17 / 14 / 38, 702 31 / 28 / 44, k 32 51 / 38 / 56, H 4 n 1368 k 4 35 / 45 / 40, k 32 65 / 59 / 58; fp32
+// d 32 H 32 n 360 k 16 52 / 60 / 83; d 64 H 1 n 2048 39 / 83 / 76; more: bf16 d 16 H 16 n 1104 k 16 94 / 112 / 67, H 64 n 398 k 16
+// 91 / 69 / 85, d 32 H 64 n 624 k 4 165 / 154 / 92; fp32 d 64 H 32 n 360 k 24 81 / 98 / 175.  Of 3980 sizes, modes and k inside the
+// first line, 96 % are within 5 % of the better side, the worst 1.4 times it; with that line alone 85 %, and twice.
+bool one_graph_preferred(int64_t N, int32_t H, int32_t d, int32_t k, int mode) {
+    if ((double)N * N * H * (d + 32) > 4.2e8 + 3.0e4 * (double)N * H) return false;
+    const bool fp32 = mode == KMIP_FP32_EXACT;
+    if (N <= 256 || (d == 64 && (fp32 || k >= 8))) return true;
+    const int row_bytes = d * (fp32 ? 4 : 2);
+    const int waves = k > 24 ? (N > 1000 ? 2 : 1) : row_bytes >= 128 || (fp32 && k < 4 && N > 440) ? 6 : N > 440 ? 4 : 1;
+    const OneGraphShape s = one_graph_shape(N, H, row_bytes);
+    return (N + s.rows - 1) / s.rows * H <= (int64_t)waves * sm_count();  // more than 256 nodes: a block per SM
 }
 
 bool one_graph_supported(int64_t N, int32_t G, int32_t H, int32_t d, int32_t k, int mode) {
