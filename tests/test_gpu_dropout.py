@@ -49,6 +49,19 @@ def test_dropout_matches_the_oracle(mode, d, k, drop):
         assert np.all(err <= pu.OUT_ATOL + pu.OUT_RTOL * np.abs(ref)), f"{name} off by {err.max():.3e}"
 
 
+@pytest.mark.parametrize("n,H,d,k,mode", [(700, 1, 32, 16, wl.MODE_BF16_TC), (700, 2, 16, 17, wl.MODE_BF16_TC), (300, 1, 64, 15, wl.MODE_FP32_EXACT),
+                                          (300, 1, 64, 32, wl.MODE_FP32_EXACT)])
+def test_dropout_in_the_one_graph_kernel(n, H, d, k, mode):
+    w = wl.iid_workload("s", 4200 + k, [n], H, d, k, mode, input_scale=1.0 / np.sqrt(d), backward=False)
+    Q, K, V, dO, offs = pu.to_device(w)
+    fb = kb.ForwardBuffers(n, 1, H, d, k, mode)
+    assert kb.kmip_attn_forward_dropout(Q, K, V, offs, k, mode, 0.5, 77, fb.out, fb.topk_idx, fb.topk_score, fb.workspace) == kb.KMIP_OK
+    assert kb.kmip_last_status(fb.workspace) == kb.KMIP_OK and kb.kmip_test_route(fb.workspace) == kb.ROUTE_SMALL
+    ref, _ = oracle.forward_given_idx(w.Q, w.K, w.V, fb.topk_idx.cpu().numpy(), drop=0.5, seed=77)
+    out = fb.out.float().cpu().numpy().astype(np.float64)
+    assert np.all(np.abs(out - ref) <= pu.OUT_ATOL + pu.OUT_RTOL * np.abs(ref))
+
+
 def test_dropout_argument_checks():
     w = wl.iid_workload("s", 4100, [64], 1, 16, 4, wl.MODE_BF16_TC)
     Q, K, V, dO, offs = pu.to_device(w)

@@ -102,8 +102,8 @@ def test_ragged_batch_with_tiny_and_empty_graphs(mode, route):
 
 @pytest.mark.parametrize("route", [FILTER, TENSOR_CORE])
 def test_item_and_ring_boundaries(route):
-    """Graphs around the 512-row and 384-row work-item sizes of the sweeps: one to four active query
-    tiles, a short last key tile, and enough key tiles per item for the accumulator buffers and their
+    """Graphs around the work-item sizes of the sweeps (128, 256 and 384 rows): one to three active query
+    tiles, several items, a short last key tile, and enough key tiles per item for the accumulator buffers and their
     barrier phases to wrap several times."""
     sizes = [383, 384, 385, 511, 512, 513, 769, 1025, 1153, 2000, 127, 128, 129]
     for d, k in ((32, 32), (16, 16)):
@@ -384,8 +384,8 @@ def test_one_graph_with_bad_offsets_is_reported():
                                           (77, 1, 128, 16, "fp32"), (301, 1, 16, 17, "bf16"), (301, 1, 32, 64, "bf16"), (301, 1, 32, 65, "bf16"),
                                           (603, 1, 16, 7, "bf16")])
 def test_rows_and_lists_by_half_warps(n, H, d, k, mode):
-    """Softmax, weighted sum and backward pass with two rows or two hit lists per warp: odd numbers of rows, k on both sides of half a
-    warp, rows too wide for it; three keys that every query takes give lists that half a warp does not take (301 hits) and, at 603
+    """Softmax, weighted sum and backward pass with two rows (k <= 16) and two hit lists per warp: odd numbers of rows, k on both sides
+    of half a warp, rows too wide for it; three keys that every query takes give lists that half a warp does not take (301 hits) and, at 603
     nodes, that a block reduces."""
     m = {"bf16": wl.MODE_BF16_TC, "fp32": wl.MODE_FP32_EXACT}[mode]
     w = wl.iid_workload("s", 6700 + n + k, [n], H, d, k, m, backward=True)
