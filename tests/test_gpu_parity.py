@@ -353,10 +353,10 @@ def test_one_graph_in_one_kernel(n, H, d, k, mode):
 
 
 @pytest.mark.parametrize("n,H,d,k,mode,route", [
-    (1024, 1, 32, 16, "fp32", kb.ROUTE_SMALL), (2048, 1, 64, 16, "fp32", kb.ROUTE_SMALL), (200, 64, 16, 32, "bf16", kb.ROUTE_SMALL),
-    (351, 8, 16, 16, "bf16", kb.ROUTE_SMALL), (430, 32, 16, 32, "fp32", kb.ROUTE_SMALL), (398, 64, 16, 7, "bf16", kb.ROUTE_SMALL),   # a warp per row
-    (1104, 16, 16, 16, "bf16", kb.ROUTE_FILTER), (788, 64, 16, 24, "fp32", kb.ROUTE_FILTER), (1389, 8, 16, 32, "bf16", kb.ROUTE_FILTER),
-    (2400, 1, 16, 8, "bf16", kb.ROUTE_SMALL), (2700, 1, 16, 17, "fp32", kb.ROUTE_SMALL)])                   # 16 rows of scores no longer fit a block
+    (1024, 1, 32, 16, "fp32", SMALL), (2048, 1, 64, 16, "fp32", SMALL), (200, 64, 16, 32, "bf16", SMALL),
+    (351, 8, 16, 16, "bf16", SMALL), (430, 32, 16, 32, "fp32", SMALL), (398, 64, 16, 7, "bf16", SMALL),   # a warp per row
+    (1104, 16, 16, 16, "bf16", FILTER), (788, 64, 16, 24, "fp32", FILTER), (1389, 8, 16, 32, "bf16", FILTER),
+    (2400, 1, 16, 8, "bf16", SMALL), (2700, 1, 16, 17, "fp32", SMALL)])                   # 16 rows of scores no longer fit a block
 def test_a_lone_graph_with_many_heads_does_not_queue_for_whole_blocks(n, H, d, k, mode, route):
     """Where the one-graph kernel's blocks come in many waves, or selection is most of their work, a warp per row or the filter
     takes the call (H 64, 788 nodes, d 16, k 32: 375 us in the one-graph kernel, 214 in the filter)."""
@@ -367,7 +367,7 @@ def test_a_lone_graph_with_many_heads_does_not_queue_for_whole_blocks(n, H, d, k
     assert kb.kmip_test_route(a.workspace) == route
     pu.check_forward(w, a)
     b = kb.forward(Q.float(), K.float(), V.float(), offs, k, kb.KMIP_FP32_EXACT, fp32_path=1)
-    assert torch.equal(a.topk_score, b.topk_score) and (route != kb.ROUTE_SMALL or torch.equal(a.topk_idx, b.topk_idx))
+    assert torch.equal(a.topk_score, b.topk_score) and (route != SMALL or torch.equal(a.topk_idx, b.topk_idx))
 
 
 def test_one_graph_with_bad_offsets_is_reported():
