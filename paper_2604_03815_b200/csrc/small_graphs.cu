@@ -537,18 +537,22 @@ cudaError_t launch_small_graphs(const FwdArgs& a) {
 // Where that beats what the call takes without it, the kernel for batches or the filter.  Its work grows with N^2 H d, the
 // filter's mostly with its launches and its rows, and its blocks of up to 32 warps want to come in one wave: from the second
 // on a warp per row fills the chip as well, without a block's barriers, unless key rows of 128 bytes and more are dear to
-// read a row at a time.  With k > 24 most of its time is selection; fp32 has no filter below k = 4.  Measured (us, CUDA graph,
+// read a row at a time.  From k = 30 on most of its time is selection (each warp keeps more candidates); fp32 has no filter below k = 4.  Measured (us, CUDA graph,
 // here / batch kernel / filter), up to one wave: fp32 d 16 H 1 n 2048 17 / 36 / 47, d 32 H 1 1184 16 / 26 / 48; 1.2 to 5 waves:
 // bf16 d 16 H 8 n 351 k 16 17 / 14 / 38, 702 31 / 28 / 44, k 32 51 / 38 / 56, H 4 n 1368 k 4 35 / 45 / 40, k 32 65 / 59 / 58; fp32
 // d 32 H 32 n 360 k 16 52 / 60 / 83; d 64 H 1 n 2048 39 / 83 / 76; more: bf16 d 16 H 16 n 1104 k 16 94 / 112 / 67, H 64 n 398 k 16
-// 91 / 69 / 85, d 32 H 64 n 624 k 4 165 / 154 / 92; fp32 d 64 H 32 n 360 k 24 81 / 98 / 175.  Of 3980 sizes, modes and k inside the
-// first line, 96 % are within 5 % of the better side, the worst 1.4 times it; with that line alone 85 %, and twice.
+// 91 / 69 / 85, d 32 H 64 n 624 k 4 165 / 154 / 92; fp32 d 64 H 32 n 360 k 24 81 / 98 / 175.  Geometric means of here /
+// the better of the others, d 16 and 32, k 24 / 28 / 30 / 32: rows below 128 bytes, n > 1000, two waves 0.77 0.80 0.85 0.97,
+// four 0.97 1.00 1.06 1.21; 512 nodes, two to four waves, k <= 28 1.06, 620 nodes 0.97; wider rows, three waves 0.81 0.83 0.86
+// 0.95.  Of 2808 such sizes and k inside the first line, 95 % are within 5 % of the better side, the worst 1.3 times it; with
+// that line alone 81 %, and with H up to 64 twice.
 bool one_graph_preferred(int64_t N, int32_t H, int32_t d, int32_t k, int mode) {
     if ((double)N * N * H * (d + 32) > 4.2e8 + 3.0e4 * (double)N * H) return false;
     const bool fp32 = mode == KMIP_FP32_EXACT;
     if (N <= 256 || (d == 64 && (fp32 || k >= 8))) return true;
     const int row_bytes = d * (fp32 ? 4 : 2);
-    const int waves = k > 24 ? (N > 1000 ? 2 : 1) : row_bytes >= 128 || (fp32 && k < 4 && N > 440) ? 6 : N > 440 ? 4 : 1;
+    const bool wide = row_bytes >= 128;
+    const int waves = k >= 30 ? (wide ? 3 : N > 1000 ? 2 : 1) : wide || (fp32 && k < 4 && N > 440) ? 6 : N > 600 ? 4 : 1;
     const OneGraphShape s = one_graph_shape(N, H, row_bytes);
     return (N + s.rows - 1) / s.rows * H <= (int64_t)waves * sm_count();  // more than 256 nodes: a block per SM
 }
