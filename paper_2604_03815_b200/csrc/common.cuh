@@ -54,7 +54,7 @@ struct StatusBlock {
     unsigned long long counters[4];
     int n_redo;      // forward, fp16 prefilter: rows the rescoring kernel sent to the exact kernel
     int redo_done[kRedoSplitMax];  // parts finished of each of the first redo rows (score_select_exact.cu)
-    int route;       // forward: Route, written by the plan kernel
+    int route;       // forward: Route, written by the plan kernel (a lone small graph: by its own kernel)
     int reserved[50 - kRedoSplitMax];
 };
 static_assert(sizeof(StatusBlock) == kStatusBytes, "status block size");
@@ -253,8 +253,8 @@ __device__ __forceinline__ bool kmip_check(bool cond, StatusBlock* sb, int code)
 // First thing in the kernels of the sweeps' routes: true if the plan kernel gave the batch to the small-graph kernel, or if
 // the call failed before.  The wait is for launches that overlap the end of the kernel before them (launch_next).
 // The tensor-core sweeps may record a problem while blocks of theirs still start, so they don't ask for the second: they find
-// no work items when the plan failed.  The half-precision one asks for neither - its loop is sensitive to what the compiler
-// makes of a line up here (100k nodes, d 16, k 16: 924 us without, 960 with) - and finds no work items in both cases.
+// no work items when the plan failed.  The half-precision one asks for neither and finds no work items in both cases; the wait
+// at its head would make no difference (100k nodes, H 1, d 16, k 16 774 us without and with it, H 4, d 32, k 16 3047 and 3052).
 __device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ bool small_route(const StatusBlock* sb) {
     wait_for_previous();

@@ -37,12 +37,14 @@
 // predicate and advances with one: a predicated store costs a warp 12 clocks, a plain one 5 (both sides of a tile's 16
 // stores, one warp: 201 and 86 clocks).
 //
-// Measured (us; before: four query tiles from shared memory, three issuers that were one warp short, predicated appends, the
-// ragged last tile masked inside the loop): 100k nodes, H 4, d 32, k 16 3425 -> 3060, k 30 4180 -> 3400; H 1, d 16, k 10
-// 911 -> 762, k 45 1041 -> 884; 50k nodes, H 4, d 64, k 20 1327 -> 1046; point clouds, H 4, d 32, k 32, 200k nodes
-// 12 130 -> 9400, 500k nodes 64 600 -> 53 000.  A round (one key tile, three query tiles, d 32) takes 546 clocks with thresholds
+// Measured (us, events around the launch; before: four query tiles from shared memory, three issuers that were one warp short,
+// predicated appends, the ragged last tile masked inside the loop): 100k nodes, H 4, d 32, k 16 3450 -> 3050, k 30
+// 4220 -> 3390; H 1, d 16, k 10 915 -> 770, k 45 1051 -> 898; 50k nodes, H 4, d 64, k 20 1348 -> 1061; point clouds, H 4, d 32,
+// k 32, 200k nodes 12 180 -> 9300, 500k nodes 65 500 -> 53 000.  Where items of 512 rows just filled one wave and those of 384 do
+// not, the whole forward pass is up to 6 % slower: 31 623 nodes, H 2, d 16, k 8 333 -> 351, 15 000, H 4, d 32 251 -> 265.  A round (one key tile, three query tiles, d 32) takes 546 clocks with thresholds
 // that nothing beats, 384 of them MMA, and 920 where every tile has hits: three chains of load, maxima, append a
-// scheduler, which fill 61 % of its issue slots.  What did not pay there (100k nodes, H 4, d 32, k 16, us, against 3060):
+// scheduler, which fill 61 % of its issue slots.  What did not pay there (100k nodes, H 4, d 32, k 16, us, against 3060 in the
+// same runs):
 // four query tiles of 112 keys in 96 registers 3360, two tiles with two buffers each 4140, five of 80 keys 3760, six of 64
 // keys 4010, the hits of a half tile kept aside and appended in batches 3670, one vote per half tile 3200, two key tiles per
 // vote 3650, six key stages 3080.
@@ -156,7 +158,7 @@ struct SelectTargets {
 // steps that interpolate (the entries above a threshold thin out exponentially), then bisection over the ordered 16-bit
 // values.  Where many entries tie and no threshold leaves a number in range, the smallest tied ones past `hi` are
 // dropped too.  `seg` >= 0: also keeps the high bytes at `hi_bytes` (the first n_old entries have one).
-// About 900 instructions a warp at CAP = 80.
+// Its instructions grow with CAP: a load, two extrema and up to 19 counts for every two entries.
 // Out of line: the loop that calls it rarely keeps its registers.
 template <int CAP>
 __device__ __noinline__ RowSel16 select_rows(RowSel16 r, uint32_t base, SelectTargets t, bool raise, unsigned char* hi_bytes, int seg) {

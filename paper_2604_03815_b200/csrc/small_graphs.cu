@@ -76,6 +76,20 @@ template <int D> struct RowDot<float, D> {
     }
 };
 
+// `best` (sorted, a lane per entry, at most k) and up to 32 more candidates, unsorted: the best k of both.
+__device__ __forceinline__ cand_t merge_sorted(cand_t best, cand_t more, int k, int lane) {
+    cand_t v[1] = {more};
+    warp_sort_desc<1>(v, lane);
+    const cand_t rev = __shfl_sync(FULL, v[0], 31 - lane);
+    cand_t m = cmax(lane < k ? best : 0ull, rev);
+#pragma unroll
+    for (int j = 16; j > 0; j >>= 1) {
+        const cand_t o = __shfl_xor_sync(FULL, m, j);
+        m = ((lane & j) == 0) ? cmax(m, o) : cmin(m, o);
+    }
+    return m;
+}
+
 // The end of a row: softmax over the kept scores (`best`: sorted, one entry per lane, 0 = none) and the weighted sum of their
 // V rows.
 template <typename T, int D>
@@ -209,18 +223,7 @@ small_forward_kernel(const T* __restrict__ Q, const T* __restrict__ K, const T* 
                         __syncwarp();
                         best = lane < cnt ? pend[lane] : 0ull;
                     } else {
-                        for (int p0 = 0; p0 < cnt; p0 += 32) {
-                            cand_t v[1] = {p0 + lane < cnt ? pend[p0 + lane] : 0ull};
-                            warp_sort_desc<1>(v, lane);
-                            const cand_t rev = __shfl_sync(FULL, v[0], 31 - lane);
-                            cand_t m = cmax(lane < k ? best : 0ull, rev);
-#pragma unroll
-                            for (int j = 16; j > 0; j >>= 1) {
-                                const cand_t o = __shfl_xor_sync(FULL, m, j);
-                                m = ((lane & j) == 0) ? cmax(m, o) : cmin(m, o);
-                            }
-                            best = m;
-                        }
+                        for (int p0 = 0; p0 < cnt; p0 += 32) best = merge_sorted(best, p0 + lane < cnt ? pend[p0 + lane] : 0ull, k, lane);
                     }
                     if (lane >= k) best = 0ull;
                     if (!last_chunk) {
@@ -265,20 +268,6 @@ __device__ __forceinline__ int lane_rank(uint32_t mine, int lane) {
         place += o > mine || (o == mine && j < lane) ? 1 : 0;
     }
     return place;
-}
-
-// `best` (sorted, a lane per entry, at most k) and up to 32 more candidates, unsorted: the best k of both.
-__device__ __forceinline__ cand_t merge_sorted(cand_t best, cand_t more, int k, int lane) {
-    cand_t v[1] = {more};
-    warp_sort_desc<1>(v, lane);
-    const cand_t rev = __shfl_sync(FULL, v[0], 31 - lane);
-    cand_t m = cmax(lane < k ? best : 0ull, rev);
-#pragma unroll
-    for (int j = 16; j > 0; j >>= 1) {
-        const cand_t o = __shfl_xor_sync(FULL, m, j);
-        m = ((lane & j) == 0) ? cmax(m, o) : cmin(m, o);
-    }
-    return m;
 }
 
 // A part of a key row (at most 64 bytes) in a lane's registers, and the chain of multiply-adds of a query row against it (index
