@@ -29,7 +29,7 @@ METRIC = "k-MIP fwd+bwd query-key scores/sec at N=500k"
 UNIT = "scores/s"
 FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustained": 1400.0}
 # kernels of a forward call by the route the library reports (kmip_test_route)
-FWD_LAUNCHES = {1: 2,       # plan, the whole forward pass of small graphs; without the plan for a single graph
+FWD_LAUNCHES = {1: 2,       # plan, the whole forward pass of small graphs; one kernel for a lone graph like configuration 1's
                 2: 7,       # plan, norm maxima, operand conversion, prefilter sweep, rescoring, exact pass, softmax+gather-V
                 3: 5,       # plan, keys by head, score+select sweep, rescoring, softmax+gather-V
                 4: 4,       # plan, sweep, rescoring, softmax+gather-V
